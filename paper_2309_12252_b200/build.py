@@ -4,14 +4,16 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import tempfile
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdeer_b200.so")
-SOURCES = ["deer_api.cu"]
+# (source, extra flags); the one-launch Newton kernels are compiled per padded state size
+SOURCES = [("deer_api.cu", []), ("newton_body.cu", [])] + [("newton_kernels.cu", [f"-DBODY_N={n}"]) for n in range(8, 65, 8)]
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
-    "-Xcompiler", "-fPIC", "-shared",
+    "-Xcompiler", "-fPIC",
 ]
 
 
@@ -27,9 +29,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     stale = (not os.path.exists(LIB)) or any(os.path.getmtime(s) > os.path.getmtime(LIB) for s in _sources())
     if force or stale:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + \
-              ["-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES]
-        subprocess.run(cmd, check=True)
+        with tempfile.TemporaryDirectory() as tmp:           # one nvcc per source, side by side, then the link
+            objs = [os.path.join(tmp, f"{k}.o") for k in range(len(SOURCES))]
+            runs = [subprocess.Popen([nvcc] + NVCC_FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) +
+                                     ["-c", os.path.join(CSRC, f), "-o", o]) for (f, extra), o in zip(SOURCES, objs)]
+            failed = [f for f, r in zip(SOURCES, runs) if r.wait() != 0]
+            if failed:
+                raise RuntimeError(f"nvcc failed on {failed}")
+            subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs, check=True)
     return LIB
 
 

@@ -75,6 +75,14 @@ static inline cudaError_t launch_pdl(bool overlap, void (*kern)(KArgs...), unsig
         }                                                          \
     } while (0)
 
+// What an evaluation reports, written by the kernel that takes the loop decision straight into page-locked host memory.
+struct HostResult {
+    int iters, done, burn;
+    unsigned err_bits;
+    float trace[28];     // err after the first bodies
+};
+constexpr int HOST_TRACE = 28;
+
 // Device-resident status of one evaluation (first 256 bytes of the workspace).
 struct StatusBlock {
     unsigned err_bits;   // max |y_new - y| of the running body, as the bits of a non-negative float
@@ -89,9 +97,11 @@ struct StatusBlock {
     int ctl_mode;        // 1: the last CTA of a single-pass scan takes the Newton loop decision
     int max_iter;
     float tol;
-    unsigned pad0;
+    int burn;            // one-launch bodies: burn-in of their chains, raised when it proves too short
     float *trace;        // err after each body (first ERR_TRACE_CAP bodies), or nullptr
-    unsigned pad[50];
+    unsigned mis_bits;   // one-launch bodies: largest mismatch between a chain's end and the start its successor assumed
+    HostResult *host;    // page-locked host memory, or nullptr
+    unsigned pad[46];
 };
 static_assert(sizeof(StatusBlock) == 256, "status block is one 256-byte line");
 constexpr int ERR_TRACE_CAP = 1024;
@@ -163,6 +173,11 @@ __device__ __forceinline__ bool loop_ended(const StatusBlock *st)
 // End of one Newton body (App. B.1 loop): record err, count the body, decide whether the loop goes on
 // (err > tol and fewer than max_iter bodies).  A NaN err fails "err > tol" and ends the loop, as in
 // the listing; an infinite err ends it too.  Single thread.
+__device__ __forceinline__ bool newton_loop_ends(float e, float tol, int k, int max_iter)
+{
+    return !(e > tol) || !(e <= 3.402823466e38f) || k + 1 >= max_iter;
+}
+
 __device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int max_iter, float *trace)
 {
     const unsigned bits = *(volatile unsigned *)&st->err_bits;
@@ -172,7 +187,12 @@ __device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int ma
     st->iters = k + 1;
     st->err_last_bits = bits;
     st->err_bits = 0u;
-    if (!(e > tol) || !(e <= 3.402823466e38f) || k + 1 >= max_iter) st->done = 1;
+    const int end = newton_loop_ends(e, tol, k, max_iter);
+    if (end) st->done = 1;
+    if (HostResult *h = st->host) {
+        if (k < HOST_TRACE) h->trace[k] = e;
+        h->iters = k + 1; h->err_bits = bits; h->burn = st->burn; h->done = end;
+    }
 }
 
 // Called by one thread of every CTA of a single-pass scan after the CTA's last global write.  The

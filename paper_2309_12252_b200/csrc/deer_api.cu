@@ -24,6 +24,7 @@
 #include "scan_fused_fwd64.cuh"
 #include "cell_wide.cuh"
 #include "vjp_wide.cuh"
+#include "newton_body.h"
 
 namespace deer {
 
@@ -645,9 +646,15 @@ struct EvalWs {
     float *trace;        // [ERR_TRACE_CAP] err after each body (device side of err_trace)
     unsigned long long *diag;   // [B] per-sequence {err bits, inverted index} of the last body
     float *u, *J, *rhs, *yalt;
+    float *edge;         // one-launch bodies: states at the boundaries between warps
+    unsigned *edge_flag;
+    unsigned long long *words;   // whole-loop launches: exchanged maxima (at most one CTA per SM)
     ScanWs scan;
     size_t bytes;
 };
+
+// chain groups of a one-launch body at the shortest chain length
+static size_t body_groups_max(int B, int T) { return ((size_t)B * ((T + BODY_L_MIN - 1) / BODY_L_MIN) + 15) / 16; }
 
 static EvalWs carve_eval(void *ws, int B, int T, int n, int m)
 {
@@ -662,6 +669,9 @@ static EvalWs carve_eval(void *ws, int B, int T, int n, int m)
     w.J = cv.take<float>(N * n * n);
     w.rhs = cv.take<float>(N * n);
     w.yalt = cv.take<float>(N * n);
+    w.edge = cv.take<float>(body_groups_max(B, T) * 2 * n);
+    w.edge_flag = cv.take<unsigned>(body_groups_max(B, T));
+    w.words = cv.take<unsigned long long>((size_t)4 * num_sms());
     w.scan = carve_scan(cv, B, T, n);
     w.bytes = cv.off;
     return w;
@@ -886,6 +896,114 @@ static int linrec_scan_impl(const float *J, const float *b, const float *y0, int
     return run_scan(a, w.scan, flags, st);
 }
 
+// A page-locked record for the result of one evaluation, from a fixed set that is made on first use (8 KB per process).
+// An evaluation that finds none free, or no page-locked memory, reads its status with a copy instead.
+class HostSlot {
+    static constexpr int COUNT = 64;
+    static HostResult *base()
+    {
+        static HostResult *b = []() -> HostResult * {
+            void *v = nullptr;
+            if (cudaHostAlloc(&v, COUNT * sizeof(HostResult), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+            return (HostResult *)v;
+        }();
+        return b;
+    }
+    static std::atomic<unsigned long long> &taken() { static std::atomic<unsigned long long> t{0}; return t; }
+    int idx = -1;
+
+public:
+    HostResult *p = nullptr;
+    explicit HostSlot(bool want)
+    {
+        if (!want || !base()) return;
+        for (unsigned long long t = taken().load(); ~t != 0ull;) {
+            const int i = __builtin_ctzll(~t);
+            if (taken().compare_exchange_weak(t, t | (1ull << i))) { idx = i; p = base() + i; return; }
+        }
+    }
+    ~HostSlot() { if (idx >= 0) taken().fetch_and(~(1ull << idx)); }
+    HostSlot(const HostSlot &) = delete;
+    HostSlot &operator=(const HostSlot &) = delete;
+};
+
+// ---- evaluations whose bodies are one launch each (newton_body.cuh)
+// The flags that ask for a particular form of the scan are served by the kernels that have that form.
+static bool body_takes(int n, int m, int flags)
+{
+    return !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
+           (body_supported(n, m, false) || body_supported(n, m, true));
+}
+
+// Runs the Newton loop until it ends or the form gives up (hs->done == BODY_FALL_BACK, the iterate after hs->iters bodies in
+// buf[hs->iters & 1]).
+template <typename CopyOut>
+static int eval_one_launch(const deer_gru_params *p, const float *x, const float *y0, int B, int T, float tol, int max_iter,
+                           const EvalWs &w, float *const (&buf)[2], int flags, cudaStream_t st, StatusBlock *hs, HostResult *hr,
+                           CopyOut copy_out)
+{
+    const int n = p->n, m = p->m;
+    const bool have_u = !body_supported(n, m, false);
+    bool u_done = false;
+    int rc, burn = body_first_burn(n, tol);
+    BodyArgs a{};
+    a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0};
+    a.x = x; a.u = have_u ? w.u : nullptr; a.y0 = y0;
+    a.buf[0] = buf[0]; a.buf[1] = buf[1];
+    a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1;
+    a.eta = body_eta(n, tol);
+    a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
+    for (int form = 0; form < 2; ++form) {               // the two-phase kernel, then the one-phase kernel
+        BodyPlan plan{};
+        if (!body_plan(&plan, form == 0, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;
+        if (burn > plan.burn_cap) { hs->done = BODY_FALL_BACK; continue; }
+        a.L = plan.L;
+        a.burn_cap = plan.burn_cap;
+        a.warm = ((flags & DEER_FLAG_WARM_START) || hs->iters > 0) ? 1 : 0;
+        StatusBlock init;
+        memset(&init, 0, sizeof(init));
+        init.max_iter = max_iter;
+        init.tol = tol;
+        init.trace = w.trace;
+        init.burn = burn;
+        init.iters = hs->iters;
+        init.host = hr;
+        if (hr) { hr->iters = hs->iters; hr->done = 0; }
+        EvalBeginArgs e{};
+        if (plan.whole_loop) {
+            e.starts = (unsigned long long *)w.edge; e.nstarts = (size_t)plan.edges * n;
+            e.agg_words = w.words; e.nagg_words = (size_t)4 * plan.max_ctas;
+        } else {
+            e.flags = w.edge_flag; e.nflags = (size_t)plan.edges;
+        }
+        const unsigned blocks = (unsigned)((e.nflags + e.nstarts + 1023) / 1024);
+        DEER_KERNEL("eval_begin_kernel", st, eval_begin_kernel<<<blocks < 1u ? 1u : blocks, 256, 0, st>>>(w.st, init, e));
+        if (have_u && !u_done) {
+            if ((rc = run_proj(p, x, w.u, (size_t)B * T, st)) != DEER_OK) return rc;
+            u_done = true;
+        }
+        for (int group = 4;; group = 2) {
+            const int left = max_iter - hs->iters;
+            for (int j = 0; j < (plan.whole_loop ? 1 : left < group ? left : group); ++j)
+                if ((rc = launch_newton_body(a, plan, st)) != DEER_OK) return rc;
+            if ((rc = copy_out()) != DEER_OK) return rc;
+            if (hr) {
+                DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+                hs->iters = hr->iters; hs->done = hr->done; hs->burn = hr->burn; hs->err_last_bits = hr->err_bits;
+                if (plan.whole_loop && !hs->done) return DEER_ERR_DEVICE_TIMEOUT;
+            } else {
+                DEER_CHECK_CUDA(cudaMemcpyAsync(hs, w.st, 48, cudaMemcpyDeviceToHost, st), "read status");
+                DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+                if (hs->flags & FLAG_TIMEOUT) return DEER_ERR_DEVICE_TIMEOUT;
+            }
+            if (hs->done) break;
+        }
+        if (hs->done == BODY_DONE) return DEER_OK;
+        burn = hs->burn;
+    }
+    return DEER_OK;                                      // (hs->done == BODY_FALL_BACK)
+}
+
 // copy_st / copy_ev (optional): the stream the copy to y_host is enqueued on, and an event to order it behind `st`.
 // y_host (optional, host memory): the result is also copied there.  The copy is enqueued behind every
 // group of bodies, after a device-side selection of the buffer that holds the current iterate, so that
@@ -901,6 +1019,35 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     int rc = check_ws(ws, ws_bytes, w.bytes);
     if (rc != DEER_OK) return rc;
     const size_t N = (size_t)B * T;
+    float *buf[2] = {y, w.yalt};
+    StatusBlock hs;
+    memset(&hs, 0, sizeof(hs));
+    // enqueued behind every group of bodies when the result goes to host memory
+    auto copy_out = [&]() -> int {
+        if (!y_host) return DEER_OK;
+        size_t words = N * n / 4;
+        unsigned blocks = (unsigned)((words + 1023) / 1024);
+        const unsigned cap = 4u * (unsigned)num_sms();
+        if (blocks > cap) blocks = cap;
+        if (blocks < 1u) blocks = 1u;
+        DEER_KERNEL("result_select_kernel", st, result_select_kernel<<<blocks, 256, 0, st>>>(w.st, y, w.yalt, N * n));
+        if (copy_st) {      // the result leaves on a stream of its own, behind the selection
+            DEER_CHECK_CUDA(cudaEventRecord(copy_ev, st), "record result event");
+            DEER_CHECK_CUDA(cudaStreamWaitEvent(copy_st, copy_ev, 0), "wait result event");
+        }
+        DEER_CHECK_CUDA(cudaMemcpyAsync(y_host, y, N * n * sizeof(float), cudaMemcpyDeviceToHost, copy_st ? copy_st : st),
+                        "copy result to host");
+        return DEER_OK;
+    };
+    const bool one_launch = body_takes(n, m, flags);
+    HostSlot slot(one_launch);
+    if (one_launch) {
+        if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, copy_out)) != DEER_OK) return rc;
+    }
+    if (!one_launch || hs.done != BODY_DONE) {
+    const int k0 = hs.iters;                   // bodies that the one-launch form has done
+    if (k0 > 0) flags |= DEER_FLAG_WARM_START;
+    hs.done = 0;
     const bool fused_proj = cell_projects(n, m) && ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
 
     ScanArgs a{};
@@ -927,6 +1074,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
         init.max_iter = max_iter;
         init.tol = tol;
         init.trace = w.trace;
+        init.iters = k0;
         // one launch: status block, zero initial guess, cleared words of the single-pass scan
         EvalBeginArgs e{};
         if (!(flags & DEER_FLAG_WARM_START)) { e.y = y; e.ny = N * n; }
@@ -950,9 +1098,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     // Newton loop (App. B.1): bodies are enqueued ahead of the convergence test -- the decision at
     // the end of each body is taken on the device, and the kernels of bodies past the end return
     // at once -- so the host only synchronises once per group of bodies.
-    float *buf[2] = {y, w.yalt};
-    int enq = 0, group = 4;
-    StatusBlock hs;
+    int enq = k0, group = 4;
     for (;;) {
         int todo = max_iter - enq;
         if (todo > group) todo = group;
@@ -969,31 +1115,21 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
                 DEER_KERNEL("newton_control_kernel", st, newton_control_kernel<<<1, 1, 0, st>>>(w.st, tol, max_iter, w.trace));
             }
         }
-        if (y_host) {
-            size_t words = N * n / 4;
-            unsigned blocks = (unsigned)((words + 1023) / 1024);
-            const unsigned cap = 4u * (unsigned)num_sms();
-            if (blocks > cap) blocks = cap;
-            if (blocks < 1u) blocks = 1u;
-            DEER_KERNEL("result_select_kernel", st, result_select_kernel<<<blocks, 256, 0, st>>>(w.st, y, w.yalt, N * n));
-            if (copy_st) {      // the result leaves on a stream of its own, behind the selection
-                DEER_CHECK_CUDA(cudaEventRecord(copy_ev, st), "record result event");
-                DEER_CHECK_CUDA(cudaStreamWaitEvent(copy_st, copy_ev, 0), "wait result event");
-            }
-            DEER_CHECK_CUDA(cudaMemcpyAsync(y_host, y, N * n * sizeof(float), cudaMemcpyDeviceToHost, copy_st ? copy_st : st),
-                            "copy result to host");
-        }
+        if ((rc = copy_out()) != DEER_OK) return rc;
         DEER_CHECK_CUDA(cudaMemcpyAsync(&hs, w.st, 32, cudaMemcpyDeviceToHost, st), "read status");
         DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
         if (hs.flags & FLAG_TIMEOUT) return DEER_ERR_DEVICE_TIMEOUT;
         if (hs.done || enq >= max_iter) break;
         group = 2;
     }
+    }
     const int k = hs.iters;
     float e;
     memcpy(&e, &hs.err_last_bits, sizeof(float));
     if ((err_b || err_argmax) && k > 0) {
-        // the last two iterates are still in the two buffers (before the result copy below)
+        // the last two iterates are still in the two buffers (before the result copy below); a zero guess may not have been
+        // written out
+        if (k == 1 && !(flags & DEER_FLAG_WARM_START)) DEER_CHECK_CUDA(cudaMemsetAsync(buf[0], 0, N * n * sizeof(float), st), "zero guess");
         std::vector<unsigned long long> keys((size_t)B);
         DEER_KERNEL("err_diag_kernel", st, err_diag_kernel<<<(unsigned)B, 256, 0, st>>>(buf[k & 1], buf[(k + 1) & 1], (size_t)T * n, w.diag));
         DEER_CHECK_CUDA(cudaMemcpyAsync(keys.data(), w.diag, sizeof(unsigned long long) * (size_t)B, cudaMemcpyDeviceToHost, st), "read diagnostics");
@@ -1011,10 +1147,12 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     }
     if ((k & 1) && !y_host)
         DEER_CHECK_CUDA(cudaMemcpyAsync(y, w.yalt, N * n * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy result");
-    if (err_trace && k > 0)
+    const bool trace_here = one_launch && slot.p && hs.done == BODY_DONE && k <= HOST_TRACE;
+    if (err_trace && k > 0 && trace_here) memcpy(err_trace, slot.p->trace, sizeof(float) * (size_t)k);
+    if (err_trace && k > 0 && !trace_here)
         DEER_CHECK_CUDA(cudaMemcpyAsync(err_trace, w.trace, sizeof(float) * (size_t)(k < ERR_TRACE_CAP ? k : ERR_TRACE_CAP),
                                         cudaMemcpyDeviceToHost, st), "read trace");
-    DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+    if (((k & 1) && !y_host) || (err_trace && !trace_here)) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
     int status = DEER_OK;
     if (!isfinite(e)) status = DEER_NONFINITE;
     else if (e > tol && !(tol < 0.0f)) status = DEER_NOT_CONVERGED;

@@ -1,0 +1,199 @@
+// Launch side of the one-launch Newton body.
+#include <algorithm>
+#include <mutex>
+#include <stdlib.h>
+#include "newton_body.h"
+
+namespace deer {
+
+BodyKernels body_kernels_8(bool, bool);
+BodyKernels body_kernels_16(bool, bool);
+BodyKernels body_kernels_24(bool, bool);
+BodyKernels body_kernels_32(bool, bool);
+BodyKernels body_kernels_40(bool, bool);
+BodyKernels body_kernels_48(bool, bool);
+BodyKernels body_kernels_56(bool, bool);
+BodyKernels body_kernels_64(bool, bool);
+
+// n = 16, 32, 64: sizes whose linear solve has always run in reduced precision (bf16 / single-TF32 chain products)
+static bool reduced(int n) { return n == 16 || n == 32 || n == 64; }
+
+// A kernel per state size (rounded up to a multiple of 8) and row alignment.
+static BodyKernels pick(int n, bool v2)
+{
+    const bool exact = !reduced(n);
+    switch ((n + 7) / 8) {
+    case 1: return body_kernels_8(v2, exact);
+    case 2: return body_kernels_16(v2, exact);
+    case 3: return body_kernels_24(v2, exact);
+    case 4: return body_kernels_32(v2, exact);
+    case 5: return body_kernels_40(v2, exact);
+    case 6: return body_kernels_48(v2, exact);
+    case 7: return body_kernels_56(v2, exact);
+    default: return body_kernels_64(v2, exact);
+    }
+}
+
+constexpr size_t BODY_SMEM_MAX = 226 * 1024;          // (dynamic; the kernels have a few static words besides)
+
+bool body_supported(int n, int m, bool have_u)
+{
+    if (n < 1 || n > 64) return false;
+    return have_u || (m <= 64 && pick(n, false).one_smem((m + 7) / 8) <= BODY_SMEM_MAX);
+}
+
+// What a body's boundaries have to be good to, as a part of its update, and the burn-in that a cell as initialised needs for
+// it (white-noise inputs).  Reduced-precision solves: a thousandth.  The others: fp32 level where the caller counts bodies
+// (tol < 0), else 1e-4 -- the loop then ends on a body whose update is below tol, so the result is good to 1e-4 of that.
+float body_eta(int n, float tol) { return reduced(n) ? 1e-3f : tol > 0.0f ? 1e-4f : 4e-6f; }
+int body_first_burn(int n, float tol) { return reduced(n) ? 24 : tol > 0.0f ? 30 : 40; }
+
+// Shared-memory opt-in and CTAs per SM of a kernel, looked up once per kernel, device and shared-memory size.
+static int occupancy_of(const void *kern, int threads, size_t smem)
+{
+    static std::mutex mu;
+    struct Entry { const void *k; size_t smem; int dev, occ; };
+    static Entry cache[128];
+    static int used = 0;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    for (int i = 0; i < used; ++i)
+        if (cache[i].k == kern && cache[i].smem == smem && cache[i].dev == dev) return cache[i].occ;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BODY_SMEM_MAX);
+    int o = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, threads, smem) != cudaSuccess || o < 1) o = 1;
+    if (used < 128) cache[used++] = {kern, smem, dev, o};
+    return o;
+}
+
+static int sm_count()
+{
+    static int sms[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    if (!sms[dev]) {
+        int v = 0;
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        sms[dev] = v > 0 ? v : 148;
+    }
+    return sms[dev];
+}
+
+// CTAs of `per_cta` chains of length L: in all, of the head that needs most, and boundaries between units of `unit` chains.
+struct Count { long long ctas, edges; int worst; };
+static Count count_ctas(int B, int T, const int *strides, int H, int L, int per_cta, int unit)
+{
+    Count c{0, 0, 0};
+    for (int h = 0; h < H; ++h) {
+        const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s;
+        const long long chains = (long long)B * s * ((Tp + L - 1) / L), k = (chains + per_cta - 1) / per_cta;
+        c.ctas += k;
+        c.edges += (chains + unit - 1) / unit;
+        c.worst = (int)std::max<long long>(c.worst, k);
+    }
+    return c;
+}
+
+static int longest(int T, const int *strides, int H)
+{
+    int w = 1;
+    for (int h = 0; h < H; ++h) w = std::max(w, (T + (strides ? strides[h] : 1) - 1) / (strides ? strides[h] : 1));
+    return w;
+}
+
+bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool have_u, const int *strides, int H)
+{
+    const int kx = have_u ? 0 : (m + 7) / 8, sms = sm_count(), Tmax = longest(T, strides, H);
+    if (!body_supported(n, m, have_u)) return false;
+    const BodyKernels k = pick(n, (n & 1) == 0);
+    if (two_phase) {
+        const size_t fixed = k.seg_fixed(kx);
+        if (fixed >= BODY_SMEM_MAX) return false;
+        const int slots = (int)((BODY_SMEM_MAX - fixed) / k.slot_bytes);
+        const int cap = std::min(96, slots / 2), own = slots - cap;
+        if (own < 80) return false;
+        p->warps = k.seg_warps;
+        p->burn_cap = cap;
+        // The shortest chains for which the problem is one wave of CTAs, one per SM: a body then takes burn + L short steps.
+        // Where none is short enough, the CTA that holds most positions.
+        for (int L = 5; ; L += 2) {
+            const int nc_fit = std::min(k.nc_max, own / L / 16 * 16);
+            if (nc_fit < 16) return p->NC > 0 && p->max_ctas > 0;
+            int NC = 16;
+            while (2 * NC <= nc_fit && count_ctas(B, T, strides, H, L, NC, NC).ctas > sms) NC *= 2;
+            const Count c = count_ctas(B, T, strides, H, L, NC, NC);
+            if (p->NC * p->L < NC * L || c.ctas <= sms) {
+                p->NC = NC; p->L = L; p->max_ctas = c.worst; p->edges = c.edges;
+                p->waves = (float)c.ctas / (float)sms;
+                p->smem = fixed + k.slot_bytes * (size_t)(cap + NC * L);
+            }
+            p->whole_loop = c.ctas <= sms;
+            if (c.ctas <= sms || L >= Tmax) return true;
+        }
+    }
+    p->NC = 0;
+    p->whole_loop = false;
+    p->warps = k.one_warps;
+    p->smem = k.one_smem(kx);
+    const long long cap = (long long)sms * occupancy_of((const void *)k.one, 32 * p->warps, p->smem);   // CTAs of one wave
+    // The whole problem is one wave of chains: the shortest chain length for which it is, but no chains that would spend
+    // most of their steps on the burn-in.
+    const long long positions = (long long)B * T * H;
+    int L = (int)std::max<long long>(16, positions / (cap * p->warps * 16));
+    while (L < Tmax && count_ctas(B, T, strides, H, L, 16 * p->warps, 16).ctas > cap) L += std::max(1, L / 64);
+    const Count c = count_ctas(B, T, strides, H, L, 16 * p->warps, 16);
+    p->L = L; p->max_ctas = c.worst; p->edges = c.edges;
+    p->waves = (float)c.ctas / (float)cap;
+    // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
+    p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * L) : std::max(320, 8 * L);
+    return true;
+}
+
+// Measured lines (B200, m = n unless stated, us per evaluation: two-phase / one-phase / multiplied-out kernels):
+//   n = 4, B = 1, T = 1,000:   75 /  -  / 104      n = 4,  B = 16, T = 3e4: 591 / 354 / 188
+//   n = 8, B = 16, T = 1e4 (m = 4): 129 / - / 231   n = 8,  B = 16, T = 3e4: 570 / 321 / 539   n = 8,  T = 1e5: 1733 / 704 / 1564
+//   n = 16, B = 8, T = 2e4:   302 / 410 / 452      n = 16, B = 16, T = 1e5: 2407 / 1108 / 2283
+//   n = 32, B = 16, T = 1e3:  128 / 887 / 353      n = 32, B = 16, T = 1e4: 876 / 1126 / 873
+//   n = 64, B = 16, T = 1e3:    - / 2369 / 1247    n = 64, B = 16, T = 1e4:   - / 2828 / 3345
+// Two-phase: one wave (then the whole loop is one launch), two waves from n = 9 on.  One-phase: from half a wave of chains on --
+// below, its steps, a whole cell each, are a serial chain that nothing fills.  States of 1, 2 and 4 pad to 8 columns, which is
+// more work than their own kernels do.  Sizes without tuned kernels of the other kind always come here.
+bool body_suits(const BodyPlan &p, int n)
+{
+    const bool tuned = (n & (n - 1)) == 0;
+    if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
+    if (!tuned) return true;
+    return n == 8 || (n > 8 && p.waves >= 0.5f);
+}
+
+int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st)
+{
+    const bool aligned = ((((uintptr_t)a.buf[0] | (uintptr_t)a.buf[1] | (uintptr_t)a.y0 | (uintptr_t)a.u) & 7) == 0);
+    const bool v2 = (a.n & 1) == 0 && aligned;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.max_ctas, (unsigned)a.H);
+    cfg.blockDim = dim3(32u * (unsigned)p.warps);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    if (p.whole_loop) {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    const BodyKernels k = pick(a.n, v2);
+    occupancy_of(p.NC > 0 ? (const void *)k.seg : (const void *)k.one, 32 * p.warps, p.smem);      // (the shared-memory opt-in on first use)
+    if (p.NC > 0) {
+        DEER_KERNEL("newton_segment_kernel", st, cudaLaunchKernelEx(&cfg, k.seg, a, p.NC, p.whole_loop ? 1 : 0));
+    } else {
+        DEER_KERNEL("newton_body_kernel", st, cudaLaunchKernelEx(&cfg, k.one, a));
+    }
+    return DEER_OK;
+}
+
+}  // namespace deer

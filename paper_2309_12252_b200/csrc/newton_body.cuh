@@ -1,0 +1,420 @@
+// One Newton body of deer_gru_eval (Eq. 3 with Eq. 5, Newton-update form of App. A.1) as ONE launch: cell, residual,
+// linear solve, new iterate and convergence maximum, with nothing but x, the old iterate and the new one in memory.
+//
+// The update solves d_t = J_t d_{t-1} + r_t, r_t = f(y_{t-1}, x_t) - y_t.  The sequences are cut into chains of L
+// positions; sixteen chains advance in lockstep as the sixteen rows of a warp's m16n8k8 MMAs, a step being
+//     [16, m] x [m, 3n] + [16, n] x [n, 3n]      gates: 3 x TF32, so f is good to fp32 level
+//     [16, n] x [n, 3n]                          J_t d_{t-1} = z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d)
+// with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragment of one step is the A
+// operand of the next by renaming the contraction index (slots t, t + 4 of a K step hold columns 2t, 2t + 1), so
+// neither J_t, nor its coefficients, nor any chain product is ever formed or stored.
+//
+// What a chain does not know is the update entering it.  It starts `burn` positions early from zero: the error of its
+// entering update is the old error carried through `burn` Jacobians, and the Jacobians of a cell that forgets make it
+// vanish.  That is not taken on trust: every chain's end state is compared with the state its successor had assumed at
+// the same position (same arithmetic on same inputs: the difference is the carried error and nothing else).  The
+// largest mismatch of the launch has to stay below eta * max(err, tol) -- the accuracy the linear solve is asked for
+// in any case, since the fixed point does not depend on it.  When it does not, the body is not counted: the burn-in is
+// raised to what the observed decay calls for and the body is run again, or, for a cell that hardly forgets, the
+// evaluation goes on with the kernels that multiply the Jacobians out (BODY_FALL_BACK).
+//
+// Nothing waits on another CTA.  Boundaries inside a warp are compared from shared memory; at a boundary between two
+// warps each side leaves its state in global memory and the one that arrives second compares.
+#pragma once
+#include "mma_tf32.cuh"
+#include "newton_body.h"
+
+namespace deer {
+
+// What becomes of a body whose update is e and whose largest boundary mismatch is mis.
+struct BodyVerdict { bool counts; int done, burn; };
+__device__ __forceinline__ BodyVerdict body_verdict(float e, float mis, float eta, int burn, int burn_cap, float tol, int iters, int max_iter)
+{
+    BodyVerdict v{true, 0, burn};
+    if (e <= 3.402823466e38f) {                          // (a NaN or Inf ends the loop)
+        const float scale = fmaxf(e, tol > 0.0f ? tol : 0.0f), thr = eta * scale;
+        // Where the loop runs to a tolerance, a body whose boundaries are good to a thousandth of its update is a good
+        // quasi-Newton step: it counts, and the next one is given the burn-in that eta asks for.
+        const float most = tol > 0.0f ? fmaxf(eta, 1e-3f) * scale : thr;
+        if (!(mis <= thr)) {
+            // the carried error is about e * rho^burn: the burn-in after which it is thr / 2
+            const float ratio = mis / e;
+            int wn = 1 << 20;
+            if (ratio < 0.7f) wn = (int)(1.1f * (float)burn * __logf(0.5f * thr / e) / __logf(ratio)) + 4;
+            if (wn <= burn) wn = burn + 8;
+            if (mis <= most) {
+                v.burn = wn < burn_cap ? wn : burn_cap;
+            } else {
+                v.counts = false;
+                v.burn = wn;
+                if (wn > burn_cap) v.done = BODY_FALL_BACK;
+                return v;
+            }
+        }
+    }
+    if (newton_loop_ends(e, tol, iters, max_iter)) v.done = BODY_DONE;
+    return v;
+}
+
+// End of a body that is a launch of its own: the last CTA's decision.  Single thread.
+__device__ __forceinline__ void body_decide(StatusBlock *st, float eta, int burn_cap)
+{
+    const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits);
+    const float mis = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
+    const BodyVerdict v = body_verdict(e, mis, eta, st->burn, burn_cap, st->tol, st->iters, st->max_iter);
+    st->mis_bits = 0u;
+    st->burn = v.burn;
+    if (v.counts) { newton_decide(st, st->tol, st->max_iter, st->trace); return; }
+    st->err_bits = 0u;
+    st->done = v.done;
+    if (HostResult *h = st->host) { h->burn = v.burn; h->done = v.done; }
+}
+
+template <int N> struct Body {
+    static constexpr int NT = N / 8;
+    static constexpr int NS = 3 * N + 2;                 // records per pair of contraction rows: = 2 (mod 8), conflict-free
+    static constexpr int SW = N + 4;                     // stride of a saved start state
+    static constexpr size_t smem(int warps, int kx)      // kx: 8-column blocks of x contracted in the kernel
+    {
+        return sizeof(float) * ((size_t)4 * (N / 2 + 4 * kx) * NS + 4 * N + (size_t)warps * 16 * SW);
+    }
+};
+
+// EXACT: the products with d are 3 x TF32 as well (n <= 8 and sizes whose solve has always been fp32-accurate); V2: rows
+// are read and written as 8-byte pairs.
+template <int N, bool V2, bool EXACT>
+__global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_body_kernel(BodyArgs a)
+{
+    using C = Body<N>;
+    constexpr int NT = C::NT, NS = C::NS, SW = C::SW;
+    extern __shared__ __align__(16) float smb[];
+    const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
+    StatusBlock *st = a.st + blockIdx.y;
+    const int n = a.n, m = a.m, H = a.H, L = a.L;
+    const bool proj = a.u == nullptr;
+    const int kx = proj ? (m + 7) >> 3 : 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+
+    // geometry of this CTA's head
+    const int s = hd.stride, Tp = (a.T + s - 1) / s, nchain = (Tp + L - 1) / L;
+    const long long total = (long long)a.B * s * nchain;
+    const long long groups = (total + 15) >> 4;
+    const unsigned nctas = (unsigned)((groups + nwarps - 1) / nwarps);
+    if (blockIdx.x >= nctas) return;
+
+    // ---- weights into shared memory as records {hi(W[c][2p]), hi(W[c][2p+1]), lo, lo}: the B operand of one column block
+    // of one K step is one 128-bit load (weights are not produced by the previous launch: this runs before its end)
+    float4 *sH = reinterpret_cast<float4 *>(smb), *sI = sH + (N / 2) * NS;
+    float *sb = smb + 4 * (size_t)(N / 2 + 4 * kx) * NS;
+    auto lo = [](float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
+    for (int idx = tid; idx < (N / 2) * 3 * N; idx += blockDim.x) {
+        const int kp = idx % (N / 2), c = idx / (N / 2), gate = c / N, i = c % N;
+        const float *wr = hd.W_h + (size_t)(gate * n + i) * n + 2 * kp;
+        const float v0 = i < n && 2 * kp < n ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < n ? wr[1] : 0.0f;
+        sH[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    }
+    for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
+        const int kp = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
+        const float *wr = hd.W_i + (size_t)(gate * n + i) * m + 2 * kp;
+        const float v0 = i < n && 2 * kp < m ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < m ? wr[1] : 0.0f;
+        sI[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    }
+    for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
+        sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
+        sb[N + i] = i < n ? hd.b_h[n + i] + (proj ? hd.b_i[n + i] : 0.0f) : 0.0f;
+        sb[2 * N + i] = i < n ? hd.b_h[2 * n + i] : 0.0f;
+        sb[3 * N + i] = i < n && proj ? hd.b_i[2 * n + i] : 0.0f;
+    }
+    float *ss = sb + 4 * N + warp * 16 * SW;             // start states of this warp's chains
+    pdl_prologue();
+    if (*(volatile int *)&st->done) return;
+    __syncthreads();
+
+    const int iters = *(volatile int *)&st->iters, burn = *(volatile int *)&st->burn;
+    const float *ycur = a.buf[iters & 1];
+    const ptrdiff_t to_new = a.buf[(iters + 1) & 1] - ycur;
+    const bool zero = iters == 0 && !a.warm;             // the guess is zero: nothing of it is read
+    const long long grp = (long long)blockIdx.x * nwarps + warp;
+    unsigned mb = 0u, mis = 0u;
+
+    if (grp < groups) {
+        // ---- rows g and g + 8 of this lane: chain c of sequence (b, phase)
+        int tt[2], t_end[2];
+        const float *yp[2], *xp[2], *y0p[2];             // pointers at position tt (not dereferenced outside the sequence)
+        bool next[2];                                    // the row's chain has a successor
+        const size_t ys = (size_t)s * H * n, xs = proj ? (size_t)s * m : (size_t)s * H * 3 * n;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const long long gid = grp * 16 + g + 8 * h;
+            const long long q = gid < total ? gid / nchain : 0;
+            const int c = gid < total ? (int)(gid - q * nchain) : 0;
+            const long long b = q / s;
+            const int ph = (int)(q - b * s);
+            const int len = gid < total ? (a.T - ph + s - 1) / s : 0;
+            t_end[h] = min(len, (c + 1) * L);
+            if (c * L >= len) t_end[h] = 0;
+            next[h] = (c + 1) * L < len;
+            tt[h] = c * L - burn;
+            const size_t e = (size_t)b * a.T + ph;
+            yp[h] = ycur + (e * H + blockIdx.y) * n + (ptrdiff_t)tt[h] * (ptrdiff_t)ys;
+            xp[h] = (proj ? a.x + e * m : a.u + (e * H + blockIdx.y) * 3 * n) + (ptrdiff_t)tt[h] * (ptrdiff_t)xs;
+            y0p[h] = a.y0 + ((size_t)b * H + blockIdx.y) * n;
+        }
+        // (a warp whose chains are all first ones has no burn-in: its earliest position is -burn)
+        const int tmax = __reduce_max_sync(0xffffffffu, max(t_end[0] > 0 ? tt[0] : -burn, t_end[1] > 0 ? tt[1] : -burn));
+        const int s_first = tmax <= -burn ? burn : 0;
+        const int s_end = __reduce_max_sync(0xffffffffu, max(t_end[0] > 0 ? t_end[0] - tt[0] : 0, t_end[1] > 0 ? t_end[1] - tt[1] : 0));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { tt[h] += s_first; yp[h] += (ptrdiff_t)s_first * (ptrdiff_t)ys; xp[h] += (ptrdiff_t)s_first * (ptrdiff_t)xs; }
+
+        auto ld2 = [&](const float *p, int col, int width) -> float2 {
+            if constexpr (V2) {
+                return col < width ? *reinterpret_cast<const float2 *>(p + col) : make_float2(0.0f, 0.0f);
+            } else {
+                return make_float2(col < width ? p[col] : 0.0f, col + 1 < width ? p[col + 1] : 0.0f);
+            }
+        };
+        const bool xv2 = (m & 1) == 0 && ((uintptr_t)a.x & 7) == 0;
+        auto ldx = [&](const float *p, int col) -> float2 {
+            if (xv2) return col < m ? __ldg(reinterpret_cast<const float2 *>(p + col)) : make_float2(0.0f, 0.0f);
+            return make_float2(col < m ? __ldg(p + col) : 0.0f, col + 1 < m ? __ldg(p + col + 1) : 0.0f);
+        };
+        // iterate at position tt + off of row h (off = -1, 0): y0 before the first position, zero where nothing is
+        auto load_y = [&](float (&dst)[NT][4], int off) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int q = tt[h] + off;
+                const bool in = q >= 0 && q < t_end[h] && !zero, first = q == -1 && t_end[h] > 0;
+                const float *p = first ? y0p[h] : yp[h] + (ptrdiff_t)off * (ptrdiff_t)ys;
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float2 v = in || first ? ld2(p, 8 * j + 2 * t, n) : make_float2(0.0f, 0.0f);
+                    dst[j][2 * h] = v.x; dst[j][2 * h + 1] = v.y;
+                }
+            }
+        };
+        float hp[NT][4], yc[NT][4], d[NT][4];
+        load_y(hp, -1);
+        load_y(yc, 0);
+#pragma unroll
+        for (int j = 0; j < NT; ++j) { d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.0f; }
+
+#pragma unroll 1
+        for (int step = s_first; step < s_end; ++step) {
+            if (step == burn) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    *reinterpret_cast<float2 *>(ss + g * SW + 8 * j + 2 * t) = make_float2(d[j][0], d[j][1]);
+                    *reinterpret_cast<float2 *>(ss + (g + 8) * SW + 8 * j + 2 * t) = make_float2(d[j][2], d[j][3]);
+                }
+            }
+            const bool act[2] = {tt[0] >= 0 && tt[0] < t_end[0], tt[1] >= 0 && tt[1] < t_end[1]};
+            // ---- input half of the gates: u from memory, or x contracted here
+            float xr[NT][4], xz[NT][4], xn[NT][4];
+            if (proj) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] = 0.0f; xz[j][q] = 0.0f; xn[j][q] = 0.0f; }
+                float2 x0 = act[0] ? ldx(xp[0], 2 * t) : make_float2(0.0f, 0.0f);
+                float2 x1 = act[1] ? ldx(xp[1], 2 * t) : make_float2(0.0f, 0.0f);
+#pragma unroll 1
+                for (int kk = 0; kk < kx; ++kk) {
+                    unsigned ah[4], al[4];
+                    split_tf32(x0.x, ah[0], al[0]);
+                    split_tf32(x1.x, ah[1], al[1]);
+                    split_tf32(x0.y, ah[2], al[2]);
+                    split_tf32(x1.y, ah[3], al[3]);
+                    if (kk + 1 < kx) {
+                        x0 = act[0] ? ldx(xp[0], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
+                        x1 = act[1] ? ldx(xp[1], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
+                    }
+                    const float4 *q0 = sI + (4 * kk + t) * NS + g;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        {
+#pragma unroll
+                            for (int gate = 0; gate < 3; ++gate) {
+                                const float4 w = q0[gate * N + 8 * j];
+                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                                float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
+                                mma_tf32(acc, al, bh, acc);
+                                mma_tf32(acc, ah, bl, acc);
+                                mma_tf32(acc, ah, bh, acc);
+                            }
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const int col = 8 * j + 2 * t;
+                        const bool on = act[h] && col < n;
+                        const float2 vr = on ? ld2(xp[h], col, n) : make_float2(0.0f, 0.0f);
+                        const float2 vz = on ? ld2(xp[h] + n, col, n) : make_float2(0.0f, 0.0f);
+                        const float2 vn = on ? ld2(xp[h] + 2 * n, col, n) : make_float2(0.0f, 0.0f);
+                        xr[j][2 * h] = vr.x; xr[j][2 * h + 1] = vr.y;
+                        xz[j][2 * h] = vz.x; xz[j][2 * h + 1] = vz.y;
+                        xn[j][2 * h] = vn.x; xn[j][2 * h + 1] = vn.y;
+                    }
+            }
+            // ---- hidden half and the update, one block of eight columns at a time
+            const bool hid = !zero || __any_sync(0xffffffffu, tt[0] == 0 || tt[1] == 0);     // zero guess: W_h 0 = 0
+            float dn[NT][4];
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                {
+                    float hr[4] = {xr[j][0], xr[j][1], xr[j][2], xr[j][3]}, hz[4] = {xz[j][0], xz[j][1], xz[j][2], xz[j][3]};
+                    float hq[4] = {0.f, 0.f, 0.f, 0.f}, ur[4] = {0.f, 0.f, 0.f, 0.f}, uz[4] = {0.f, 0.f, 0.f, 0.f}, un[4] = {0.f, 0.f, 0.f, 0.f};
+                    const float4 *q0 = sH + t * NS + 8 * j + g;
+#pragma unroll
+                    for (int kk = 0; kk < NT; ++kk) {
+                        {
+                            unsigned ah[4], al[4], dh[4], dl[4];
+                            split_tf32(d[kk][0], dh[0], dl[0]); split_tf32(d[kk][2], dh[1], dl[1]);
+                            split_tf32(d[kk][1], dh[2], dl[2]); split_tf32(d[kk][3], dh[3], dl[3]);
+                            split_tf32(hp[kk][0], ah[0], al[0]); split_tf32(hp[kk][2], ah[1], al[1]);
+                            split_tf32(hp[kk][1], ah[2], al[2]); split_tf32(hp[kk][3], ah[3], al[3]);
+#pragma unroll
+                            for (int gate = 0; gate < 3; ++gate) {
+                                const float4 w = q0[4 * kk * NS + gate * N];
+                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                                float (&hacc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
+                                float (&uacc)[4] = gate == 0 ? ur : gate == 1 ? uz : un;
+                                if (hid) {
+                                    mma_tf32(hacc, al, bh, hacc);
+                                    mma_tf32(hacc, ah, bl, hacc);
+                                    mma_tf32(hacc, ah, bh, hacc);
+                                }
+                                if constexpr (EXACT) {
+                                    mma_tf32(uacc, dl, bh, uacc);
+                                    mma_tf32(uacc, dh, bl, uacc);
+                                }
+                                mma_tf32(uacc, dh, bh, uacc);
+                            }
+                        }
+                    }
+                    const int col = 8 * j + 2 * t;
+                    const float2 bR = *reinterpret_cast<const float2 *>(sb + col), bZ = *reinterpret_cast<const float2 *>(sb + N + col);
+                    const float2 bQ = *reinterpret_cast<const float2 *>(sb + 2 * N + col), bN = *reinterpret_cast<const float2 *>(sb + 3 * N + col);
+                    const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float2 h2 = make_float2(hp[j][2 * h], hp[j][2 * h + 1]), y2 = make_float2(yc[j][2 * h], yc[j][2 * h + 1]);
+                        const float2 d2 = make_float2(d[j][2 * h], d[j][2 * h + 1]);
+                        const float2 q = fadd2(make_float2(hq[2 * h], hq[2 * h + 1]), bQ);
+                        const float2 r = sigmoid2_gate(fadd2(make_float2(hr[2 * h], hr[2 * h + 1]), bR));
+                        const float2 z = sigmoid2_gate(fadd2(make_float2(hz[2 * h], hz[2 * h + 1]), bZ));
+                        const float2 c = tanh2_gate(ffma2(r, q, fadd2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), bN)));
+                        const float2 omz = ffma2(z, mone, one), omr = ffma2(r, mone, one);
+                        const float2 f = ffma2(omz, c, fmul2(z, h2));
+                        const float2 az = fmul2(fmul2(ffma2(c, mone, h2), z), omz);
+                        const float2 an = fmul2(omz, ffma2(fmul2(c, mone), c, one));
+                        const float2 kn = fmul2(an, r);
+                        const float2 kr = fmul2(fmul2(kn, q), omr);
+                        float2 v = ffma2(y2, mone, f);                                          // r_t = f - y
+                        v = ffma2(z, d2, v);
+                        v = ffma2(kr, make_float2(ur[2 * h], ur[2 * h + 1]), v);
+                        v = ffma2(az, make_float2(uz[2 * h], uz[2 * h + 1]), v);
+                        v = ffma2(kn, make_float2(un[2 * h], un[2 * h + 1]), v);
+                        dn[j][2 * h] = v.x; dn[j][2 * h + 1] = v.y;
+                        if (step >= burn && act[h]) {
+                            const float2 yn = fadd2(y2, v);
+                            float *o = const_cast<float *>(yp[h]) + to_new + col;
+                            if constexpr (V2) {
+                                if (col < n) {
+                                    mb = max(mb, max(absdiff_bits(yn.x, y2.x), absdiff_bits(yn.y, y2.y)));
+                                    *reinterpret_cast<float2 *>(o) = yn;
+                                }
+                            } else {
+                                if (col < n) { mb = max(mb, absdiff_bits(yn.x, y2.x)); o[0] = yn.x; }
+                                if (col + 1 < n) { mb = max(mb, absdiff_bits(yn.y, y2.y)); o[1] = yn.y; }
+                            }
+                        }
+                    }
+                }
+            }
+            // ---- advance
+#pragma unroll
+            for (int h = 0; h < 2; ++h) { ++tt[h]; yp[h] += ys; xp[h] += xs; }
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        d[j][q] = act[q >> 1] ? dn[j][q] : d[j][q];
+                        hp[j][q] = yc[j][q];
+                    }
+                }
+            }
+            if (step + 1 < s_end) load_y(yc, 0);
+        }
+        // ---- boundaries: this row's end state against the state its successor assumed
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = g + 8 * h;
+            if (next[h] && row < 15) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float2 v = *reinterpret_cast<const float2 *>(ss + (row + 1) * SW + 8 * j + 2 * t);
+                    mis = max(mis, max(absdiff_bits(v.x, d[j][2 * h]), absdiff_bits(v.y, d[j][2 * h + 1])));
+                }
+            }
+        }
+        const bool has_next = __shfl_sync(0xffffffffu, (int)next[1], 28) != 0;                   // row 15
+        const bool has_prev = __shfl_sync(0xffffffffu, (int)(t_end[0] > 0 && grp > 0 && (grp * 16) % nchain != 0), 0) != 0;   // row 0
+        __syncwarp();
+        if (has_next) {                                  // row 15's end state takes the place of row 15's start state
+            if (g == 7) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    *reinterpret_cast<float2 *>(ss + 15 * SW + 8 * j + 2 * t) = make_float2(d[j][2], d[j][3]);
+            }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {           // 0: left of the boundary behind this group, 1: right of the one before it
+            if (side == 0 ? !has_next : !has_prev) continue;
+            const size_t edge = (size_t)hd.first_edge + (size_t)grp - side;
+            const float *own = ss + (side == 0 ? 15 : 0) * SW;
+            float *slot = a.edge + edge * 2 * n;
+            for (int i = lane; i < n; i += 32) __stcg(slot + side * n + i, own[i]);
+            __threadfence();
+            __syncwarp();
+            unsigned old = 0;
+            if (lane == 0) old = atomicAdd(a.edge_flag + edge, 1u);
+            old = __shfl_sync(0xffffffffu, old, 0);
+            if (old == 1u) {
+                __threadfence();
+                for (int i = lane; i < n; i += 32) mis = max(mis, absdiff_bits(own[i], __ldcg(slot + (side ^ 1) * n + i)));
+                if (lane == 0) a.edge_flag[edge] = 0u;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+        mis = max(mis, __shfl_xor_sync(0xffffffffu, mis, o));
+    }
+    if (lane == 0) {
+        if (mb) atomicMax(&st->err_bits, mb);
+        if (mis) atomicMax(&st->mis_bits, mis);
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(&st->exit_counter, 1u);
+        if (prev + 1u == nctas) {
+            __threadfence();
+            st->exit_counter = 0u;
+            body_decide(st, a.eta, a.burn_cap);
+        }
+    }
+}
+
+}  // namespace deer

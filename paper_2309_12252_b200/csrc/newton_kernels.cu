@@ -1,0 +1,33 @@
+// The one-launch Newton kernels of one padded state size: compiled once per size with -DBODY_N=8, 16, ... 64 (build.py).
+#include "newton_segment.cuh"
+
+#ifndef BODY_N
+#error "BODY_N: state size, a multiple of 8 up to 64"
+#endif
+
+namespace deer {
+
+// v2: rows as 8-byte pairs; exact: products with the update at fp32 level
+template <int N> static BodyKernels kernels_of(bool v2, bool exact)
+{
+    BodyKernels k{};
+    k.one = v2 ? newton_body_kernel<N, true, true> : newton_body_kernel<N, false, true>;
+    k.seg = v2 ? newton_segment_kernel<N, true, true> : newton_segment_kernel<N, false, true>;
+    if constexpr (N == 16 || N == 32 || N == 64) {
+        // single-TF32 products with the update: the sizes whose solve has always run in reduced precision
+        if (v2 && !exact) { k.one = newton_body_kernel<N, true, false>; k.seg = newton_segment_kernel<N, true, false>; }
+    }
+    k.one_warps = N > 32 ? 8 : 4;
+    k.seg_warps = Seg<N>::WARPS;
+    k.nc_max = Seg<N>::NC_MAX;
+    k.slot_bytes = Seg<N>::SZ * sizeof(float);
+    k.one_smem = [](int kx) { return Body<N>::smem(N > 32 ? 8 : 4, kx); };
+    k.seg_fixed = [](int kx) { return Seg<N>::fixed(kx); };
+    return k;
+}
+
+#define BODY_CAT_(a, b) a##b
+#define BODY_CAT(a, b) BODY_CAT_(a, b)
+BodyKernels BODY_CAT(body_kernels_, BODY_N)(bool v2, bool exact) { return kernels_of<BODY_N>(v2, exact); }
+
+}  // namespace deer
