@@ -200,8 +200,9 @@ constexpr int PROJ_PP = 8;
 
 __global__ void __launch_bounds__(256) proj_tiled_kernel(const float *__restrict__ x, const float *__restrict__ W_i,
                                                          const float *__restrict__ b_i, float *__restrict__ u,
-                                                         size_t N, int m, int n3, int G, int wt_given)
+                                                         size_t N, int m, int n3, int G, int wt_given, const StatusBlock *st)
 {
+    if (loop_ended(st)) return;
     extern __shared__ __align__(16) float smp[];
     float *sWT = smp;                    // [m][n3]
     float *sX = sWT + (size_t)m * n3;    // [G*PP][m+1]

@@ -101,7 +101,8 @@ struct StatusBlock {
     float *trace;        // err after each body (first ERR_TRACE_CAP bodies), or nullptr
     unsigned mis_bits;   // one-launch bodies: largest mismatch between a chain's end and the start its successor assumed
     HostResult *host;    // page-locked host memory, or nullptr
-    unsigned pad[46];
+    unsigned top_end_bits, mis_end_bits;     // adjoint launch: max|dy0|, largest mismatch near the first time step
+    unsigned pad[44];
 };
 static_assert(sizeof(StatusBlock) == 256, "status block is one 256-byte line");
 constexpr int ERR_TRACE_CAP = 1024;

@@ -454,7 +454,7 @@ static int run_scan(ScanArgs a, const ScanWs &w, int flags, cudaStream_t st, boo
 // tensor-core affine map (K = inputs, nout = outputs; see affine_mma_kernel)
 template <int NB_MAX, bool WT>
 static int launch_affine_mma(const float *in, const float *W, const float *bias, float *out, size_t N, int K, int nout,
-                             cudaStream_t st)
+                             cudaStream_t st, const StatusBlock *unless)
 {
     const size_t sm = sizeof(float) * 2 * (size_t)K * (nout + 4);
     int rc;
@@ -463,24 +463,25 @@ static int launch_affine_mma(const float *in, const float *W, const float *bias,
     const size_t per_sm = sm > 110 * 1024 ? 1 : 2;
     const size_t cap = (size_t)num_sms() * per_sm;
     const unsigned blocks = (unsigned)(tiles < cap ? tiles : cap);
-    DEER_KERNEL("affine_mma_kernel", st, (affine_mma_kernel<NB_MAX, WT><<<blocks, 256, sm, st>>>(in, W, bias, out, N, K, nout)));
+    DEER_KERNEL("affine_mma_kernel", st, (affine_mma_kernel<NB_MAX, WT><<<blocks, 256, sm, st>>>(in, W, bias, out, N, K, nout, unless)));
     return DEER_OK;
 }
 
-// out[e][g] = bias[g] + sum_k W[g][k] in[e][k]   (wt_given: W is stored [k][g]; bias may be null)
+// out[e][g] = bias[g] + sum_k W[g][k] in[e][k]   (wt_given: W is stored [k][g]; bias may be null; unless: nothing to do once
+// that block's done is set)
 static int run_affine(const float *in, const float *W, const float *bias, float *out, size_t N, int m, int n3,
-                      int wt_given, cudaStream_t st)
+                      int wt_given, cudaStream_t st, const StatusBlock *unless = nullptr)
 {
     // tensor-core path: K and the output count multiples of 8, 8-byte aligned rows, weights fit shared memory
     const bool aligned8 = (((uintptr_t)in | (uintptr_t)out) & 7) == 0;
     if (aligned8 && m % 8 == 0 && m >= 16 && n3 % 8 == 0 && n3 <= 192 &&
         sizeof(float) * 2 * (size_t)m * (n3 + 4) <= 200 * 1024) {
-        if (n3 <= 64) return wt_given ? launch_affine_mma<8, true>(in, W, bias, out, N, m, n3, st)
-                                      : launch_affine_mma<8, false>(in, W, bias, out, N, m, n3, st);
-        if (n3 <= 96) return wt_given ? launch_affine_mma<12, true>(in, W, bias, out, N, m, n3, st)
-                                      : launch_affine_mma<12, false>(in, W, bias, out, N, m, n3, st);
-        return wt_given ? launch_affine_mma<24, true>(in, W, bias, out, N, m, n3, st)
-                        : launch_affine_mma<24, false>(in, W, bias, out, N, m, n3, st);
+        if (n3 <= 64) return wt_given ? launch_affine_mma<8, true>(in, W, bias, out, N, m, n3, st, unless)
+                                      : launch_affine_mma<8, false>(in, W, bias, out, N, m, n3, st, unless);
+        if (n3 <= 96) return wt_given ? launch_affine_mma<12, true>(in, W, bias, out, N, m, n3, st, unless)
+                                      : launch_affine_mma<12, false>(in, W, bias, out, N, m, n3, st, unless);
+        return wt_given ? launch_affine_mma<24, true>(in, W, bias, out, N, m, n3, st, unless)
+                        : launch_affine_mma<24, false>(in, W, bias, out, N, m, n3, st, unless);
     }
     int G = 256 / n3;
     while (G > 1 && sizeof(float) * (size_t)G * PROJ_PP * (m + 1) > 64 * 1024) --G;
@@ -493,18 +494,18 @@ static int run_affine(const float *in, const float *W, const float *bias, float 
     const unsigned blocks = (unsigned)(tiles < cap ? tiles : cap);
     const int threads = (n3 * G + 31) / 32 * 32;
     DEER_KERNEL("proj_tiled_kernel", st,
-                proj_tiled_kernel<<<blocks, threads, sm, st>>>(in, W, bias, out, N, m, n3, G, wt_given));
+                proj_tiled_kernel<<<blocks, threads, sm, st>>>(in, W, bias, out, N, m, n3, G, wt_given, unless));
     return DEER_OK;
 }
 
-static int run_proj(const deer_gru_params *p, const float *x, float *u, size_t N, cudaStream_t st)
+static int run_proj(const deer_gru_params *p, const float *x, float *u, size_t N, cudaStream_t st, const StatusBlock *unless = nullptr)
 {
     const int n3 = 3 * p->n, m = p->m;
     if (n3 <= 256 && sizeof(float) * ((size_t)m * n3 + (size_t)PROJ_PP * (m + 1)) <= 200 * 1024)
-        return run_affine(x, p->W_i, p->b_i, u, N, m, n3, 0, st);
+        return run_affine(x, p->W_i, p->b_i, u, N, m, n3, 0, st, unless);
     size_t total = N * (size_t)n3;
     unsigned blocks = (unsigned)((total + 255) / 256);
-    DEER_KERNEL("proj_kernel", st, proj_kernel<<<blocks, 256, 0, st>>>(x, p->W_i, p->b_i, u, N, m, n3));
+    DEER_KERNEL("proj_kernel", st, proj_kernel<<<blocks, 256, 0, st>>>(x, p->W_i, p->b_i, u, N, m, n3, unless));
     return DEER_OK;
 }
 
@@ -656,6 +657,9 @@ struct EvalWs {
 // chain groups of a one-launch body at the shortest chain length
 static size_t body_groups_max(int B, int T) { return ((size_t)B * ((T + BODY_L_MIN - 1) / BODY_L_MIN) + 15) / 16; }
 
+// ... and of an adjoint launch (its chains are 16 positions at least), idle warps of the last CTA included
+static size_t adjoint_groups_max(int B, int T) { return ((size_t)B * ((T + 15) / 16) + 15) / 16 + 8; }
+
 static EvalWs carve_eval(void *ws, int B, int T, int n, int m)
 {
     (void)m;
@@ -697,6 +701,8 @@ constexpr int WGRAD_P = 592;   // slices of the position axis in the parameter-g
 
 struct VjpWs {
     StatusBlock *st;
+    unsigned *edge_flag;         // directly behind the status block: cleared with it
+    float *edge, *starts;
     float *u, *J, *rhs, *lam, *dGi, *dGh, *partial, *partial2;
     ScanWs scan;
     size_t bytes;
@@ -708,6 +714,9 @@ static VjpWs carve_vjp(void *ws, int B, int T, int n, int m)
     VjpWs w;
     size_t N = (size_t)B * T;
     w.st = cv.take<StatusBlock>(1);
+    w.edge_flag = cv.take<unsigned>(body_groups_max(B, T));
+    w.edge = cv.take<float>(body_groups_max(B, T) * 2 * n);
+    w.starts = cv.take<float>(adjoint_groups_max(B, T) * adjoint_starts(n));
     w.u = cv.take<float>(N * 3 * n);
     w.J = cv.take<float>(N * n * n);
     w.lam = cv.take<float>(N * n);
@@ -1209,12 +1218,33 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     int rc = check_ws(ws, ws_bytes, w.bytes);
     if (rc != DEER_OK) return rc;
     const size_t N = (size_t)B * T;
-    DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock), st), "memset status");
+    const bool have_u = !adjoint_supported(n, m, false);
+    BodyPlan plan{};
+    const bool adj = !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
+                     adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && adjoint_suits(plan, n);
+    DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj ? (size_t)plan.edges * sizeof(unsigned) : 0), st), "memset status");
     // small n and m: the cell projects x itself and one kernel does the cell VJP, the slices of the
     // parameter-gradient reduction and dx (no u, dG_i, dG_h arrays)
     const bool small = cell_projects(n, m) && !(flags & DEER_FLAG_GENERIC) && y0 != nullptr &&
                        ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
-    if (!small && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
+    const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
+    if (adj) {
+        if (have_u && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
+        AdjArgs a{};
+        a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0, 0};
+        a.x = x; a.u = have_u ? w.u : nullptr; a.y0 = y0; a.y = y; a.gy = gy;
+        a.lam = small ? w.lam : nullptr; a.dGi = w.dGi; a.dGh = w.dGh;
+        a.dy0 = dy0; a.dy0_by_head = 1;
+        a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1; a.L = plan.L;
+        a.eta = ADJ_ETA;
+        a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = w.starts;
+        for (int k = 0; k < ADJ_TRIES; ++k) {
+            a.burn = ADJ_BURN[k];
+            if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
+        }
+        unless = w.st;
+    }
+    if (!small && !(adj && have_u) && (rc = run_proj(p, x, w.u, N, st, unless)) != DEER_OK) return rc;
     ScanArgs a{};
     a.J = w.J; a.b = gy; a.y0 = nullptr; a.y = w.lam; a.yold = nullptr;
     a.B = B; a.T = T; a.n = n; a.reverse = 1;
@@ -1225,7 +1255,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     const bool gen_J = (n == 16 || n == 32) && !(flags & DEER_FLAG_MATERIALIZE) && scan_is_single_pass(a, w.scan, flags) &&
                        ((((uintptr_t)y | (uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0);
     if (gen_J) a.Wh = p->W_h;
-    CellArgs c{p->W_h, p->b_h, small ? nullptr : w.u, x, p->W_i, p->b_i, m, y, y0, w.J, nullptr, B, T, n, nullptr,
+    CellArgs c{p->W_h, p->b_h, small ? nullptr : w.u, x, p->W_i, p->b_i, m, y, y0, w.J, nullptr, B, T, n, unless,
                gen_J ? 1 : 0};
     if ((rc = run_cell(c, st)) != DEER_OK) return rc;
     if ((rc = run_scan(a, w.scan, flags, st)) != DEER_OK) return rc;
@@ -1237,12 +1267,12 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
         DEER_KERNEL("wgrad_final_kernel", st, wgrad_final_kernel<<<(n3 * (m + 1) + 7) / 8, 256, 0, st>>>(w.partial, P, n3, m, g->dW_i, g->db_i));
         DEER_KERNEL("wgrad_final_kernel", st, wgrad_final_kernel<<<(n3 * (n + 1) + 7) / 8, 256, 0, st>>>(w.partial2, P, n3, n, g->dW_h, g->db_h));
         if (dy0) {
-            DEER_KERNEL("vjp_dy0_kernel", st, vjp_dy0_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, w.lam, dy0, B, T, n));
+            DEER_KERNEL("vjp_dy0_kernel", st, vjp_dy0_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, w.lam, dy0, B, T, n, unless));
         }
         return DEER_OK;
     }
     {
-        VjpArgs v{p->W_h, p->b_h, w.u, y, y0, w.lam, w.dGi, w.dGh, B, T, n};
+        VjpArgs v{p->W_h, p->b_h, w.u, y, y0, w.lam, w.dGi, w.dGh, B, T, n, unless};
         const bool aligned = (((uintptr_t)y | (uintptr_t)y0) & 15) == 0;
         if (aligned && (n == 16 || n == 32 || n == 64)) {
             if ((rc = launch_vjp_cell_wide(v, st)) != DEER_OK) return rc;
@@ -1299,9 +1329,9 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     }
     if (dy0) {
         if (gen_J) {
-            DEER_KERNEL("vjp_dy0_coef_kernel", st, vjp_dy0_coef_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, p->W_h, w.lam, dy0, B, T, n));
+            DEER_KERNEL("vjp_dy0_coef_kernel", st, vjp_dy0_coef_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, p->W_h, w.lam, dy0, B, T, n, unless));
         } else {
-            DEER_KERNEL("vjp_dy0_kernel", st, vjp_dy0_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, w.lam, dy0, B, T, n));
+            DEER_KERNEL("vjp_dy0_kernel", st, vjp_dy0_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, w.lam, dy0, B, T, n, unless));
         }
     }
     return DEER_OK;
@@ -1688,7 +1718,7 @@ int deer_lstm_eval(const deer_lstm_params *p, const float *x, const float *s0, i
         if ((rc = run_affine(x, p->W_i, p->b, w.u, N, m, 4 * k, 0, st)) != DEER_OK) return rc;
     } else {
         const size_t total = N * (size_t)(4 * k);
-        DEER_KERNEL("proj_kernel", st, proj_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(x, p->W_i, p->b, w.u, N, m, 4 * k));
+        DEER_KERNEL("proj_kernel", st, proj_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(x, p->W_i, p->b, w.u, N, m, 4 * k, nullptr));
     }
     const size_t sm = sizeof(float) * 4 * (size_t)k * (k + 1);
     if ((rc = opt_in_smem((const void *)lstm_cell_kernel, sm)) != DEER_OK) return rc;

@@ -13,8 +13,9 @@ constexpr int GEN_THREADS = 128;
 // ------------------------------------------------------------------ a0: u = x W_i^T + b_i
 __global__ void proj_kernel(const float *__restrict__ x, const float *__restrict__ W_i,
                             const float *__restrict__ b_i, float *__restrict__ u, size_t N, int m,
-                            int n3)
+                            int n3, const StatusBlock *st)
 {
+    if (loop_ended(st)) return;
     size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= N * (size_t)n3) return;
     size_t e = idx / n3;
@@ -400,10 +401,12 @@ struct VjpArgs {
     const float *W_h, *b_h, *u, *y, *y0, *lam;   // lam [B,T,n] = dL/df at every position
     float *dGi, *dGh;                            // [B,T,3n] gradients w.r.t. u and w.r.t. W_h h + b_h
     int B, T, n;
+    const StatusBlock *st;                       // nullptr, or: nothing to do once st->done is set
 };
 
 __global__ void vjp_cell_kernel(VjpArgs a)
 {
+    if (loop_ended(a.st)) return;
     extern __shared__ float sW[];
     const int n = a.n, ld = n + 1;
     float *sb = sW + 3 * n * ld;
@@ -595,8 +598,9 @@ __global__ void vjp_dx_kernel(const float *__restrict__ dGi, const float *__rest
 
 // dy0[b][j] = sum_i J[b][0][i][j] lam[b][0][i]
 __global__ void vjp_dy0_kernel(const float *__restrict__ J, const float *__restrict__ lam,
-                               float *__restrict__ dy0, int B, int T, int n)
+                               float *__restrict__ dy0, int B, int T, int n, const StatusBlock *st)
 {
+    if (loop_ended(st)) return;
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= B * n) return;
     int seq = idx / n, j = idx % n;
@@ -610,8 +614,10 @@ __global__ void vjp_dy0_kernel(const float *__restrict__ J, const float *__restr
 // the same from the coefficient rows {k_r, a_z, k_n, z}[n] of position 0 (J = diag(k_r) W_hr + diag(a_z) W_hz +
 // diag(k_n) W_hn + diag(z), evaluated in the order of the cell's Jacobian phase)
 __global__ void vjp_dy0_coef_kernel(const float *__restrict__ coef, const float *__restrict__ W_h,
-                                    const float *__restrict__ lam, float *__restrict__ dy0, int B, int T, int n)
+                                    const float *__restrict__ lam, float *__restrict__ dy0, int B, int T, int n,
+                                    const StatusBlock *st)
 {
+    if (loop_ended(st)) return;
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= B * n) return;
     int seq = idx / n, j = idx % n;

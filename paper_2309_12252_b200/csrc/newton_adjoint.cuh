@@ -1,0 +1,423 @@
+// The gradient's adjoint solve as ONE launch (Eq. 7; the dual operator of Sec. 3.1.1): gates at the trajectory,
+// lambda_t = gy_t + J_{t+1}^T lambda_{t+1}, and the gradients w.r.t. the pre-activations -- no projected inputs, Jacobians,
+// coefficient rows or lambda in memory.
+//
+// Chains in lockstep, burn-in and verified boundaries as in newton_body.cuh, in descending time.  The state that a chain
+// carries is mu_t = J_{t+1}^T lambda_{t+1}.  With the gates at t and lambda = gy + mu, the hidden-side gradients of the three
+// pre-activations are p = (k_r.lambda, a_z.lambda, k_n.lambda) -- what dW_h, dW_i, dx are contractions of -- and
+//     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands.
+// All products are 3 x TF32 (a one-shot solve).  A boundary mismatch above eta * max|lambda| leaves StatusBlock::done at 0:
+// the launches enqueued behind this one (a longer burn-in, then the kernels that multiply the Jacobians out) do the work.
+// dy0 is an output with a scale of its own: where dL/dy is zero near the start of the sequences, dy0 may be many orders of
+// magnitude below max|lambda|.  So the boundaries that dy0 can still feel -- those less than DY0_REACH burn-ins from the
+// sequence's first step -- are held to eta * max|dy0| as well.
+#pragma once
+#include "newton_body.cuh"
+
+namespace deer {
+
+constexpr int DY0_REACH = 8;     // a burn-in takes an error down by about 1e-6 or more; behind eight of them it is below any fp32
+
+template <int N> struct Adj {
+    static constexpr int NT = N / 8;
+    static constexpr int NS = 3 * N + 2, NS2 = N + 2;    // = 2 (mod 8) records
+    static constexpr int SW = N + 4;
+    static constexpr bool SS_GLOBAL = N > 48;            // start states in the workspace: the weights of both contractions fill
+                                                         // the shared memory
+    static constexpr size_t smem(int warps, int kx)
+    {
+        if (SS_GLOBAL) warps = 0;
+        return sizeof(float) * ((size_t)4 * (N / 2 + 4 * kx) * NS + (size_t)4 * (3 * N / 2) * NS2 + 4 * N + (size_t)warps * 16 * SW);
+    }
+};
+
+// End of the launch: were the boundaries good enough?  Single thread.
+__device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool dy0)
+{
+    auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
+    const float top = take(st->err_bits), mis = take(st->mis_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
+    if (mis <= eta * top && (!dy0 || mis_end <= eta * top_end)) st->done = BODY_DONE;
+}
+
+template <int N, bool V2>
+__global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 3) newton_adjoint_kernel(AdjArgs a)
+{
+    using C = Adj<N>;
+    constexpr int NT = C::NT, NS = C::NS, NS2 = C::NS2, SW = C::SW;
+    extern __shared__ __align__(16) float smb[];
+    const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
+    StatusBlock *st = a.st + blockIdx.y;
+    const int n = a.n, m = a.m, H = a.H, L = a.L;
+    const bool proj = a.u == nullptr;
+    const int kx = proj ? (m + 7) >> 3 : 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+
+    // geometry of this CTA's head
+    const int s = hd.stride, Tp = (a.T + s - 1) / s, nchain = (Tp + L - 1) / L;
+    const long long total = (long long)a.B * s * nchain;
+    const long long groups = (total + 15) >> 4;
+    const unsigned nctas = (unsigned)((groups + nwarps - 1) / nwarps);
+    if (blockIdx.x >= nctas) return;
+
+    // ---- weights into shared memory as records {hi(W[c][2p]), hi(W[c][2p+1]), lo, lo}: the B operand of one column block
+    // of one K step is one 128-bit load (weights are not produced by the previous launch: this runs before its end)
+    float4 *sH = reinterpret_cast<float4 *>(smb), *sI = sH + (N / 2) * NS;
+    float4 *sT = sI + 4 * kx * NS;                       // W_h by pairs of rows: the B operand of p W_h
+    float *sb = reinterpret_cast<float *>(sT + (3 * N / 2) * NS2);
+    auto lo = [](float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
+    for (int idx = tid; idx < (N / 2) * 3 * N; idx += blockDim.x) {
+        const int kp = idx % (N / 2), c = idx / (N / 2), gate = c / N, i = c % N;
+        const float *wr = hd.W_h + (size_t)(gate * n + i) * n + 2 * kp;
+        const float v0 = i < n && 2 * kp < n ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < n ? wr[1] : 0.0f;
+        sH[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    }
+    for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
+        const int kp = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
+        const float *wr = hd.W_i + (size_t)(gate * n + i) * m + 2 * kp;
+        const float v0 = i < n && 2 * kp < m ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < m ? wr[1] : 0.0f;
+        sI[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    }
+    for (int idx = tid; idx < (3 * N / 2) * N; idx += blockDim.x) {
+        const int c = idx % N, kp = idx / N, gate = 2 * kp / N, i = 2 * kp % N;
+        const float v0 = c < n && i < n ? hd.W_h[(size_t)(gate * n + i) * n + c] : 0.0f;
+        const float v1 = c < n && i + 1 < n ? hd.W_h[(size_t)(gate * n + i + 1) * n + c] : 0.0f;
+        sT[kp * NS2 + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    }
+    for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
+        sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
+        sb[N + i] = i < n ? hd.b_h[n + i] + (proj ? hd.b_i[n + i] : 0.0f) : 0.0f;
+        sb[2 * N + i] = i < n ? hd.b_h[2 * n + i] : 0.0f;
+        sb[3 * N + i] = i < n && proj ? hd.b_i[2 * n + i] : 0.0f;
+    }
+    float *ss = sb + 4 * N + warp * 16 * SW;             // start states of this warp's chains
+    if constexpr (C::SS_GLOBAL) ss = a.starts + ((size_t)hd.first_edge + (size_t)blockIdx.x * nwarps + warp) * 16 * SW;
+    pdl_prologue();
+    if (*(volatile int *)&st->done) return;
+    __syncthreads();
+
+    const int burn = a.burn;
+    const long long grp = (long long)blockIdx.x * nwarps + warp;
+    unsigned mb = 0u, mis = 0u, mb_end = 0u, mis_end = 0u;
+
+    if (grp < groups) {
+        // ---- rows g and g + 8 of this lane: chain c of sequence (b, phase); scan position q is time step len - 1 - q
+        int tt[2], t_end[2], len[2];
+        const float *yp[2], *xp[2], *gp[2], *y0p[2];     // pointers at scan position tt (not dereferenced outside the sequence)
+        long long row[2];                                // row of the scan position in [B,T]
+        bool next[2];
+        const long long ys = (long long)s * H * n, xs = (long long)s * (proj ? m : H * 3 * n);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const long long gid = grp * 16 + g + 8 * h;
+            const long long q = gid < total ? gid / nchain : 0;
+            const int c = gid < total ? (int)(gid - q * nchain) : 0;
+            const long long b = q / s;
+            const int ph = (int)(q - b * s);
+            len[h] = gid < total ? (a.T - ph + s - 1) / s : 0;
+            t_end[h] = min(len[h], (c + 1) * L);
+            if (c * L >= len[h]) t_end[h] = 0;
+            next[h] = (c + 1) * L < len[h];
+            tt[h] = c * L - burn;
+            const long long e = b * a.T + ph + (long long)(len[h] - 1 - tt[h]) * s;
+            row[h] = e;
+            yp[h] = a.y + (e * H + blockIdx.y) * n;
+            gp[h] = a.gy + (e * H + blockIdx.y) * n;
+            xp[h] = proj ? a.x + e * m : a.u + (e * H + blockIdx.y) * 3 * n;
+            y0p[h] = a.y0 + ((size_t)b * H + blockIdx.y) * n;
+        }
+        // boundaries behind rows g, g + 8 and the one before row 0: close enough to the first time step for dy0 to feel them
+        const int reach = DY0_REACH * burn;
+        const bool near[2] = {len[0] - t_end[0] < reach, len[1] - t_end[1] < reach};
+        const bool near_prev = __shfl_sync(0xffffffffu, (int)(len[0] - (tt[0] + burn) < reach), 0) != 0;
+        // (a warp whose chains are all first ones has no burn-in: its earliest position is -burn)
+        const int tmax = __reduce_max_sync(0xffffffffu, max(t_end[0] > 0 ? tt[0] : -burn, t_end[1] > 0 ? tt[1] : -burn));
+        const int s_first = tmax <= -burn ? burn : 0;
+        const int s_end = __reduce_max_sync(0xffffffffu, max(t_end[0] > 0 ? t_end[0] - tt[0] : 0, t_end[1] > 0 ? t_end[1] - tt[1] : 0));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { tt[h] += s_first; row[h] -= (long long)s_first * s; yp[h] -= s_first * ys; gp[h] -= s_first * ys; xp[h] -= s_first * xs; }
+
+        auto ld2 = [&](const float *p, int col, int width) -> float2 {
+            if constexpr (V2) {
+                return col < width ? *reinterpret_cast<const float2 *>(p + col) : make_float2(0.0f, 0.0f);
+            } else {
+                return make_float2(col < width ? p[col] : 0.0f, col + 1 < width ? p[col + 1] : 0.0f);
+            }
+        };
+        const bool xv2 = (m & 1) == 0 && ((uintptr_t)a.x & 7) == 0;
+        auto ldx = [&](const float *p, int col) -> float2 {
+            if (xv2) return col < m ? __ldg(reinterpret_cast<const float2 *>(p + col)) : make_float2(0.0f, 0.0f);
+            return make_float2(col < m ? __ldg(p + col) : 0.0f, col + 1 < m ? __ldg(p + col + 1) : 0.0f);
+        };
+        // at scan position tt: the state before it (y0 before the first time step), dL/dy
+        auto load_h = [&](float (&dst)[NT][4]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool in = tt[h] >= 0 && tt[h] < t_end[h];
+                const float *p = tt[h] == len[h] - 1 ? y0p[h] : yp[h] - ys;
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float2 v = in ? ld2(p, 8 * j + 2 * t, n) : make_float2(0.0f, 0.0f);
+                    dst[j][2 * h] = v.x; dst[j][2 * h + 1] = v.y;
+                }
+            }
+        };
+        auto load_g = [&](float (&dst)[NT][4]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool in = tt[h] >= 0 && tt[h] < t_end[h];
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float2 v = in ? ld2(gp[h], 8 * j + 2 * t, n) : make_float2(0.0f, 0.0f);
+                    dst[j][2 * h] = v.x; dst[j][2 * h + 1] = v.y;
+                }
+            }
+        };
+        float hp[NT][4], gy[NT][4], d[NT][4];            // d: mu
+        load_h(hp);
+        load_g(gy);
+#pragma unroll
+        for (int j = 0; j < NT; ++j) { d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.0f; }
+
+#pragma unroll 1
+        for (int step = s_first; step < s_end; ++step) {
+            if (step == burn) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    *reinterpret_cast<float2 *>(ss + g * SW + 8 * j + 2 * t) = make_float2(d[j][0], d[j][1]);
+                    *reinterpret_cast<float2 *>(ss + (g + 8) * SW + 8 * j + 2 * t) = make_float2(d[j][2], d[j][3]);
+                }
+            }
+            const bool act[2] = {tt[0] >= 0 && tt[0] < t_end[0], tt[1] >= 0 && tt[1] < t_end[1]};
+            // ---- input half of the gates: u from memory, or x contracted here
+            float xr[NT][4], xz[NT][4], xn[NT][4];
+            if (proj) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] = 0.0f; xz[j][q] = 0.0f; xn[j][q] = 0.0f; }
+                float2 x0 = act[0] ? ldx(xp[0], 2 * t) : make_float2(0.0f, 0.0f);
+                float2 x1 = act[1] ? ldx(xp[1], 2 * t) : make_float2(0.0f, 0.0f);
+#pragma unroll 1
+                for (int kk = 0; kk < kx; ++kk) {
+                    unsigned ah[4], al[4];
+                    split_tf32(x0.x, ah[0], al[0]);
+                    split_tf32(x1.x, ah[1], al[1]);
+                    split_tf32(x0.y, ah[2], al[2]);
+                    split_tf32(x1.y, ah[3], al[3]);
+                    if (kk + 1 < kx) {
+                        x0 = act[0] ? ldx(xp[0], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
+                        x1 = act[1] ? ldx(xp[1], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
+                    }
+                    const float4 *q0 = sI + (4 * kk + t) * NS + g;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        {
+#pragma unroll
+                            for (int gate = 0; gate < 3; ++gate) {
+                                const float4 w = q0[gate * N + 8 * j];
+                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                                float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
+                                mma_tf32(acc, al, bh, acc);
+                                mma_tf32(acc, ah, bl, acc);
+                                mma_tf32(acc, ah, bh, acc);
+                            }
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const int col = 8 * j + 2 * t;
+                        const bool on = act[h] && col < n;
+                        const float2 vr = on ? ld2(xp[h], col, n) : make_float2(0.0f, 0.0f);
+                        const float2 vz = on ? ld2(xp[h] + n, col, n) : make_float2(0.0f, 0.0f);
+                        const float2 vn = on ? ld2(xp[h] + 2 * n, col, n) : make_float2(0.0f, 0.0f);
+                        xr[j][2 * h] = vr.x; xr[j][2 * h + 1] = vr.y;
+                        xz[j][2 * h] = vz.x; xz[j][2 * h + 1] = vz.y;
+                        xn[j][2 * h] = vn.x; xn[j][2 * h + 1] = vn.y;
+                    }
+            }
+            // ---- hidden half, gates, lambda and the pre-activation gradients, one block of eight columns at a time
+            float p[3][NT][4], zl[NT][4];
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                float (&hr)[4] = xr[j], (&hz)[4] = xz[j];
+                float hq[4] = {0.f, 0.f, 0.f, 0.f};
+                const float4 *q0 = sH + t * NS + 8 * j + g;
+#pragma unroll
+                for (int kk = 0; kk < NT; ++kk) {
+                    unsigned ah[4], al[4];
+                    split_tf32(hp[kk][0], ah[0], al[0]); split_tf32(hp[kk][2], ah[1], al[1]);
+                    split_tf32(hp[kk][1], ah[2], al[2]); split_tf32(hp[kk][3], ah[3], al[3]);
+#pragma unroll
+                    for (int gate = 0; gate < 3; ++gate) {
+                        const float4 w = q0[4 * kk * NS + gate * N];
+                        const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                        float (&acc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
+                        mma_tf32(acc, al, bh, acc);
+                        mma_tf32(acc, ah, bl, acc);
+                        mma_tf32(acc, ah, bh, acc);
+                    }
+                }
+                const int col = 8 * j + 2 * t;
+                const float2 bR = *reinterpret_cast<const float2 *>(sb + col), bZ = *reinterpret_cast<const float2 *>(sb + N + col);
+                const float2 bQ = *reinterpret_cast<const float2 *>(sb + 2 * N + col), bN = *reinterpret_cast<const float2 *>(sb + 3 * N + col);
+                const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 h2 = make_float2(hp[j][2 * h], hp[j][2 * h + 1]);
+                    const float2 l2 = fadd2(make_float2(gy[j][2 * h], gy[j][2 * h + 1]), make_float2(d[j][2 * h], d[j][2 * h + 1]));
+                    const float2 q = fadd2(make_float2(hq[2 * h], hq[2 * h + 1]), bQ);
+                    const float2 r = sigmoid2_gate(fadd2(make_float2(hr[2 * h], hr[2 * h + 1]), bR));
+                    const float2 z = sigmoid2_gate(fadd2(make_float2(hz[2 * h], hz[2 * h + 1]), bZ));
+                    const float2 c = tanh2_gate(ffma2(r, q, fadd2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), bN)));
+                    const float2 omz = ffma2(z, mone, one), omr = ffma2(r, mone, one);
+                    const float2 pz = fmul2(fmul2(fmul2(ffma2(c, mone, h2), z), omz), l2);
+                    const float2 pa = fmul2(fmul2(omz, ffma2(fmul2(c, mone), c, one)), l2);          // w.r.t. W_in x + b_in
+                    const float2 pn = fmul2(pa, r);                                                  // w.r.t. W_hn h + b_hn
+                    const float2 pr = fmul2(fmul2(pn, q), omr);
+                    const float2 zz = fmul2(z, l2);
+                    p[0][j][2 * h] = pr.x; p[0][j][2 * h + 1] = pr.y;
+                    p[1][j][2 * h] = pz.x; p[1][j][2 * h + 1] = pz.y;
+                    p[2][j][2 * h] = pn.x; p[2][j][2 * h + 1] = pn.y;
+                    zl[j][2 * h] = zz.x; zl[j][2 * h + 1] = zz.y;
+                    if (step >= burn && act[h]) {
+                        if (col < n) mb = max(mb, __float_as_uint(fabsf(l2.x)));
+                        if (col + 1 < n) mb = max(mb, __float_as_uint(fabsf(l2.y)));
+                        const long long o = row[h] * H + blockIdx.y;
+                        auto st2 = [&](float *dst, float2 v) {
+                            if constexpr (V2) { if (col < n) *reinterpret_cast<float2 *>(dst) = v; }
+                            else { if (col < n) dst[0] = v.x; if (col + 1 < n) dst[1] = v.y; }
+                        };
+                        if (a.lam) {
+                            st2(a.lam + o * n + col, l2);
+                        } else {
+                            float *gi = a.dGi + o * 3 * n + col, *gh = a.dGh + o * 3 * n + col;
+                            st2(gi, pr); st2(gi + n, pz); st2(gi + 2 * n, pa);
+                            st2(gh, pr); st2(gh + n, pz); st2(gh + 2 * n, pn);
+                        }
+                    }
+                }
+            }
+            // ---- advance; the next position's state and dL/dy are requested while p W_h runs
+#pragma unroll
+            for (int h = 0; h < 2; ++h) { ++tt[h]; row[h] -= s; yp[h] -= ys; gp[h] -= ys; xp[h] -= xs; }
+            if (step + 1 < s_end) { load_h(hp); load_g(gy); }
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                float acc[4] = {zl[j][0], zl[j][1], zl[j][2], zl[j][3]}, cr[4] = {0.f, 0.f, 0.f, 0.f};
+                const float4 *q0 = sT + t * NS2 + 8 * j + g;
+#pragma unroll
+                for (int gate = 0; gate < 3; ++gate)
+#pragma unroll
+                    for (int kk = 0; kk < NT; ++kk) {
+                        unsigned ph[4], pl[4];
+                        split_tf32(p[gate][kk][0], ph[0], pl[0]); split_tf32(p[gate][kk][2], ph[1], pl[1]);
+                        split_tf32(p[gate][kk][1], ph[2], pl[2]); split_tf32(p[gate][kk][3], ph[3], pl[3]);
+                        const float4 w = q0[(gate * N / 2 + 4 * kk) * NS2];
+                        const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                        mma_tf32(cr, pl, bh, cr);
+                        mma_tf32(cr, ph, bl, cr);
+                        mma_tf32(acc, ph, bh, acc);
+                    }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? acc[q] + cr[q] : d[j][q];
+            }
+        }
+        // ---- the state that leaves the first time step: the gradient w.r.t. y0
+        if (a.dy0) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (t_end[h] > 0 && !next[h]) {
+                    const long long q = (grp * 16 + g + 8 * h) / nchain;
+                    float *o = a.dy0 + (a.dy0_by_head ? q * H + blockIdx.y : hd.first_seq + q) * n;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const int col = 8 * j + 2 * t;
+                        mb_end = max(mb_end, max(__float_as_uint(fabsf(d[j][2 * h])), __float_as_uint(fabsf(d[j][2 * h + 1]))));
+                        if (col < n) o[col] = d[j][2 * h];
+                        if (col + 1 < n) o[col + 1] = d[j][2 * h + 1];
+                    }
+                }
+        }
+        // ---- boundaries: this row's end state against the state its successor assumed
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = g + 8 * h;
+            if (next[h] && row < 15) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const float2 v = *reinterpret_cast<const float2 *>(ss + (row + 1) * SW + 8 * j + 2 * t);
+                    const unsigned q = max(absdiff_bits(v.x, d[j][2 * h]), absdiff_bits(v.y, d[j][2 * h + 1]));
+                    mis = max(mis, q);
+                    if (near[h]) mis_end = max(mis_end, q);
+                }
+            }
+        }
+        const bool near_next = __shfl_sync(0xffffffffu, (int)near[1], 28) != 0;
+        const bool has_next = __shfl_sync(0xffffffffu, (int)next[1], 28) != 0;                   // row 15
+        const bool has_prev = __shfl_sync(0xffffffffu, (int)(t_end[0] > 0 && grp > 0 && (grp * 16) % nchain != 0), 0) != 0;   // row 0
+        __syncwarp();
+        if (has_next) {                                  // row 15's end state takes the place of row 15's start state
+            if (g == 7) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    *reinterpret_cast<float2 *>(ss + 15 * SW + 8 * j + 2 * t) = make_float2(d[j][2], d[j][3]);
+            }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {           // 0: left of the boundary behind this group, 1: right of the one before it
+            if (side == 0 ? !has_next : !has_prev) continue;
+            const size_t edge = (size_t)hd.first_edge + (size_t)grp - side;
+            const float *own = ss + (side == 0 ? 15 : 0) * SW;
+            float *slot = a.edge + edge * 2 * n;
+            for (int i = lane; i < n; i += 32) __stcg(slot + side * n + i, own[i]);
+            __threadfence();
+            __syncwarp();
+            unsigned old = 0;
+            if (lane == 0) old = atomicAdd(a.edge_flag + edge, 1u);
+            old = __shfl_sync(0xffffffffu, old, 0);
+            if (old == 1u) {
+                __threadfence();
+                const bool near_here = side == 0 ? near_next : near_prev;
+                for (int i = lane; i < n; i += 32) {
+                    const unsigned q = absdiff_bits(own[i], __ldcg(slot + (side ^ 1) * n + i));
+                    mis = max(mis, q);
+                    if (near_here) mis_end = max(mis_end, q);
+                }
+                if (lane == 0) a.edge_flag[edge] = 0u;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+        mis = max(mis, __shfl_xor_sync(0xffffffffu, mis, o));
+        mb_end = max(mb_end, __shfl_xor_sync(0xffffffffu, mb_end, o));
+        mis_end = max(mis_end, __shfl_xor_sync(0xffffffffu, mis_end, o));
+    }
+    if (lane == 0) {
+        if (mb) atomicMax(&st->err_bits, mb);
+        if (mis) atomicMax(&st->mis_bits, mis);
+        if (mb_end) atomicMax(&st->top_end_bits, mb_end);
+        if (mis_end) atomicMax(&st->mis_end_bits, mis_end);
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(&st->exit_counter, 1u);
+        if (prev + 1u == nctas) {
+            __threadfence();
+            st->exit_counter = 0u;
+            adjoint_decide(st, a.eta, a.dy0 != nullptr);
+        }
+    }
+}
+
+}  // namespace deer

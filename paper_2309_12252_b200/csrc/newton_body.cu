@@ -103,6 +103,24 @@ static int longest(int T, const int *strides, int H)
     return w;
 }
 
+// One-phase plans: the whole problem is one wave of chains -- the shortest chain length for which it is, but no chains that
+// would spend most of their steps on the burn-in.
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t smem, int B, int T, const int *strides, int H)
+{
+    const int Tmax = longest(T, strides, H);
+    p->NC = 0;
+    p->whole_loop = false;
+    p->warps = warps;
+    p->smem = smem;
+    const long long cap = (long long)sm_count() * occupancy_of(kern, 32 * warps, smem);      // CTAs of one wave
+    const long long positions = (long long)B * T * H;
+    int L = (int)std::max<long long>(16, positions / (cap * warps * 16));
+    while (L < Tmax && count_ctas(B, T, strides, H, L, 16 * warps, 16).ctas > cap) L += std::max(1, L / 64);
+    const Count c = count_ctas(B, T, strides, H, L, 16 * warps, 16);
+    p->L = L; p->max_ctas = c.worst; p->edges = c.edges;
+    p->waves = (float)c.ctas / (float)cap;
+}
+
 bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool have_u, const int *strides, int H)
 {
     const int kx = have_u ? 0 : (m + 7) / 8, sms = sm_count(), Tmax = longest(T, strides, H);
@@ -133,22 +151,47 @@ bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool hav
             if (c.ctas <= sms || L >= Tmax) return true;
         }
     }
-    p->NC = 0;
-    p->whole_loop = false;
-    p->warps = k.one_warps;
-    p->smem = k.one_smem(kx);
-    const long long cap = (long long)sms * occupancy_of((const void *)k.one, 32 * p->warps, p->smem);   // CTAs of one wave
-    // The whole problem is one wave of chains: the shortest chain length for which it is, but no chains that would spend
-    // most of their steps on the burn-in.
-    const long long positions = (long long)B * T * H;
-    int L = (int)std::max<long long>(16, positions / (cap * p->warps * 16));
-    while (L < Tmax && count_ctas(B, T, strides, H, L, 16 * p->warps, 16).ctas > cap) L += std::max(1, L / 64);
-    const Count c = count_ctas(B, T, strides, H, L, 16 * p->warps, 16);
-    p->L = L; p->max_ctas = c.worst; p->edges = c.edges;
-    p->waves = (float)c.ctas / (float)cap;
+    one_wave_of_chains(p, (const void *)k.one, k.one_warps, k.one_smem(kx), B, T, strides, H);
     // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
-    p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * L) : std::max(320, 8 * L);
+    p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
     return true;
+}
+
+bool adjoint_supported(int n, int m, bool have_u)
+{
+    if (n < 1 || n > 64) return false;
+    return have_u || (m <= 64 && pick(n, false).adj_smem((m + 7) / 8) <= BODY_SMEM_MAX);
+}
+
+bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const int *strides, int H)
+{
+    if (!adjoint_supported(n, m, have_u)) return false;
+    const BodyKernels k = pick(n, (n & 1) == 0);
+    if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
+    one_wave_of_chains(p, (const void *)k.adj, k.one_warps, k.adj_smem(have_u ? 0 : (m + 7) / 8), B, T, strides, H);
+    return true;
+}
+
+size_t adjoint_starts(int n) { return n > 48 ? 16 * (size_t)((n + 7) / 8 * 8 + 4) : 0; }
+
+// Where the kernels that multiply the Jacobians out are tuned (powers of two), half a wave of chains or more; for n >= 32 their
+// 3 x TF32 products are so much more work that a part of a wave is enough.  n <= 4 pads to 8 columns and stays with its own.
+// (B200, us per gradient, here / there: n = 8, B = 16, T = 1e4 117 / 92; n = 32, T = 1e5 2210 / 5046)
+bool adjoint_suits(const BodyPlan &p, int n)
+{
+    if ((n & (n - 1)) != 0) return true;
+    return n <= 4 ? false : n <= 16 ? p.waves >= 0.6f : p.waves >= 0.1f;
+}
+
+int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
+{
+    const bool aligned = (((uintptr_t)a.y | (uintptr_t)a.gy | (uintptr_t)a.y0 | (uintptr_t)a.u | (uintptr_t)a.lam | (uintptr_t)a.dGi |
+                           (uintptr_t)a.dGh) & 7) == 0;
+    const BodyKernels k = pick(a.n, (a.n & 1) == 0 && aligned);
+    occupancy_of((const void *)k.adj, 32 * p.warps, p.smem);
+    DEER_KERNEL("newton_adjoint_kernel", st,
+                k.adj<<<dim3((unsigned)p.max_ctas, (unsigned)a.H), 32 * p.warps, p.smem, st>>>(a));
+    return DEER_OK;
 }
 
 // Measured lines (B200, m = n unless stated, us per evaluation: two-phase / one-phase / multiplied-out kernels):

@@ -9,6 +9,7 @@ struct BodyHead {
     const float *W_i, *W_h, *b_i, *b_h;
     int stride;              // a head of stride s runs s interleaved sequences per batch entry
     int first_edge;          // offset of the head's chain groups in the edge buffers
+    long long first_seq;     // sequences of the heads before this one (adjoint: rows of dy0)
 };
 
 struct BodyArgs {
@@ -29,15 +30,34 @@ struct BodyArgs {
     unsigned long long *words;   // [H][2][CTAs][2]  maxima exchanged at the end of a body (whole-loop launches)
 };
 
+// The adjoint solve of the gradient as one launch (newton_adjoint.cuh).
+struct AdjArgs {
+    BodyHead h0;
+    const BodyHead *heads;
+    const float *x, *u, *y0; // as in BodyArgs
+    const float *y, *gy;     // [B,T,H,n] trajectory, dL/dy
+    float *lam;              // [B,T,H,n] out: lambda; or nullptr:
+    float *dGi, *dGh;        // [B,T,H,3n] out: gradients w.r.t. the input-side and hidden-side pre-activations
+    float *dy0;              // or nullptr; row b * H + head (dy0_by_head), else first_seq + sequence
+    int dy0_by_head;
+    int B, T, n, m, H, L, burn;
+    float eta;               // largest boundary mismatch that is accepted, as a part of max|lambda|
+    StatusBlock *st;         // [H]; done = 1 where the launch has done the work (it returns at once where it is set)
+    float *edge;
+    unsigned *edge_flag;
+    float *starts;           // [groups][16][n + 4 of the padded size], n > 48 only (adjoint_starts)
+};
+
 constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2;       // StatusBlock::done: the loop ended / this form gives up
 
 // The kernels of one padded state size (newton_kernels.cu).
 struct BodyKernels {
     void (*one)(BodyArgs);                     // one-phase (newton_body.cuh)
     void (*seg)(BodyArgs, int, int);           // two-phase (newton_segment.cuh)
+    void (*adj)(AdjArgs);                      // adjoint, one-phase (newton_adjoint.cuh)
     int one_warps, seg_warps, nc_max;
     size_t slot_bytes;
-    size_t (*one_smem)(int kx), (*seg_fixed)(int kx);
+    size_t (*one_smem)(int kx), (*seg_fixed)(int kx), (*adj_smem)(int kx);
 };
 
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
@@ -66,5 +86,16 @@ bool body_suits(const BodyPlan &p, int n);
 int body_first_burn(int n, float tol);
 float body_eta(int n, float tol);
 int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st);
+
+bool adjoint_supported(int n, int m, bool have_u);
+bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const int *strides, int H);
+// floats of AdjArgs::starts per chain group (0: not used)
+size_t adjoint_starts(int n);
+bool adjoint_suits(const BodyPlan &p, int n);
+int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st);
+// Burn-ins that are tried one after the other, and the accuracy asked of the boundaries (a one-shot solve: fp32 level).
+constexpr int ADJ_TRIES = 2;
+constexpr int ADJ_BURN[ADJ_TRIES] = {44, 128};
+constexpr float ADJ_ETA = 4e-6f;
 
 }  // namespace deer

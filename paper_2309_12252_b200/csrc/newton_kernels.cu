@@ -1,5 +1,6 @@
 // The one-launch Newton kernels of one padded state size: compiled once per size with -DBODY_N=8, 16, ... 64 (build.py).
 #include "newton_segment.cuh"
+#include "newton_adjoint.cuh"
 
 #ifndef BODY_N
 #error "BODY_N: state size, a multiple of 8 up to 64"
@@ -17,11 +18,13 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
         // single-TF32 products with the update: the sizes whose solve has always run in reduced precision
         if (v2 && !exact) { k.one = newton_body_kernel<N, true, false>; k.seg = newton_segment_kernel<N, true, false>; }
     }
+    k.adj = v2 ? newton_adjoint_kernel<N, true> : newton_adjoint_kernel<N, false>;
     k.one_warps = N > 32 ? 8 : 4;
     k.seg_warps = Seg<N>::WARPS;
     k.nc_max = Seg<N>::NC_MAX;
     k.slot_bytes = Seg<N>::SZ * sizeof(float);
     k.one_smem = [](int kx) { return Body<N>::smem(N > 32 ? 8 : 4, kx); };
+    k.adj_smem = [](int kx) { return Adj<N>::smem(N > 32 ? 8 : 4, kx); };
     k.seg_fixed = [](int kx) { return Seg<N>::fixed(kx); };
     return k;
 }

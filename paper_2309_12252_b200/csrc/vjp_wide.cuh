@@ -11,6 +11,7 @@ namespace deer {
 template <int N>
 __global__ void __launch_bounds__(256) vjp_cell_wide_kernel(VjpArgs a)
 {
+    if (loop_ended(a.st)) return;
     using C = CellWide<N>;
     extern __shared__ __align__(16) float sm[];
     float *sWT = sm;                           // [N][3N]
@@ -291,8 +292,9 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
 template <int NB_MAX, bool WT_GIVEN>
 __global__ void __launch_bounds__(256) affine_mma_kernel(const float *__restrict__ in, const float *__restrict__ W,
                                                          const float *__restrict__ bias, float *__restrict__ out,
-                                                         size_t N, int K, int NOUT)
+                                                         size_t N, int K, int NOUT, const StatusBlock *st)
 {
+    if (loop_ended(st)) return;
     extern __shared__ __align__(16) float smw[];
     const int NS = NOUT + 4;                  // row stride: 2 * NS = 8 (mod 32) words
     float *sBh = smw, *sBl = smw + (size_t)K * NS;
