@@ -25,6 +25,8 @@
 #include "cell_wide.cuh"
 #include "vjp_wide.cuh"
 #include "newton_body.h"
+#include "affine_tiled.cuh"
+#include "multihead.cuh"
 
 namespace deer {
 
@@ -498,6 +500,19 @@ static int run_affine(const float *in, const float *W, const float *bias, float 
     return DEER_OK;
 }
 
+template <bool WT>
+static int launch_affine_tiled(const float *in, const float *W, const float *bias, float *out, size_t N, int K, int nout, cudaStream_t st)
+{
+    int rc;
+    if ((rc = opt_in_smem((const void *)affine_tiled_kernel<WT>, AffineTile::SMEM)) != DEER_OK) return rc;
+    const int vec = K % 4 == 0 && (!WT || nout % 4 == 0) && (((uintptr_t)in | (uintptr_t)W) & 15) == 0;
+    const size_t blocks = ((N + AffineTile::MT - 1) / AffineTile::MT) * ((nout + AffineTile::NT - 1) / AffineTile::NT);
+    if (blocks > 0x7fffffffu) return DEER_ERR_UNSUPPORTED_N;
+    DEER_KERNEL("affine_tiled_kernel", st, (affine_tiled_kernel<WT><<<(unsigned)blocks, AffineTile::THREADS, AffineTile::SMEM, st>>>(
+                                               in, W, bias, out, N, K, nout, vec)));
+    return DEER_OK;
+}
+
 static int run_proj(const deer_gru_params *p, const float *x, float *u, size_t N, cudaStream_t st, const StatusBlock *unless = nullptr)
 {
     const int n3 = 3 * p->n, m = p->m;
@@ -809,7 +824,20 @@ struct MhWs {
     float *xs, *y0s, *ys, *gys, *dxs, *dy0s;
     void *inner;
     size_t inner_bytes, bytes;
+    // all heads as one batch
+    BodyHead *heads;
+    MhGrad *grads;
+    StatusBlock *st;         // [H]
+    float *Wc, *bc;          // input weights and biases side by side
+    float *u, *yalt, *dGi, *dGh, *edge, *starts, *dy0all, *partial;
+    unsigned *edge_flag;
+    unsigned long long *words;
+    size_t groups;
 };
+
+constexpr int MH_P_IN = 32;  // slices of the positions in the reduction of the stacked input weights
+// ... and of a head's hidden weights: about 16 CTAs per SM over all heads
+static int mh_p_hidden(int H) { return std::max(8, std::min(128, 2368 / H)); }
 
 static MhWs carve_mh(void *ws, int H, const int *strides, int B, int T, int n, int m)
 {
@@ -834,6 +862,30 @@ static MhWs carve_mh(void *ws, int H, const int *strides, int B, int T, int n, i
     w.dy0s = cv.take<float>(maxB * n);
     w.inner_bytes = inner;
     w.inner = cv.take<char>(inner);
+    const size_t N = (size_t)B * T, n3 = 3 * (size_t)n;
+    size_t agroups = 0, seqs = 0;
+    w.groups = 0;
+    for (int h = 0; h < H; ++h) {
+        const int Bs = B * strides[h], Tp = (T + strides[h] - 1) / strides[h];
+        w.groups += body_groups_max(Bs, Tp) + 1;
+        agroups += adjoint_groups_max(Bs, Tp);
+        seqs += (size_t)Bs;
+    }
+    w.heads = cv.take<BodyHead>(H);
+    w.grads = cv.take<MhGrad>(H);
+    w.st = cv.take<StatusBlock>(H);
+    w.Wc = cv.take<float>(H * n3 * m);
+    w.bc = cv.take<float>(H * n3);
+    w.u = cv.take<float>(N * H * n3);
+    w.yalt = cv.take<float>(N * H * n);
+    w.dGi = cv.take<float>(N * H * n3);
+    w.dGh = cv.take<float>(N * H * n3);
+    w.edge = cv.take<float>(w.groups * 2 * n);
+    w.edge_flag = cv.take<unsigned>(w.groups);
+    w.words = cv.take<unsigned long long>((size_t)4 * num_sms());
+    w.starts = cv.take<float>(agroups * adjoint_starts(n));
+    w.dy0all = cv.take<float>(seqs * n);
+    w.partial = cv.take<float>(std::max((size_t)MH_P_IN * H * n3 * (m + 1), (size_t)mh_p_hidden(H) * H * n3 * (n + 1)));
     w.bytes = cv.off;
     return w;
 }
@@ -1013,6 +1065,12 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     return DEER_OK;                                      // (hs->done == BODY_FALL_BACK)
 }
 
+static int eval_status(float e, float tol)
+{
+    if (!isfinite(e)) return DEER_NONFINITE;
+    return e > tol && !(tol < 0.0f) ? DEER_NOT_CONVERGED : DEER_OK;
+}
+
 // copy_st / copy_ev (optional): the stream the copy to y_host is enqueued on, and an event to order it behind `st`.
 // y_host (optional, host memory): the result is also copied there.  The copy is enqueued behind every
 // group of bodies, after a device-side selection of the buffer that holds the current iterate, so that
@@ -1021,7 +1079,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
                          float tol, int max_iter, float *y, int *iters, float *err,
                          float *err_trace, void *ws, size_t ws_bytes, int flags, cudaStream_t st,
                          float *y_host = nullptr, float *err_b = nullptr, unsigned long long *err_argmax = nullptr,
-                         cudaStream_t copy_st = nullptr, cudaEvent_t copy_ev = nullptr)
+                         cudaStream_t copy_st = nullptr, cudaEvent_t copy_ev = nullptr, int bodies_done = 0)
 {
     const int n = p->n, m = p->m;
     EvalWs w = carve_eval(ws, B, T, n, m);
@@ -1048,7 +1106,11 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
                         "copy result to host");
         return DEER_OK;
     };
-    const bool one_launch = body_takes(n, m, flags);
+    // bodies_done > 0: y holds the iterate after that many bodies of the one-launch form, which has given up
+    hs.iters = bodies_done;
+    if (bodies_done & 1)
+        DEER_CHECK_CUDA(cudaMemcpyAsync(w.yalt, y, N * n * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy iterate");
+    const bool one_launch = bodies_done == 0 && body_takes(n, m, flags);
     HostSlot slot(one_launch);
     if (one_launch) {
         if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, copy_out)) != DEER_OK) return rc;
@@ -1162,12 +1224,9 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
         DEER_CHECK_CUDA(cudaMemcpyAsync(err_trace, w.trace, sizeof(float) * (size_t)(k < ERR_TRACE_CAP ? k : ERR_TRACE_CAP),
                                         cudaMemcpyDeviceToHost, st), "read trace");
     if (((k & 1) && !y_host) || (err_trace && !trace_here)) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
-    int status = DEER_OK;
-    if (!isfinite(e)) status = DEER_NONFINITE;
-    else if (e > tol && !(tol < 0.0f)) status = DEER_NOT_CONVERGED;
     if (iters) *iters = k;
     if (err) *err = e;
-    return status;
+    return eval_status(e, tol);
 }
 
 // cell VJP, parameter-gradient slices and dx in one pass (n, m in {1,2,4,8}); P = slices written
@@ -1810,6 +1869,155 @@ static std::vector<int> mh_order(const int *strides, int H)
     return order;
 }
 
+// ---- all heads in one batch: the body, adjoint and contraction kernels take the head as a grid dimension
+static bool mh_batched(int n, int H, int flags)
+{
+    return H <= 1024 && body_supported(n, 1, true) &&
+           !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS));
+}
+
+// The heads' table on the device; first_edge by the units of `unit` chains of length L (0: none).
+static int mh_table(const deer_gru_params *heads, const int *strides, int H, int B, int T, int L, int unit, const MhWs &w, cudaStream_t st)
+{
+    std::vector<BodyHead> t((size_t)H);
+    long long edge = 0, seq = 0;
+    for (int h = 0; h < H; ++h) {
+        const int s = strides[h], Tp = (T + s - 1) / s;
+        t[h] = BodyHead{heads[h].W_i, heads[h].W_h, heads[h].b_i, heads[h].b_h, s, (int)edge, seq};
+        if (unit) edge += ((long long)B * s * ((Tp + L - 1) / L) + unit - 1) / unit;
+        seq += (long long)B * s;
+    }
+    if ((size_t)edge > w.groups) return DEER_ERR_WORKSPACE;
+    DEER_CHECK_CUDA(cudaMemcpyAsync(w.heads, t.data(), sizeof(BodyHead) * (size_t)H, cudaMemcpyHostToDevice, st), "copy heads");
+    return DEER_OK;
+}
+
+// u = x W_i^T + b_i of all heads: one contraction [N, m] x [m, H*3n]
+static int mh_project(const MhWs &w, const float *x, size_t N, int H, int n, int m, cudaStream_t st)
+{
+    DEER_KERNEL("mh_gather_kernel", st, mh_gather_kernel<<<mh_blocks((size_t)H * 3 * n * m), 256, 0, st>>>(w.heads, H, 3 * n, m, w.Wc, w.bc));
+    return launch_affine_tiled<false>(x, w.Wc, w.bc, w.u, N, m, H * 3 * n, st);
+}
+
+// The Newton loops of all heads; hs[h].done tells how head h ended (its iterate after hs[h].iters bodies is in y, or, where
+// that is odd, in w.yalt).
+static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int H, const float *x, const float *y0, int B, int T,
+                           float tol, int max_iter, float *y, const MhWs &w, int flags, cudaStream_t st, std::vector<StatusBlock> &hs)
+{
+    const int n = heads[0].n, m = heads[0].m;
+    const size_t N = (size_t)B * T;
+    int rc;
+    BodyPlan plan{};
+    // the two-phase kernel where it is the whole loop in one launch, else the one-phase kernel
+    if (!body_plan(&plan, true, B, T, n, m, true, strides, H) || !plan.whole_loop) {
+        plan = BodyPlan{};
+        if (!body_plan(&plan, false, B, T, n, m, true, strides, H)) return DEER_ERR_UNSUPPORTED_N;
+    }
+    if ((rc = mh_table(heads, strides, H, B, T, plan.L, plan.NC > 0 ? plan.NC : 16, w, st)) != DEER_OK) return rc;
+    StatusBlock init;
+    memset(&init, 0, sizeof(init));
+    init.max_iter = max_iter;
+    init.tol = tol;
+    init.burn = body_first_burn(n, tol);
+    const size_t nw = plan.whole_loop ? (size_t)plan.edges * n : 0, nflags = plan.whole_loop ? 0 : (size_t)plan.edges;
+    DEER_KERNEL("mh_begin_kernel", st, mh_begin_kernel<<<mh_blocks(nw + nflags + H), 256, 0, st>>>(
+                                           w.st, init, H, w.edge_flag, nflags, (unsigned long long *)w.edge, nw, w.words,
+                                           plan.whole_loop ? (size_t)4 * H * plan.max_ctas : 0));
+    if ((rc = mh_project(w, x, N, H, n, m, st)) != DEER_OK) return rc;
+    BodyArgs a{};
+    a.heads = w.heads;
+    a.u = w.u; a.y0 = y0;
+    a.buf[0] = y; a.buf[1] = w.yalt;
+    a.B = B; a.T = T; a.n = n; a.m = m; a.H = H; a.L = plan.L;
+    a.warm = (flags & DEER_FLAG_WARM_START) ? 1 : 0;
+    a.eta = body_eta(n, tol);
+    a.burn_cap = plan.burn_cap;
+    a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
+    hs.assign((size_t)H, StatusBlock{});
+    for (int group = 4, most = 0;; group = 2) {
+        for (int j = 0; j < (plan.whole_loop ? 1 : std::min(group, max_iter - most)); ++j)
+            if ((rc = launch_newton_body(a, plan, st)) != DEER_OK) return rc;
+        DEER_CHECK_CUDA(cudaMemcpyAsync(hs.data(), w.st, sizeof(StatusBlock) * (size_t)H, cudaMemcpyDeviceToHost, st), "read status");
+        DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+        bool all = true;
+        most = max_iter;                                 // bodies of the head that is least far
+        for (const StatusBlock &h : hs) {
+            if (h.flags & FLAG_TIMEOUT) return DEER_ERR_DEVICE_TIMEOUT;
+            if (!h.done) { all = false; most = std::min(most, h.iters); }
+        }
+        if (all) return DEER_OK;
+        if (plan.whole_loop) return DEER_ERR_DEVICE_TIMEOUT;
+    }
+}
+
+static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int H, const float *x, const float *y0, const float *y,
+                          const float *gy, int B, int T, const deer_gru_grads *dheads, float *dx, float *dy0, const MhWs &w,
+                          cudaStream_t st, bool *did)
+{
+    const int n = heads[0].n, m = heads[0].m, n3 = 3 * n;
+    const size_t N = (size_t)B * T;
+    *did = false;
+    int rc;
+    BodyPlan plan{};
+    if (!adjoint_plan(&plan, B, T, n, m, true, strides, H)) return DEER_OK;
+    if ((rc = mh_table(heads, strides, H, B, T, plan.L, 16, w, st)) != DEER_OK) return rc;
+    std::vector<MhGrad> gr((size_t)H);
+    for (int h = 0; h < H; ++h) gr[h] = MhGrad{dheads[h].dW_i, dheads[h].dW_h, dheads[h].db_i, dheads[h].db_h};
+    DEER_CHECK_CUDA(cudaMemcpyAsync(w.grads, gr.data(), sizeof(MhGrad) * (size_t)H, cudaMemcpyHostToDevice, st), "copy gradient table");
+    StatusBlock init;
+    memset(&init, 0, sizeof(init));
+    DEER_KERNEL("mh_begin_kernel", st, mh_begin_kernel<<<mh_blocks((size_t)plan.edges + H), 256, 0, st>>>(
+                                           w.st, init, H, w.edge_flag, (size_t)plan.edges, nullptr, 0, nullptr, 0));
+    if ((rc = mh_project(w, x, N, H, n, m, st)) != DEER_OK) return rc;
+    AdjArgs a{};
+    a.heads = w.heads;
+    a.u = w.u; a.y0 = y0; a.y = y; a.gy = gy;
+    a.dGi = w.dGi; a.dGh = w.dGh;
+    a.dy0 = dy0 ? w.dy0all : nullptr;
+    a.B = B; a.T = T; a.n = n; a.m = m; a.H = H; a.L = plan.L;
+    a.eta = ADJ_ETA;
+    a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = w.starts;
+    for (int k = 0; k < ADJ_TRIES; ++k) {
+        a.burn = ADJ_BURN[k];
+        if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
+    }
+    // dW_i, db_i of all heads: one contraction of dG_i [N, H*3n] with x [N, m]
+    WgradArgs wa{};
+    wa.dG = w.dGi; wa.V = x; wa.T = T; wa.n3 = H * n3; wa.K = m; wa.N = N;
+    const int P = (int)std::min(N, (size_t)MH_P_IN);
+    wa.slice = (N + P - 1) / P;
+    wa.partial = w.partial;
+    const int rows = std::min(192, wa.n3);
+    const dim3 grid(P, (m + 63) / 64, (wa.n3 + 191) / 192);
+    if ((((uintptr_t)x | (uintptr_t)w.dGi) & 15) == 0 && wa.n3 % 4 == 0 && m % 4 == 0) {
+        const size_t sm = wgrad_staged_smem(rows);
+        if ((rc = opt_in_smem((const void *)wgrad_mma_staged_kernel, sm)) != DEER_OK) return rc;
+        DEER_KERNEL("wgrad_mma_kernel", st, wgrad_mma_staged_kernel<<<grid, 32 * ((rows + 15) / 16), sm, st>>>(wa));
+    } else {
+        DEER_KERNEL("wgrad_mma_kernel", st, wgrad_mma_kernel<<<grid, 32 * ((rows + 15) / 16), 0, st>>>(wa));
+    }
+    const size_t outs = (size_t)H * n3 * (m + 1);
+    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs + 7) / 8), 256, 0, st>>>(w.partial, P, n3, m, H, w.grads, 0));
+    // dW_h, db_h: a contraction per head
+    WgradArgs wh{};
+    wh.dG = w.dGh; wh.V = y; wh.y0 = y0; wh.shifted = 1; wh.T = T; wh.n3 = n3; wh.K = n; wh.N = N;
+    const int Ph = (int)std::min(N, (size_t)mh_p_hidden(H));
+    wh.slice = (N + Ph - 1) / Ph;
+    wh.partial = w.partial;
+    wh.heads = w.heads; wh.H = H;
+    DEER_KERNEL("wgrad_mma_kernel", st, wgrad_mma_kernel<<<dim3(Ph, (n + 63) / 64, H), 32 * ((n3 + 15) / 16), 0, st>>>(wh));
+    const size_t outs_h = (size_t)H * n3 * (n + 1);
+    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs_h + 7) / 8), 256, 0, st>>>(w.partial, Ph, n3, n, H, w.grads, 1));
+    if (dx && (rc = launch_affine_tiled<true>(w.dGi, w.Wc, nullptr, dx, N, H * n3, m, st)) != DEER_OK) return rc;
+    if (dy0) DEER_KERNEL("mh_dy0_sum_kernel", st, mh_dy0_sum_kernel<<<mh_blocks((size_t)B * H * n), 256, 0, st>>>(w.heads, w.dy0all, dy0, B, T, n, H));
+    std::vector<StatusBlock> hs((size_t)H);
+    DEER_CHECK_CUDA(cudaMemcpyAsync(hs.data(), w.st, sizeof(StatusBlock) * (size_t)H, cudaMemcpyDeviceToHost, st), "read status");
+    DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+    *did = true;
+    for (const StatusBlock &h : hs) *did = *did && h.done == BODY_DONE;    // (a head whose Jacobians hardly decay: head by head)
+    return DEER_OK;
+}
+
 int deer_gru_multihead_eval(const deer_gru_params *heads, const int *strides, int H, const float *x, const float *y0,
                             int B, int T, float tol, int max_iter, float *y, int *iters, void *ws, size_t ws_bytes,
                             int flags, void *stream)
@@ -1822,22 +2030,43 @@ int deer_gru_multihead_eval(const deer_gru_params *heads, const int *strides, in
     MhWs w = carve_mh(ws, H, strides, B, T, n, m);
     if ((rc = check_ws(ws, ws_bytes, w.bytes)) != DEER_OK) return rc;
     int worst = DEER_OK;
+    std::vector<StatusBlock> hs;
+    const bool batched = mh_batched(n, H, flags);
+    if (batched) {
+        if ((rc = mh_eval_batched(heads, strides, H, x, y0, B, T, tol, max_iter, y, w, flags, st, hs)) != DEER_OK) return rc;
+        bool odd = false, all = true;
+        for (int h = 0; h < H; ++h) {
+            odd = odd || (hs[h].iters & 1);
+            if (hs[h].done != BODY_DONE) { all = false; continue; }
+            float e;
+            memcpy(&e, &hs[h].err_last_bits, sizeof(float));
+            worst = std::max(worst, eval_status(e, tol));
+            if (iters) iters[h] = hs[h].iters;
+        }
+        if (odd) DEER_KERNEL("mh_select_kernel", st, mh_select_kernel<<<mh_blocks((size_t)B * T * H * n), 256, 0, st>>>(w.st, y, w.yalt, (size_t)B * T, H, n));
+        if (all) {
+            if (odd) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+            return worst;
+        }
+    }
     int packed_stride = 1;                     // stride whose dense batch of x is in w.xs (stride 1: x itself)
     const std::vector<int> order = mh_order(strides, H);
     for (int oi = 0; oi < H; ++oi) {
         const int h = order[(size_t)oi];
         const int s = strides[h], Tp = (T + s - 1) / s, Bs = B * s;
+        if (batched && hs[h].done == BODY_DONE) continue;
+        const int k0 = batched ? hs[h].iters : 0;      // bodies done before the batched form gave this head up
         if (s != packed_stride) {              // heads of equal stride read the same dense batch of x
             { if ((rc = mh_pack(x, w.xs, B, T, s, Tp, m, m, 0, st)) != DEER_OK) return rc; }
             packed_stride = s;
         }
         const float *xs = s == 1 ? x : w.xs;
         DEER_KERNEL("mh_y0_pack_kernel", st, mh_y0_pack_kernel<<<mh_blocks((size_t)Bs * n), 256, 0, st>>>(y0, w.y0s, B, s, n, H, h));
-        if (flags & DEER_FLAG_WARM_START)
+        if ((flags & DEER_FLAG_WARM_START) || k0 > 0)
             { if ((rc = mh_pack(y, w.ys, B, T, s, Tp, n, H * n, h * n, st)) != DEER_OK) return rc; }
         int it = 0;
         rc = gru_eval_impl(&heads[h], xs, w.y0s, Bs, Tp, tol, max_iter, w.ys, &it, nullptr, nullptr, w.inner, w.inner_bytes,
-                           flags, st);
+                           flags, st, nullptr, nullptr, nullptr, nullptr, nullptr, k0);
         if (rc < 0) return rc;
         if (iters) iters[h] = it;
         if (rc > worst) worst = rc;
@@ -1860,6 +2089,11 @@ int deer_gru_multihead_vjp(const deer_gru_params *heads, const int *strides, int
     cudaStream_t st = (cudaStream_t)stream;
     MhWs w = carve_mh(ws, H, strides, B, T, n, m);
     if ((rc = check_ws(ws, ws_bytes, w.bytes)) != DEER_OK) return rc;
+    if (mh_batched(n, H, flags)) {
+        bool did = false;
+        if ((rc = mh_vjp_batched(heads, strides, H, x, y0, y, gy, B, T, dheads, dx, dy0, w, st, &did)) != DEER_OK) return rc;
+        if (did) return DEER_OK;
+    }
     unsigned timeout_flags = 0;
     int packed_stride = 1;                     // (stride 1: x itself)
     const std::vector<int> order = mh_order(strides, H);

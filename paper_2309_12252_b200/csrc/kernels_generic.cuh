@@ -5,6 +5,7 @@
 // where they apply.
 #pragma once
 #include "common.cuh"
+#include "newton_body.h"
 
 namespace deer {
 
@@ -642,6 +643,10 @@ struct WgradArgs {
     int shifted, T, n3, K, tile;
     size_t N, slice;
     float *partial;      // [P][n3*(K+1)]
+    // Multi-head unit (heads != nullptr, blockIdx.z = head): columns h*n3.. of dG [N, H*n3] with columns h*K.. of
+    // V = y [N, H*K], shifted by the head's stride; partial [H][P][n3*(K+1)].  Tensor-core kernels only.
+    const BodyHead *heads;
+    int H;
 };
 
 __global__ void wgrad_partial_kernel(WgradArgs a)

@@ -1,0 +1,82 @@
+// Multi-head unit as ONE batch over its heads (Sec. 4.4: the heads are independent): helpers around the body, adjoint and
+// contraction kernels, which take the heads as a second grid dimension.
+#pragma once
+#include "newton_body.h"
+#include "vjp_wide.cuh"
+
+namespace deer {
+
+struct MhGrad { float *dW_i, *dW_h, *db_i, *db_h; };
+
+// The heads' input weights and biases side by side: Wc [H*3n][m], bc [H*3n]
+__global__ void mh_gather_kernel(const BodyHead *__restrict__ heads, int H, int n3, int m, float *__restrict__ Wc, float *__restrict__ bc)
+{
+    const size_t per = (size_t)n3 * m, total = per * H;
+    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = i0; i < total; i += stride) Wc[i] = heads[i / per].W_i[i % per];
+    for (size_t i = i0; i < (size_t)H * n3; i += stride) bc[i] = heads[i / n3].b_i[i % n3];
+}
+
+// Status blocks and edge flags of a call over all heads.
+__global__ void mh_begin_kernel(StatusBlock *st, StatusBlock init, int H, unsigned *flags, size_t nflags, unsigned long long *w0, size_t n0,
+                                unsigned long long *w1, size_t n1)
+{
+    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = i0; i < (size_t)H; i += stride) st[i] = init;
+    for (size_t i = i0; i < nflags; i += stride) flags[i] = 0u;
+    for (size_t i = i0; i < n0; i += stride) w0[i] = 0ull;
+    for (size_t i = i0; i < n1; i += stride) w1[i] = 0ull;
+}
+
+// Heads that ended after an odd number of bodies have their result in the other buffer.
+__global__ void mh_select_kernel(const StatusBlock *__restrict__ st, float *__restrict__ y, const float *__restrict__ yalt, size_t N, int H, int n)
+{
+    const int Hn = H * n;
+    const size_t total = N * Hn, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        const int h = (int)(i % Hn) / n;
+        if (st[h].iters & 1) y[i] = yalt[i];
+    }
+}
+
+// dy0[b, h, i] = sum over the phases p, in order, of dy0s[first_seq[h] + b s + p, i]
+__global__ void mh_dy0_sum_kernel(const BodyHead *__restrict__ heads, const float *__restrict__ dy0s, float *__restrict__ dy0, int B, int T, int n, int H)
+{
+    const size_t total = (size_t)B * H * n;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i % n), h = (int)(i / n % H);
+        const long long b = (long long)(i / n / H);
+        const int s = heads[h].stride;
+        const float *src = dy0s + (heads[h].first_seq + b * s) * n + c;
+        float acc = 0.0f;
+        for (int p = 0; p < s && p < T; ++p) acc += src[(size_t)p * n];          // (phases that have positions)
+        dy0[i] = acc;
+    }
+}
+
+// Second stage of the parameter-gradient reductions over all heads (wgrad_final_kernel with the heads' own outputs):
+// hidden = 0: rows g = h * n3 + ... of ONE contraction [P][H*n3][K+1]; 1: a contraction per head, [H][P][n3][K+1].
+__global__ void mh_wgrad_final_kernel(const float *__restrict__ partial, int P, int n3, int K, int H, const MhGrad *__restrict__ out, int hidden)
+{
+    const int K1 = K + 1, per = n3 * K1;
+    const size_t outs = (size_t)per * H;
+    const size_t o = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (o >= outs) return;
+    const int h = (int)(o / per), r = (int)(o % per);
+    const float *src = hidden ? partial + (size_t)h * P * per + r : partial + o;
+    const size_t pitch = hidden ? (size_t)per : outs;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int p = lane; p < P; p += 32) acc += src[p * pitch];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+    if (lane == 0) {
+        const int g = r / K1, k = r % K1;
+        float *dW = hidden ? out[h].dW_h : out[h].dW_i, *db = hidden ? out[h].db_h : out[h].db_i;
+        if (k < K) dW[(size_t)g * K + k] = acc;
+        else db[g] = acc;
+    }
+}
+
+}  // namespace deer

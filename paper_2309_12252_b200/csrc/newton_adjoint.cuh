@@ -179,6 +179,28 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
 #pragma unroll
         for (int j = 0; j < NT; ++j) { d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.0f; }
 
+        // projected inputs at position tt + ahead
+        constexpr bool U_AHEAD = NT <= 2;                // a step ahead where the registers allow it
+        auto load_u = [&](float (&vr)[NT][4], float (&vz)[NT][4], float (&vn)[NT][4], int ahead) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool on = tt[h] + ahead >= 0 && tt[h] + ahead < t_end[h];
+                const float *q = xp[h] - ahead * (ptrdiff_t)xs;
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const int col = 8 * j + 2 * t;
+                    const float2 a0 = on ? ld2(q, col, n) : make_float2(0.0f, 0.0f);
+                    const float2 a1 = on && col < n ? ld2(q + n, col, n) : make_float2(0.0f, 0.0f);
+                    const float2 a2 = on && col < n ? ld2(q + 2 * n, col, n) : make_float2(0.0f, 0.0f);
+                    vr[j][2 * h] = a0.x; vr[j][2 * h + 1] = a0.y;
+                    vz[j][2 * h] = a1.x; vz[j][2 * h + 1] = a1.y;
+                    vn[j][2 * h] = a2.x; vn[j][2 * h + 1] = a2.y;
+                }
+            }
+        };
+        float ur_n[U_AHEAD ? NT : 1][4], uz_n[U_AHEAD ? NT : 1][4], un_n[U_AHEAD ? NT : 1][4];
+        if constexpr (U_AHEAD) { if (!proj) load_u(ur_n, uz_n, un_n, 0); }
+
 #pragma unroll 1
         for (int step = s_first; step < s_end; ++step) {
             if (step == burn) {
@@ -225,20 +247,14 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                         }
                     }
                 }
+            } else if constexpr (U_AHEAD) {              // (requested a step ago; the next one's now)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] = ur_n[j][q]; xz[j][q] = uz_n[j][q]; xn[j][q] = un_n[j][q]; }
+                if (step + 1 < s_end) load_u(ur_n, uz_n, un_n, 1);
             } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int j = 0; j < NT; ++j) {
-                        const int col = 8 * j + 2 * t;
-                        const bool on = act[h] && col < n;
-                        const float2 vr = on ? ld2(xp[h], col, n) : make_float2(0.0f, 0.0f);
-                        const float2 vz = on ? ld2(xp[h] + n, col, n) : make_float2(0.0f, 0.0f);
-                        const float2 vn = on ? ld2(xp[h] + 2 * n, col, n) : make_float2(0.0f, 0.0f);
-                        xr[j][2 * h] = vr.x; xr[j][2 * h + 1] = vr.y;
-                        xz[j][2 * h] = vz.x; xz[j][2 * h + 1] = vz.y;
-                        xn[j][2 * h] = vn.x; xn[j][2 * h + 1] = vn.y;
-                    }
+                load_u(xr, xz, xn, 0);
             }
             // ---- hidden half, gates, lambda and the pre-activation gradients, one block of eight columns at a time
             float p[3][NT][4], zl[NT][4];

@@ -1,4 +1,5 @@
 // Launch side of the one-launch Newton body.
+#include <math.h>
 #include <algorithm>
 #include <mutex>
 #include <stdlib.h>
@@ -103,9 +104,10 @@ static int longest(int T, const int *strides, int H)
     return w;
 }
 
-// One-phase plans: the whole problem is one wave of chains -- the shortest chain length for which it is, but no chains that
-// would spend most of their steps on the burn-in.
-static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t smem, int B, int T, const int *strides, int H)
+// One-phase plans: the chain length with the least estimated time.  Every CTA runs its chains' steps (burn-in and L, or the
+// whole sequence where it is no longer than L) and `cap` of them run at a time, so the launch takes the longest CTA's steps or
+// the sum over CTAs / cap, whichever is more.
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t smem, int burn, int B, int T, const int *strides, int H)
 {
     const int Tmax = longest(T, strides, H);
     p->NC = 0;
@@ -113,12 +115,23 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t 
     p->warps = warps;
     p->smem = smem;
     const long long cap = (long long)sm_count() * occupancy_of(kern, 32 * warps, smem);      // CTAs of one wave
-    const long long positions = (long long)B * T * H;
-    int L = (int)std::max<long long>(16, positions / (cap * warps * 16));
-    while (L < Tmax && count_ctas(B, T, strides, H, L, 16 * warps, 16).ctas > cap) L += std::max(1, L / 64);
-    const Count c = count_ctas(B, T, strides, H, L, 16 * warps, 16);
-    p->L = L; p->max_ctas = c.worst; p->edges = c.edges;
-    p->waves = (float)c.ctas / (float)cap;
+    double best = 0.0;
+    for (int L = 16; ; L += std::max(1, L / 32)) {
+        double sum = 0.0, top = 0.0;
+        for (int h = 0; h < H; ++h) {
+            const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s, nch = (Tp + L - 1) / L;
+            const double ctas = (double)(((long long)B * s * nch + 16 * warps - 1) / (16 * warps)), steps = nch > 1 ? L + burn : Tp;
+            sum += ctas * steps;
+            top = std::max(top, steps);
+        }
+        // (a launch of a little more than one wave takes two: whole waves, as far as a few of them go)
+        const double waves = sum / top / (double)cap, whole = waves <= 4.0 ? ceil(waves - 1e-9) : waves;
+        const double cost = top * std::max(1.0, whole);
+        if (best == 0.0 || cost < best) { best = cost; p->L = L; p->waves = (float)waves; }
+        if (L >= Tmax || (best > 0.0 && top > best)) break;
+    }
+    const Count c = count_ctas(B, T, strides, H, p->L, 16 * warps, 16);
+    p->max_ctas = c.worst; p->edges = c.edges;
 }
 
 bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool have_u, const int *strides, int H)
@@ -147,11 +160,11 @@ bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool hav
                 p->waves = (float)c.ctas / (float)sms;
                 p->smem = fixed + k.slot_bytes * (size_t)(cap + NC * L);
             }
-            p->whole_loop = c.ctas <= sms;
+            p->whole_loop = (long long)c.worst * H <= sms;      // (the grid is max_ctas x H)
             if (c.ctas <= sms || L >= Tmax) return true;
         }
     }
-    one_wave_of_chains(p, (const void *)k.one, k.one_warps, k.one_smem(kx), B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.one, k.one_warps, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
     // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
     p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
     return true;
@@ -168,7 +181,7 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, k.one_warps, k.adj_smem(have_u ? 0 : (m + 7) / 8), B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.adj, k.one_warps, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
     return true;
 }
 

@@ -74,12 +74,18 @@ __global__ void __launch_bounds__(256) vjp_cell_wide_kernel(VjpArgs a)
 // position: per step of 8 positions the A fragment is dG^T (rows = gates), the B fragments are V; both
 // are read straight from global memory as 32-byte row segments.  Products use the 3 x TF32 split
 // (fp32-level accuracy); the bias column is the running sum of the A fragment (chunk 0 writes it).
-// blockDim.x = 32 * ceil(n3 / 16), gridDim.y = ceil(K / 64).
+// blockDim.x = 32 * ceil(min(n3, 192) / 16), gridDim.y = ceil(K / 64), gridDim.z = ceil(n3 / 192) or, multi-head, H.
 __global__ void __launch_bounds__(384) wgrad_mma_kernel(WgradArgs a)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const int n3 = a.n3, K = a.K, K1 = K + 1;
+    const int K = a.K, K1 = K + 1;
+    // rows gr0 .. gr0 + n3 - 1 of the outputs: all of them, a block of 192 (blockIdx.z), or one head's (heads)
+    const int gr0 = a.heads ? 0 : 192 * blockIdx.z, n3 = a.heads ? a.n3 : min(192, a.n3 - gr0);
+    const int head = a.heads ? blockIdx.z : 0, H = a.heads ? a.H : 1;
+    const size_t ldG = (size_t)H * a.n3, ldV = (size_t)H * K;
+    const float *dG = a.dG + (a.heads ? (size_t)head * a.n3 : (size_t)gr0), *V = a.V + (size_t)head * K;
+    const int shift = a.heads ? a.heads[head].stride : 1;
     const int kb = 64 * blockIdx.y;
     const int nb = min(8, (K - kb + 7) >> 3);
     const size_t e0 = (size_t)blockIdx.x * a.slice;
@@ -93,20 +99,24 @@ __global__ void __launch_bounds__(384) wgrad_mma_kernel(WgradArgs a)
     const int row = 16 * warp + g;
     const bool rv0 = row < n3, rv1 = row + 8 < n3;
     auto vrow = [&](size_t e) -> const float * {
-        if (!a.shifted) return a.V + e * K;
+        if (!a.shifted) return V + e * ldV;
+        if (a.heads) {
+            const size_t seq = e / (size_t)a.T;
+            return (int)(e - seq * (size_t)a.T) < shift ? a.y0 + (seq * H + head) * K : V + (e - shift) * ldV;
+        }
         size_t seq;
-        return seq_start(e, a.T, seq) ? a.y0 + seq * K : a.V + (e - 1) * K;
+        return seq_start(e, a.T, seq) ? a.y0 + seq * K : V + (e - 1) * ldV;
     };
 #pragma unroll 1
     for (size_t e = e0; e < e1; e += 8) {
         const size_t p0 = e + t, p1 = e + t + 4;
         const bool v0 = p0 < e1, v1 = p1 < e1;
         float av[4];
-        av[0] = (v0 && rv0) ? __ldg(a.dG + p0 * n3 + row) : 0.0f;
-        av[1] = (v0 && rv1) ? __ldg(a.dG + p0 * n3 + row + 8) : 0.0f;
-        av[2] = (v1 && rv0) ? __ldg(a.dG + p1 * n3 + row) : 0.0f;
-        av[3] = (v1 && rv1) ? __ldg(a.dG + p1 * n3 + row + 8) : 0.0f;
-        const float *r0 = v0 ? vrow(p0) : a.V, *r1 = v1 ? vrow(p1) : a.V;
+        av[0] = (v0 && rv0) ? __ldg(dG + p0 * ldG + row) : 0.0f;
+        av[1] = (v0 && rv1) ? __ldg(dG + p0 * ldG + row + 8) : 0.0f;
+        av[2] = (v1 && rv0) ? __ldg(dG + p1 * ldG + row) : 0.0f;
+        av[3] = (v1 && rv1) ? __ldg(dG + p1 * ldG + row + 8) : 0.0f;
+        const float *r0 = v0 ? vrow(p0) : V, *r1 = v1 ? vrow(p1) : V;
         float bv[8][2];
 #pragma unroll
         for (int nn = 0; nn < 8; ++nn) {
@@ -132,7 +142,7 @@ __global__ void __launch_bounds__(384) wgrad_mma_kernel(WgradArgs a)
             }
         }
     }
-    float *out = a.partial + (size_t)blockIdx.x * n3 * K1;
+    float *out = a.partial + (((size_t)head * gridDim.x + blockIdx.x) * a.n3 + gr0) * K1;
 #pragma unroll
     for (int nn = 0; nn < 8; ++nn) {
         if (nn < nb) {
@@ -172,7 +182,8 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
     extern __shared__ __align__(16) float wg_sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
     const int g = lane >> 2, t = lane & 3;
-    const int n3 = a.n3, K = a.K, K1 = K + 1;
+    const int gr0 = 192 * blockIdx.z, n3 = min(192, a.n3 - gr0), ldG = a.n3;      // (output rows in blocks of 192)
+    const int K = a.K, K1 = K + 1;
     const int GS = wgrad_gs(n3);
     const int kb = 64 * blockIdx.y;
     const int kc = min(64, K - kb);                    // columns of this chunk (a multiple of 4)
@@ -196,7 +207,7 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
             for (int c = tid; c < WG_S * gq; c += nthr) {
                 const int r = c / gq, cc = c - r * gq;
                 float *dst = sG + r * GS + 4 * cc;
-                if (pb + r < e1) cp_async16(dst, a.dG + (pb + r) * n3 + 4 * cc);
+                if (pb + r < e1) cp_async16(dst, a.dG + (pb + r) * ldG + gr0 + 4 * cc);
                 else *reinterpret_cast<float4 *>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
             for (int c = tid; c < WG_S * vq; c += nthr) {
@@ -255,7 +266,7 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
         }
     }
     cp_async_wait_0();
-    float *out = a.partial + (size_t)blockIdx.x * n3 * K1;
+    float *out = a.partial + ((size_t)blockIdx.x * a.n3 + gr0) * K1;
 #pragma unroll
     for (int nn = 0; nn < 8; ++nn) {
         if (nn < nb) {
