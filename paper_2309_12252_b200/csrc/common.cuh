@@ -275,6 +275,8 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b)
 __device__ __forceinline__ float ex2_approx(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rcp_approx(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
+__device__ __forceinline__ float min_nan(float x) { float y; asm("min.NaN.f32 %0, %1, 0f42700000;" : "=f"(y) : "f"(x)); return y; }   // min(x, 60), NaN kept
+
 // The gate activations on a pair of values: the arithmetic around the two special-function-unit results (the scaling of
 // the exponent, 1 +- e, the final product) runs as packed f32x2 instructions; same approximate units as the scalar forms.
 __device__ __forceinline__ float2 sigmoid2_gate(float2 a)

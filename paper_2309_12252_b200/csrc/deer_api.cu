@@ -1004,19 +1004,29 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
                            CopyOut copy_out)
 {
     const int n = p->n, m = p->m;
-    const bool have_u = !body_supported(n, m, false);
+    const bool need_u = !body_supported(n, m, false);
     bool u_done = false;
     int rc, burn = body_first_burn(n, tol);
     BodyArgs a{};
     a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0};
-    a.x = x; a.u = have_u ? w.u : nullptr; a.y0 = y0;
+    a.x = x; a.y0 = y0;
     a.buf[0] = buf[0]; a.buf[1] = buf[1];
     a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1;
     a.eta = body_eta(n, tol);
     a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
-    for (int form = 0; form < 2; ++form) {               // the two-phase kernel, then the one-phase kernel
+    a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
+    const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
+    bool tiles = false;
+    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::ONE_PHASE}) {
         BodyPlan plan{};
-        if (!body_plan(&plan, form == 0, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;
+        if (form == BodyForm::TILE && !aligned32) continue;
+        if (form == BodyForm::ONE_PHASE && tiles) break; // (what the tiles give up is for the kernels that multiply the Jacobians out)
+        const bool have_u = need_u && form != BodyForm::TILE;
+        if (!body_plan(&plan, form, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;
+        a.u = have_u ? w.u : nullptr;
+        // n = 32, 64: the two-phase kernel only where it is the whole loop in one launch
+        if (form == BodyForm::TWO_PHASE && (n == 32 || n == 64) && aligned32 && m <= 64 && !plan.whole_loop) continue;
+        tiles = form == BodyForm::TILE;
         if (burn > plan.burn_cap) { hs->done = BODY_FALL_BACK; continue; }
         a.L = plan.L;
         a.burn_cap = plan.burn_cap;
@@ -1112,8 +1122,10 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
         DEER_CHECK_CUDA(cudaMemcpyAsync(w.yalt, y, N * n * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy iterate");
     const bool one_launch = bodies_done == 0 && body_takes(n, m, flags);
     HostSlot slot(one_launch);
+    bool ended_there = false;                  // the one-launch form ran to the end
     if (one_launch) {
         if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, copy_out)) != DEER_OK) return rc;
+        ended_there = hs.done == BODY_DONE;
     }
     if (!one_launch || hs.done != BODY_DONE) {
     const int k0 = hs.iters;                   // bodies that the one-launch form has done
@@ -1218,7 +1230,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     }
     if ((k & 1) && !y_host)
         DEER_CHECK_CUDA(cudaMemcpyAsync(y, w.yalt, N * n * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy result");
-    const bool trace_here = one_launch && slot.p && hs.done == BODY_DONE && k <= HOST_TRACE;
+    const bool trace_here = ended_there && slot.p && k <= HOST_TRACE;
     if (err_trace && k > 0 && trace_here) memcpy(err_trace, slot.p->trace, sizeof(float) * (size_t)k);
     if (err_trace && k > 0 && !trace_here)
         DEER_CHECK_CUDA(cudaMemcpyAsync(err_trace, w.trace, sizeof(float) * (size_t)(k < ERR_TRACE_CAP ? k : ERR_TRACE_CAP),
@@ -1909,9 +1921,9 @@ static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int
     int rc;
     BodyPlan plan{};
     // the two-phase kernel where it is the whole loop in one launch, else the one-phase kernel
-    if (!body_plan(&plan, true, B, T, n, m, true, strides, H) || !plan.whole_loop) {
+    if (!body_plan(&plan, BodyForm::TWO_PHASE, B, T, n, m, true, strides, H) || !plan.whole_loop) {
         plan = BodyPlan{};
-        if (!body_plan(&plan, false, B, T, n, m, true, strides, H)) return DEER_ERR_UNSUPPORTED_N;
+        if (!body_plan(&plan, BodyForm::ONE_PHASE, B, T, n, m, true, strides, H)) return DEER_ERR_UNSUPPORTED_N;
     }
     if ((rc = mh_table(heads, strides, H, B, T, plan.L, plan.NC > 0 ? plan.NC : 16, w, st)) != DEER_OK) return rc;
     StatusBlock init;

@@ -107,20 +107,20 @@ static int longest(int T, const int *strides, int H)
 // One-phase plans: the chain length with the least estimated time.  Every CTA runs its chains' steps (burn-in and L, or the
 // whole sequence where it is no longer than L) and `cap` of them run at a time, so the launch takes the longest CTA's steps or
 // the sum over CTAs / cap, whichever is more.
-static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t smem, int burn, int B, int T, const int *strides, int H)
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, size_t smem, int burn, int B, int T, const int *strides, int H)
 {
     const int Tmax = longest(T, strides, H);
     p->NC = 0;
     p->whole_loop = false;
-    p->warps = warps;
+    p->warps = threads / 32;
     p->smem = smem;
-    const long long cap = (long long)sm_count() * occupancy_of(kern, 32 * warps, smem);      // CTAs of one wave
+    const long long cap = (long long)sm_count() * occupancy_of(kern, threads, smem);      // CTAs of one wave
     double best = 0.0;
     for (int L = 16; ; L += std::max(1, L / 32)) {
         double sum = 0.0, top = 0.0;
         for (int h = 0; h < H; ++h) {
             const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s, nch = (Tp + L - 1) / L;
-            const double ctas = (double)(((long long)B * s * nch + 16 * warps - 1) / (16 * warps)), steps = nch > 1 ? L + burn : Tp;
+            const double ctas = (double)(((long long)B * s * nch + chains - 1) / chains), steps = nch > 1 ? L + burn : Tp;
             sum += ctas * steps;
             top = std::max(top, steps);
         }
@@ -130,16 +130,24 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int warps, size_t 
         if (best == 0.0 || cost < best) { best = cost; p->L = L; p->waves = (float)waves; }
         if (L >= Tmax || (best > 0.0 && top > best)) break;
     }
-    const Count c = count_ctas(B, T, strides, H, p->L, 16 * warps, 16);
+    const Count c = count_ctas(B, T, strides, H, p->L, chains, edge_unit);
     p->max_ctas = c.worst; p->edges = c.edges;
 }
 
-bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool have_u, const int *strides, int H)
+bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H)
 {
     const int kx = have_u ? 0 : (m + 7) / 8, sms = sm_count(), Tmax = longest(T, strides, H);
-    if (!body_supported(n, m, have_u)) return false;
+    if (form != BodyForm::TILE && !body_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
-    if (two_phase) {
+    p->form = form;
+    if (form == BodyForm::TILE) {
+        if (!(n == 32 || n == 64) || have_u || m > 64 || H != 1 || strides) return false;
+        if (k.tile_smem(m) > BODY_SMEM_MAX) return false;
+        one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H);
+        p->burn_cap = std::max(96, 2 * p->L);
+        return true;
+    }
+    if (form == BodyForm::TWO_PHASE) {
         const size_t fixed = k.seg_fixed(kx);
         if (fixed >= BODY_SMEM_MAX) return false;
         const int slots = (int)((BODY_SMEM_MAX - fixed) / k.slot_bytes);
@@ -164,7 +172,7 @@ bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool hav
             if (c.ctas <= sms || L >= Tmax) return true;
         }
     }
-    one_wave_of_chains(p, (const void *)k.one, k.one_warps, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
     // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
     p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
     return true;
@@ -181,7 +189,7 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, k.one_warps, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
     return true;
 }
 
@@ -218,6 +226,7 @@ int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 // more work than their own kernels do.  Sizes without tuned kernels of the other kind always come here.
 bool body_suits(const BodyPlan &p, int n)
 {
+    if (p.form == BodyForm::TILE) return true;
     const bool tuned = (n & (n - 1)) == 0;
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
@@ -243,6 +252,11 @@ int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st)
     }
     cfg.attrs = attr; cfg.numAttrs = 1;
     const BodyKernels k = pick(a.n, v2);
+    if (p.form == BodyForm::TILE) {
+        occupancy_of((const void *)k.tile(a.m), 32 * p.warps, p.smem);
+        DEER_KERNEL("newton_tile_kernel", st, k.tile(a.m)<<<(unsigned)p.max_ctas, 32 * p.warps, p.smem, st>>>(a));
+        return DEER_OK;
+    }
     occupancy_of(p.NC > 0 ? (const void *)k.seg : (const void *)k.one, 32 * p.warps, p.smem);      // (the shared-memory opt-in on first use)
     if (p.NC > 0) {
         DEER_KERNEL("newton_segment_kernel", st, cudaLaunchKernelEx(&cfg, k.seg, a, p.NC, p.whole_loop ? 1 : 0));

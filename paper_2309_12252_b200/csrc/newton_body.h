@@ -27,6 +27,7 @@ struct BodyArgs {
     StatusBlock *st;         // [H]
     float *edge;             // [groups][2][n]  states either side of a boundary between two warps
     unsigned *edge_flag;     // [groups]        arrivals at it (left cleared)
+    float *starts;           // [chains][n]     tile kernel: update that each chain assumed at its first own position
     unsigned long long *words;   // [H][2][CTAs][2]  maxima exchanged at the end of a body (whole-loop launches)
 };
 
@@ -55,6 +56,9 @@ struct BodyKernels {
     void (*one)(BodyArgs);                     // one-phase (newton_body.cuh)
     void (*seg)(BodyArgs, int, int);           // two-phase (newton_segment.cuh)
     void (*adj)(AdjArgs);                      // adjoint, one-phase (newton_adjoint.cuh)
+    void (*(*tile)(int m))(BodyArgs);          // 128 chains per tcgen05 tile (newton_tile.cuh); n = 32, 64 only
+    size_t (*tile_smem)(int m);
+    int tile_threads, tile_chains;
     int one_warps, seg_warps, nc_max;
     size_t slot_bytes;
     size_t (*one_smem)(int kx), (*seg_fixed)(int kx), (*adj_smem)(int kx);
@@ -62,8 +66,12 @@ struct BodyKernels {
 
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
 
+// The forms of a body.
+enum class BodyForm { TWO_PHASE, TILE, ONE_PHASE };
+
 // How a body is launched.
 struct BodyPlan {
+    BodyForm form;
     int NC;                  // > 0: the two-phase kernel, chains per CTA (newton_segment.cuh); 0: the one-phase kernel
     int L;                   // positions per chain
     int warps;               // warps per CTA
@@ -77,9 +85,9 @@ struct BodyPlan {
 
 // Does the kernel take these sizes?
 bool body_supported(int n, int m, bool have_u);
-// Chain length and launch shape; strides == nullptr: one head of stride 1.  two_phase: the form to plan for; returns
-// false when it does not take these sizes.
-bool body_plan(BodyPlan *p, bool two_phase, int B, int T, int n, int m, bool have_u, const int *strides, int H);
+// Chain length and launch shape of a form; strides == nullptr: one head of stride 1.  False when the form does not take these
+// sizes.
+bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H);
 // Does the form the plan stands for suit the problem, or are the kernels that multiply the Jacobians out faster?
 bool body_suits(const BodyPlan &p, int n);
 // Burn-in a call starts with, and the accuracy asked of the boundaries.

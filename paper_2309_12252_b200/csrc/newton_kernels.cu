@@ -1,6 +1,7 @@
 // The one-launch Newton kernels of one padded state size: compiled once per size with -DBODY_N=8, 16, ... 64 (build.py).
 #include "newton_segment.cuh"
 #include "newton_adjoint.cuh"
+#include "newton_tile.cuh"
 
 #ifndef BODY_N
 #error "BODY_N: state size, a multiple of 8 up to 64"
@@ -19,6 +20,12 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
         if (v2 && !exact) { k.one = newton_body_kernel<N, true, false>; k.seg = newton_segment_kernel<N, true, false>; }
     }
     k.adj = v2 ? newton_adjoint_kernel<N, true> : newton_adjoint_kernel<N, false>;
+    if constexpr (N == 32 || N == 64) {
+        k.tile = [](int m) -> void (*)(BodyArgs) { return m <= 32 ? newton_tile_kernel<N, 1, true> : newton_tile_kernel<N, 64 / N, false>; };
+        k.tile_threads = TileBody<N>::THREADS;
+        k.tile_chains = TileBody<N>::GROUPS * TileBody<N>::ROWS;
+        k.tile_smem = [](int m) { return TileBody<N>::smem((m + 15) & ~15); };
+    }
     k.one_warps = N > 32 ? 8 : 4;
     k.seg_warps = Seg<N>::WARPS;
     k.nc_max = Seg<N>::NC_MAX;
