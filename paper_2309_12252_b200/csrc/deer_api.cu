@@ -456,7 +456,7 @@ static int run_scan(ScanArgs a, const ScanWs &w, int flags, cudaStream_t st, boo
 // tensor-core affine map (K = inputs, nout = outputs; see affine_mma_kernel)
 template <int NB_MAX, bool WT>
 static int launch_affine_mma(const float *in, const float *W, const float *bias, float *out, size_t N, int K, int nout,
-                             cudaStream_t st, const StatusBlock *unless)
+                             cudaStream_t st, const StatusBlock *unless, const StatusBlock *packed)
 {
     const size_t sm = sizeof(float) * 2 * (size_t)K * (nout + 4);
     int rc;
@@ -465,25 +465,25 @@ static int launch_affine_mma(const float *in, const float *W, const float *bias,
     const size_t per_sm = sm > 110 * 1024 ? 1 : 2;
     const size_t cap = (size_t)num_sms() * per_sm;
     const unsigned blocks = (unsigned)(tiles < cap ? tiles : cap);
-    DEER_KERNEL("affine_mma_kernel", st, (affine_mma_kernel<NB_MAX, WT><<<blocks, 256, sm, st>>>(in, W, bias, out, N, K, nout, unless)));
+    DEER_KERNEL("affine_mma_kernel", st, (affine_mma_kernel<NB_MAX, WT><<<blocks, 256, sm, st>>>(in, W, bias, out, N, K, nout, unless, packed)));
     return DEER_OK;
 }
 
 // out[e][g] = bias[g] + sum_k W[g][k] in[e][k]   (wt_given: W is stored [k][g]; bias may be null; unless: nothing to do once
-// that block's done is set)
+// that block's done is set; packed: see affine_mma_kernel, tensor-core path only)
 static int run_affine(const float *in, const float *W, const float *bias, float *out, size_t N, int m, int n3,
-                      int wt_given, cudaStream_t st, const StatusBlock *unless = nullptr)
+                      int wt_given, cudaStream_t st, const StatusBlock *unless = nullptr, const StatusBlock *packed = nullptr)
 {
     // tensor-core path: K and the output count multiples of 8, 8-byte aligned rows, weights fit shared memory
     const bool aligned8 = (((uintptr_t)in | (uintptr_t)out) & 7) == 0;
     if (aligned8 && m % 8 == 0 && m >= 16 && n3 % 8 == 0 && n3 <= 192 &&
         sizeof(float) * 2 * (size_t)m * (n3 + 4) <= 200 * 1024) {
-        if (n3 <= 64) return wt_given ? launch_affine_mma<8, true>(in, W, bias, out, N, m, n3, st, unless)
-                                      : launch_affine_mma<8, false>(in, W, bias, out, N, m, n3, st, unless);
-        if (n3 <= 96) return wt_given ? launch_affine_mma<12, true>(in, W, bias, out, N, m, n3, st, unless)
-                                      : launch_affine_mma<12, false>(in, W, bias, out, N, m, n3, st, unless);
-        return wt_given ? launch_affine_mma<24, true>(in, W, bias, out, N, m, n3, st, unless)
-                        : launch_affine_mma<24, false>(in, W, bias, out, N, m, n3, st, unless);
+        if (n3 <= 64) return wt_given ? launch_affine_mma<8, true>(in, W, bias, out, N, m, n3, st, unless, packed)
+                                      : launch_affine_mma<8, false>(in, W, bias, out, N, m, n3, st, unless, packed);
+        if (n3 <= 96) return wt_given ? launch_affine_mma<12, true>(in, W, bias, out, N, m, n3, st, unless, packed)
+                                      : launch_affine_mma<12, false>(in, W, bias, out, N, m, n3, st, unless, packed);
+        return wt_given ? launch_affine_mma<24, true>(in, W, bias, out, N, m, n3, st, unless, packed)
+                        : launch_affine_mma<24, false>(in, W, bias, out, N, m, n3, st, unless, packed);
     }
     int G = 256 / n3;
     while (G > 1 && sizeof(float) * (size_t)G * PROJ_PP * (m + 1) > 64 * 1024) --G;
@@ -1291,27 +1291,32 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     const size_t N = (size_t)B * T;
     const bool have_u = !adjoint_supported(n, m, false);
     BodyPlan plan{};
-    const bool adj = !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
+    // n = 32, 64: 128 chains per tcgen05 tile; else sixteen per warp
+    BodyPlan tplan{};
+    const bool exact_flags = (flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) != 0;
+    const bool tile = !exact_flags && (((uintptr_t)y | (uintptr_t)y0 | (uintptr_t)gy | (uintptr_t)x | (uintptr_t)p->W_h | (uintptr_t)p->W_i | (uintptr_t)dx) & 15) == 0 &&
+                      adjoint_tile_plan(&tplan, B, T, n, m);
+    const bool adj = !tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
                      adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && adjoint_suits(plan, n);
-    DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj ? (size_t)plan.edges * sizeof(unsigned) : 0), st), "memset status");
+    DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj || tile ? (size_t)(tile ? tplan : plan).edges * sizeof(unsigned) : 0), st), "memset status");
     // small n and m: the cell projects x itself and one kernel does the cell VJP, the slices of the
     // parameter-gradient reduction and dx (no u, dG_i, dG_h arrays)
     const bool small = cell_projects(n, m) && !(flags & DEER_FLAG_GENERIC) && y0 != nullptr &&
                        ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
     const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
-    if (adj) {
-        if (have_u && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
+    if (adj || tile) {
+        if (!tile && have_u && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
         AdjArgs a{};
         a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0, 0};
-        a.x = x; a.u = have_u ? w.u : nullptr; a.y0 = y0; a.y = y; a.gy = gy;
+        a.x = x; a.u = !tile && have_u ? w.u : nullptr; a.y0 = y0; a.y = y; a.gy = gy;
         a.lam = small ? w.lam : nullptr; a.dGi = w.dGi; a.dGh = w.dGh;
         a.dy0 = dy0; a.dy0_by_head = 1;
-        a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1; a.L = plan.L;
+        a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1; a.L = tile ? tplan.L : plan.L;
         a.eta = ADJ_ETA;
-        a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = w.starts;
+        a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = tile ? w.J : w.starts;
         for (int k = 0; k < ADJ_TRIES; ++k) {
             a.burn = ADJ_BURN[k];
-            if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
+            if ((rc = tile ? launch_adjoint_tile(a, tplan, st) : launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
         }
         unless = w.st;
     }
@@ -1365,6 +1370,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
         wa.T = T; wa.n3 = n3; wa.K = side == 0 ? m : n;
         wa.N = N; wa.slice = (N + P - 1) / P;
         wa.partial = w.partial;
+        if (tile) { wa.packed = w.st; wa.dG_packed = w.dGi; }
         int outs = n3 * (wa.K + 1);
         if (n3 <= 32 && wa.K <= 8) {
             DEER_KERNEL("wgrad_small_kernel", st, wgrad_small_kernel<<<P, 256, 0, st>>>(wa));
@@ -1391,11 +1397,11 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
                                                                 side == 0 ? g->db_i : g->db_h));
     }
     if (dx) {
-        if (m >= 32 && m <= 256) {
-            if ((rc = run_affine(w.dGi, p->W_i, nullptr, dx, N, n3, m, 1, st)) != DEER_OK) return rc;
+        if (m >= 32 && m <= 256 && (!tile || m % 8 == 0)) {      // (packed rows: the tensor-core kernel or the plain one)
+            if ((rc = run_affine(w.dGi, p->W_i, nullptr, dx, N, n3, m, 1, st, nullptr, tile ? w.st : nullptr)) != DEER_OK) return rc;
         } else {
             size_t total = N * (size_t)m;
-            DEER_KERNEL("vjp_dx_kernel", st, vjp_dx_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(w.dGi, p->W_i, dx, N, m, n3));
+            DEER_KERNEL("vjp_dx_kernel", st, vjp_dx_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(w.dGi, p->W_i, dx, N, m, n3, tile ? w.st : nullptr));
         }
     }
     if (dy0) {

@@ -215,6 +215,23 @@ int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
     return DEER_OK;
 }
 
+bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m)
+{
+    if (!(n == 32 || n == 64) || m > 64) return false;
+    const BodyKernels k = pick(n, true);
+    if (k.adj_tile_smem(m) > BODY_SMEM_MAX) return false;
+    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, k.adj_tile_smem(m), ADJ_BURN[0], B, T, nullptr, 1);
+    return true;
+}
+
+int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
+{
+    const BodyKernels k = pick(a.n, true);
+    occupancy_of((const void *)k.adj_tile(a.m), 32 * p.warps, p.smem);
+    DEER_KERNEL("adjoint_tile_kernel", st, k.adj_tile(a.m)<<<(unsigned)p.max_ctas, 32 * p.warps, p.smem, st>>>(a));
+    return DEER_OK;
+}
+
 // Measured lines (B200, m = n unless stated, us per evaluation: two-phase / one-phase / multiplied-out kernels):
 //   n = 4, B = 1, T = 1,000:   75 /  -  / 104      n = 4,  B = 16, T = 3e4: 591 / 354 / 188
 //   n = 8, B = 16, T = 1e4 (m = 4): 129 / - / 231   n = 8,  B = 16, T = 3e4: 570 / 321 / 539   n = 8,  T = 1e5: 1733 / 704 / 1564

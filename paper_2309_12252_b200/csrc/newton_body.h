@@ -59,6 +59,8 @@ struct BodyKernels {
     void (*(*tile)(int m))(BodyArgs);          // 128 chains per tcgen05 tile (newton_tile.cuh); n = 32, 64 only
     size_t (*tile_smem)(int m);
     int tile_threads, tile_chains;
+    void (*(*adj_tile)(int m))(AdjArgs);
+    size_t (*adj_tile_smem)(int m);
     int one_warps, seg_warps, nc_max;
     size_t slot_bytes;
     size_t (*one_smem)(int kx), (*seg_fixed)(int kx), (*adj_smem)(int kx);
@@ -101,6 +103,9 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
 size_t adjoint_starts(int n);
 bool adjoint_suits(const BodyPlan &p, int n);
 int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st);
+// The same with 128 chains per tcgen05 tile (adjoint_tile.cuh): n = 32, 64; AdjArgs::dGi receives packed rows [4n].
+bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m);
+int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st);
 // Burn-ins that are tried one after the other, and the accuracy asked of the boundaries (a one-shot solve: fp32 level).
 constexpr int ADJ_TRIES = 2;
 constexpr int ADJ_BURN[ADJ_TRIES] = {44, 128};

@@ -56,6 +56,21 @@ __device__ __forceinline__ void tile_mma(unsigned tmem_d, uint64_t a, uint64_t b
         : "memory");
 }
 
+// A from tensor memory (row = lane, two f16 per 32-bit column); B K-major, or MN-major with tile_idesc's bit 16
+__device__ __forceinline__ void tile_mma_ta(unsigned tmem_d, unsigned tmem_a, uint64_t b, unsigned idesc, unsigned accumulate)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p; \n\t"
+        "}\n"
+        :
+        : "r"(tmem_d), "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+constexpr unsigned TILE_B_MN = 1u << 16;
+
 __device__ __forceinline__ void tile_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -68,6 +83,11 @@ __device__ __forceinline__ void tile_ld4(unsigned taddr, float2 (&v)[2])
                  : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y)
                  : "r"(taddr));
 }
+__device__ __forceinline__ void tile_st2(unsigned taddr, unsigned a, unsigned b)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void tile_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tile_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tile_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tile_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
