@@ -1073,11 +1073,11 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
     const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
     bool tiles = false;
-    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::ONE_PHASE}) {
+    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE}) {
         BodyPlan plan{};
         if (form == BodyForm::TILE && !aligned32) continue;
-        if (form == BodyForm::ONE_PHASE && tiles) break; // (what the tiles give up is for the kernels that multiply the Jacobians out)
-        const bool have_u = need_u && form != BodyForm::TILE;
+        if (form == BodyForm::ONE_PHASE && (tiles || n <= 8)) break; // (what the tiles give up is for the kernels that multiply the Jacobians out)
+        const bool have_u = form == BodyForm::LANE ? m > 8 : need_u && form != BodyForm::TILE;
         if (!body_plan(&plan, form, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;
         a.u = have_u ? w.u : nullptr;
         // n = 32, 64: the two-phase kernel only where it is the whole loop in one launch
@@ -1985,9 +1985,9 @@ static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int
     // the two-phase kernel where it is the whole loop in one launch, else the one-phase kernel
     if (!body_plan(&plan, BodyForm::TWO_PHASE, B, T, n, m, true, strides, H) || !plan.whole_loop) {
         plan = BodyPlan{};
-        if (!body_plan(&plan, BodyForm::ONE_PHASE, B, T, n, m, true, strides, H)) return DEER_ERR_UNSUPPORTED_N;
+        if (!body_plan(&plan, n <= 8 ? BodyForm::LANE : BodyForm::ONE_PHASE, B, T, n, m, true, strides, H)) return DEER_ERR_UNSUPPORTED_N;
     }
-    if ((rc = mh_table(heads, strides, H, B, T, plan.L, plan.NC > 0 ? plan.NC : 16, w, st)) != DEER_OK) return rc;
+    if ((rc = mh_table(heads, strides, H, B, T, plan.L, plan.NC > 0 ? plan.NC : plan.form == BodyForm::LANE ? 32 : 16, w, st)) != DEER_OK) return rc;
     StatusBlock init;
     memset(&init, 0, sizeof(init));
     init.max_iter = max_iter;

@@ -107,7 +107,7 @@ static int longest(int T, const int *strides, int H)
 // One-phase plans: the chain length with the least estimated time.  Every CTA runs its chains' steps (burn-in and L, or the
 // whole sequence where it is no longer than L) and `cap` of them run at a time, so the launch takes the longest CTA's steps or
 // the sum over CTAs / cap, whichever is more.
-static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, size_t smem, int burn, int B, int T, const int *strides, int H)
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, int gran, size_t smem, int burn, int B, int T, const int *strides, int H)
 {
     const int Tmax = longest(T, strides, H);
     p->NC = 0;
@@ -116,7 +116,8 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
     p->smem = smem;
     const long long cap = (long long)sm_count() * occupancy_of(kern, threads, smem);      // CTAs of one wave
     double best = 0.0;
-    for (int L = 16; ; L += std::max(1, L / 32)) {
+    // (gran: what the chain length is a multiple of)
+    for (int L = std::max(16, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
         double sum = 0.0, top = 0.0;
         for (int h = 0; h < H; ++h) {
             const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s, nch = (Tp + L - 1) / L;
@@ -137,13 +138,21 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
 bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H)
 {
     const int kx = have_u ? 0 : (m + 7) / 8, sms = sm_count(), Tmax = longest(T, strides, H);
-    if (form != BodyForm::TILE && !body_supported(n, m, have_u)) return false;
+    if (form != BodyForm::TILE && form != BodyForm::LANE && !body_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     p->form = form;
+    if (form == BodyForm::LANE) {
+        if (n > 8 || (!have_u && m > 8)) return false;
+        const LaneKernel lk = lane_kernel(n, m, have_u);
+        const int burn = (body_first_burn(n, 1.0f) + lk.W - 1) / lk.W * lk.W;
+        one_wave_of_chains(p, (const void *)lk.kern, 128, 128, 32, lk.W, lk.smem, burn, B, T, strides, H);
+        p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
+        return true;
+    }
     if (form == BodyForm::TILE) {
         if (!(n == 32 || n == 64) || have_u || m > 64 || H != 1 || strides) return false;
         if (k.tile_smem(m) > BODY_SMEM_MAX) return false;
-        one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H);
+        one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, 1, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H);
         p->burn_cap = std::max(96, 2 * p->L);
         return true;
     }
@@ -172,7 +181,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
             if (c.ctas <= sms || L >= Tmax) return true;
         }
     }
-    one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
     // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
     p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
     return true;
@@ -189,7 +198,7 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
     return true;
 }
 
@@ -220,7 +229,7 @@ bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m)
     if (!(n == 32 || n == 64) || m > 64) return false;
     const BodyKernels k = pick(n, true);
     if (k.adj_tile_smem(m) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, k.adj_tile_smem(m), ADJ_BURN[0], B, T, nullptr, 1);
+    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, 1, k.adj_tile_smem(m), ADJ_BURN[0], B, T, nullptr, 1);
     return true;
 }
 
@@ -243,7 +252,7 @@ int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 // more work than their own kernels do.  Sizes without tuned kernels of the other kind always come here.
 bool body_suits(const BodyPlan &p, int n)
 {
-    if (p.form == BodyForm::TILE) return true;
+    if (p.form == BodyForm::TILE || p.form == BodyForm::LANE) return true;
     const bool tuned = (n & (n - 1)) == 0;
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
@@ -272,6 +281,12 @@ int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st)
     if (p.form == BodyForm::TILE) {
         occupancy_of((const void *)k.tile(a.m), 32 * p.warps, p.smem);
         DEER_KERNEL("newton_tile_kernel", st, k.tile(a.m)<<<(unsigned)p.max_ctas, 32 * p.warps, p.smem, st>>>(a));
+        return DEER_OK;
+    }
+    if (p.form == BodyForm::LANE) {
+        const LaneKernel lk = lane_kernel(a.n, a.m, a.u != nullptr);
+        occupancy_of((const void *)lk.kern, 128, p.smem);
+        DEER_KERNEL("newton_lane_kernel", st, cudaLaunchKernelEx(&cfg, lk.kern, a));
         return DEER_OK;
     }
     occupancy_of(p.NC > 0 ? (const void *)k.seg : (const void *)k.one, 32 * p.warps, p.smem);      // (the shared-memory opt-in on first use)

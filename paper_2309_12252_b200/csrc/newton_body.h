@@ -69,7 +69,7 @@ struct BodyKernels {
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
 
 // The forms of a body.
-enum class BodyForm { TWO_PHASE, TILE, ONE_PHASE };
+enum class BodyForm { TWO_PHASE, TILE, LANE, ONE_PHASE };
 
 // How a body is launched.
 struct BodyPlan {
@@ -84,6 +84,10 @@ struct BodyPlan {
     long long edges;         // boundaries between warps (one-phase) or CTAs (two-phase) of all heads at most
     size_t smem;
 };
+
+// A thread per chain (newton_lane.cuh): n up to 8; inputs of up to 8 channels contracted in the kernel, else projected.
+struct LaneKernel { void (*kern)(BodyArgs); size_t smem; int W; };
+LaneKernel lane_kernel(int n, int m, bool have_u);
 
 // Does the kernel take these sizes?
 bool body_supported(int n, int m, bool have_u);

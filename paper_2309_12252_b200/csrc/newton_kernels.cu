@@ -1,6 +1,7 @@
 // The one-launch Newton kernels of one padded state size: compiled once per size with -DBODY_N=8, 16, ... 64 (build.py).
 #include "newton_segment.cuh"
 #include "newton_adjoint.cuh"
+#include "newton_lane.cuh"
 #include "newton_tile.cuh"
 #include "adjoint_tile.cuh"
 
@@ -38,6 +39,19 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
     k.seg_fixed = [](int kx) { return Seg<N>::fixed(kx); };
     return k;
 }
+
+#if BODY_N == 8
+template <int N, int M> static LaneKernel lane_of() { return {newton_lane_kernel<N, M>, Lane<N, M>::SMEM, Lane<N, M>::W}; }
+template <int N> static LaneKernel lane_m(int m, bool have_u)
+{
+    if (have_u) return lane_of<N, 0>();
+    return m <= 1 ? lane_of<N, 1>() : m <= 2 ? lane_of<N, 2>() : m <= 4 ? lane_of<N, 4>() : lane_of<N, 8>();
+}
+LaneKernel lane_kernel(int n, int m, bool have_u)
+{
+    return n <= 1 ? lane_m<1>(m, have_u) : n <= 2 ? lane_m<2>(m, have_u) : n <= 4 ? lane_m<4>(m, have_u) : lane_m<8>(m, have_u);
+}
+#endif
 
 #define BODY_CAT_(a, b) a##b
 #define BODY_CAT(a, b) BODY_CAT_(a, b)
