@@ -15,21 +15,23 @@ namespace deer {
 template <int N, int M> struct Lane {                    // M: input channels, padded (1, 2, 4, 8), or 0: projected inputs u
     static constexpr int WARPS = 4, THREADS = 128;
     static constexpr int XW = M > 0 ? M : 3 * N;         // floats of input per position
-    static constexpr int W = M > 0 ? 32 / (N > M ? N : M) : 16 / N;              // positions of a window
+    static constexpr int W0 = M > 0 ? (N <= 2 ? 16 : 32) / (N > M ? N : M) : 16 / N;
+    static constexpr int W = N == 1 && W0 < 4 ? 4 : W0;  // positions of a window
     static constexpr int P = N < 4 ? 4 / N : 1;          // positions per 16 bytes of state
+    static constexpr int Q = N == 1 && W % 8 == 0 ? 8 : N == 1 ? 4 : N == 2 ? (W % 4 == 0 ? 4 : 2) : N == 4 ? 2 : 1;      // positions whose cells are evaluated side by side
     __host__ __device__ static constexpr int stride(int w) { return (((w + 3) / 4) | 1) * 4; }
     static constexpr int YR = stride(W * N), XR = stride(W * XW);
     static constexpr int ROW = 3 * N + 3 * M + 4;        // weights and biases of a state component, padded to 16 bytes
     static constexpr int ROWP = (ROW + 3) / 4 * 4;
     static constexpr size_t SMEM = sizeof(float) * ((size_t)N * ROWP + (size_t)WARPS * 2 * 32 * (YR + XR));
-    static_assert(W % P == 0, "windows are whole pieces");
+    static_assert(W % P == 0 && W % Q == 0 && Q * N % 4 == 0, "windows are whole pieces");
 };
 
 template <int N, int M>
 __global__ void __launch_bounds__(128) newton_lane_kernel(BodyArgs a)
 {
     using C = Lane<N, M>;
-    constexpr int W = C::W, P = C::P, YR = C::YR, XR = C::XR, XW = C::XW, ROWP = C::ROWP;
+    constexpr int W = C::W, P = C::P, YR = C::YR, XR = C::XR, XW = C::XW, ROWP = C::ROWP, Q = C::Q;
     constexpr float LOG2E = 1.4426950408889634f;
     extern __shared__ __align__(16) float smb[];
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
@@ -193,36 +195,44 @@ __global__ void __launch_bounds__(128) newton_lane_kernel(BodyArgs a)
         float *sy = ring + (w & 1) * 32 * (YR + XR) + lane * YR;
         const float *sx = ring + (w & 1) * 32 * (YR + XR) + 32 * YR + lane * XR;
 #pragma unroll 1
-        for (int i0 = 0; i0 < W; i0 += P) {
-            float yv[P * N], xv[P * XW];
+        for (int i0 = 0; i0 < W; i0 += Q) {
+            float yv[Q * N], xv[Q * XW];
 #pragma unroll
-            for (int k = 0; k < P * N / 4; ++k) {
+            for (int k = 0; k < Q * N / 4; ++k) {
                 const float4 v = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4 *>(sy + i0 * N + 4 * k);
                 yv[4 * k] = v.x; yv[4 * k + 1] = v.y; yv[4 * k + 2] = v.z; yv[4 * k + 3] = v.w;
             }
-            if constexpr (P * XW % 4 == 0) {
+            if constexpr (Q * XW % 4 == 0) {
 #pragma unroll
-                for (int k = 0; k < P * XW / 4; ++k) {
+                for (int k = 0; k < Q * XW / 4; ++k) {
                     const float4 v = *reinterpret_cast<const float4 *>(sx + i0 * XW + 4 * k);
                     xv[4 * k] = v.x; xv[4 * k + 1] = v.y; xv[4 * k + 2] = v.z; xv[4 * k + 3] = v.w;
                 }
             } else {
 #pragma unroll
-                for (int k = 0; k < P * XW; ++k) xv[k] = sx[i0 * XW + k];
+                for (int k = 0; k < Q * XW; ++k) xv[k] = sx[i0 * XW + k];
             }
+            const int t0 = ts + W * w + i0;
+            const bool own = W * w >= burn;
+            // The cells of the Q positions depend on the old iterate only: side by side.  z, k_r, k_z, k_n, f of position p,
+            // component i; one component at a time, its weights from registers or shared memory (broadcast).
+            float cz[Q][N], ckr[Q][N], ckz[Q][N], ckn[Q][N], cf[Q][N];
+            float hq[Q][N];
 #pragma unroll
-            for (int p = 0; p < P; ++p) {
-                const int t = ts + W * w + i0 + p;
-                const bool act = t >= 0 && t < te, keep = act && W * w >= burn;
-                float dn[N];
+            for (int p = 0; p < Q; ++p)
 #pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    float wr[ROWP];                      // this component's weights
+                for (int k = 0; k < N; ++k) hq[p][k] = p == 0 ? h[k] : t0 + p - 1 >= 0 ? yv[(p - 1) * N + k] : h[k];
+            float dn[N];                                 // (Q == 1: the update beside the cell, weights read once)
 #pragma unroll
-                    for (int k = 0; k < ROWP / 4; ++k) {
-                        const float4 v = REG ? wreg[REG ? i * ROWP / 4 + k : 0] : reinterpret_cast<const float4 *>(sw)[i * ROWP / 4 + k];
-                        wr[4 * k] = v.x; wr[4 * k + 1] = v.y; wr[4 * k + 2] = v.z; wr[4 * k + 3] = v.w;
-                    }
+            for (int i = 0; i < N; ++i) {
+                float wr[ROWP];
+#pragma unroll
+                for (int k = 0; k < ROWP / 4; ++k) {
+                    const float4 v = REG ? wreg[REG ? i * ROWP / 4 + k : 0] : reinterpret_cast<const float4 *>(sw)[i * ROWP / 4 + k];
+                    wr[4 * k] = v.x; wr[4 * k + 1] = v.y; wr[4 * k + 2] = v.z; wr[4 * k + 3] = v.w;
+                }
+#pragma unroll
+                for (int p = 0; p < Q; ++p) {
                     float ar = wr[3 * N + 3 * M], az = wr[3 * N + 3 * M + 1], aq = wr[3 * N + 3 * M + 2], an = wr[3 * N + 3 * M + 3];
                     if constexpr (M > 0) {
 #pragma unroll
@@ -237,25 +247,63 @@ __global__ void __launch_bounds__(128) newton_lane_kernel(BodyArgs a)
                     float ur = 0.0f, uz = 0.0f, un = 0.0f;
 #pragma unroll
                     for (int k = 0; k < N; ++k) {
-                        ar = fmaf(wr[k], h[k], ar);
-                        az = fmaf(wr[N + k], h[k], az);
-                        aq = fmaf(wr[2 * N + k], h[k], aq);
-                        ur = fmaf(wr[k], d[k], ur);
-                        uz = fmaf(wr[N + k], d[k], uz);
-                        un = fmaf(wr[2 * N + k], d[k], un);
+                        ar = fmaf(wr[k], hq[p][k], ar);
+                        az = fmaf(wr[N + k], hq[p][k], az);
+                        aq = fmaf(wr[2 * N + k], hq[p][k], aq);
+                        if constexpr (Q == 1) {
+                            ur = fmaf(wr[k], d[k], ur);
+                            uz = fmaf(wr[N + k], d[k], uz);
+                            un = fmaf(wr[2 * N + k], d[k], un);
+                        }
                     }
                     const float r = rcp_approx(1.0f + ex2_approx(-LOG2E * ar)), z = rcp_approx(1.0f + ex2_approx(-LOG2E * az));
                     const float cc = fmaf(rcp_approx(1.0f + ex2_approx(2.0f * LOG2E * fmaf(r, aq, an))), -2.0f, 1.0f);         // tanh
-                    const float omz = 1.0f - z, hc = h[i] - cc;
-                    const float kn = omz * fmaf(-cc, cc, 1.0f) * r, kr = kn * aq * (1.0f - r), kz = z * omz * hc;
-                    const float yn = fmaf(z, d[i], fmaf(kr, ur, fmaf(kz, uz, fmaf(kn, un, fmaf(z, hc, cc)))));
-                    dn[i] = yn - yv[p * N + i];
-                    if (act) sy[(i0 + p) * N + i] = yn;
-                    if (keep && i < n) mb = max(mb, __float_as_uint(fabsf(dn[i])));
+                    const float omz = 1.0f - z, hc = hq[p][i] - cc;
+                    const float kn = omz * fmaf(-cc, cc, 1.0f) * r, kr = kn * aq * (1.0f - r), kz = z * omz * hc, f = fmaf(z, hc, cc);
+                    if constexpr (Q == 1) {
+                        dn[i] = fmaf(z, d[i], fmaf(kr, ur, fmaf(kz, uz, fmaf(kn, un, f))));
+                    } else {
+                        cz[p][i] = z; ckr[p][i] = kr; ckz[p][i] = kz; ckn[p][i] = kn; cf[p][i] = f;
+                    }
+                }
+            }
+            // the updates, one position after the other
+#pragma unroll
+            for (int p = 0; p < Q; ++p) {
+                const bool act = t0 + p >= 0 && t0 + p < te;
+                if constexpr (Q > 1) {
+#pragma unroll
+                    for (int i = 0; i < N; ++i) {
+                        float ur = 0.0f, uz = 0.0f, un = 0.0f;
+                        float wr[3 * N];
+#pragma unroll
+                        for (int k = 0; k < (3 * N + 3) / 4; ++k) {
+                            const float4 v = REG ? wreg[REG ? i * ROWP / 4 + k : 0] : reinterpret_cast<const float4 *>(sw)[i * ROWP / 4 + k];
+                            if (4 * k < 3 * N) wr[4 * k] = v.x;
+                            if (4 * k + 1 < 3 * N) wr[4 * k + 1] = v.y;
+                            if (4 * k + 2 < 3 * N) wr[4 * k + 2] = v.z;
+                            if (4 * k + 3 < 3 * N) wr[4 * k + 3] = v.w;
+                        }
+#pragma unroll
+                        for (int k = 0; k < N; ++k) {
+                            ur = fmaf(wr[k], d[k], ur);
+                            uz = fmaf(wr[N + k], d[k], uz);
+                            un = fmaf(wr[2 * N + k], d[k], un);
+                        }
+                        dn[i] = fmaf(cz[p][i], d[i], fmaf(ckr[p][i], ur, fmaf(ckz[p][i], uz, fmaf(ckn[p][i], un, cf[p][i]))));
+                    }
                 }
 #pragma unroll
-                for (int i = 0; i < N; ++i)
-                    if (act) { d[i] = dn[i]; h[i] = yv[p * N + i]; }
+                for (int i = 0; i < N; ++i) {            // dn: the new iterate
+                    const float v = dn[i] - yv[p * N + i];
+                    if (own && act && i < n) mb = max(mb, __float_as_uint(fabsf(v)));
+                    if (act) { d[i] = v; h[i] = yv[p * N + i]; yv[p * N + i] = dn[i]; }
+                }
+            }
+            if constexpr (Q * N % 4 == 0) {
+#pragma unroll
+                for (int k = 0; k < Q * N / 4; ++k)
+                    *reinterpret_cast<float4 *>(sy + i0 * N + 4 * k) = make_float4(yv[4 * k], yv[4 * k + 1], yv[4 * k + 2], yv[4 * k + 3]);
             }
         }
         __syncwarp();
