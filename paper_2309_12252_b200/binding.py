@@ -148,8 +148,9 @@ def _f32(t):
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None:          # (the raw handle: a Stream object costs 3 us a call)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 @dataclass
@@ -168,11 +169,12 @@ class GruParamsDev:
         return GruParamsDev(p.n, p.m, mk(p.W_i), mk(p.W_h), mk(p.b_i), mk(p.b_h))
 
     def c_struct(self):
-        for t, shape in ((self.W_i, (3 * self.n, self.m)), (self.W_h, (3 * self.n, self.n)),
-                         (self.b_i, (3 * self.n,)), (self.b_h, (3 * self.n,))):
-            assert tuple(t.shape) == shape and t.dtype == torch.float32 and t.is_cuda and t.is_contiguous()
-        return _Params(self.n, self.m, self.W_i.data_ptr(), self.W_h.data_ptr(), self.b_i.data_ptr(),
-                       self.b_h.data_ptr())
+        n, n3 = self.n, 3 * self.n
+        W_i, W_h, b_i, b_h = self.W_i, self.W_h, self.b_i, self.b_h
+        assert W_i.shape == (n3, self.m) and W_h.shape == (n3, n) and b_i.shape == (n3,) and b_h.shape == (n3,)
+        for t in (W_i, W_h, b_i, b_h):
+            assert t.dtype is torch.float32 and t.is_cuda and t.is_contiguous()
+        return _Params(n, self.m, W_i.data_ptr(), W_h.data_ptr(), b_i.data_ptr(), b_h.data_ptr())
 
 
 def deer_status_string(status: int) -> str:
@@ -436,10 +438,13 @@ def deer_gru_multihead_vjp(heads, strides, x, y0, y, gy, ws=None, flags=0, strea
     H, ps, st = _mh_args(heads, strides)
     n = heads[0].n
     dev = x.device
-    g = dict(dW_i=[torch.empty((3 * n, m), device=dev) for _ in range(H)], dW_h=[torch.empty((3 * n, n), device=dev) for _ in range(H)],
-             db_i=[torch.empty((3 * n,), device=dev) for _ in range(H)], db_h=[torch.empty((3 * n,), device=dev) for _ in range(H)])
-    gs = (_Grads * H)(*[_Grads(g["dW_i"][h].data_ptr(), g["dW_h"][h].data_ptr(), g["db_i"][h].data_ptr(),
-                               g["db_h"][h].data_ptr()) for h in range(H)])
+    # one allocation per kind, the heads' gradients its slices
+    whole = (torch.empty((H, 3 * n, m), device=dev), torch.empty((H, 3 * n, n), device=dev), torch.empty((H, 3 * n), device=dev),
+             torch.empty((H, 3 * n), device=dev))
+    g = {k: list(t.unbind(0)) for k, t in zip(("dW_i", "dW_h", "db_i", "db_h"), whole)}
+    base = [t.data_ptr() for t in whole]
+    step = [4 * t[0].numel() for t in whole]
+    gs = (_Grads * H)(*[_Grads(*[b + h * s for b, s in zip(base, step)]) for h in range(H)])
     dx = torch.empty_like(x)
     dy0 = torch.empty_like(y0)
     if ws is None:

@@ -1345,6 +1345,10 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     int rc = check_ws(ws, ws_bytes, w.bytes);
     if (rc != DEER_OK) return rc;
     const size_t N = (size_t)B * T;
+    // small n and m: the cell projects x itself and one kernel does the cell VJP, the slices of the
+    // parameter-gradient reduction and dx (no u, dG_i, dG_h arrays)
+    const bool small = cell_projects(n, m) && !(flags & DEER_FLAG_GENERIC) && y0 != nullptr &&
+                       ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
     const bool have_u = !adjoint_supported(n, m, false);
     BodyPlan plan{};
     // n = 32, 64: 128 chains per tcgen05 tile; else sixteen per warp
@@ -1352,31 +1356,29 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     const bool exact_flags = (flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) != 0;
     const bool tile = !exact_flags && (((uintptr_t)y | (uintptr_t)y0 | (uintptr_t)gy | (uintptr_t)x | (uintptr_t)p->W_h | (uintptr_t)p->W_i | (uintptr_t)dx) & 15) == 0 &&
                       adjoint_tile_plan(&tplan, B, T, n, m);
-    const bool adj = !tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
-                     adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && adjoint_suits(plan, n);
+    const bool lanes = small && !exact_flags && (((uintptr_t)gy) & 3) == 0 && rows_adjoint_plan(&plan, B, T, n, m, WGRAD_P);     // all in one launch
+    const bool adj = lanes || (!tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
+                     adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && adjoint_suits(plan, n));
     DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj || tile ? (size_t)(tile ? tplan : plan).edges * sizeof(unsigned) : 0), st), "memset status");
-    // small n and m: the cell projects x itself and one kernel does the cell VJP, the slices of the
-    // parameter-gradient reduction and dx (no u, dG_i, dG_h arrays)
-    const bool small = cell_projects(n, m) && !(flags & DEER_FLAG_GENERIC) && y0 != nullptr &&
-                       ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
     const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
     if (adj || tile) {
-        if (!tile && have_u && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
+        if (!tile && !lanes && have_u && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
         AdjArgs a{};
         a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0, 0};
-        a.x = x; a.u = !tile && have_u ? w.u : nullptr; a.y0 = y0; a.y = y; a.gy = gy;
+        a.x = x; a.u = !tile && !lanes && have_u ? w.u : nullptr; a.y0 = y0; a.y = y; a.gy = gy;
         a.lam = small ? w.lam : nullptr; a.dGi = w.dGi; a.dGh = w.dGh;
         a.dy0 = dy0; a.dy0_by_head = 1;
         a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1; a.L = tile ? tplan.L : plan.L;
         a.eta = ADJ_ETA;
         a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = tile ? w.J : w.starts;
-        for (int k = 0; k < ADJ_TRIES; ++k) {
+        // (small cells: one try, the passes behind it are cheap)
+        for (int k = 0; k < (lanes ? 1 : ADJ_TRIES); ++k) {
             a.burn = ADJ_BURN[k];
-            if ((rc = tile ? launch_adjoint_tile(a, tplan, st) : launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
+            if ((rc = tile ? launch_adjoint_tile(a, tplan, st) : lanes ? launch_rows_adjoint(a, plan, w.partial, w.partial2, dx, st) : launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
         }
         unless = w.st;
     }
-    if (!small && !(adj && have_u) && (rc = run_proj(p, x, w.u, N, st, unless)) != DEER_OK) return rc;
+    if (!small && !(adj && !lanes && have_u) && (rc = run_proj(p, x, w.u, N, st, unless)) != DEER_OK) return rc;
     ScanArgs a{};
     a.J = w.J; a.b = gy; a.y0 = nullptr; a.y = w.lam; a.yold = nullptr;
     a.B = B; a.T = T; a.n = n; a.reverse = 1;
@@ -1393,11 +1395,11 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     if ((rc = run_scan(a, w.scan, flags, st, true, unless == nullptr)) != DEER_OK) return rc;
 
     if (small) {
-        VjpSmallArgs v{p->W_h, p->b_h, p->W_i, p->b_i, x, y, y0, w.lam, dx, w.partial, w.partial2, B, T};
+        VjpSmallArgs v{p->W_h, p->b_h, p->W_i, p->b_i, x, y, y0, w.lam, dx, w.partial, w.partial2, B, T, lanes ? unless : nullptr};
         int P = 0;
         if ((rc = launch_vjp_small(v, n, m, &P, st)) != DEER_OK) return rc;
-        DEER_KERNEL("wgrad_final_kernel", st, wgrad_final_kernel<<<(n3 * (m + 1) + 7) / 8, 256, 0, st>>>(w.partial, P, n3, m, g->dW_i, g->db_i));
-        DEER_KERNEL("wgrad_final_kernel", st, wgrad_final_kernel<<<(n3 * (n + 1) + 7) / 8, 256, 0, st>>>(w.partial2, P, n3, n, g->dW_h, g->db_h));
+        const int oi = n3 * (m + 1), oh = n3 * (n + 1);
+        DEER_KERNEL("wgrad_final_kernel", st, wgrad_final2_kernel<<<(oi + oh + 7) / 8, 256, 0, st>>>(w.partial, w.partial2, P, lanes ? unless : nullptr, plan.max_ctas, n3, m, n, g->dW_i, g->db_i, g->dW_h, g->db_h));
         if (dy0) {
             DEER_KERNEL("vjp_dy0_kernel", st, vjp_dy0_kernel<<<(B * n + 127) / 128, 128, 0, st>>>(w.J, w.lam, dy0, B, T, n, unless));
         }

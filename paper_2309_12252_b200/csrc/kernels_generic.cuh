@@ -458,11 +458,13 @@ struct VjpSmallArgs {
     float *partial_i;          // [P][3n*(m+1)]
     float *partial_h;          // [P][3n*(n+1)]
     int B, T;
+    const StatusBlock *st;     // nullptr, or: nothing to do once st->done is set
 };
 
 template <int N, int M>
 __global__ void __launch_bounds__(256, 2) vjp_small_kernel(VjpSmallArgs a)
 {
+    if (loop_ended(a.st)) return;
     constexpr int EPB = 256 / N;                       // positions per block per step
     constexpr int VI = 3 * (M + 1), VH = 3 * (N + 1), VALS = VI + VH;
     extern __shared__ float red[];                     // [256][VALS + 1]
@@ -773,6 +775,32 @@ __global__ void wgrad_final_kernel(const float *__restrict__ partial, int P, int
         const int g = o / K1, k = o % K1;
         if (k < K) dW[(size_t)g * K + k] = acc;
         else db[g] = acc;
+    }
+}
+
+// The second stages of both contractions of a small cell in one launch.
+// (P_done slices instead of P where st's done is set: the fused gradient wrote them)
+__global__ void wgrad_final2_kernel(const float *__restrict__ pi, const float *__restrict__ ph, int P, const StatusBlock *st, int P_done, int n3, int m, int n,
+                                    float *__restrict__ dW_i, float *__restrict__ db_i, float *__restrict__ dW_h, float *__restrict__ db_h)
+{
+    if (loop_ended(st)) P = P_done;
+    const int oi = n3 * (m + 1), oh = n3 * (n + 1);
+    int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (o >= oi + oh) return;
+    const bool hid = o >= oi;
+    if (hid) o -= oi;
+    const float *partial = hid ? ph : pi;
+    const int outs = hid ? oh : oi, K = hid ? n : m, K1 = K + 1;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int p = lane; p < P; p += 32) acc += partial[(size_t)p * outs + o];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+    if (lane == 0) {
+        const int g = o / K1, k = o % K1;
+        if (k < K) (hid ? dW_h : dW_i)[(size_t)g * K + k] = acc;
+        else (hid ? db_h : db_i)[g] = acc;
     }
 }
 

@@ -61,7 +61,7 @@ static int occupancy_of(const void *kern, int threads, size_t smem)
     std::lock_guard<std::mutex> lk(mu);
     for (int i = 0; i < used; ++i)
         if (cache[i].k == kern && cache[i].smem == smem && cache[i].dev == dev) return cache[i].occ;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BODY_SMEM_MAX);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BODY_SMEM_MAX);
     int o = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, threads, smem) != cudaSuccess || o < 1) o = 1;
     if (used < 128) cache[used++] = {kern, smem, dev, o};
@@ -107,14 +107,14 @@ static int longest(int T, const int *strides, int H)
 // One-phase plans: the chain length with the least estimated time.  Every CTA runs its chains' steps (burn-in and L, or the
 // whole sequence where it is no longer than L) and `cap` of them run at a time, so the launch takes the longest CTA's steps or
 // the sum over CTAs / cap, whichever is more.
-static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, int gran, size_t smem, int burn, int B, int T, const int *strides, int H)
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, int gran, size_t smem, int burn, int B, int T, const int *strides, int H, int occ_cap = 64)
 {
     const int Tmax = longest(T, strides, H);
     p->NC = 0;
     p->whole_loop = false;
     p->warps = threads / 32;
     p->smem = smem;
-    const long long cap = (long long)sm_count() * occupancy_of(kern, threads, smem);      // CTAs of one wave
+    const long long cap = (long long)sm_count() * std::min(occ_cap, occupancy_of(kern, threads, smem));      // CTAs of one wave
     double best = 0.0;
     // (gran: what the chain length is a multiple of)
     for (int L = std::max(16, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
@@ -222,6 +222,14 @@ int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
     DEER_KERNEL("newton_adjoint_kernel", st,
                 k.adj<<<dim3((unsigned)p.max_ctas, (unsigned)a.H), 32 * p.warps, p.smem, st>>>(a));
     return DEER_OK;
+}
+
+bool rows_adjoint_plan(BodyPlan *p, int B, int T, int n, int m, int max_ctas)
+{
+    auto small = [](int v) { return v == 1 || v == 2 || v == 4 || v == 8; };
+    if (!small(n) || !small(m)) return false;
+    one_wave_of_chains(p, (const void *)rows_adjoint_of(n, m), 128, 128 / n, 32 / n, 4, 0, ADJ_BURN[0], B, T, nullptr, 1, std::max(1, max_ctas / sm_count()));
+    return p->max_ctas <= max_ctas;
 }
 
 bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m)

@@ -85,6 +85,13 @@ struct BodyPlan {
     size_t smem;
 };
 
+// The whole gradient of a small cell in one launch (rows_adjoint.cuh): n, m in {1, 2, 4, 8}; the launch writes
+// plan.max_ctas slices of the parameter gradients.
+struct RowsAdjOut;
+bool rows_adjoint_plan(BodyPlan *p, int B, int T, int n, int m, int max_ctas);
+int launch_rows_adjoint(const AdjArgs &a, const BodyPlan &p, float *partial_i, float *partial_h, float *dx, cudaStream_t st);
+void (*rows_adjoint_of(int n, int m))(AdjArgs, RowsAdjOut);
+
 // A thread per chain (newton_lane.cuh): n up to 8; inputs of up to 8 channels contracted in the kernel, else projected.
 struct LaneKernel { void (*kern)(BodyArgs); size_t smem; int W; };
 LaneKernel lane_kernel(int n, int m, bool have_u);

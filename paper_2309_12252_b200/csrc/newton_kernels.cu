@@ -2,6 +2,7 @@
 #include "newton_segment.cuh"
 #include "newton_adjoint.cuh"
 #include "newton_lane.cuh"
+#include "rows_adjoint.cuh"
 #include "newton_tile.cuh"
 #include "adjoint_tile.cuh"
 
@@ -50,6 +51,15 @@ template <int N> static LaneKernel lane_m(int m, bool have_u)
 LaneKernel lane_kernel(int n, int m, bool have_u)
 {
     return n <= 1 ? lane_m<1>(m, have_u) : n <= 2 ? lane_m<2>(m, have_u) : n <= 4 ? lane_m<4>(m, have_u) : lane_m<8>(m, have_u);
+}
+using RowsAdjKernel = void (*)(AdjArgs, RowsAdjOut);
+template <int N> static RowsAdjKernel rows_m(int m) { return m == 1 ? rows_adjoint_kernel<N, 1> : m == 2 ? rows_adjoint_kernel<N, 2> : m == 4 ? rows_adjoint_kernel<N, 4> : rows_adjoint_kernel<N, 8>; }
+void (*rows_adjoint_of(int n, int m))(AdjArgs, RowsAdjOut) { return n == 1 ? rows_m<1>(m) : n == 2 ? rows_m<2>(m) : n == 4 ? rows_m<4>(m) : rows_m<8>(m); }
+int launch_rows_adjoint(const AdjArgs &a, const BodyPlan &p, float *partial_i, float *partial_h, float *dx, cudaStream_t st)
+{
+    const RowsAdjOut out{partial_i, partial_h, dx};
+    DEER_KERNEL("rows_adjoint_kernel", st, rows_adjoint_of(a.n, a.m)<<<(unsigned)p.max_ctas, 128, 0, st>>>(a, out));
+    return DEER_OK;
 }
 #endif
 
