@@ -1,4 +1,4 @@
-// The gradient's adjoint solve for n = 32 and 64 as one launch: the algorithm of newton_adjoint.cuh (see there: chains in
+// The gradient's adjoint solve for n = 64 as one launch: the algorithm of newton_adjoint.cuh (see there: chains in
 // descending time with a burn-in and verified boundaries, mu_t = J_{t+1}^T lambda_{t+1} as the state) with 128 chains in
 // lockstep as the rows of a tcgen05 tile, in the manner of newton_tile.cuh.
 //
@@ -18,55 +18,51 @@
 
 namespace deer {
 
-template <int N> struct TileAdj {
-    static constexpr int GROUPS = N == 32 ? 2 : 1, GT = 8 * N, THREADS = GROUPS * GT, ROWS = 128;
+struct TileAdj {
+    static constexpr int N = 64, THREADS = 8 * N, ROWS = 128;
     static constexpr int CG = N / 16;                    // threads of a row
     static constexpr int LPR = N / 4, GS = N + 4;
     static constexpr unsigned PANEL = 128 * 128, HP = 2 * N / 64, WROWS = 3 * N;
-    static constexpr unsigned TMEM = 512, TCOLS = 8 * N; // columns of a group: q r z un (n each), mu (n), p hi and lo (3n / 2 each)
+    static constexpr unsigned TMEM = 512;                // columns: q r z un (n each), mu (n), p hi and lo (3n / 2 each)
     __host__ __device__ static constexpr unsigned xp(int kx) { return (2 * kx + 63) / 64; }
     static constexpr size_t smem(int kx)
     {
-        return 1024 + GROUPS * (size_t)PANEL * (HP + xp(kx)) + (size_t)WROWS * 128 * (HP + xp(kx)) +
-               sizeof(float) * (GROUPS * (ROWS * GS + CG * ROWS) + 4 * N) + GROUPS * sizeof(TileRow) * ROWS;
+        return 1024 + (size_t)PANEL * (HP + xp(kx)) + (size_t)WROWS * 128 * (HP + xp(kx)) +
+               sizeof(float) * (ROWS * GS + CG * ROWS + 4 * N) + sizeof(TileRow) * ROWS;
     }
 };
 
-template <int N, int XJ>
-__global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(AdjArgs a)
+__global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjArgs a)
 {
-    using C = TileAdj<N>;
+    using C = TileAdj;
+    constexpr int N = C::N;
     constexpr unsigned WR = C::WROWS;
     constexpr float LOG2E = 1.4426950408889634f;
     StatusBlock *st = a.st;
-    if (*(volatile int *)&st->done) return;
+    const int burn = adjoint_burn(a, st);
+    if (*(volatile int *)&st->done || burn == 0) return;
 
     extern __shared__ __align__(16) unsigned char smem_tile[];
-    __shared__ __align__(8) uint64_t s_bars[C::GROUPS][2];
+    __shared__ __align__(8) uint64_t bar1, bar2;
     __shared__ unsigned s_tmem, s_top;
-    __shared__ int s_aborts[C::GROUPS][2], s_sides[C::GROUPS][2];
+    __shared__ int s_abort[2], s_side[2];               // s_abort: a wait for products 1, 2 ran out (each read behind a sync that
+                                                         // follows its writes, and before one that precedes the next)
     unsigned char *sm = (unsigned char *)(((uintptr_t)smem_tile + 1023) & ~(uintptr_t)1023);
     const int m = a.m, kx = (m + 15) & ~15;
-    const int all = threadIdx.x, grp = all / C::GT, tid = all % C::GT, lane = tid & 31, warp = tid >> 5;       // (tid, warp: of the group)
-    const unsigned operands = C::PANEL * (C::HP + C::xp(kx));
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned char *sWh = sm, *sWi = sWh + WR * 128 * C::HP;
-    unsigned char *sH = sWi + WR * 128 * C::xp(kx) + grp * operands, *sX = sH + C::PANEL * C::HP;
-    float *sb = reinterpret_cast<float *>(sWi + WR * 128 * C::xp(kx) + C::GROUPS * operands);
-    float *sG = sb + 4 * N + grp * (C::ROWS * C::GS + C::CG * C::ROWS), *sMax = sG + C::ROWS * C::GS;
-    TileRow *rows = reinterpret_cast<TileRow *>(sb + 4 * N + C::GROUPS * (C::ROWS * C::GS + C::CG * C::ROWS)) + grp * C::ROWS;
-    uint64_t &bar1 = s_bars[grp][0], &bar2 = s_bars[grp][1];
-    int *s_abort = s_aborts[grp];                        // a wait for products 1, 2 ran out (each read behind a sync that follows
-                                                         // its writes, and before one that precedes the next)
-    int *s_side = s_sides[grp];
-    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(C::GT) : "memory"); };
-    const int L = a.L, T = a.T, nchain = (T + L - 1) / L, burn = a.burn;
+    unsigned char *sH = sWi + WR * 128 * C::xp(kx), *sX = sH + C::PANEL * C::HP;
+    float *sb = reinterpret_cast<float *>(sX + C::PANEL * C::xp(kx));
+    float *sG = sb + 4 * N, *sMax = sG + C::ROWS * C::GS;
+    TileRow *rows = reinterpret_cast<TileRow *>(sMax + C::CG * C::ROWS);
+    const int L = a.L, T = a.T, nchain = (T + L - 1) / L;
     const long long total = (long long)a.B * nchain;
-    const long long tile = (long long)blockIdx.x * C::GROUPS + grp;
+    const long long tile = blockIdx.x;
 
     // ---- weights, biases, geometry, tensor memory
     const float wscale = tile_weight_scale(a.h0.W_h, 3 * N * N, a.h0.W_i, 3 * N * m, &s_top);
     const float kS = 1.0f / (wscale * TILE_OP_SCALE);
-    for (int i = all; i < (int)WR * (N / 2); i += C::THREADS) {          // rows of W_h in the order n, r, z
+    for (int i = tid; i < (int)WR * (N / 2); i += C::THREADS) {          // rows of W_h in the order n, r, z
         const int k = 2 * (i % (N / 2)), r = i / (N / 2), gate = r < N ? 2 : r / N - 1;
         const float2 v = *reinterpret_cast<const float2 *>(a.h0.W_h + (size_t)(gate * N + r % N) * N + k);
         unsigned hi, lo;
@@ -74,7 +70,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         *reinterpret_cast<unsigned *>(sWh + panel_off(WR, r, k)) = hi;
         *reinterpret_cast<unsigned *>(sWh + panel_off(WR, r, N + k)) = lo;
     }
-    for (int i = all; i < (int)WR * (kx / 2); i += C::THREADS) {         // rows of W_i in the order r, z, n
+    for (int i = tid; i < (int)WR * (kx / 2); i += C::THREADS) {         // rows of W_i in the order r, z, n
         const int k = 2 * (i % (kx / 2)), r = i / (kx / 2);
         const float *w = a.h0.W_i + (size_t)r * m + k;
         unsigned hi, lo;
@@ -82,7 +78,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, k)) = hi;
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, kx + k)) = lo;
     }
-    for (int i = all; i < N; i += C::THREADS) {
+    for (int i = tid; i < N; i += C::THREADS) {
         sb[i] = -LOG2E * (a.h0.b_h[i] + a.h0.b_i[i]);
         sb[N + i] = -LOG2E * (a.h0.b_h[N + i] + a.h0.b_i[N + i]);
         sb[2 * N + i] = a.h0.b_h[2 * N + i];
@@ -102,19 +98,19 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         rows[tid] = r;
     }
     if (tid == 0) { mbar_init(&bar1, 1); mbar_init(&bar2, 1); s_abort[0] = s_abort[1] = 0; s_side[0] = s_side[1] = 0; }
-    if (all < 32) {
+    if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(C::TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tile_fence_before();
     __syncthreads();
     tile_fence_after();
-    const unsigned tmem = s_tmem + (unsigned)grp * C::TCOLS;
+    const unsigned tmem = s_tmem;
     const int xv = (m & 3) == 0 && ((uintptr_t)a.x & 15) == 0 ? 4 : (m & 1) == 0 && ((uintptr_t)a.x & 7) == 0 ? 2 : 1;
 
-    // ---- loader mapping: rows lr + 32 i, columns 4 lc .. 4 lc + 3 (of x also 4 lc + N ..)
+    // ---- loader mapping: rows lr + 32 i, columns 4 lc .. 4 lc + 3
     const int lr = tid / C::LPR, lc = tid % C::LPR;
-    float4 yv[4], xr[4][XJ];
+    float4 yv[4], xr[4];
     unsigned x_in = 0u;                                  // rows (bit i) that are inside their chain
     auto load = [&](int step) {                          // the state before every row's time step, and x there
         x_in = 0u;
@@ -129,25 +125,22 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
             const float *h = (in && !first ? a.y : a.y0) + (size_t)(unsigned)(in && !first ? r.e - step - 1 : r.b) * N;
             yv[i] = __ldg(reinterpret_cast<const float4 *>(h) + lc);
         }
+        const int c = 4 * lc;
+        if (xv == 4) {
+            const int cc = min(c, m - 4);
 #pragma unroll
-        for (int j = 0; j < XJ; ++j) {
-            const int c = 4 * lc + N * j;
-            if (xv == 4) {
-                const int cc = min(c, m - 4);
+            for (int i = 0; i < 4; ++i) xr[i] = __ldg(reinterpret_cast<const float4 *>(p[i] + cc));
+        } else if (xv == 2) {
+            const int ca = min(c, m - 2), cb = min(c + 2, m - 2);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) xr[i][j] = __ldg(reinterpret_cast<const float4 *>(p[i] + cc));
-            } else if (xv == 2) {
-                const int ca = min(c, m - 2), cb = min(c + 2, m - 2);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 u = __ldg(reinterpret_cast<const float2 *>(p[i] + ca)), v = __ldg(reinterpret_cast<const float2 *>(p[i] + cb));
-                    xr[i][j] = make_float4(u.x, u.y, v.x, v.y);
-                }
-            } else {
-                const int c1 = min(c, m - 1), c2 = min(c + 1, m - 1), c3 = min(c + 2, m - 1), c4 = min(c + 3, m - 1);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xr[i][j] = make_float4(__ldg(p[i] + c1), __ldg(p[i] + c2), __ldg(p[i] + c3), __ldg(p[i] + c4));
+            for (int i = 0; i < 4; ++i) {
+                const float2 u = __ldg(reinterpret_cast<const float2 *>(p[i] + ca)), v = __ldg(reinterpret_cast<const float2 *>(p[i] + cb));
+                xr[i] = make_float4(u.x, u.y, v.x, v.y);
             }
+        } else {
+            const int c1 = min(c, m - 1), c2 = min(c + 1, m - 1), c3 = min(c + 2, m - 1), c4 = min(c + 3, m - 1);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xr[i] = make_float4(__ldg(p[i] + c1), __ldg(p[i] + c2), __ldg(p[i] + c3), __ldg(p[i] + c4));
         }
     };
     auto load_g = [&](int step) {                        // dL/dy of every row's step straight into sG (zeros outside the chain)
@@ -174,16 +167,13 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
     auto put_operands = [&]() {
 #pragma unroll
         for (int i = 0; i < 4; ++i) put(sH, lr + 32 * i, 4 * lc, N, wanted((x_in >> i) & 1u, yv[i]));
+        const int c = 4 * lc;
+        if (c >= kx) return;
 #pragma unroll
-        for (int j = 0; j < XJ; ++j) {
-            const int c = 4 * lc + N * j;
-            if (c >= kx) continue;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float4 v = wanted((x_in >> i) & 1u && c < m, xr[i][j]);
-                if (!whole) { v.y = c + 1 < m ? v.y : 0.f; v.z = c + 2 < m ? v.z : 0.f; v.w = c + 3 < m ? v.w : 0.f; }
-                put(sX, lr + 32 * i, c, kx, v);
-            }
+        for (int i = 0; i < 4; ++i) {
+            float4 v = wanted((x_in >> i) & 1u && c < m, xr[i]);
+            if (!whole) { v.y = c + 1 < m ? v.y : 0.f; v.z = c + 2 < m ? v.z : 0.f; v.w = c + 3 < m ? v.w : 0.f; }
+            put(sX, lr + 32 * i, c, kx, v);
         }
     };
 
@@ -221,7 +211,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         cp_async_wait_0();
         fence_proxy_async();
         tile_fence_before();
-        group_sync();                                    // operands and dL/dy of this step are there
+        __syncthreads();                                    // operands and dL/dy of this step are there
         if (*(volatile int *)&s_abort[1]) break;
         if (uwarp == 0) {
             tile_fence_after();
@@ -257,7 +247,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         for (int j = 0; j < 8; ++j) top = max(top, max(__float_as_uint(fabsf(l[j].x)), __float_as_uint(fabsf(l[j].y))));
         if (keep) mb = max(mb, top);
         sMax[cg * C::ROWS + row] = __uint_as_float(top);
-        group_sync();
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < C::CG; ++k) top = max(top, __float_as_uint(sMax[k * C::ROWS + row]));
         // p up to about 2^8 (|p| <= |lambda| / 4 or so): exponent of the row's largest |lambda| to 2^9
@@ -331,13 +321,13 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         }
         tile_wait_st();
         tile_fence_before();
-        group_sync();                                    // p of every row is in tensor memory; the operands are free
+        __syncthreads();                                    // p of every row is in tensor memory; the operands are free
         if (*(volatile int *)&s_abort[0]) break;
         if (uwarp == 0) {
             tile_fence_after();
             if (tile_elect()) {
                 // p W_h: K steps of 16 gate rows; B MN-major: 16 rows of W_h's operand, n contiguous (lo half: n f16 further on)
-                const uint64_t lo_at = N == 32 ? (uint64_t)(64 >> 4) : (uint64_t)((WR * 128) >> 4);
+                const uint64_t lo_at = (uint64_t)((WR * 128) >> 4);
 #pragma unroll
                 for (int k = 0; k < 3 * N; k += 16) {
                     const uint64_t b = dWh + (uint64_t)((k * 128) >> 4);
@@ -366,7 +356,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         }
     }
     cp_async_wait_0();
-    group_sync();
+    __syncthreads();
 
     // ---- the state that leaves the first time step: the gradient w.r.t. y0
     if (a.dy0 && own.te > 0 && !has_next) {
@@ -405,7 +395,7 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
         s_side[1] = T - chain * L < reach ? 2 : 1;
         __threadfence();
     }
-    group_sync();
+    __syncthreads();
     if (warp < 2 && s_side[warp]) {
         const size_t edge = (size_t)tile - warp;
         unsigned old = 0;
@@ -442,14 +432,14 @@ __global__ void __launch_bounds__(TileAdj<N>::THREADS, 1) adjoint_tile_kernel(Ad
     tile_fence_before();
     __syncthreads();
     tile_fence_after();
-    if (all < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(C::TMEM) : "memory");
-    if (all == 0) {
+    if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(C::TMEM) : "memory");
+    if (tid == 0) {
         __threadfence();
         const unsigned prev = atomicAdd(&st->exit_counter, 1u);
         if (prev + 1u == gridDim.x) {
             __threadfence();
             st->exit_counter = 0u;
-            adjoint_decide(st, a.eta, a.dy0 != nullptr);
+            adjoint_decide(st, a.eta, a.dy0 != nullptr, burn);
         }
     }
 }

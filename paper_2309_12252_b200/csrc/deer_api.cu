@@ -1057,11 +1057,10 @@ static bool body_takes(int n, int m, int flags)
 template <typename CopyOut>
 static int eval_one_launch(const deer_gru_params *p, const float *x, const float *y0, int B, int T, float tol, int max_iter,
                            const EvalWs &w, float *const (&buf)[2], int flags, cudaStream_t st, StatusBlock *hs, HostResult *hr,
-                           CopyOut copy_out)
+                           bool &u_done, CopyOut copy_out)
 {
     const int n = p->n, m = p->m;
     const bool need_u = !body_supported(n, m, false);
-    bool u_done = false;
     int rc, burn = body_first_burn(n, tol);
     BodyArgs a{};
     a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0};
@@ -1102,6 +1101,12 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
             e.agg_words = w.words; e.nagg_words = (size_t)4 * plan.max_ctas;
         } else {
             e.flags = w.edge_flag; e.nflags = (size_t)plan.edges;
+        }
+        if (T > plan.burn_cap) {
+            // a cell initialised to remember for long: where its slowest state, by the bias of its update gate, keeps a tenth
+            // over the longest burn-in, no try is made
+            e.b_i = p->b_i; e.b_h = p->b_h; e.n = n;
+            e.slow = powf(0.1f, 1.0f / (float)plan.burn_cap);
         }
         const unsigned blocks = (unsigned)((e.nflags + e.nstarts + 1023) / 1024);
         DEER_KERNEL("eval_begin_kernel", st, eval_begin_kernel<<<blocks < 1u ? 1u : blocks, 256, 0, st>>>(w.st, init, e));
@@ -1145,7 +1150,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
                          float tol, int max_iter, float *y, int *iters, float *err,
                          float *err_trace, void *ws, size_t ws_bytes, int flags, cudaStream_t st,
                          float *y_host = nullptr, float *err_b = nullptr, unsigned long long *err_argmax = nullptr,
-                         cudaStream_t copy_st = nullptr, cudaEvent_t copy_ev = nullptr, int bodies_done = 0)
+                         cudaStream_t copy_st = nullptr, cudaEvent_t copy_ev = nullptr, int bodies_done = 0, int *burn_in = nullptr)
 {
     const int n = p->n, m = p->m;
     EvalWs w = carve_eval(ws, B, T, n, m);
@@ -1178,10 +1183,12 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
         DEER_CHECK_CUDA(cudaMemcpyAsync(w.yalt, y, N * n * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy iterate");
     const bool one_launch = bodies_done == 0 && body_takes(n, m, flags);
     HostSlot slot(one_launch);
+    bool u_done = false;                       // w.u holds the projected inputs
     bool ended_there = false;                  // the one-launch form ran to the end
     if (one_launch) {
-        if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, copy_out)) != DEER_OK) return rc;
+        if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, u_done, copy_out)) != DEER_OK) return rc;
         ended_there = hs.done == BODY_DONE;
+        if (burn_in) *burn_in = hs.burn;       // what the last body had or would have needed
     }
     if (!one_launch || hs.done != BODY_DONE) {
     const int k0 = hs.iters;                   // bodies that the one-launch form has done
@@ -1232,7 +1239,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
         DEER_KERNEL("eval_begin_kernel", st, eval_begin_kernel<<<blocks, 256, 0, st>>>(w.st, init, e));
     }
     const bool cell_proj = gen_J && coef_cell_projects(n, m, x);     // (n = 32: the coefficient cell contracts x W_i^T itself)
-    if (!fused_proj && !cell_proj && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
+    if (!fused_proj && !cell_proj && !u_done && (rc = run_proj(p, x, w.u, N, st)) != DEER_OK) return rc;
 
     // Newton loop (App. B.1): bodies are enqueued ahead of the convergence test -- the decision at
     // the end of each body is taken on the device, and the kernels of bodies past the end return
@@ -1338,7 +1345,7 @@ static int launch_vjp_small(const VjpSmallArgs &v, int n, int m, int *P, cudaStr
 
 static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y0, const float *y,
                         const float *gy, int B, int T, const deer_gru_grads *g, float *dx,
-                        float *dy0, void *ws, size_t ws_bytes, int flags, cudaStream_t st)
+                        float *dy0, void *ws, size_t ws_bytes, int flags, cudaStream_t st, int burn_hint = 0)
 {
     const int n = p->n, m = p->m, n3 = 3 * n;
     VjpWs w = carve_vjp(ws, B, T, n, m);
@@ -1351,14 +1358,16 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
                        ((((uintptr_t)y | (uintptr_t)y0) & 15) == 0);
     const bool have_u = !adjoint_supported(n, m, false);
     BodyPlan plan{};
-    // n = 32, 64: 128 chains per tcgen05 tile; else sixteen per warp
+    // n = 64: 128 chains per tcgen05 tile; else sixteen per warp
     BodyPlan tplan{};
     const bool exact_flags = (flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) != 0;
+    const int first_burn = std::max(burn_hint, ADJ_BURN);
+    auto worth = [&](const BodyPlan &q) { return first_burn <= adjoint_burn_cap(n, m, (long long)B * T, q.L); };
     const bool tile = !exact_flags && (((uintptr_t)y | (uintptr_t)y0 | (uintptr_t)gy | (uintptr_t)x | (uintptr_t)p->W_h | (uintptr_t)p->W_i | (uintptr_t)dx) & 15) == 0 &&
-                      adjoint_tile_plan(&tplan, B, T, n, m);
+                      adjoint_tile_plan(&tplan, B, T, n, m) && worth(tplan);
     const bool lanes = small && !exact_flags && (((uintptr_t)gy) & 3) == 0 && rows_adjoint_plan(&plan, B, T, n, m, WGRAD_P);     // all in one launch
     const bool adj = lanes || (!tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
-                     adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && adjoint_suits(plan, n));
+                     adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && worth(plan));
     DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj || tile ? (size_t)(tile ? tplan : plan).edges * sizeof(unsigned) : 0), st), "memset status");
     const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
     if (adj || tile) {
@@ -1372,8 +1381,9 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
         a.eta = ADJ_ETA;
         a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = tile ? w.J : w.starts;
         // (small cells: one try, the passes behind it are cheap)
+        a.burn = lanes ? ADJ_BURN : first_burn;
+        a.burn_cap = lanes ? 0 : adjoint_burn_cap(n, m, (long long)B * T, a.L);
         for (int k = 0; k < (lanes ? 1 : ADJ_TRIES); ++k) {
-            a.burn = ADJ_BURN[k];
             if ((rc = tile ? launch_adjoint_tile(a, tplan, st) : lanes ? launch_rows_adjoint(a, plan, w.partial, w.partial2, dx, st) : launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
         }
         unless = w.st;
@@ -1689,6 +1699,14 @@ int deer_gru_vjp(const deer_gru_params *p, const float *x, const float *y0, cons
     return gru_vjp_impl(p, x, y0, y, gy, B, T, g, dx, dy0, ws, ws_bytes, flags, (cudaStream_t)stream);
 }
 
+// The burn-in that a gradient's boundaries need, from the one that the evaluation of the same trajectory came to (0: the
+// evaluation tells nothing beyond its first one): the accuracy asked for goes with the burn-in's logarithm.
+static int adjoint_burn_hint(int burn, int n, float tol)
+{
+    if (burn <= body_first_burn(n, tol)) return 0;
+    return (int)fminf(1e6f, (float)burn * logf(0.5f * ADJ_ETA) / logf(0.5f * body_eta(n, tol)));
+}
+
 int deer_gru_classifier_step(const deer_gru_params *l1, const deer_gru_params *l2, const float *W_o,
                              const float *b_o, int ncls, const float *x, const int *labels, int B,
                              int T, float tol, int max_iter, float *loss, int *iters,
@@ -1706,16 +1724,21 @@ int deer_gru_classifier_step(const deer_gru_params *l1, const deer_gru_params *l
     ClsWs w = carve_cls(ws, B, T, n, m, 64);
     int rc = check_ws(ws, ws_bytes, w.bytes);
     if (rc != DEER_OK) return rc;
+    for (const deer_gru_params *l : {l1, l2})
+        if (!l->W_i || !l->W_h || !l->b_i || !l->b_h || l->m <= 0 || !valid_sizes(B, T, l->n, l->m)) return DEER_ERR_INVALID_ARG;
+    for (const deer_gru_grads *g : {g1, g2})
+        if (!g->dW_i || !g->dW_h || !g->db_i || !g->db_h) return DEER_ERR_INVALID_ARG;
     const size_t N = (size_t)B * T;
     // zero initial states live at the head of gyB until the backward pass needs it
     float *zero0 = w.gyB;
     DEER_CHECK_CUDA(cudaMemsetAsync(zero0, 0, (size_t)B * n * sizeof(float), st), "memset y0");
     int it[2] = {0, 0};
-    int s1 = deer_gru_eval(l1, x, zero0, B, T, tol, max_iter, w.y1, &it[0], nullptr, nullptr, w.inner,
-                           w.inner_bytes, flags, stream);
+    int burn1 = 0, burn2 = 0;
+    int s1 = gru_eval_impl(l1, x, zero0, B, T, tol, max_iter, w.y1, &it[0], nullptr, nullptr, w.inner,
+                           w.inner_bytes, flags, st, nullptr, nullptr, nullptr, nullptr, nullptr, 0, &burn1);
     if (s1 < 0) return s1;
-    int s2 = deer_gru_eval(l2, w.y1, zero0, B, T, tol, max_iter, w.y2, &it[1], nullptr, nullptr,
-                           w.inner, w.inner_bytes, flags, stream);
+    int s2 = gru_eval_impl(l2, w.y1, zero0, B, T, tol, max_iter, w.y2, &it[1], nullptr, nullptr,
+                           w.inner, w.inner_bytes, flags, st, nullptr, nullptr, nullptr, nullptr, nullptr, 0, &burn2);
     if (s2 < 0) return s2;
     if (iters) { iters[0] = it[0]; iters[1] = it[1]; }
     int seg_len = (T + POOL_SEGS - 1) / POOL_SEGS;
@@ -1730,12 +1753,12 @@ int deer_gru_classifier_step(const deer_gru_params *l1, const deer_gru_params *l
     // the backward passes are asynchronous and share one status block: the flags word of each is
     // saved beside the loss before the next call clears it, and both are read after the final sync
     const unsigned *vflags = &reinterpret_cast<const StatusBlock *>(w.inner)->flags;
-    rc = deer_gru_vjp(l2, w.y1, zero1, w.y2, w.gyA, B, T, g2, w.gyB, nullptr, w.inner, w.inner_bytes,
-                      flags, stream);
+    rc = gru_vjp_impl(l2, w.y1, zero1, w.y2, w.gyA, B, T, g2, w.gyB, nullptr, w.inner, w.inner_bytes,
+                      flags, st, adjoint_burn_hint(burn2, n, tol));
     if (rc != DEER_OK) return rc;
     DEER_CHECK_CUDA(cudaMemcpyAsync(w.loss + 1, vflags, sizeof(unsigned), cudaMemcpyDeviceToDevice, st), "save status");
-    rc = deer_gru_vjp(l1, x, zero1, w.y1, w.gyB, B, T, g1, nullptr, nullptr, w.inner, w.inner_bytes,
-                      flags, stream);
+    rc = gru_vjp_impl(l1, x, zero1, w.y1, w.gyB, B, T, g1, nullptr, nullptr, w.inner, w.inner_bytes,
+                      flags, st, adjoint_burn_hint(burn1, n, tol));
     if (rc != DEER_OK) return rc;
     DEER_CHECK_CUDA(cudaMemcpyAsync(w.loss + 2, vflags, sizeof(unsigned), cudaMemcpyDeviceToDevice, st), "save status");
     float tail[3];
@@ -2053,10 +2076,10 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     a.B = B; a.T = T; a.n = n; a.m = m; a.H = H; a.L = plan.L;
     a.eta = ADJ_ETA;
     a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = w.starts;
-    for (int k = 0; k < ADJ_TRIES; ++k) {
-        a.burn = ADJ_BURN[k];
+    a.burn = ADJ_BURN;
+    a.burn_cap = 512;                                    // (what comes behind goes head by head)
+    for (int k = 0; k < ADJ_TRIES; ++k)
         if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
-    }
     // dW_i, db_i of all heads: one contraction of dG_i [N, H*3n] with x [N, m]
     WgradArgs wa{};
     wa.dG = w.dGi; wa.V = x; wa.T = T; wa.n3 = H * n3; wa.K = m; wa.N = N;

@@ -324,12 +324,26 @@ struct EvalBeginArgs {
     unsigned *flags; size_t nflags;              // single-pass scan words (nullptr / 0 when not used)
     unsigned long long *starts; size_t nstarts;
     unsigned long long *agg_words; size_t nagg_words;
+    const float *b_i, *b_h; int n; float slow;  // one-launch bodies (or nullptr): they give up at once where an update gate's
+                                                // bias alone keeps more than `slow` of a state per step
 };
 __global__ void eval_begin_kernel(StatusBlock *st, StatusBlock init, EvalBeginArgs e)
 {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 == 0) *st = init;
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        float z = 0.0f;
+        if (e.b_i) for (int i = threadIdx.x; i < e.n; i += 32) z = fmaxf(z, 1.0f / (1.0f + __expf(-(e.b_i[e.n + i] + e.b_h[e.n + i]))));
+        z = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z)));
+        if (threadIdx.x == 0) {
+            if (e.b_i && z > e.slow) {
+                init.done = BODY_FALL_BACK;
+                init.burn = (int)fminf(1e6f, -2.3f / __logf(z)) + 1;             // until a tenth is left
+                if (init.host) { init.host->burn = init.burn; init.host->done = init.done; }
+            }
+            *st = init;
+        }
+    }
     if (e.y) {
         if (((uintptr_t)e.y & 15) == 0) {
             float4 *y4 = reinterpret_cast<float4 *>(e.y);
@@ -597,7 +611,8 @@ __global__ void vjp_dx_kernel(const float *__restrict__ dGi, const float *__rest
     int k = (int)(idx - e * m);
     const float *g = dGi + e * ld;
     float acc = 0.0f;
-    for (int j = 0; j < n3; ++j) acc = fmaf(W_i[(size_t)j * m + k], g[j < gap_at ? j : j + gap], acc);
+    for (int j = 0; j < gap_at; ++j) acc = fmaf(W_i[(size_t)j * m + k], g[j], acc);
+    for (int j = gap_at; j < n3; ++j) acc = fmaf(W_i[(size_t)j * m + k], g[j + gap], acc);
     dx[idx] = acc;
 }
 

@@ -31,12 +31,25 @@ template <int N> struct Adj {
     }
 };
 
+// The burn-in of this launch: the call's, or what the launch before this one found to be needed (0: more than is worth trying).
+__device__ __forceinline__ int adjoint_burn(const AdjArgs &a, const StatusBlock *st)
+{
+    const int want = *(const volatile int *)&st->burn;
+    return want == 0 ? a.burn : want <= a.burn_cap ? want : 0;
+}
+
 // End of the launch: were the boundaries good enough?  Single thread.
-__device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool dy0)
+__device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool dy0, int burn)
 {
     auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
     const float top = take(st->err_bits), mis = take(st->mis_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
-    if (mis <= eta * top && (!dy0 || mis_end <= eta * top_end)) st->done = BODY_DONE;
+    const bool inner = mis <= eta * top, end = !dy0 || mis_end <= eta * top_end;
+    if (inner && end) { st->done = BODY_DONE; return; }
+    // the carried error is about max|lambda| * rho^burn: the burn-in after which it is half of what is accepted
+    int want = 1 << 20;
+    if (inner) want = 3 * burn;
+    else if (mis < 0.7f * top) want = (int)(1.1f * (float)burn * __logf(0.5f * eta) / __logf(mis / top)) + 4;
+    st->burn = max(want, burn + 8);
 }
 
 template <int N, bool V2>
@@ -93,10 +106,10 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     float *ss = sb + 4 * N + warp * 16 * SW;             // start states of this warp's chains
     if constexpr (C::SS_GLOBAL) ss = a.starts + ((size_t)hd.first_edge + (size_t)blockIdx.x * nwarps + warp) * 16 * SW;
     pdl_prologue();
-    if (*(volatile int *)&st->done) return;
+    const int burn = adjoint_burn(a, st);
+    if (*(volatile int *)&st->done || burn == 0) return;
     __syncthreads();
 
-    const int burn = a.burn;
     const long long grp = (long long)blockIdx.x * nwarps + warp;
     unsigned mb = 0u, mis = 0u, mb_end = 0u, mis_end = 0u;
 
@@ -431,7 +444,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            adjoint_decide(st, a.eta, a.dy0 != nullptr);
+            adjoint_decide(st, a.eta, a.dy0 != nullptr, burn);
         }
     }
 }

@@ -115,6 +115,7 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
     p->warps = threads / 32;
     p->smem = smem;
     const long long cap = (long long)sm_count() * std::min(occ_cap, occupancy_of(kern, threads, smem));      // CTAs of one wave
+    p->share = (float)((double)B * T * H / ((double)cap * chains));
     double best = 0.0;
     // (gran: what the chain length is a multiple of)
     for (int L = std::max(16, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
@@ -135,6 +136,29 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
     p->max_ctas = c.worst; p->edges = c.edges;
 }
 
+// Burn-ins that are worth trying.  A launch takes burn + L steps, whatever its size while it is one wave; the kernels that
+// multiply the Jacobians out take `a` such steps' time for a small problem and `b` for every position of `share` more (B200, us
+// per body, here per step / there, positions in thousands, m = 4 or 8):
+//   n = 1   0.6-1.0 / 34 (192) 44 (1,600)              n = 16  2.8-3.2 / 148 (240) 280 (640)
+//   n = 2   0.6-0.8 / 32 (192) 66 (1,600)              n = 32  4.6 / 106 (32) 193 (128) 554 (640)
+//   n = 4   0.75-0.9 / 39 (192) 120 (1,600)            n = 64  5.0-6.4 / 311 (16) 714 (128) 1508 (320)
+//   n = 8   1.5-2.1 / 72 (192) 178 (640) 396 (1,600)
+// Only the powers of two have tuned kernels of that kind; the others' are an order of magnitude slower.
+static int worth_trying(const BodyPlan &p, int n)
+{
+    float a, b;
+    switch (n) {
+    case 1: case 2: a = 45.0f; b = 2.0f; break;
+    case 4: a = 30.0f; b = 2.7f; break;
+    case 8: a = 24.0f; b = 4.0f; break;
+    case 16: a = 30.0f; b = 2.6f; break;
+    case 32: a = 15.0f; b = 6.7f; break;
+    case 64: a = 36.0f; b = 13.0f; break;
+    default: return std::max(320, 8 * p.L);
+    }
+    return (int)(a + b * p.share) - p.L;
+}
+
 bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H)
 {
     const int kx = have_u ? 0 : (m + 7) / 8, sms = sm_count(), Tmax = longest(T, strides, H);
@@ -146,14 +170,15 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         const LaneKernel lk = lane_kernel(n, m, have_u);
         const int burn = (body_first_burn(n, 1.0f) + lk.W - 1) / lk.W * lk.W;
         one_wave_of_chains(p, (const void *)lk.kern, 128, 128, 32, lk.W, lk.smem, burn, B, T, strides, H);
-        p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
+        p->burn_cap = worth_trying(*p, n);
         return true;
     }
     if (form == BodyForm::TILE) {
         if (!(n == 32 || n == 64) || have_u || m > 64 || H != 1 || strides) return false;
         if (k.tile_smem(m) > BODY_SMEM_MAX) return false;
         one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, 1, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H);
-        p->burn_cap = std::max(96, 2 * p->L);
+        if (p->edges <= sms) p->max_ctas = (int)p->edges;      // (two tiles per CTA only where there are more than SMs)
+        p->burn_cap = worth_trying(*p, n);
         return true;
     }
     if (form == BodyForm::TWO_PHASE) {
@@ -168,7 +193,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         // Where none is short enough, the CTA that holds most positions.
         for (int L = 5; ; L += 2) {
             const int nc_fit = std::min(k.nc_max, own / L / 16 * 16);
-            if (nc_fit < 16) return p->NC > 0 && p->max_ctas > 0;
+            if (nc_fit < 16) break;
             int NC = 16;
             while (2 * NC <= nc_fit && count_ctas(B, T, strides, H, L, NC, NC).ctas > sms) NC *= 2;
             const Count c = count_ctas(B, T, strides, H, L, NC, NC);
@@ -178,12 +203,17 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
                 p->smem = fixed + k.slot_bytes * (size_t)(cap + NC * L);
             }
             p->whole_loop = (long long)c.worst * H <= sms;      // (the grid is max_ctas x H)
-            if (c.ctas <= sms || L >= Tmax) return true;
+            if (c.ctas <= sms || L >= Tmax) break;
         }
+        if (!(p->NC > 0 && p->max_ctas > 0)) return false;
+        // A step of a chain takes an eighth of a microsecond (n <= 8) to a half; a body of the other kernels 30 to 90 us.  The
+        // slots that the CTA's own positions leave are there for longer burn-ins.
+        p->burn_cap = std::max(cap, std::min(slots - p->NC * p->L, (n & (n - 1)) != 0 ? 512 : n <= 8 ? 128 : 224));
+        p->smem = fixed + k.slot_bytes * (size_t)(p->burn_cap + p->NC * p->L);
+        return true;
     }
     one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
-    // (tuned kernels that multiply the Jacobians out exist for the powers of two; the any-n kernels are an order of magnitude slower)
-    p->burn_cap = (n & (n - 1)) == 0 ? std::max(96, 2 * p->L) : std::max(320, 8 * p->L);
+    p->burn_cap = worth_trying(*p, n);
     return true;
 }
 
@@ -198,19 +228,38 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN[0], B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN, B, T, strides, H);
     return true;
 }
 
 size_t adjoint_starts(int n) { return n > 48 ? 16 * (size_t)((n + 7) / 8 * 8 + 4) : 0; }
 
-// Where the kernels that multiply the Jacobians out are tuned (powers of two), half a wave of chains or more; for n >= 32 their
-// 3 x TF32 products are so much more work that a part of a wave is enough.  n <= 4 pads to 8 columns and stays with its own.
-// (B200, us per gradient, here / there: n = 8, B = 16, T = 1e4 117 / 92; n = 32, T = 1e5 2210 / 5046)
-bool adjoint_suits(const BodyPlan &p, int n)
+// From how many positions on is the adjoint launch faster than the kernels that multiply the Jacobians out?  Its time is that
+// of its steps (44 + 16 of them, some 3 us each, more with the channels that a step contracts) until the chains fill the GPU.
+// (B200, us per gradient, here / there, B = 8: n = 9, m = 8 202 / 138 at 6,400 positions, 208 / 200 at 20,000; n = 20, m = 8
+// 228 / 244 at 6,400; n = 28, m = 60 530 / 400 at 6,400, 561 / 737 at 20,000; n = 16, m = 3 219 / 180 at 80,000, 295 / 305 at
+// 160,000; n = 32, m = 3 395 / 263 at 40,000, 436 / 411 at 80,000, m = 64 653 / 465 and 849 / 762 at 80,000 and 160,000;
+// n = 64, here a tile, 728 / 525 at 20,000, 793 / 722 at 40,000, 819 / 881 at 56,000 whatever m.)
+// n <= 4 pads to 8 columns where its own kernels are tuned; n = 64 with m > 64 is no tile's (nor worth its spills early).
+static float adjoint_line(int n, int m)
 {
-    if ((n & (n - 1)) != 0) return true;
-    return n <= 4 ? false : n <= 16 ? p.waves >= 0.6f : p.waves >= 0.1f;
+    const float c = (float)m;
+    switch (n) {
+    case 1: case 2: case 4: return 1e30f;
+    case 8: return 270000.0f;
+    case 16: return 120000.0f * (1.0f + c / 20.0f);
+    case 32: return 70000.0f * (1.0f + c / 35.0f);
+    case 64: return m <= 64 ? 50000.0f : 250000.0f;
+    }
+    if (n < 8) return 4000.0f * (1.0f + c / 8.0f);
+    if (n < 16) return 180000.0f / (float)n * (1.0f + c / 40.0f);
+    return 4000.0f * (1.0f + c / 30.0f);
+}
+
+// The other kernels' time grows with the positions: at k times the line it is that of k (44 + 16) steps.
+int adjoint_burn_cap(int n, int m, long long positions, int L)
+{
+    return (int)fminf(512.0f, (float)(ADJ_BURN + 16) * ((float)positions / adjoint_line(n, m))) - L;
 }
 
 int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
@@ -228,16 +277,17 @@ bool rows_adjoint_plan(BodyPlan *p, int B, int T, int n, int m, int max_ctas)
 {
     auto small = [](int v) { return v == 1 || v == 2 || v == 4 || v == 8; };
     if (!small(n) || !small(m)) return false;
-    one_wave_of_chains(p, (const void *)rows_adjoint_of(n, m), 128, 128 / n, 32 / n, 4, 0, ADJ_BURN[0], B, T, nullptr, 1, std::max(1, max_ctas / sm_count()));
+    one_wave_of_chains(p, (const void *)rows_adjoint_of(n, m), 128, 128 / n, 32 / n, 4, 0, ADJ_BURN, B, T, nullptr, 1, std::max(1, max_ctas / sm_count()));
     return p->max_ctas <= max_ctas;
 }
 
+// (n = 32 gains nothing over sixteen chains per warp: 2270 / 2286 us at 1.6e6 positions.)
 bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m)
 {
-    if (!(n == 32 || n == 64) || m > 64) return false;
+    if (n != 64 || m > 64) return false;
     const BodyKernels k = pick(n, true);
     if (k.adj_tile_smem(m) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, 1, k.adj_tile_smem(m), ADJ_BURN[0], B, T, nullptr, 1);
+    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, 1, k.adj_tile_smem(m), ADJ_BURN, B, T, nullptr, 1);
     return true;
 }
 
@@ -260,8 +310,9 @@ int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 // more work than their own kernels do.  Sizes without tuned kernels of the other kind always come here.
 bool body_suits(const BodyPlan &p, int n)
 {
-    if (p.form == BodyForm::TILE || p.form == BodyForm::LANE) return true;
+    if (p.form == BodyForm::TILE) return true;
     const bool tuned = (n & (n - 1)) == 0;
+    if (p.form == BodyForm::LANE) return !tuned || p.share >= (n == 1 ? 30.0f : n == 2 ? 26.0f : n == 4 ? 13.0f : 10.0f);
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
     return n == 8 || (n > 8 && p.waves >= 0.5f);

@@ -41,7 +41,8 @@ struct AdjArgs {
     float *dGi, *dGh;        // [B,T,H,3n] out: gradients w.r.t. the input-side and hidden-side pre-activations
     float *dy0;              // or nullptr; row b * H + head (dy0_by_head), else first_seq + sequence
     int dy0_by_head;
-    int B, T, n, m, H, L, burn;
+    int B, T, n, m, H, L;
+    int burn, burn_cap;      // burn-in of the first try; longest that another one is worth
     float eta;               // largest boundary mismatch that is accepted, as a part of max|lambda|
     StatusBlock *st;         // [H]; done = 1 where the launch has done the work (it returns at once where it is set)
     float *edge;
@@ -81,6 +82,7 @@ struct BodyPlan {
     int burn_cap;            // longest burn-in the launch can hold or is worth trying
     bool whole_loop;         // the whole Newton loop is one (cooperative) launch
     float waves;             // CTAs of the launch / CTAs that the GPU holds
+    float share;             // positions per chain if every chain that the GPU holds at a time had the same (one-phase, tile, lane)
     long long edges;         // boundaries between warps (one-phase) or CTAs (two-phase) of all heads at most
     size_t smem;
 };
@@ -112,14 +114,15 @@ bool adjoint_supported(int n, int m, bool have_u);
 bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const int *strides, int H);
 // floats of AdjArgs::starts per chain group (0: not used)
 size_t adjoint_starts(int n);
-bool adjoint_suits(const BodyPlan &p, int n);
+// Longest burn-in for which a launch of chains of L beats the kernels that multiply the Jacobians out.
+int adjoint_burn_cap(int n, int m, long long positions, int L);
 int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st);
-// The same with 128 chains per tcgen05 tile (adjoint_tile.cuh): n = 32, 64; AdjArgs::dGi receives packed rows [4n].
+// The same with 128 chains per tcgen05 tile (adjoint_tile.cuh): n = 64; AdjArgs::dGi receives packed rows [4n].
 bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m);
 int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st);
-// Burn-ins that are tried one after the other, and the accuracy asked of the boundaries (a one-shot solve: fp32 level).
-constexpr int ADJ_TRIES = 2;
-constexpr int ADJ_BURN[ADJ_TRIES] = {44, 128};
+// Launches of a gradient (the second with the burn-in that the first one found), the first one's burn-in, and the accuracy
+// asked of the boundaries (a one-shot solve: fp32 level).
+constexpr int ADJ_TRIES = 2, ADJ_BURN = 44;
 constexpr float ADJ_ETA = 4e-6f;
 
 }  // namespace deer

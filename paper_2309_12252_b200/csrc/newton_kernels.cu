@@ -4,10 +4,12 @@
 #include "newton_lane.cuh"
 #include "rows_adjoint.cuh"
 #include "newton_tile.cuh"
-#include "adjoint_tile.cuh"
 
 #ifndef BODY_N
 #error "BODY_N: state size, a multiple of 8 up to 64"
+#endif
+#if BODY_N == 64
+#include "adjoint_tile.cuh"
 #endif
 
 namespace deer {
@@ -27,10 +29,12 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
         k.tile = [](int m) -> void (*)(BodyArgs) { return m <= 32 ? newton_tile_kernel<N, 1, true> : newton_tile_kernel<N, 64 / N, false>; };
         k.tile_threads = TileBody<N>::THREADS;
         k.tile_chains = TileBody<N>::GROUPS * TileBody<N>::ROWS;
-        k.adj_tile = [](int m) -> void (*)(AdjArgs) { return m <= N ? adjoint_tile_kernel<N, 1> : adjoint_tile_kernel<N, 64 / N>; };
-        k.adj_tile_smem = [](int m) { return TileAdj<N>::smem((m + 15) & ~15); };
         k.tile_smem = [](int m) { return TileBody<N>::smem((m + 15) & ~15); };
     }
+#if BODY_N == 64
+    k.adj_tile = [](int m) -> void (*)(AdjArgs) { return adjoint_tile_kernel; };
+    k.adj_tile_smem = [](int m) { return TileAdj::smem((m + 15) & ~15); };
+#endif
     k.one_warps = N > 32 ? 8 : 4;
     k.seg_warps = Seg<N>::WARPS;
     k.nc_max = Seg<N>::NC_MAX;

@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         }
         const unsigned eb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[2][lane] : 0u);
         const unsigned qb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[3][lane] : 0u);
-        const BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, tol, iters, max_iter);
+        const BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter);
         if (blockIdx.x == 0 && tid == 0) {
             if (v.counts) {
                 if (st->trace && iters < ERR_TRACE_CAP) st->trace[iters] = __uint_as_float(eb);
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap);
+            body_decide(st, a.eta, a.burn_cap, a.T);
         }
     }
     return;

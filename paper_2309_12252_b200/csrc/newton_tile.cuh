@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
     int &s_abort = s_aborts[grp];
     int *s_side = s_sides[grp];
     auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(C::GT) : "memory"); };
-    const long long tile = (long long)blockIdx.x * C::GROUPS + grp;
+    const long long tile = (long long)grp * gridDim.x + blockIdx.x;      // (few tiles: each on an SM of its own)
     const int L = a.L, T = a.T, nchain = (T + L - 1) / L;
     const long long total = (long long)a.B * nchain;
 
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
                 st->done = BODY_FALL_BACK;
                 if (HostResult *h = st->host) h->done = BODY_FALL_BACK;
             } else {
-                body_decide(st, a.eta, a.burn_cap);
+                body_decide(st, a.eta, a.burn_cap, a.T);
             }
         }
     }

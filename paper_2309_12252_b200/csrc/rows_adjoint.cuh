@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         if (prevc + 1u == gridDim.x) {
             __threadfence();
             st->exit_counter = 0u;
-            adjoint_decide(st, a.eta, a.dy0 != nullptr);
+            adjoint_decide(st, a.eta, a.dy0 != nullptr, burn);
         }
     }
 }
