@@ -112,12 +112,16 @@ static int onepass_tile_len(int n, int B, int T, int *sw)
     }
 }
 
-// Sizes for which chains with a verified burn-in pay: enough matrices that reading them is what the scan takes.  (n = 8: 32,768
-// positions.  Below, the two launches that return at once behind it cost more than it gives; n <= 2: the one-thread-per-chain
-// scan already runs at 0.7 of the copy rate.)
+// Sizes for which chains with a verified burn-in pay: enough matrices that reading them is what the scan takes; its 128 steps
+// and the launches behind it that return at once take some 30 us (n = 32: 60).  The chunked scan's time goes with the length of
+// a sequence.  (B200, us here / there: n = 4, B = 8, T = 4e4 32 / 25, T = 1e5 42 / 42, B = 1, T = 5e5 34 / 108; n = 8, B = 8,
+// T = 5e3 26 / 23, T = 2e4 36 / 38, T = 4e4 43 / 58; n = 16, B = 8, T = 5e3 44 / 41, T = 1e4 51 / 58; n = 32, B = 8, T = 2e3
+// 67 / 58, T = 3e3 71 / 76, B = 1, T = 4e3 41 / 49; n = 64, B = 1, T = 1e3 86 / 208.)  n <= 2: the one-thread-per-chain scan
+// already runs at 0.7 of the copy rate.
 static bool vscan_takes(int n, int B, int T)
 {
-    return (n == 4 || n == 8 || n == 16 || n == 32 || n == 64) && T >= 3 * VSCAN_L_MIN && (double)B * T * n * n * 4 >= 8e6;
+    const double from = n == 64 || B <= 2 ? 8e6 : n == 32 ? 80e6 : 45e6;      // bytes of J
+    return (n == 4 || n == 8 || n == 16 || n == 32 || n == 64) && T >= 3 * VSCAN_L_MIN && (double)B * T * n * n * 4 >= from;
 }
 
 static ScanWs carve_scan(Carver &cv, int B, int T, int n)

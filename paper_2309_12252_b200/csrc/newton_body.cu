@@ -106,8 +106,10 @@ static int longest(int T, const int *strides, int H)
 
 // One-phase plans: the chain length with the least estimated time.  Every CTA runs its chains' steps (burn-in and L, or the
 // whole sequence where it is no longer than L) and `cap` of them run at a time, so the launch takes the longest CTA's steps or
-// the sum over CTAs / cap, whichever is more.
-static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, int gran, size_t smem, int burn, int B, int T, const int *strides, int H, int occ_cap = 64)
+// the sum over CTAs / cap, whichever is more.  `alone`: time of a step of a nearly empty GPU as a part of a full one's (thread
+// and warp chains: n = 1 0.57 us at 0.1 waves, 1.0 at 0.75; n = 8 1.5 at 0.3, 2.1 at 0.8; n = 16 2.8 at 0.5, 3.2 at 1); below
+// zero: of a CTA that has half of its tiles, else the same throughout (n = 32 tiles: 3.5 us, 4.6 with both).
+static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int chains, int edge_unit, int gran, size_t smem, int burn, int B, int T, const int *strides, int H, float alone = 0.6f, int occ_cap = 64)
 {
     const int Tmax = longest(T, strides, H);
     p->NC = 0;
@@ -118,7 +120,7 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
     p->share = (float)((double)B * T * H / ((double)cap * chains));
     double best = 0.0;
     // (gran: what the chain length is a multiple of)
-    for (int L = std::max(16, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
+    for (int L = std::max(4, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
         double sum = 0.0, top = 0.0;
         for (int h = 0; h < H; ++h) {
             const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s, nch = (Tp + L - 1) / L;
@@ -128,9 +130,9 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
         }
         // (a launch of a little more than one wave takes two: whole waves, as far as a few of them go)
         const double waves = sum / top / (double)cap, whole = waves <= 4.0 ? ceil(waves - 1e-9) : waves;
-        const double cost = top * std::max(1.0, whole);
+        const double cost = top * (waves >= 1.0 ? whole : alone < 0.0f ? (waves <= 0.5 ? -alone : 1.0) : alone + (1.0 - alone) * waves);
         if (best == 0.0 || cost < best) { best = cost; p->L = L; p->waves = (float)waves; }
-        if (L >= Tmax || (best > 0.0 && top > best)) break;
+        if (L >= Tmax || (best > 0.0 && fabsf(alone) * top > best)) break;
     }
     const Count c = count_ctas(B, T, strides, H, p->L, chains, edge_unit);
     p->max_ctas = c.worst; p->edges = c.edges;
@@ -140,11 +142,11 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
 // multiply the Jacobians out take `a` such steps' time for a small problem and `b` for every position of `share` more (B200, us
 // per body, here per step / there, positions in thousands, m = 4 or 8):
 //   n = 1   0.6-1.0 / 34 (192) 44 (1,600)              n = 16  2.8-3.2 / 148 (240) 280 (640)
-//   n = 2   0.6-0.8 / 32 (192) 66 (1,600)              n = 32  4.6 / 106 (32) 193 (128) 554 (640)
+//   n = 2   0.6-0.8 / 32 (192) 66 (1,600)              n = 32  3.5-4.6 / 106 (32) 193 (128) 554 (640)
 //   n = 4   0.75-0.9 / 39 (192) 120 (1,600)            n = 64  5.0-6.4 / 311 (16) 714 (128) 1508 (320)
 //   n = 8   1.5-2.1 / 72 (192) 178 (640) 396 (1,600)
 // Only the powers of two have tuned kernels of that kind; the others' are an order of magnitude slower.
-static int worth_trying(const BodyPlan &p, int n)
+static int worth_trying(const BodyPlan &p, int n, int m)
 {
     float a, b;
     switch (n) {
@@ -152,7 +154,7 @@ static int worth_trying(const BodyPlan &p, int n)
     case 4: a = 30.0f; b = 2.7f; break;
     case 8: a = 24.0f; b = 4.0f; break;
     case 16: a = 30.0f; b = 2.6f; break;
-    case 32: a = 15.0f; b = 6.7f; break;
+    case 32: a = 2700.0f / (float)(128 + m); b = 1000.0f / (float)(128 + m); break;      // (a step of m = 32 takes 4.5 us)
     case 64: a = 36.0f; b = 13.0f; break;
     default: return std::max(320, 8 * p.L);
     }
@@ -170,15 +172,15 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         const LaneKernel lk = lane_kernel(n, m, have_u);
         const int burn = (body_first_burn(n, 1.0f) + lk.W - 1) / lk.W * lk.W;
         one_wave_of_chains(p, (const void *)lk.kern, 128, 128, 32, lk.W, lk.smem, burn, B, T, strides, H);
-        p->burn_cap = worth_trying(*p, n);
+        p->burn_cap = worth_trying(*p, n, m);
         return true;
     }
     if (form == BodyForm::TILE) {
         if (!(n == 32 || n == 64) || have_u || m > 64 || H != 1 || strides) return false;
         if (k.tile_smem(m) > BODY_SMEM_MAX) return false;
-        one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, 1, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H);
+        one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, 1, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H, n == 32 ? -0.75f : 1.0f);
         if (p->edges <= sms) p->max_ctas = (int)p->edges;      // (two tiles per CTA only where there are more than SMs)
-        p->burn_cap = worth_trying(*p, n);
+        p->burn_cap = worth_trying(*p, n, m);
         return true;
     }
     if (form == BodyForm::TWO_PHASE) {
@@ -213,7 +215,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         return true;
     }
     one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
-    p->burn_cap = worth_trying(*p, n);
+    p->burn_cap = worth_trying(*p, n, m);
     return true;
 }
 
@@ -228,7 +230,7 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN, B, T, strides, H);
+    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN, B, T, strides, H, 0.8f);
     return true;
 }
 
@@ -277,7 +279,7 @@ bool rows_adjoint_plan(BodyPlan *p, int B, int T, int n, int m, int max_ctas)
 {
     auto small = [](int v) { return v == 1 || v == 2 || v == 4 || v == 8; };
     if (!small(n) || !small(m)) return false;
-    one_wave_of_chains(p, (const void *)rows_adjoint_of(n, m), 128, 128 / n, 32 / n, 4, 0, ADJ_BURN, B, T, nullptr, 1, std::max(1, max_ctas / sm_count()));
+    one_wave_of_chains(p, (const void *)rows_adjoint_of(n, m), 128, 128 / n, 32 / n, 4, 0, ADJ_BURN, B, T, nullptr, 1, 0.6f, std::max(1, max_ctas / sm_count()));
     return p->max_ctas <= max_ctas;
 }
 
@@ -287,7 +289,7 @@ bool adjoint_tile_plan(BodyPlan *p, int B, int T, int n, int m)
     if (n != 64 || m > 64) return false;
     const BodyKernels k = pick(n, true);
     if (k.adj_tile_smem(m) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, 1, k.adj_tile_smem(m), ADJ_BURN, B, T, nullptr, 1);
+    one_wave_of_chains(p, (const void *)k.adj_tile(m), k.tile_threads, k.tile_chains, 128, 1, k.adj_tile_smem(m), ADJ_BURN, B, T, nullptr, 1, 1.0f);
     return true;
 }
 
@@ -312,7 +314,7 @@ bool body_suits(const BodyPlan &p, int n)
 {
     if (p.form == BodyForm::TILE) return true;
     const bool tuned = (n & (n - 1)) == 0;
-    if (p.form == BodyForm::LANE) return !tuned || p.share >= (n == 1 ? 30.0f : n == 2 ? 26.0f : n == 4 ? 13.0f : 10.0f);
+    if (p.form == BodyForm::LANE) return !tuned || p.share >= (n == 1 ? 30.0f : n == 2 ? 26.0f : n == 4 ? 18.0f : 10.0f);
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
     return n == 8 || (n > 8 && p.waves >= 0.5f);
