@@ -577,16 +577,39 @@ def measure_workload(bd, torch, synth, idx, rank, device, dist, steps, warmup, f
     tot = sum(v["total_ms"] for v in prof.values()) or 1.0
     kernels = {k: dict(launches_per_step=v["launches"] / prof_steps, us_per_launch=1e3 * v["total_ms"] / v["launches"],
                        share=v["total_ms"] / tot) for k, v in prof.items()}
-    return dict(cfg=cfg, B=B, T=T, n=n, m=m, iters=iters, err=r.err, value=total_units / (total_ms * 1e-3),
+    return dict(cfg=cfg, B=B, T=T, n=n, dim_in=m, iters=iters, err=r.err, value=total_units / (total_ms * 1e-3),
                 ms_per_step=total_ms / steps, launches=int(launches),
                 e2e=dict(value=e2e_units / (e2e_ms * 1e-3), unit=UNIT, h2d_bytes_per_step=int(x_host.numel() * 4),
                          d2h_bytes_per_step=int(y_host.numel() * 4), ms_per_step=e2e_ms / steps),
                 kernels=kernels, prof=prof, prof_steps=prof_steps)
 
 
+def body_bytes_per_position(n: int, m: int) -> int:
+    """A Newton body as one launch: x and the iterate read once, the new iterate written once."""
+    return 4 * (m + 2 * n)
+
+
+def adjoint_bytes_per_position(n: int, m: int) -> int:
+    """The gradient's adjoint as one launch (n = 64): x, y, dL/dy read, packed pre-activation gradients [4n] written."""
+    return 4 * (m + 2 * n + 4 * n)
+
+
+def roofline_of_launch(kernel, bytes_per_launch, ms, pk, extra=None):
+    """Algorithmic bytes of a launch against the measured HBM copy rate (its products' tensor bound is far below)."""
+    gbs = bytes_per_launch / (ms * 1e-3) / 1e9
+    return dict(bound="hbm", kernel=kernel, achieved=gbs, peak=pk["hbm_gbs"], unit="GB/s", frac=gbs / pk["hbm_gbs"],
+                peak_source=pk["source"], ms_per_launch=ms, bytes_per_launch=bytes_per_launch, traffic=None, **(extra or {}))
+
+
 def step_scan_roofline(m, pk):
-    """Roofline of the scan inside the measured step (the dominant kernel), from the profiled pass."""
+    """Roofline of the dominant kernel of the measured step, from the profiled pass: a body's one launch, or the scan."""
     prof = m["prof"]
+    top = max(prof, key=lambda k: prof[k]["total_ms"]) if prof else ""
+    if top.startswith("newton_"):
+        bodies = m["iters"] * m["prof_steps"]            # (a launch may be several bodies, and launches behind the last return at once)
+        nbytes = body_bytes_per_position(m["n"], m["dim_in"]) * m["B"] * m["T"]
+        return roofline_of_launch(top, nbytes, prof[top]["total_ms"] / bodies, pk,
+                                  dict(note="per Newton body; bound by issue slots and the special-function unit (gates), not by HBM"))
     names = [k for k in prof if is_scan_kernel(k)]
     scan_ms = sum(prof[k]["total_ms"] for k in names)
     launches = sum(prof[k]["launches"] for k in names if k.startswith("scan_")) or (m["prof_steps"] * m["iters"])
@@ -703,18 +726,15 @@ def main():
         # ---- config 4: full training step of the 2-layer n = 64 classifier
         c4 = time_classifier(bd, synth, torch, device, 32, 17_984, 0, 3, 2)
         k4 = c4["kernels"]
-        per4 = lambda name: k4[name]["ms"] / k4[name]["launches"] if name in k4 else None
-        fwd_ms = (per4("scan_fused_reduce64_kernel") or 0.0) + (per4("scan_fused_apply_kernel") or 0.0)
+        N4 = 32 * 17_984                                                 # (layer 1: 6 inputs, layer 2: 64)
+        body4 = sum(k * body_bytes_per_position(64, m) * N4 for k, m in zip(c4["iters"], (6, 64)))
+        adj4 = sum(adjoint_bytes_per_position(64, m) * N4 for m in (6, 64))
+        roof4 = lambda name, nbytes: roofline_of_launch(name, nbytes, k4[name]["ms"], pk, dict(note="all launches of the step")) if name in k4 else None
         extras["config4_training_step"] = dict(
             workload="config4: 2-layer GRU n=64 m=6 B=32 T=17984, mean-pool, 5-class head; loss + all gradients",
             ms_per_step=c4["ms"], value=c4["steps_per_s"], unit=UNIT, newton_iters=c4["iters"], loss=c4["loss"],
             kernels=k4,
-            forward_scan=dict(ms_per_scan=fwd_ms, kernels="scan_fused_reduce64_kernel + scan_fused_apply_kernel",
-                              bytes_per_position=fused_scan_bytes_per_position(64),
-                              hbm_frac=fused_scan_bytes_per_position(64) * 32 * 17_984 / (pk["hbm_gbs"] * 1e9) * 1e3 / max(fwd_ms, 1e-9),
-                              tensor_frac_bf16=scan_flops_per_position(64) * 32 * 17_984 / (pk["bf16_tflops"] * 1e12) * 1e3 / max(fwd_ms, 1e-9)),
-            reverse_scan_roofline=roofline_of_scan(64, 32 * 17_984, per4("scan_cta64_kernel") or 1.0, pk, scan_bytes_per_position(64),
-                                                   NCU_SCAN_TRAFFIC_PER_POSITION[64], "scan_cta64_kernel (reverse, 3 x TF32)"))
+            forward_roofline=roof4("newton_tile_kernel", body4), adjoint_roofline=roof4("adjoint_tile_kernel", adj4))
         torch.cuda.empty_cache()
         # ---- the multi-head GRU unit of the paper's sequential-image model
         extras["multihead_unit"] = time_multihead(bd, synth, torch, device, 32, 1024, 32, 8, 256, 5, 2, cpu_seconds=2.0)
@@ -724,12 +744,16 @@ def main():
         for s in SCANS_HBM:
             for reverse in (0, 1):
                 ms = time_scan(bd, torch, device, s["n"], s["B"], s["T"], reverse, 0, 10, 3)
+                chains = s["n"] >= 4                                     # (burn-in chains read J once, matrix-vector steps)
                 rl = roofline_of_scan(s["n"], s["B"] * s["T"], ms, pk, scan_bytes_per_position(s["n"]),
-                                      NCU_SCAN_TRAFFIC_PER_POSITION[s["n"]], scan_kernel_name(s["n"]),
+                                      None if chains else NCU_SCAN_TRAFFIC_PER_POSITION[s["n"]],
+                                      "scan_verified_kernel" if chains else scan_kernel_name(s["n"]),
                                       dict(workload=f"n={s['n']} B={s['B']} T={s['T']} reverse={reverse} "
                                                     f"(J {4 * s['n'] ** 2 * s['B'] * s['T'] / 1e9:.2f} GB, inputs > L2)",
                                            reverse=reverse, n=s["n"],
-                                           traffic_note="ncu capture of the forward kernel at smaller T scaled by positions (profiles/)"))
+                                           **(dict(flops_per_position=2 * s["n"] ** 2,
+                                                   tensor_frac=None, achieved_tflops=2 * s["n"] ** 2 * s["B"] * s["T"] / ms / 1e9) if chains else
+                                              dict(traffic_note="ncu capture of the forward kernel at smaller T scaled by positions (profiles/)"))))
                 scans.append(rl)
                 torch.cuda.empty_cache()
     clocks = sampler.stop()

@@ -1,0 +1,122 @@
+"""Chains with a verified burn-in (bodies, adjoints and stand-alone scans as one launch each) at the sizes where they can go
+wrong: remainders of chains, tiles and CTAs, the ends of a dispatch range, inputs and cells for which a burn-in is raised or
+the launch gives up.  Every case states the kernel it is meant for, and that kernel has to have run."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2309_12252_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2309_12252_b200 import binding
+    binding.lib()
+    return binding
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def launched(bd, call):
+    """The call's result and the names of the kernels that it launched."""
+    from bench import read_profile
+    bd.lib().deer_profile_enable(1)
+    try:
+        r = call()
+        torch.cuda.synchronize()
+    finally:
+        bd.lib().deer_profile_enable(0)
+    return r, set(read_profile(bd))
+
+
+def walk(x):
+    x = np.cumsum(x.astype(np.float64), axis=1)
+    return ((x - x.mean(1, keepdims=True)) / x.std(1, keepdims=True)).astype(np.float32)
+
+
+SEG, ONE, TILE, LANE = "newton_segment_kernel", "newton_body_kernel", "newton_tile_kernel", "newton_lane_kernel"
+
+
+@pytest.mark.parametrize("n,m,B,T,x_kind,kernel", [
+    (1, 1, 1, 3, "noise", SEG), (3, 70, 2, 129, "noise", SEG), (12, 5, 3, 401, "walk", SEG), (31, 3, 1, 80, "noise", SEG),
+    (32, 64, 2, 97, "walk", SEG), (40, 7, 2, 51, "noise", SEG),
+    (16, 3, 16, 5001, "noise", SEG), (24, 10, 16, 6001, "noise", SEG),                       # a launch per body
+    (16, 5, 16, 15001, "noise", ONE), (50, 1, 4, 663, "noise", ONE), (43, 64, 5, 2003, "walk", ONE),
+    (32, 33, 16, 6001, "noise", TILE), (32, 3, 3, 40001, "walk", TILE), (32, 64, 17, 16001, "noise", TILE),
+    (64, 1, 1, 16001, "noise", TILE), (64, 64, 7, 2801, "walk", TILE),
+    (1, 1, 16, 300001, "noise", LANE), (3, 2, 5, 50001, "noise", LANE), (4, 3, 16, 50003, "noise", LANE), (5, 9, 16, 20001, "walk", LANE),
+    (8, 8, 16, 30001, "noise", LANE), (2, 2, 16, 100001, "walk", None)])
+def test_bodies(bd, n, m, B, T, x_kind, kernel):
+    p = synth.gru_params(n, m, seed=3, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=3, tag="c/x")
+    if x_kind == "walk":
+        x = walk(x)
+    y0 = synth.normal(3, "c/y0", (B, n)) * 0.5
+    pd, xd, yd = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(pd, xd, yd))
+    assert kernel is None or kernel in names, names
+    assert r.status == 0 and r.err <= 1e-4
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-4
+
+
+@pytest.mark.parametrize("n,m,B,T", [(1, 1, 16, 300001), (8, 4, 4, 1000), (16, 8, 8, 20000), (24, 3, 2, 700), (32, 8, 16, 8000), (64, 6, 2, 9000)])
+def test_cell_that_remembers_for_long(bd, n, m, B, T):
+    """The update gate's bias alone keeps the state: no burn-in is tried, the Jacobians are multiplied out."""
+    p = synth.gru_params(n, m, seed=4, tag="c/gru")
+    p.b_i[n:2 * n] += 6.0
+    x = synth.x_gaussian(B, T, m, seed=4, tag="c/x")
+    y0 = synth.normal(4, "c/y0", (B, n)) * 0.5
+    r = bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0))
+    assert r.status == 0
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-3
+
+
+WARP, MMA_TILE, ROWS = "newton_adjoint_kernel", "adjoint_tile_kernel", "rows_adjoint_kernel"
+
+
+@pytest.mark.parametrize("n,m,B,T,dense,x_kind,kernel", [
+    (3, 7, 2, 5001, True, "noise", WARP), (12, 5, 8, 3001, True, "walk", WARP), (9, 60, 4, 15001, True, "noise", WARP),
+    (16, 8, 16, 20001, True, "noise", WARP), (24, 3, 1, 6001, False, "noise", WARP), (32, 32, 16, 10001, True, "walk", WARP),
+    (40, 7, 2, 4001, False, "noise", WARP), (56, 1, 3, 3001, True, "noise", WARP),
+    (64, 6, 3, 20001, True, "walk", MMA_TILE), (64, 64, 16, 4003, False, "noise", MMA_TILE),
+    (1, 8, 5, 20003, True, "noise", ROWS), (8, 1, 1, 45, False, "walk", ROWS), (2, 4, 64, 67, True, "noise", ROWS)])
+def test_adjoints(bd, n, m, B, T, dense, x_kind, kernel):
+    p = synth.gru_params(n, m, 5, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 5, tag="c/x")
+    if x_kind == "walk":
+        x = walk(x)
+    y0 = synth.normal(5, "c/y0", (B, n)) * 0.3
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    gy = synth.normal(5, "c/gy", (B, T, n))
+    if not dense:                      # a loss on the last step: dy0 is far below max|lambda|
+        gy[:, :-1] = 0.0
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True))
+    assert kernel in names, names
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        a, b = got[k].cpu().numpy().astype(np.float64), want[k]
+        assert np.max(np.abs(a - b)) <= 1e-3 * max(np.max(np.abs(b)), 1e-30), k
+
+
+@pytest.mark.parametrize("n,B,T", [(4, 2, 65537), (8, 3, 60001), (16, 1, 9001), (32, 2, 1111), (32, 16, 1300), (64, 1, 515), (64, 5, 193)])
+@pytest.mark.parametrize("reverse", [False, True])
+@pytest.mark.parametrize("decays", [True, False])
+def test_scans(bd, n, B, T, reverse, decays):
+    """Matrices whose products hardly decay make the boundaries differ: the chunked scan behind does the work."""
+    J = synth.contractive_J(B, T, n, seed=n + T, tag="c/J", scale=1.0)
+    if not decays:
+        J = 0.05 * J + 0.95 * np.eye(n, dtype=np.float32) * np.float32(1.04)
+    b = synth.normal(n + T, "c/b", (B, T, n))
+    y0 = synth.normal(n + T, "c/y0", (B, n))
+    want = oracle.linrec(J, b, y0, reverse=reverse, dtype=np.float64)
+    args = dev(J), dev(b), dev(y0)
+    got, names = launched(bd, lambda: bd.deer_linrec_scan(*args, reverse=reverse))
+    assert "scan_verified_kernel" in names, names
+    tol = 1e-5 if decays else 1e-4     # (sums over some eighty positions instead of two)
+    assert np.max(np.abs(got.cpu().numpy() - want)) <= tol * max(1.0, float(np.max(np.abs(want))))
