@@ -1192,7 +1192,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     if (one_launch) {
         if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, u_done, copy_out)) != DEER_OK) return rc;
         ended_there = hs.done == BODY_DONE;
-        if (burn_in) *burn_in = hs.burn;       // what the last body had or would have needed
+        if (burn_in) *burn_in = ended_there ? hs.burn : -hs.burn;      // of the last body; negative: it gave up, what it would have needed
     }
     if (!one_launch || hs.done != BODY_DONE) {
     const int k0 = hs.iters;                   // bodies that the one-launch form has done
@@ -1365,8 +1365,8 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     // n = 64: 128 chains per tcgen05 tile; else sixteen per warp
     BodyPlan tplan{};
     const bool exact_flags = (flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) != 0;
-    const int first_burn = std::max(burn_hint, ADJ_BURN);
-    auto worth = [&](const BodyPlan &q) { return first_burn <= adjoint_burn_cap(n, m, (long long)B * T, q.L); };
+    // (where the evaluation gave up, no try is made below what it would have needed)
+    auto worth = [&](const BodyPlan &q) { return std::max(-burn_hint, ADJ_BURN) <= adjoint_burn_cap(n, m, (long long)B * T, q.L); };
     const bool tile = !exact_flags && (((uintptr_t)y | (uintptr_t)y0 | (uintptr_t)gy | (uintptr_t)x | (uintptr_t)p->W_h | (uintptr_t)p->W_i | (uintptr_t)dx) & 15) == 0 &&
                       adjoint_tile_plan(&tplan, B, T, n, m) && worth(tplan);
     const bool lanes = small && !exact_flags && (((uintptr_t)gy) & 3) == 0 && rows_adjoint_plan(&plan, B, T, n, m, WGRAD_P);     // all in one launch
@@ -1385,7 +1385,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
         a.eta = ADJ_ETA;
         a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = tile ? w.J : w.starts;
         // (small cells: one try, the passes behind it are cheap)
-        a.burn = lanes ? ADJ_BURN : first_burn;
+        a.burn = !lanes && burn_hint > ADJ_BURN && burn_hint <= adjoint_burn_cap(n, m, (long long)B * T, a.L) ? burn_hint : ADJ_BURN;
         a.burn_cap = lanes ? 0 : adjoint_burn_cap(n, m, (long long)B * T, a.L);
         for (int k = 0; k < (lanes ? 1 : ADJ_TRIES); ++k) {
             if ((rc = tile ? launch_adjoint_tile(a, tplan, st) : lanes ? launch_rows_adjoint(a, plan, w.partial, w.partial2, dx, st) : launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
@@ -1704,11 +1704,11 @@ int deer_gru_vjp(const deer_gru_params *p, const float *x, const float *y0, cons
 }
 
 // The burn-in that a gradient's boundaries need, from the one that the evaluation of the same trajectory came to (0: the
-// evaluation tells nothing beyond its first one): the accuracy asked for goes with the burn-in's logarithm.
+// evaluation tells nothing beyond its first one; negative: it gave up): it goes with the logarithm of the accuracy asked for.
 static int adjoint_burn_hint(int burn, int n, float tol)
 {
-    if (burn <= body_first_burn(n, tol)) return 0;
-    return (int)fminf(1e6f, (float)burn * logf(0.5f * ADJ_ETA) / logf(0.5f * body_eta(n, tol)));
+    if (abs(burn) <= body_first_burn(n, tol)) return 0;
+    return (int)fmaxf(-1e6f, fminf(1e6f, (float)burn * logf(0.5f * ADJ_ETA) / logf(0.5f * body_eta(n, tol))));
 }
 
 int deer_gru_classifier_step(const deer_gru_params *l1, const deer_gru_params *l2, const float *W_o,

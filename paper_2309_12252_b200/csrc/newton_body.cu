@@ -146,9 +146,11 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
 //   n = 4   0.75-0.9 / 39 (192) 120 (1,600)            n = 64  5.0-6.4 / 311 (16) 714 (128) 1508 (320)
 //   n = 8   1.5-2.1 / 72 (192) 178 (640) 396 (1,600)
 // Only the powers of two have tuned kernels of that kind; the others' are an order of magnitude slower.
-static int worth_trying(const BodyPlan &p, int n, int m)
+// The two-launch scans of n >= 16 take as long for one sequence as for four (n = 32, B = 1, T = 6.4e4: 340 us per body).
+static int worth_trying(const BodyPlan &p, int n, int m, int B)
 {
     float a, b;
+    const float share = n >= 16 && B < 4 ? p.share * 4.0f / (float)B : p.share;
     switch (n) {
     case 1: case 2: a = 45.0f; b = 2.0f; break;
     case 4: a = 30.0f; b = 2.7f; break;
@@ -158,7 +160,7 @@ static int worth_trying(const BodyPlan &p, int n, int m)
     case 64: a = 36.0f; b = 13.0f; break;
     default: return std::max(320, 8 * p.L);
     }
-    return (int)(a + b * p.share) - p.L;
+    return (int)(a + b * share) - p.L;
 }
 
 bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H)
@@ -172,7 +174,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         const LaneKernel lk = lane_kernel(n, m, have_u);
         const int burn = (body_first_burn(n, 1.0f) + lk.W - 1) / lk.W * lk.W;
         one_wave_of_chains(p, (const void *)lk.kern, 128, 128, 32, lk.W, lk.smem, burn, B, T, strides, H);
-        p->burn_cap = worth_trying(*p, n, m);
+        p->burn_cap = worth_trying(*p, n, m, B);
         return true;
     }
     if (form == BodyForm::TILE) {
@@ -180,7 +182,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         if (k.tile_smem(m) > BODY_SMEM_MAX) return false;
         one_wave_of_chains(p, (const void *)k.tile(m), k.tile_threads, k.tile_chains, 128, 1, k.tile_smem(m), body_first_burn(n, 1.0f), B, T, strides, H, n == 32 ? -0.75f : 1.0f);
         if (p->edges <= sms) p->max_ctas = (int)p->edges;      // (two tiles per CTA only where there are more than SMs)
-        p->burn_cap = worth_trying(*p, n, m);
+        p->burn_cap = worth_trying(*p, n, m, B);
         return true;
     }
     if (form == BodyForm::TWO_PHASE) {
@@ -215,7 +217,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         return true;
     }
     one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
-    p->burn_cap = worth_trying(*p, n, m);
+    p->burn_cap = worth_trying(*p, n, m, B);
     return true;
 }
 

@@ -205,31 +205,51 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
     float bs0 = 0.0f, bs1 = 0.0f;
     const int row = 16 * warp + g;
     const bool rv0 = row < n3, rv1 = row + 8 < n3;
+    // The pieces of a thread: column g_c (v_c) of every g_rows-th (v_rows-th) row, the same in every stage, so that a stage
+    // costs it an addition per pointer.  (A division per piece and stage, and one more for the sequence's start, were half of
+    // this kernel's 517 instructions per warp and stage at n3 = 96, K = 32; it is bound by their issue.)
     const int gq = n3 >> 2, vq = kc >> 2;              // 16-byte pieces per row of the two tiles
+    const int g_rows = nthr / gq, v_rows = nthr / vq;
+    const int g_r = tid / gq, g_c = 4 * (tid - g_r * gq), v_r = tid / vq, v_c = 4 * (tid - v_r * vq);
+    const float *gsrc = dG + (e0 + g_r) * ldG + (g_c < gap_at ? g_c : g_c + a.n3 / 3);
+    const float *vsrc = a.V + (ptrdiff_t)(e0 + v_r - (a.shifted ? 1 : 0)) * K + kb + v_c;
+    size_t v_seq = 0;                                  // shifted: sequence and time step of row v_r
+    int v_t = 1;
+    if (a.shifted) { v_seq = (e0 + v_r) / a.T; v_t = (int)(e0 + v_r - v_seq * a.T); }
     auto issue = [&](int s) {
         if (s < nst) {
             float *sG = wg_sm + (size_t)(s % WG_STAGES) * WG_S * (GS + WG_VS), *sV = sG + WG_S * GS;
-            const size_t pb = e0 + (size_t)s * WG_S;
-            for (int c = tid; c < WG_S * gq; c += nthr) {
-                const int r = c / gq, cc = c - r * gq;
-                float *dst = sG + r * GS + 4 * cc;
-                if (pb + r < e1) cp_async16(dst, dG + (pb + r) * ldG + (4 * cc < gap_at ? 4 * cc : 4 * cc + a.n3 / 3));
-                else *reinterpret_cast<float4 *>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-            for (int c = tid; c < WG_S * vq; c += nthr) {
-                const int r = c / vq, cc = c - r * vq;
-                float *dst = sV + r * WG_VS + 4 * cc;
-                const size_t e = pb + r;
-                if (e < e1) {
-                    const float *src = a.V + e * K;
-                    if (a.shifted) {
-                        size_t seq;
-                        src = seq_start(e, a.T, seq) ? a.y0 + seq * K : a.V + (e - 1) * K;
-                    }
-                    cp_async16(dst, src + kb + 4 * cc);
-                } else {
-                    *reinterpret_cast<float4 *>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const int left = (int)min((size_t)WG_S, e1 - (e0 + (size_t)s * WG_S));
+            if (g_r < g_rows) {
+                const float *src = gsrc;
+                for (int r = g_r; r < WG_S; r += g_rows, src += (size_t)g_rows * ldG) {
+                    float *dst = sG + r * GS + g_c;
+                    if (r < left) cp_async16(dst, src);
+                    else *reinterpret_cast<float4 *>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 }
+            }
+            if (v_r < v_rows) {
+                const float *src = vsrc;
+                for (int r = v_r; r < WG_S; r += v_rows, src += (size_t)v_rows * K) {
+                    float *dst = sV + r * WG_VS + v_c;
+                    if (r < left) {
+                        const float *from = src;
+                        if (a.shifted) {
+                            int tt = v_t + r - v_r, sq = 0;
+                            while (tt >= a.T) { tt -= a.T; ++sq; }
+                            if (tt == 0) from = a.y0 + (v_seq + sq) * K + kb + v_c;
+                        }
+                        cp_async16(dst, from);
+                    } else {
+                        *reinterpret_cast<float4 *>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    }
+                }
+            }
+            gsrc += (size_t)WG_S * ldG;
+            vsrc += (size_t)WG_S * K;
+            if (a.shifted) {
+                v_t += WG_S;
+                while (v_t >= a.T) { v_t -= a.T; ++v_seq; }
             }
         }
         cp_async_commit();
@@ -246,11 +266,7 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
 #pragma unroll
         for (int sub = 0; sub < WG_S / 8; ++sub) {
             const float *g0 = sG + (8 * sub + t) * GS + row, *g1 = g0 + 4 * GS;
-            float av[4];
-            av[0] = rv0 ? g0[0] : 0.0f;
-            av[1] = rv1 ? g0[8] : 0.0f;
-            av[2] = rv0 ? g1[0] : 0.0f;
-            av[3] = rv1 ? g1[8] : 0.0f;
+            const float av[4] = {g0[0], g0[8], g1[0], g1[8]};       // (rows and columns past the end are not written out)
             bs0 += av[0] + av[2];
             bs1 += av[1] + av[3];
             unsigned ah[4], al[4];
@@ -260,10 +276,9 @@ __global__ void __launch_bounds__(384) wgrad_mma_staged_kernel(WgradArgs a)
 #pragma unroll
             for (int nn = 0; nn < 8; ++nn) {
                 if (nn < nb) {
-                    const bool cv = 8 * nn + g < kc;
                     unsigned bh[2], bl[2];
-                    split_tf32(cv ? v0[8 * nn] : 0.0f, bh[0], bl[0]);
-                    split_tf32(cv ? v1[8 * nn] : 0.0f, bh[1], bl[1]);
+                    split_tf32(v0[8 * nn], bh[0], bl[0]);
+                    split_tf32(v1[8 * nn], bh[1], bl[1]);
                     mma_tf32(acc[nn], al, bh, acc[nn]);
                     mma_tf32(acc[nn], ah, bl, acc[nn]);
                     mma_tf32(acc[nn], ah, bh, acc[nn]);
