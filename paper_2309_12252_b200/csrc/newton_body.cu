@@ -317,6 +317,9 @@ bool body_suits(const BodyPlan &p, int n)
     if (p.form == BodyForm::TILE) return true;
     const bool tuned = (n & (n - 1)) == 0;
     if (p.form == BodyForm::LANE) return !tuned || p.share >= (n == 1 ? 30.0f : n == 2 ? 26.0f : n == 4 ? 18.0f : 10.0f);
+    // (n = 1, B = 8, T = 3e3 80 / 92, T = 1e4 96 / 99; n = 2, T = 6e3 114 / 140, T = 1.5e4 142 / 152: above, what a failed try costs
+    // on slowly varying inputs, 20 to 30 us, outweighs it)
+    if (p.NC > 0 && n <= 2 && (long long)p.max_ctas * p.NC * p.L > (n == 1 ? 20000 : 64000)) return false;
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
     return n == 8 || (n > 8 && p.waves >= 0.5f);
