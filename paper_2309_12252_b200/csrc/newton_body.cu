@@ -310,8 +310,8 @@ int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 //   n = 32, B = 16, T = 1e3:  128 / 887 / 353      n = 32, B = 16, T = 1e4: 876 / 1126 / 873
 //   n = 64, B = 16, T = 1e3:    - / 2369 / 1247    n = 64, B = 16, T = 1e4:   - / 2828 / 3345
 // Two-phase: one wave (then the whole loop is one launch), two waves from n = 9 on.  One-phase: from half a wave of chains on --
-// below, its steps, a whole cell each, are a serial chain that nothing fills.  States of 1, 2 and 4 pad to 8 columns, which is
-// more work than their own kernels do.  Sizes without tuned kernels of the other kind always come here.
+// below, its steps, a whole cell each, are a serial chain that nothing fills (n <= 8 never comes here: a thread per chain).
+// Sizes without tuned kernels of the other kind always come here.
 bool body_suits(const BodyPlan &p, int n)
 {
     if (p.form == BodyForm::TILE) return true;
@@ -322,7 +322,7 @@ bool body_suits(const BodyPlan &p, int n)
     if (p.NC > 0 && n <= 2 && (long long)p.max_ctas * p.NC * p.L > (n == 1 ? 20000 : 64000)) return false;
     if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
     if (!tuned) return true;
-    return n == 8 || (n > 8 && p.waves >= 0.5f);
+    return p.waves >= 0.5f;
 }
 
 int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st)
