@@ -92,6 +92,7 @@ struct ScanWs {
 };
 
 constexpr int VSCAN_L_MIN = 64, VSCAN_BURN = 64, VSCAN_WARPS = 12;
+static_assert(VSCAN_WINDOW <= VSCAN_BURN && VSCAN_BURN <= VSCAN_L_MIN, "every chain but the first has a whole window before it");
 
 static int num_sms();
 
@@ -147,7 +148,7 @@ static ScanWs carve_scan(Carver &cv, int B, int T, int n)
     }
     w.bytes_without = cv.off;
     w.vchains = vscan_takes(n, B, T) ? (size_t)B * ((T + VSCAN_L_MIN - 1) / VSCAN_L_MIN) : 0;
-    w.vedge = cv.take<float>(w.vchains * 2 * n);
+    w.vedge = cv.take<float>(w.vchains * 3 * n);
     w.vflag = cv.take<unsigned>(w.vchains);
     return w;
 }

@@ -1,9 +1,12 @@
 // The linear recurrence y_t = J_t y_{t-1} + b_t (Eq. 10; either direction) without matrix products: chains that start `burn`
 // positions early from zero, each a plain sequence of matrix-vector steps, J read once (and a burn-in's worth of it twice).
 // What a chain's start lacks is the state entering its burn-in, carried through `burn` Jacobians; that this vanished is
-// verified: every chain's end state is compared with the start its successor assumed, relative to their own size.  One
-// boundary that differs by more than eta leaves StatusBlock::done at 0, and the chunked scan enqueued behind this launch
-// (which multiplies the matrices out, Eq. 9) does the work; otherwise it returns at once.
+// verified: every chain's end state is compared with the start its successor assumed.  One boundary that differs by more than
+// eta leaves StatusBlock::done at 0, and the chunked scan enqueued behind this launch (which multiplies the matrices out,
+// Eq. 9) does the work; otherwise it returns at once.
+// A state's components may have units of their own, and the chunked scan is good to fp32 in each: a component's difference is
+// held to eta of that component's largest value over the VSCAN_WINDOW positions before the boundary (one position alone may be
+// a zero crossing; more would measure a decayed value by what it decayed from), and to eta of the states' largest component.
 //
 // G lanes per chain (n up to 32, a warp for n = 64); a matrix is read as consecutive 16-byte pieces: lane (sub, q) holds the
 // columns 4q .. 4q+3 of the rows RP k + sub.  The next U positions' matrices are on their way in registers.
@@ -24,13 +27,15 @@ template <int N> struct VScan {
     static constexpr int CPW = 32 / G, WARPS = 4;
 };
 
+constexpr int VSCAN_WINDOW = 16;                         // (shorter than any burn-in and any chain)
+
 struct VScanArgs {
     const float *J, *b, *y0;
     float *y;
     int B, T, L, burn;
     float eta;
     StatusBlock *st;
-    float *edge;             // [chains][2][n]
+    float *edge;             // [chains][3][n]  end of the chain before, start and scale of the one behind
     unsigned *edge_flag;     // [chains]
 };
 
@@ -78,9 +83,9 @@ __global__ void __launch_bounds__(128) scan_verified_kernel(VScanArgs a)
     float y[OWN];                                        // the lane's rows of the state
 #pragma unroll
     for (int e = 0; e < OWN; ++e) y[e] = c == 0 && a.y0 ? a.y0[(size_t)seq * N + row[e]] : 0.0f;
-    float start[OWN];
+    float start[OWN], scale[OWN];                        // scale: largest |y| of the last VSCAN_WINDOW positions before the own ones
 #pragma unroll
-    for (int e = 0; e < OWN; ++e) start[e] = y[e];
+    for (int e = 0; e < OWN; ++e) { start[e] = y[e]; scale[e] = 0.0f; }
 #pragma unroll
     for (int u = 0; u < U; ++u) fetch(first + u, Jb[u], bb[u]);
 
@@ -144,6 +149,7 @@ __global__ void __launch_bounds__(128) scan_verified_kernel(VScanArgs a)
 #pragma unroll
             for (int e = 0; e < OWN; ++e) {
                 y[e] = in ? z[e] + bb[u][e] : y[e];
+                if (s < own) scale[e] = fmaxf(s == own - VSCAN_WINDOW ? 0.0f : scale[e], fabsf(y[e]));
                 if (in && s >= own && live) yseq[(size_t)(REV ? T - 1 - s : s) * N + row[e]] = y[e];
             }
             fetch(s + U, Jb[u], bb[u]);
@@ -157,10 +163,13 @@ __global__ void __launch_bounds__(128) scan_verified_kernel(VScanArgs a)
     for (int side = 0; side < 2; ++side) {               // 0: behind this chain, 1: before it
         const bool there = live && (side == 0 ? c + 1 < nchain : c > 0);
         const size_t edge = (size_t)(gid - side) ;
-        float *slot = a.edge + edge * 2 * N;
+        float *slot = a.edge + edge * 3 * N;
         if (there) {
 #pragma unroll
-            for (int e = 0; e < OWN; ++e) __stcg(slot + side * N + row[e], side == 0 ? y[e] : start[e]);
+            for (int e = 0; e < OWN; ++e) {
+                __stcg(slot + side * N + row[e], side == 0 ? y[e] : start[e]);
+                if (side == 1) __stcg(slot + 2 * N + row[e], scale[e]);
+            }
             __threadfence();
         }
         __syncwarp();
@@ -168,14 +177,14 @@ __global__ void __launch_bounds__(128) scan_verified_kernel(VScanArgs a)
         if (there && cl == 0) { __threadfence(); old = atomicAdd(a.edge_flag + edge, 1u); }
         old = __shfl_sync(FULL, old, base);
         float diff = 0.0f, size = 0.0f;
-        bool nan = false;
+        bool off = false;
         if (there && old == 1u) {
             __threadfence();
 #pragma unroll
             for (int e = 0; e < OWN; ++e) {
                 const float mine = side == 0 ? y[e] : start[e], other = __ldcg(slot + (side ^ 1) * N + row[e]);
-                const float dv = fabsf(mine - other);
-                nan = nan || !(dv <= 3.402823466e38f);
+                const float dv = fabsf(mine - other), sc = side == 0 ? __ldcg(slot + 2 * N + row[e]) : scale[e];
+                off = off || !(dv <= a.eta * sc);        // (a NaN too)
                 diff = fmaxf(diff, dv);
                 size = fmaxf(size, fmaxf(fabsf(mine), fabsf(other)));
             }
@@ -186,7 +195,7 @@ __global__ void __launch_bounds__(128) scan_verified_kernel(VScanArgs a)
             diff = fmaxf(diff, __shfl_xor_sync(FULL, diff, o));
             size = fmaxf(size, __shfl_xor_sync(FULL, size, o));
         }
-        if (nan || diff > a.eta * size) bad = 1u;
+        if (off || diff > a.eta * size) bad = 1u;
     }
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -120,3 +120,20 @@ def test_scans(bd, n, B, T, reverse, decays):
     assert "scan_verified_kernel" in names, names
     tol = 1e-5 if decays else 1e-4     # (sums over some eighty positions instead of two)
     assert np.max(np.abs(got.cpu().numpy() - want)) <= tol * max(1.0, float(np.max(np.abs(want))))
+
+
+@pytest.mark.parametrize("n,B,T", [(4, 2, 65537), (8, 3, 60001), (16, 1, 9001), (32, 16, 1300), (64, 1, 515)])
+@pytest.mark.parametrize("reverse", [False, True])
+def test_scan_components_of_unequal_size(bd, n, B, T, reverse):
+    """Every other component is large and forgets at once, the ones between are 1e9 times smaller and remember: each is good to
+    fp32 in its own size (sums over some hundred positions: a hundred roundings of 6e-8, six of them allowed for each)."""
+    J = np.zeros((B, T, n, n), np.float32)
+    i = np.arange(n)
+    J[:, :, i, i] = np.where(i % 2 == 0, 0.5, 0.99)
+    b = synth.normal(n + T, "c/b", (B, T, n)) * np.where(i % 2 == 0, 1e6, 1e-3).astype(np.float32)
+    want = oracle.linrec(J, b, None, reverse=reverse, dtype=np.float64)
+    args = dev(J), dev(b)
+    got, names = launched(bd, lambda: bd.deer_linrec_scan(*args, reverse=reverse))
+    assert "scan_verified_kernel" in names, names
+    off = np.max(np.abs(got.cpu().numpy() - want), axis=(0, 1)) / np.max(np.abs(want), axis=(0, 1))
+    assert np.max(off) <= 4e-5, off
