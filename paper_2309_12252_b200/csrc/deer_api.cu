@@ -732,8 +732,8 @@ struct EvalWs {
 // chain groups of a one-launch body at the shortest chain length
 static size_t body_groups_max(int B, int T) { return ((size_t)B * ((T + BODY_L_MIN - 1) / BODY_L_MIN) + 15) / 16; }
 
-// ... and of an adjoint launch (its chains are 16 positions at least), idle warps of the last CTA included
-static size_t adjoint_groups_max(int B, int T) { return ((size_t)B * ((T + 15) / 16) + 15) / 16 + 8; }
+// ... and of an adjoint launch, idle warps of the last CTA included
+static size_t adjoint_groups_max(int B, int T) { return ((size_t)B * ((T + CHAIN_L_MIN - 1) / CHAIN_L_MIN) + 15) / 16 + 8; }
 
 static EvalWs carve_eval(void *ws, int B, int T, int n, int m)
 {
@@ -778,6 +778,7 @@ struct VjpWs {
     StatusBlock *st;
     unsigned *edge_flag;         // directly behind the status block: cleared with it
     float *edge, *starts;
+    size_t start_groups;         // chain groups that `starts` has room for
     float *u, *J, *rhs, *lam, *dGi, *dGh, *partial, *partial2;
     ScanWs scan;
     size_t bytes;
@@ -791,7 +792,8 @@ static VjpWs carve_vjp(void *ws, int B, int T, int n, int m)
     w.st = cv.take<StatusBlock>(1);
     w.edge_flag = cv.take<unsigned>(body_groups_max(B, T));
     w.edge = cv.take<float>(body_groups_max(B, T) * 2 * n);
-    w.starts = cv.take<float>(adjoint_groups_max(B, T) * adjoint_starts(n));
+    w.start_groups = adjoint_groups_max(B, T);
+    w.starts = cv.take<float>(w.start_groups * adjoint_starts(n));
     w.u = cv.take<float>(N * 3 * n);
     w.J = cv.take<float>(N * n * n);
     w.lam = cv.take<float>(N * n);
@@ -892,7 +894,7 @@ struct MhWs {
     float *u, *yalt, *dGi, *dGh, *edge, *starts, *dy0all, *partial;
     unsigned *edge_flag;
     unsigned long long *words;
-    size_t groups;
+    size_t groups, start_groups;
 };
 
 constexpr int MH_P_IN = 32;  // slices of the positions in the reduction of the stacked input weights
@@ -943,6 +945,7 @@ static MhWs carve_mh(void *ws, int H, const int *strides, int B, int T, int n, i
     w.edge = cv.take<float>(w.groups * 2 * n);
     w.edge_flag = cv.take<unsigned>(w.groups);
     w.words = cv.take<unsigned long long>((size_t)4 * num_sms());
+    w.start_groups = agroups;
     w.starts = cv.take<float>(agroups * adjoint_starts(n));
     w.dy0all = cv.take<float>(seqs * n);
     w.partial = cv.take<float>(std::max((size_t)MH_P_IN * H * n3 * (m + 1), (size_t)mh_p_hidden(H) * H * n3 * (n + 1)));
@@ -1373,6 +1376,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     const bool lanes = small && !exact_flags && (((uintptr_t)gy) & 3) == 0 && rows_adjoint_plan(&plan, B, T, n, m, WGRAD_P);     // all in one launch
     const bool adj = lanes || (!tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
                      adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && worth(plan));
+    if (adj && !lanes && (size_t)plan.edges > w.start_groups) return DEER_ERR_WORKSPACE;
     DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj || tile ? (size_t)(tile ? tplan : plan).edges * sizeof(unsigned) : 0), st), "memset status");
     const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
     if (adj || tile) {
@@ -2064,6 +2068,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     int rc;
     BodyPlan plan{};
     if (!adjoint_plan(&plan, B, T, n, m, true, strides, H)) return DEER_OK;
+    if ((size_t)plan.edges > w.start_groups) return DEER_ERR_WORKSPACE;
     if ((rc = mh_table(heads, strides, H, B, T, plan.L, 16, w, st)) != DEER_OK) return rc;
     std::vector<MhGrad> gr((size_t)H);
     for (int h = 0; h < H; ++h) gr[h] = MhGrad{dheads[h].dW_i, dheads[h].dW_h, dheads[h].db_i, dheads[h].db_h};

@@ -120,7 +120,7 @@ static void one_wave_of_chains(BodyPlan *p, const void *kern, int threads, int c
     p->share = (float)((double)B * T * H / ((double)cap * chains));
     double best = 0.0;
     // (gran: what the chain length is a multiple of)
-    for (int L = std::max(4, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
+    for (int L = std::max(CHAIN_L_MIN, gran); ; L += std::max(gran, L / 32 / gran * gran)) {
         double sum = 0.0, top = 0.0;
         for (int h = 0; h < H; ++h) {
             const int s = strides ? strides[h] : 1, Tp = (T + s - 1) / s, nch = (Tp + L - 1) / L;

@@ -68,6 +68,7 @@ struct BodyKernels {
 };
 
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
+constexpr int CHAIN_L_MIN = 4;   // ... those of every form but the two-phase one: what boundaries and start states are sized by
 
 // The forms of a body.
 enum class BodyForm { TWO_PHASE, TILE, LANE, ONE_PHASE };

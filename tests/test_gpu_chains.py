@@ -137,3 +137,27 @@ def test_scan_components_of_unequal_size(bd, n, B, T, reverse):
     assert "scan_verified_kernel" in names, names
     off = np.max(np.abs(got.cpu().numpy() - want), axis=(0, 1)) / np.max(np.abs(want), axis=(0, 1))
     assert np.max(off) <= 4e-5, off
+
+
+def accepted(ws):
+    """StatusBlock::done of the call that last used the workspace: set where a launch with verified boundaries did the work."""
+    return int(ws[:16].view(torch.int32)[3].item())
+
+
+@pytest.mark.parametrize("n,m,B,T", [(50, 70, 4, 5000), (56, 100, 6, 4003), (64, 65, 8, 30001)])
+def test_adjoint_of_wide_states_with_projected_inputs(bd, n, m, B, T):
+    """Chains of four positions: the start states of all of them have room beside the projected inputs that the launch and the
+    kernels behind it read."""
+    p = synth.gru_params(n, m, 6, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 6, tag="c/x")
+    y0 = synth.normal(6, "c/y0", (B, n)) * 0.3
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    gy = synth.normal(6, "c/gy", (B, T, n))
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    ws = bd.alloc_workspace(bd.DEER_OP_VJP, B, T, n, m)
+    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True, ws=ws))
+    assert WARP in names and accepted(ws) == 1, names
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        a, b = got[k].cpu().numpy().astype(np.float64), want[k]
+        assert np.max(np.abs(a - b)) <= 1e-3 * np.max(np.abs(b)), k
