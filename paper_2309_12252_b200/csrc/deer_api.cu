@@ -735,6 +735,13 @@ static size_t body_groups_max(int B, int T) { return ((size_t)B * ((T + BODY_L_M
 // ... and of an adjoint launch, idle warps of the last CTA included
 static size_t adjoint_groups_max(int B, int T) { return ((size_t)B * ((T + CHAIN_L_MIN - 1) / CHAIN_L_MIN) + 15) / 16 + 8; }
 
+// boundaries of any of a gradient's launches: those of rows_adjoint.cuh lie between warps of 32 / n chains
+static size_t adjoint_edges_max(int B, int T, int n)
+{
+    const size_t chains = (size_t)B * ((T + CHAIN_L_MIN - 1) / CHAIN_L_MIN), unit = n == 4 || n == 8 ? 32 / n : 16;
+    return (chains + unit - 1) / unit;
+}
+
 static EvalWs carve_eval(void *ws, int B, int T, int n, int m)
 {
     (void)m;
@@ -778,7 +785,7 @@ struct VjpWs {
     StatusBlock *st;
     unsigned *edge_flag;         // directly behind the status block: cleared with it
     float *edge, *starts;
-    size_t start_groups;         // chain groups that `starts` has room for
+    size_t edges, start_groups;  // boundaries and chain groups that there is room for
     float *u, *J, *rhs, *lam, *dGi, *dGh, *partial, *partial2;
     ScanWs scan;
     size_t bytes;
@@ -790,8 +797,9 @@ static VjpWs carve_vjp(void *ws, int B, int T, int n, int m)
     VjpWs w;
     size_t N = (size_t)B * T;
     w.st = cv.take<StatusBlock>(1);
-    w.edge_flag = cv.take<unsigned>(body_groups_max(B, T));
-    w.edge = cv.take<float>(body_groups_max(B, T) * 2 * n);
+    w.edges = adjoint_edges_max(B, T, n);
+    w.edge_flag = cv.take<unsigned>(w.edges);
+    w.edge = cv.take<float>(w.edges * 2 * n);
     w.start_groups = adjoint_groups_max(B, T);
     w.starts = cv.take<float>(w.start_groups * adjoint_starts(n));
     w.u = cv.take<float>(N * 3 * n);
@@ -1376,7 +1384,8 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     const bool lanes = small && !exact_flags && (((uintptr_t)gy) & 3) == 0 && rows_adjoint_plan(&plan, B, T, n, m, WGRAD_P);     // all in one launch
     const bool adj = lanes || (!tile && !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
                      adjoint_plan(&plan, B, T, n, m, have_u, nullptr, 1) && worth(plan));
-    if (adj && !lanes && (size_t)plan.edges > w.start_groups) return DEER_ERR_WORKSPACE;
+    if ((adj && !lanes && (size_t)plan.edges > w.start_groups) || ((adj || tile) && (size_t)(tile ? tplan : plan).edges > w.edges))
+        return DEER_ERR_WORKSPACE;
     DEER_CHECK_CUDA(cudaMemsetAsync(w.st, 0, sizeof(StatusBlock) + (adj || tile ? (size_t)(tile ? tplan : plan).edges * sizeof(unsigned) : 0), st), "memset status");
     const StatusBlock *unless = nullptr;       // set: the launches that take it do nothing where the adjoint launch has done the work
     if (adj || tile) {

@@ -161,3 +161,22 @@ def test_adjoint_of_wide_states_with_projected_inputs(bd, n, m, B, T):
     for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
         a, b = got[k].cpu().numpy().astype(np.float64), want[k]
         assert np.max(np.abs(a - b)) <= 1e-3 * np.max(np.abs(b)), k
+
+
+@pytest.mark.parametrize("n,m,B,T", [(8, 8, 64, 1000), (8, 1, 3, 4001), (8, 4, 16, 2300), (4, 2, 33, 701), (2, 1, 9, 500), (1, 4, 40, 777)])
+def test_adjoint_of_small_cells_in_short_chains(bd, n, m, B, T):
+    """Chains of four or eight positions, a boundary per four to thirty-two of them: all are told apart, and the launch's result
+    is taken."""
+    p = synth.gru_params(n, m, 7, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 7, tag="c/x")
+    y0 = synth.normal(7, "c/y0", (B, n)) * 0.3
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    gy = synth.normal(7, "c/gy", (B, T, n))
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    ws = bd.alloc_workspace(bd.DEER_OP_VJP, B, T, n, m)
+    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True, ws=ws))
+    assert ROWS in names and accepted(ws) == 1, names
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        a, b = got[k].cpu().numpy().astype(np.float64), want[k]
+        assert np.max(np.abs(a - b)) <= 1e-4 * np.max(np.abs(b)), k
