@@ -255,7 +255,13 @@ int deer_gru_eval_host_chunk(int B, int T);
  * trajectory y, lambda = gy L_G^{-1} by ONE reverse scan with the Jacobians
  * recomputed at y (Sec. 3.1.1 allows saving or recomputing them), then the
  * cell's vector-Jacobian product at every position, summed over positions in
- * a fixed order (bit-reproducible).
+ * a fixed order (bit-reproducible).  Where the reverse scan runs as chains
+ * that start early from zero, what a chain's start lacks is checked at every
+ * boundary: at most 4e-6 of the largest |lambda| of the call and 1.6e-5 of the
+ * largest |lambda| over the eight steps around the boundary, so that dx and dy0
+ * are good to that wherever they are small, too (a sequence whose loss weighs a
+ * millionth of another's, steps far from a loss on the last one); otherwise the
+ * scan multiplies the Jacobians out.
  *   y  [B,T,n] trajectory (normally deer_gru_eval's output)   gy [B,T,n]
  *   dparams : device arrays, overwritten       dx  [B,T,m] or NULL
  *   dy0 [B,n] or NULL

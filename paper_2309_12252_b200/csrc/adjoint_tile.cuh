@@ -198,9 +198,12 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     const unsigned utmem = __shfl_sync(0xffffffffu, tmem, 0), usH = __shfl_sync(0xffffffffu, smem_u32(sH), 0);
     const uint64_t dH = tile_desc(usH), dX = tile_desc(usH + C::PANEL * C::HP), dWh = tile_desc(smem_u32(sWh)), dWi = tile_desc(smem_u32(sWi));
 
-    unsigned mb = 0u, phase = 0u, mb_end = 0u;
+    unsigned mb = 0u, phase = 0u, mb_end = 0u;          // mb: the row's largest |lambda|, from the window on
+    float scale = 0.0f;                                  // ... over the window: of the boundary before this chain
 #pragma unroll 1
     for (int step = s0; step < s_end; ++step) {
+        if (step == burn - ADJ_WINDOW) mb = 0u;
+        if (step == burn) scale = __uint_as_float(mb);
         if (step == burn && own.te > 0) {                // what this chain assumed at its first own position
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -245,11 +248,11 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) top = max(top, max(__float_as_uint(fabsf(l[j].x)), __float_as_uint(fabsf(l[j].y))));
-        if (keep) mb = max(mb, top);
         sMax[cg * C::ROWS + row] = __uint_as_float(top);
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < C::CG; ++k) top = max(top, __float_as_uint(sMax[k * C::ROWS + row]));
+        mb = max(mb, top);                                  // (outside the chain: zero, or what it ended with)
         // p up to about 2^8 (|p| <= |lambda| / 4 or so): exponent of the row's largest |lambda| to 2^9
         const int ex = min(max((int)(top >> 23), 20), 240);
         const float sc = __uint_as_float((unsigned)(127 + 9 - (ex - 127)) << 23), inv = __uint_as_float((unsigned)(127 - 9 + (ex - 127)) << 23);
@@ -357,6 +360,8 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     }
     cp_async_wait_0();
     __syncthreads();
+    if (cg == 0) sMax[row] = scale;
+    __syncthreads();
 
     // ---- the state that leaves the first time step: the gradient w.r.t. y0
     if (a.dy0 && own.te > 0 && !has_next) {
@@ -369,29 +374,31 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     }
     // ---- boundaries: this row's end state against what its successor assumed
     const int reach = DY0_REACH * burn;
-    unsigned mis = 0u, mis_end = 0u;
+    unsigned mis = 0u, rel = 0u, mis_end = 0u;
     if (has_next && row + 1 < C::ROWS) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float4 v = __ldcg(reinterpret_cast<const float4 *>(a.starts + (gid + 1) * N + c0) + j);
             mis = max(mis, max(max(absdiff_bits(v.x, d[2 * j].x), absdiff_bits(v.y, d[2 * j].y)), max(absdiff_bits(v.z, d[2 * j + 1].x), absdiff_bits(v.w, d[2 * j + 1].y))));
         }
+        rel = boundary_ratio(mis, sMax[row + 1]);
         if (T - own.te < reach) mis_end = mis;
     }
     if (row == C::ROWS - 1 && has_next) {                // the boundary behind this tile: side 0 of edge `tile`
-        float *slot = a.edge + (size_t)tile * 2 * N + c0;
+        float *slot = a.edge + (size_t)tile * ADJ_EDGE(N) + c0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) { __stcg(slot + 2 * j, d[j].x); __stcg(slot + 2 * j + 1, d[j].y); }
         s_side[0] = T - own.te < reach ? 2 : 1;
         __threadfence();
     }
     if (row == 0 && has_prev && tile > 0) {              // ... and the one before it: side 1 of edge tile - 1
-        float *slot = a.edge + (size_t)(tile - 1) * 2 * N + N + c0;
+        float *slot = a.edge + (size_t)(tile - 1) * ADJ_EDGE(N) + N + c0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float4 v = __ldcg(reinterpret_cast<const float4 *>(a.starts + gid * N + c0) + j);
             __stcg(slot + 4 * j, v.x); __stcg(slot + 4 * j + 1, v.y); __stcg(slot + 4 * j + 2, v.z); __stcg(slot + 4 * j + 3, v.w);
         }
+        if (cg == 0) __stcg(slot + N, scale);
         s_side[1] = T - chain * L < reach ? 2 : 1;
         __threadfence();
     }
@@ -403,10 +410,11 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         old = __shfl_sync(0xffffffffu, old, 0);
         if (old == 1u) {
             __threadfence();
-            const float *slot = a.edge + edge * 2 * N;
+            const float *slot = a.edge + edge * ADJ_EDGE(N);
             for (int i = lane; i < N; i += 32) {
                 const unsigned q = absdiff_bits(__ldcg(slot + i), __ldcg(slot + N + i));
                 mis = max(mis, q);
+                rel = max(rel, boundary_ratio(q, __ldcg(slot + 2 * N)));
                 if (s_side[warp] == 2) mis_end = max(mis_end, q);
             }
             if (lane == 0) a.edge_flag[edge] = 0u;
@@ -414,11 +422,13 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     }
     mb = __reduce_max_sync(0xffffffffu, mb);
     mis = __reduce_max_sync(0xffffffffu, mis);
+    rel = __reduce_max_sync(0xffffffffu, rel);
     mb_end = __reduce_max_sync(0xffffffffu, mb_end);
     mis_end = __reduce_max_sync(0xffffffffu, mis_end);
     if (lane == 0) {
         if (mb) atomicMax(&st->err_bits, mb);
         if (mis) atomicMax(&st->mis_bits, mis);
+        if (rel) atomicMax(&st->rel_bits, rel);
         if (mb_end) atomicMax(&st->top_end_bits, mb_end);
         if (mis_end) atomicMax(&st->mis_end_bits, mis_end);
         __threadfence();

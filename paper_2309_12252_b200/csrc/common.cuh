@@ -102,7 +102,8 @@ struct StatusBlock {
     unsigned mis_bits;   // one-launch bodies: largest mismatch between a chain's end and the start its successor assumed
     HostResult *host;    // page-locked host memory, or nullptr
     unsigned top_end_bits, mis_end_bits;     // adjoint launch: max|dy0|, largest mismatch near the first time step
-    unsigned pad[44];
+    unsigned rel_bits;   // ... largest mismatch as a part of |lambda| there
+    unsigned pad[43];
 };
 static_assert(sizeof(StatusBlock) == 256, "status block is one 256-byte line");
 constexpr int ERR_TRACE_CAP = 1024;

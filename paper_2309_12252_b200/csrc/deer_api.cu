@@ -799,7 +799,7 @@ static VjpWs carve_vjp(void *ws, int B, int T, int n, int m)
     w.st = cv.take<StatusBlock>(1);
     w.edges = adjoint_edges_max(B, T, n);
     w.edge_flag = cv.take<unsigned>(w.edges);
-    w.edge = cv.take<float>(w.edges * 2 * n);
+    w.edge = cv.take<float>(w.edges * ADJ_EDGE(n));
     w.start_groups = adjoint_groups_max(B, T);
     w.starts = cv.take<float>(w.start_groups * adjoint_starts(n));
     w.u = cv.take<float>(N * 3 * n);
@@ -950,7 +950,7 @@ static MhWs carve_mh(void *ws, int H, const int *strides, int B, int T, int n, i
     w.yalt = cv.take<float>(N * H * n);
     w.dGi = cv.take<float>(N * H * n3);
     w.dGh = cv.take<float>(N * H * n3);
-    w.edge = cv.take<float>(w.groups * 2 * n);
+    w.edge = cv.take<float>(w.groups * ADJ_EDGE(n));
     w.edge_flag = cv.take<unsigned>(w.groups);
     w.words = cv.take<unsigned long long>((size_t)4 * num_sms());
     w.start_groups = agroups;

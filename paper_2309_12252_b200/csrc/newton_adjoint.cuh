@@ -6,17 +6,31 @@
 // carries is mu_t = J_{t+1}^T lambda_{t+1}.  With the gates at t and lambda = gy + mu, the hidden-side gradients of the three
 // pre-activations are p = (k_r.lambda, a_z.lambda, k_n.lambda) -- what dW_h, dW_i, dx are contractions of -- and
 //     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands.
-// All products are 3 x TF32 (a one-shot solve).  A boundary mismatch above eta * max|lambda| leaves StatusBlock::done at 0:
-// the launches enqueued behind this one (a longer burn-in, then the kernels that multiply the Jacobians out) do the work.
-// dy0 is an output with a scale of its own: where dL/dy is zero near the start of the sequences, dy0 may be many orders of
-// magnitude below max|lambda|.  So the boundaries that dy0 can still feel -- those less than DY0_REACH burn-ins from the
-// sequence's first step -- are held to eta * max|dy0| as well.
+// All products are 3 x TF32 (a one-shot solve).  lambda has no scale that holds everywhere: a sequence's loss may weigh a
+// millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
+// the first one.  So a boundary is held to eta of the largest |lambda| of all and, besides, to ADJ_LOCAL eta of the largest
+// |lambda| just before it, over the last ADJ_WINDOW positions of its successor's burn-in (one position alone may be near zero
+// where n is small; more would measure a decayed lambda by what it decayed from).  Where all losses weigh alike the window's
+// largest is some third of the largest of all, so that the first rule decides there.
+// One boundary that differs by more leaves StatusBlock::done at 0: the launches enqueued behind this one (a longer burn-in,
+// then the kernels that multiply the Jacobians out) do the work.
+// The boundaries that dy0 can still feel -- those less than DY0_REACH burn-ins from the sequence's first step -- are held to
+// eta * max|dy0| as well.
 #pragma once
 #include "newton_body.cuh"
 
 namespace deer {
 
 constexpr int DY0_REACH = 8;     // a burn-in takes an error down by about 1e-6 or more; behind eight of them it is below any fp32
+constexpr int ADJ_WINDOW = 8;    // positions before a boundary whose largest |lambda| is its scale
+constexpr float ADJ_LOCAL = 4.0f;
+static_assert(ADJ_WINDOW <= ADJ_BURN && (ADJ_BURN - ADJ_WINDOW) % 4 == 0, "the window is whole steps of every kernel's burn-in");
+
+// A boundary's mismatch as a part of its scale, as the bits of a non-negative float (a NaN stays above all numbers).
+__device__ __forceinline__ unsigned boundary_ratio(unsigned diff, float scale)
+{
+    return diff == 0u ? 0u : __float_as_uint(fabsf(__uint_as_float(diff) / scale));
+}
 
 template <int N> struct Adj {
     static constexpr int NT = N / 8;
@@ -42,13 +56,13 @@ __device__ __forceinline__ int adjoint_burn(const AdjArgs &a, const StatusBlock 
 __device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool dy0, int burn)
 {
     auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
-    const float top = take(st->err_bits), mis = take(st->mis_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
-    const bool inner = mis <= eta * top, end = !dy0 || mis_end <= eta * top_end;
+    const float top = take(st->err_bits), mis = take(st->mis_bits), rel = take(st->rel_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
+    const bool inner = mis <= eta * top && rel <= ADJ_LOCAL * eta, end = !dy0 || mis_end <= eta * top_end;
     if (inner && end) { st->done = BODY_DONE; return; }
-    // the carried error is about max|lambda| * rho^burn: the burn-in after which it is half of what is accepted
+    // the carried error is about |lambda| * rho^burn: the burn-in after which it is half of what is accepted
     int want = 1 << 20;
     if (inner) want = 3 * burn;
-    else if (mis < 0.7f * top) want = (int)(1.1f * (float)burn * __logf(0.5f * eta) / __logf(mis / top)) + 4;
+    else if (mis < 0.7f * top && rel < 0.7f) want = (int)(1.1f * (float)burn * __logf(0.5f * eta) / __logf(fmaxf(mis / top, rel / ADJ_LOCAL))) + 4;
     st->burn = max(want, burn + 8);
 }
 
@@ -111,7 +125,8 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     __syncthreads();
 
     const long long grp = (long long)blockIdx.x * nwarps + warp;
-    unsigned mb = 0u, mis = 0u, mb_end = 0u, mis_end = 0u;
+    unsigned mb = 0u, mis = 0u, rel = 0u, mb_end = 0u, mis_end = 0u;
+    unsigned top[2] = {0u, 0u};                          // largest |mu| of this lane's columns of its two rows over the window
 
     if (grp < groups) {
         // ---- rows g and g + 8 of this lane: chain c of sequence (b, phase); scan position q is time step len - 1 - q
@@ -216,11 +231,17 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
 
 #pragma unroll 1
         for (int step = s_first; step < s_end; ++step) {
-            if (step == burn) {
+            if (step == burn) {                          // start states, and the scales of the boundaries before them
 #pragma unroll
                 for (int j = 0; j < NT; ++j) {
                     *reinterpret_cast<float2 *>(ss + g * SW + 8 * j + 2 * t) = make_float2(d[j][0], d[j][1]);
                     *reinterpret_cast<float2 *>(ss + (g + 8) * SW + 8 * j + 2 * t) = make_float2(d[j][2], d[j][3]);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    unsigned q = max(top[h], __shfl_xor_sync(0xffffffffu, top[h], 1));
+                    q = max(q, __shfl_xor_sync(0xffffffffu, q, 2));
+                    if (t == 0) ss[(g + 8 * h) * SW + N] = __uint_as_float(q);
                 }
             }
             const bool act[2] = {tt[0] >= 0 && tt[0] < t_end[0], tt[1] >= 0 && tt[1] < t_end[1]};
@@ -355,6 +376,14 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
 #pragma unroll
                 for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? acc[q] + cr[q] : d[j][q];
             }
+            // (mu stands for lambda = gy + mu here: work for eight steps instead of for every one; n = m = 32, 1.6e6 positions: 7 us of
+            // the gradient's 2,015 instead of 16)
+            if (step >= burn - ADJ_WINDOW && step < burn) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) top[q >> 1] = max(top[q >> 1], __float_as_uint(fabsf(d[j][q])));
+            }
         }
         // ---- the state that leaves the first time step: the gradient w.r.t. y0
         if (a.dy0) {
@@ -378,13 +407,16 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
         for (int h = 0; h < 2; ++h) {
             const int row = g + 8 * h;
             if (next[h] && row < 15) {
+                unsigned off = 0u;
 #pragma unroll
                 for (int j = 0; j < NT; ++j) {
                     const float2 v = *reinterpret_cast<const float2 *>(ss + (row + 1) * SW + 8 * j + 2 * t);
                     const unsigned q = max(absdiff_bits(v.x, d[j][2 * h]), absdiff_bits(v.y, d[j][2 * h + 1]));
-                    mis = max(mis, q);
-                    if (near[h]) mis_end = max(mis_end, q);
+                    off = max(off, q);
                 }
+                mis = max(mis, off);
+                rel = max(rel, boundary_ratio(off, ss[(row + 1) * SW + N]));
+                if (near[h]) mis_end = max(mis_end, off);
             }
         }
         const bool near_next = __shfl_sync(0xffffffffu, (int)near[1], 28) != 0;
@@ -404,8 +436,9 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
             if (side == 0 ? !has_next : !has_prev) continue;
             const size_t edge = (size_t)hd.first_edge + (size_t)grp - side;
             const float *own = ss + (side == 0 ? 15 : 0) * SW;
-            float *slot = a.edge + edge * 2 * n;
+            float *slot = a.edge + edge * ADJ_EDGE(n);
             for (int i = lane; i < n; i += 32) __stcg(slot + side * n + i, own[i]);
+            if (side == 1 && lane == 0) __stcg(slot + 2 * n, own[N]);
             __threadfence();
             __syncwarp();
             unsigned old = 0;
@@ -414,9 +447,11 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
             if (old == 1u) {
                 __threadfence();
                 const bool near_here = side == 0 ? near_next : near_prev;
+                const float scale = side == 0 ? __ldcg(slot + 2 * n) : own[N];
                 for (int i = lane; i < n; i += 32) {
                     const unsigned q = absdiff_bits(own[i], __ldcg(slot + (side ^ 1) * n + i));
                     mis = max(mis, q);
+                    rel = max(rel, boundary_ratio(q, scale));
                     if (near_here) mis_end = max(mis_end, q);
                 }
                 if (lane == 0) a.edge_flag[edge] = 0u;
@@ -427,12 +462,14 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     for (int o = 16; o > 0; o >>= 1) {
         mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
         mis = max(mis, __shfl_xor_sync(0xffffffffu, mis, o));
+        rel = max(rel, __shfl_xor_sync(0xffffffffu, rel, o));
         mb_end = max(mb_end, __shfl_xor_sync(0xffffffffu, mb_end, o));
         mis_end = max(mis_end, __shfl_xor_sync(0xffffffffu, mis_end, o));
     }
     if (lane == 0) {
         if (mb) atomicMax(&st->err_bits, mb);
         if (mis) atomicMax(&st->mis_bits, mis);
+        if (rel) atomicMax(&st->rel_bits, rel);
         if (mb_end) atomicMax(&st->top_end_bits, mb_end);
         if (mis_end) atomicMax(&st->mis_end_bits, mis_end);
         __threadfence();

@@ -43,12 +43,14 @@ struct AdjArgs {
     int dy0_by_head;
     int B, T, n, m, H, L;
     int burn, burn_cap;      // burn-in of the first try; longest that another one is worth
-    float eta;               // largest boundary mismatch that is accepted, as a part of max|lambda|
+    float eta;               // largest boundary mismatch that is accepted, as a part of max|lambda| (and see ADJ_LOCAL)
     StatusBlock *st;         // [H]; done = 1 where the launch has done the work (it returns at once where it is set)
-    float *edge;
+    float *edge;             // [boundaries][ADJ_EDGE(n)]  end state of the chain before, start state and scale of the one behind
     unsigned *edge_flag;
     float *starts;           // [groups][16][n + 4 of the padded size], n > 48 only (adjoint_starts)
 };
+
+__host__ __device__ constexpr int ADJ_EDGE(int n) { return 2 * n + 1; }
 
 constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2;       // StatusBlock::done: the loop ended / this form gives up
 

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         for (int k = 0; k < M; ++k) x[k] = __ldg(xp + k);
         g = __ldg(gb + (size_t)t * N + i);
     };
-    float mu = 0.0f, start = 0.0f;
+    float mu = 0.0f, start = 0.0f, scale = 0.0f;         // scale: of the boundary before this chain
     unsigned mb = 0u;
     float ai[3][M + 1], ah[3][N + 1];
 #pragma unroll
@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         const float r = rcp_approx(1.0f + ex2_approx(-LOG2E * ar)), z = rcp_approx(1.0f + ex2_approx(-LOG2E * az));
         const float cc = fmaf(rcp_approx(1.0f + ex2_approx(2.0f * LOG2E * fmaf(r, aq, an))), -2.0f, 1.0f);       // tanh
         const float lam = gv[u] + mu, lo = (1.0f - z) * lam;
+        if (act) mb = max(mb, __float_as_uint(fabsf(lam)));
         float pz = lo * z * (h - cc), pa = lo * fmaf(-cc, cc, 1.0f), pn = pa * r, pr = pn * aq * (1.0f - r);
         float sh[N];
 #pragma unroll
@@ -124,7 +125,6 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         reduce_scatter<N, N>(sh, i);
         if constexpr (OWN) {
             if (!act) { pr = 0.0f; pz = 0.0f; pn = 0.0f; pa = 0.0f; }
-            else mb = max(mb, __float_as_uint(fabsf(lam)));
 #pragma unroll
             for (int k = 0; k < M; ++k) { ai[0][k] = fmaf(pr, xv[u][k], ai[0][k]); ai[1][k] = fmaf(pz, xv[u][k], ai[1][k]); ai[2][k] = fmaf(pa, xv[u][k], ai[2][k]); }
 #pragma unroll
@@ -155,10 +155,15 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         for (int u = 0; u < U; ++u) fetch(ts + s0 + u, hb[u], xv[u], gv[u]);
 #pragma unroll 1
         for (int s = s0; s < burn; s += U) {
+            if (s == burn - ADJ_WINDOW) mb = 0u;
 #pragma unroll
             for (int u = 0; u < U; ++u) { step(s + u, u, No{}); fetch(ts + s + U + u, hb[u], xv[u], gv[u]); }
         }
         start = mu;
+        unsigned top = mb;
+#pragma unroll
+        for (int o = N / 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(FULL, top, o));
+        scale = __uint_as_float(top);
 #pragma unroll 1
         for (int s = burn; s < s_end; s += U) {
 #pragma unroll
@@ -186,23 +191,31 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
         else out.partial_h[(size_t)blockIdx.x * (3 * N * (N + 1)) + (((v - VI) / (N + 1)) * N + row) * (N + 1) + (v - VI) % (N + 1)] = sum;
     }
     // ---- the gradient w.r.t. y0, and the boundaries
-    unsigned mb_end = 0u, mis = 0u, mis_end = 0u;
+    unsigned mb_end = 0u, mis = 0u, rel = 0u, mis_end = 0u;
     if (a.dy0 && te > 0 && !next) {
         a.dy0[(size_t)b * N + i] = mu;
         mb_end = __float_as_uint(fabsf(mu));
     }
     const int reach = DY0_REACH * burn;
     if constexpr (N < 32) {                              // the next chain of this warp
-        const float sn = __shfl_down_sync(FULL, start, N);
-        if (next && lane + N < 32) { mis = absdiff_bits(sn, mu); if (T - te < reach) mis_end = mis; }
+        const float sn = __shfl_down_sync(FULL, start, N), sc = __shfl_down_sync(FULL, scale, N);
+        if (next && lane + N < 32) {
+            mis = absdiff_bits(sn, mu);
+            rel = boundary_ratio(mis, sc);
+            if (T - te < reach) mis_end = mis;
+        }
     }
     const long long wg = (long long)blockIdx.x * 4 + warp;
 #pragma unroll 1
     for (int side = 0; side < 2; ++side) {               // 0: behind this warp's chains, 1: before them
         const bool mine = side == 0 ? lane >= 32 - N && next : lane < N && prev && wg > 0;
         const size_t edge = (size_t)(wg - side);
-        float *slot = a.edge + edge * 2 * N;
-        if (mine) { __stcg(slot + side * N + i, side == 0 ? mu : start); __threadfence(); }
+        float *slot = a.edge + edge * ADJ_EDGE(N);
+        if (mine) {
+            __stcg(slot + side * N + i, side == 0 ? mu : start);
+            if (side == 1 && i == 0) __stcg(slot + 2 * N, scale);
+            __threadfence();
+        }
         __syncwarp();
         unsigned old = 0u;
         const int leader = side == 0 ? 32 - N : 0;
@@ -212,17 +225,20 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
             __threadfence();
             const unsigned q = absdiff_bits(side == 0 ? mu : start, __ldcg(slot + (side ^ 1) * N + i));
             mis = max(mis, q);
+            rel = max(rel, boundary_ratio(q, side == 0 ? __ldcg(slot + 2 * N) : scale));
             if (T - (side == 0 ? te : c * L) < reach) mis_end = max(mis_end, q);
             if (lane == leader) a.edge_flag[edge] = 0u;
         }
     }
     mb = __reduce_max_sync(FULL, mb);
     mis = __reduce_max_sync(FULL, mis);
+    rel = __reduce_max_sync(FULL, rel);
     mb_end = __reduce_max_sync(FULL, mb_end);
     mis_end = __reduce_max_sync(FULL, mis_end);
     if (lane == 0) {
         if (mb) atomicMax(&st->err_bits, mb);
         if (mis) atomicMax(&st->mis_bits, mis);
+        if (rel) atomicMax(&st->rel_bits, rel);
         if (mb_end) atomicMax(&st->top_end_bits, mb_end);
         if (mis_end) atomicMax(&st->mis_end_bits, mis_end);
         __threadfence();

@@ -180,3 +180,60 @@ def test_adjoint_of_small_cells_in_short_chains(bd, n, m, B, T):
     for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
         a, b = got[k].cpu().numpy().astype(np.float64), want[k]
         assert np.max(np.abs(a - b)) <= 1e-4 * np.max(np.abs(b)), k
+
+
+def gradient(bd, p, x, y0, gy, **kw):
+    """deer_gru_vjp at the sequential trajectory, the fp64 gradients, the kernels launched, whether their result was taken."""
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    B, T, m = x.shape
+    ws = bd.alloc_workspace(bd.DEER_OP_VJP, B, T, p.b_i.size // 3, m)
+    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True, ws=ws, **kw))
+    got = {k: v.cpu().numpy().astype(np.float64) for k, v in got.items() if v is not None}
+    return got, want, names, accepted(ws)
+
+
+SCALES = [(8, 4, 16, 10001, ROWS), (2, 1, 16, 40001, ROWS), (24, 3, 2, 6001, WARP), (32, 8, 16, 9001, WARP), (64, 6, 4, 20001, MMA_TILE)]
+
+
+@pytest.mark.parametrize("n,m,B,T,kernel", SCALES)
+def test_adjoint_of_sequences_of_unequal_weight(bd, n, m, B, T, kernel):
+    """The first sequence's loss weighs most and its inputs make the cell forget; the others weigh a millionth or less and
+    remember.  Each has its own dx and dy0 to a thousandth, the tolerance that gradients have everywhere."""
+    p = synth.gru_params(n, m, 8, tag="c/gru")
+    p.W_i[n:2 * n, 0] = 1.0
+    x = synth.x_gaussian(B, T, m, 8, tag="c/x")
+    x[:, :, 0] = 2.0 + 0.25 * x[:, :, 0]
+    x[0, :, 0] -= 6.0
+    y0 = synth.normal(8, "c/y0", (B, n)) * 0.3
+    gy = synth.normal(8, "c/gy", (B, T, n))
+    gy[1::2] *= np.float32(1e-6)
+    gy[2::2] *= np.float32(1e-12)
+    got, want, names, _ = gradient(bd, p, x, y0, gy)
+    assert kernel in names, names
+    for k in ("dx", "dy0"):
+        for b in range(B):
+            assert np.max(np.abs(got[k][b] - want[k][b])) <= 1e-3 * np.max(np.abs(want[k][b])), (k, b)
+
+
+@pytest.mark.parametrize("n,m,B,T,kernel", SCALES)
+def test_adjoint_behind_a_loss_on_the_last_step(bd, n, m, B, T, kernel):
+    """lambda decays through every magnitude towards the first step: dx is right at each, compared in blocks of eight steps as
+    long as it is an ordinary fp32 number (products of up to some hundred Jacobians, each good to about 1e-5)."""
+    p = synth.gru_params(n, m, 9, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 9, tag="c/x")
+    y0 = synth.normal(9, "c/y0", (B, n)) * 0.3
+    gy = np.zeros((B, T, n), np.float32)
+    gy[:, -1] = synth.normal(9, "c/gy", (B, n))
+    got, want, names, _ = gradient(bd, p, x, y0, gy)
+    assert kernel in names, names
+    blocks = 0
+    for b in range(B):
+        for t in range(T - 8, T - 400, -8):
+            top = np.max(np.abs(want["dx"][b, t:t + 8]))
+            if top < 1e-25:
+                break
+            assert np.max(np.abs(got["dx"][b, t:t + 8] - want["dx"][b, t:t + 8])) <= 1e-2 * top, (b, T - t)
+            blocks += 1
+    assert blocks > 6 * B              # (n = 2 decays by 1e-25 within some sixty steps)
