@@ -363,13 +363,15 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     if (cg == 0) sMax[row] = scale;
     __syncthreads();
 
-    // ---- the state that leaves the first time step: the gradient w.r.t. y0
-    if (a.dy0 && own.te > 0 && !has_next) {
-        float *o = a.dy0 + (size_t)own.b * N + c0;
+    // ---- the state that leaves the first time step: the gradient w.r.t. y0.  Wanted or not, it shows an input beyond f16's range
+    // at that step, which reaches no boundary.
+    if (own.te > 0 && !has_next) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            mb_end = max(mb_end, max(__float_as_uint(fabsf(d[j].x)), __float_as_uint(fabsf(d[j].y))));
-            o[2 * j] = d[j].x; o[2 * j + 1] = d[j].y;
+        for (int j = 0; j < 8; ++j) mb_end = max(mb_end, max(__float_as_uint(fabsf(d[j].x)), __float_as_uint(fabsf(d[j].y))));
+        if (a.dy0) {
+            float *o = a.dy0 + (size_t)own.b * N + c0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { o[2 * j] = d[j].x; o[2 * j + 1] = d[j].y; }
         }
     }
     // ---- boundaries: this row's end state against what its successor assumed

@@ -57,7 +57,8 @@ __device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool 
 {
     auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
     const float top = take(st->err_bits), mis = take(st->mis_bits), rel = take(st->rel_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
-    const bool inner = mis <= eta * top && rel <= ADJ_LOCAL * eta, end = !dy0 || mis_end <= eta * top_end;
+    // (at the first time step a NaN reaches no boundary and no lambda any more, only the final state and the gradients there)
+    const bool inner = top_end <= 3.402823466e38f && mis <= eta * top && rel <= ADJ_LOCAL * eta, end = !dy0 || mis_end <= eta * top_end;
     if (inner && end) { st->done = BODY_DONE; return; }
     // the carried error is about |lambda| * rho^burn: the burn-in after which it is half of what is accepted
     int want = 1 << 20;
@@ -385,22 +386,23 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                     for (int q = 0; q < 4; ++q) top[q >> 1] = max(top[q >> 1], __float_as_uint(fabsf(d[j][q])));
             }
         }
-        // ---- the state that leaves the first time step: the gradient w.r.t. y0
-        if (a.dy0) {
+        // ---- the state that leaves the first time step: the gradient w.r.t. y0 (wanted or not, it shows what is not finite there)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if (t_end[h] > 0 && !next[h]) {
+        for (int h = 0; h < 2; ++h)
+            if (t_end[h] > 0 && !next[h]) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mb_end = max(mb_end, max(__float_as_uint(fabsf(d[j][2 * h])), __float_as_uint(fabsf(d[j][2 * h + 1]))));
+                if (a.dy0) {
                     const long long q = (grp * 16 + g + 8 * h) / nchain;
                     float *o = a.dy0 + (a.dy0_by_head ? q * H + blockIdx.y : hd.first_seq + q) * n;
 #pragma unroll
                     for (int j = 0; j < NT; ++j) {
                         const int col = 8 * j + 2 * t;
-                        mb_end = max(mb_end, max(__float_as_uint(fabsf(d[j][2 * h])), __float_as_uint(fabsf(d[j][2 * h + 1]))));
                         if (col < n) o[col] = d[j][2 * h];
                         if (col + 1 < n) o[col + 1] = d[j][2 * h + 1];
                     }
                 }
-        }
+            }
         // ---- boundaries: this row's end state against the state its successor assumed
         __syncwarp();
 #pragma unroll

@@ -192,9 +192,9 @@ __global__ void __launch_bounds__(128, (RowsAdj<N, M>::CTAS)) rows_adjoint_kerne
     }
     // ---- the gradient w.r.t. y0, and the boundaries
     unsigned mb_end = 0u, mis = 0u, rel = 0u, mis_end = 0u;
-    if (a.dy0 && te > 0 && !next) {
-        a.dy0[(size_t)b * N + i] = mu;
-        mb_end = __float_as_uint(fabsf(mu));
+    if (te > 0 && !next) {
+        if (a.dy0) a.dy0[(size_t)b * N + i] = mu;
+        mb_end = __float_as_uint(fabsf(mu));             // (wanted or not: see adjoint_decide)
     }
     const int reach = DY0_REACH * burn;
     if constexpr (N < 32) {                              // the next chain of this warp

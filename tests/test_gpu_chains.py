@@ -237,3 +237,19 @@ def test_adjoint_behind_a_loss_on_the_last_step(bd, n, m, B, T, kernel):
             assert np.max(np.abs(got["dx"][b, t:t + 8] - want["dx"][b, t:t + 8])) <= 1e-2 * top, (b, T - t)
             blocks += 1
     assert blocks > 6 * B              # (n = 2 decays by 1e-25 within some sixty steps)
+
+
+@pytest.mark.parametrize("t", [0, 1, 1000, 12000])
+def test_adjoint_tile_beyond_the_range_of_its_operands(bd, t):
+    """Inputs that f16 halves cannot hold make the tile's result a NaN, at the first time step only in the gradients there: the
+    launch has to see it whether dy0 is wanted or not, and the kernels behind do the work."""
+    n, m, B, T = 64, 6, 5, 12001
+    p = synth.gru_params(n, m, 10, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 10, tag="c/x")
+    x[1, t] *= np.float32(2e4)
+    gy = synth.normal(10, "c/gy", (B, T, n))
+    for want_dy0 in (False, True):
+        got, want, names, done = gradient(bd, p, x, np.zeros((B, n), np.float32), gy, want_dy0=want_dy0)
+        assert MMA_TILE in names and done == 0, names
+        for k in got:
+            assert np.max(np.abs(got[k] - want[k])) <= 1e-3 * np.max(np.abs(want[k])), k
