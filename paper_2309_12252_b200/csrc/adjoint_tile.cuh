@@ -436,8 +436,7 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         __threadfence();
     }
     if ((s_abort[0] || s_abort[1]) && tid == 0) {                           // a wait for the tensor core ran out: let what is in flight end
-        tile_wait(&bar1, phase ^ 1u);
-        tile_wait(&bar2, phase ^ 1u);
+        if (s_abort[0]) tile_wait(&bar1, phase); else tile_wait(&bar2, phase ^ 1u);
         atomicOr(&st->flags, FLAG_TIMEOUT);
         __threadfence();
     }
