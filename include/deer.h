@@ -93,8 +93,12 @@ enum {
                                    and every wait gives up after a few polls, so the scan drains
                                    and the call reports DEER_ERR_DEVICE_TIMEOUT (outputs invalid).
                                    Nothing traps or hangs; the workspace can be used again */
-    DEER_FLAG_COEF_ROWS  = 32   /* deer_gru_cell_jac, n = 16, 32 and 64: write the four coefficient
+    DEER_FLAG_COEF_ROWS  = 32,  /* deer_gru_cell_jac, n = 16, 32 and 64: write the four coefficient
                                    vectors per position instead of the matrices (see there) */
+    DEER_FLAG_EXPIRE_BODY_WAITS = 64 /* the same test aid for the kernels that run a Newton body, the
+                                   whole loop or the adjoint solve as one launch (evaluations and
+                                   gradients): a CTA's wait for the others of a whole-loop launch
+                                   and for its tensor-core products give up */
 };
 
 /* Bytes of workspace needed by `op` at the given sizes (0 if the sizes are

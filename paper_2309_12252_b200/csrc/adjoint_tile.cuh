@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         const float sc = __uint_as_float((unsigned)(127 + 9 - (ex - 127)) << 23), inv = __uint_as_float((unsigned)(127 - 9 + (ex - 127)) << 23);
         const float kM = inv / wscale;
         if (step + 1 < s_end) { load(step + 1); load_g(step + 1); }
-        if (!tile_wait(&bar1, phase)) s_abort[0] = 1;
+        if (a.expire || !tile_wait(&bar1, phase)) s_abort[0] = 1;
         tile_fence_after();
         // ---- gates, pre-activation gradients
         float *go = a.dGi + (ptrdiff_t)(own.e - step) * (4 * N) + c0;

@@ -1084,6 +1084,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     a.buf[0] = buf[0]; a.buf[1] = buf[1];
     a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1;
     a.eta = body_eta(n, tol);
+    a.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0;
     a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
     a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
     const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
@@ -1138,7 +1139,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
             if (hr) {
                 DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
                 hs->iters = hr->iters; hs->done = hr->done; hs->burn = hr->burn; hs->err_last_bits = hr->err_bits;
-                if (plan.whole_loop && !hs->done) return DEER_ERR_DEVICE_TIMEOUT;
+                if (hs->done == BODY_TIMED_OUT || (plan.whole_loop && !hs->done)) return DEER_ERR_DEVICE_TIMEOUT;
             } else {
                 DEER_CHECK_CUDA(cudaMemcpyAsync(hs, w.st, 48, cudaMemcpyDeviceToHost, st), "read status");
                 DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
@@ -1397,6 +1398,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
         a.dy0 = dy0; a.dy0_by_head = 1;
         a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1; a.L = tile ? tplan.L : plan.L;
         a.eta = ADJ_ETA;
+        a.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0;
         a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.starts = tile ? w.J : w.starts;
         // (small cells: one try, the passes behind it are cheap)
         a.burn = !lanes && burn_hint > ADJ_BURN && burn_hint <= adjoint_burn_cap(n, m, (long long)B * T, a.L) ? burn_hint : ADJ_BURN;
@@ -2049,6 +2051,7 @@ static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int
     a.warm = (flags & DEER_FLAG_WARM_START) ? 1 : 0;
     a.eta = body_eta(n, tol);
     a.burn_cap = plan.burn_cap;
+    a.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0;
     a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
     hs.assign((size_t)H, StatusBlock{});
     for (int group = 4, most = 0;; group = 2) {

@@ -57,6 +57,7 @@ __device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool 
 {
     auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
     const float top = take(st->err_bits), mis = take(st->mis_bits), rel = take(st->rel_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
+    if (*(volatile unsigned *)&st->flags & FLAG_TIMEOUT) { st->burn = 1 << 20; return; }         // (unfinished rows: the kernels behind do the work)
     // (at the first time step a NaN reaches no boundary and no lambda any more, only the final state and the gradients there)
     const bool inner = top_end <= 3.402823466e38f && mis <= eta * top && rel <= ADJ_LOCAL * eta, end = !dy0 || mis_end <= eta * top_end;
     if (inner && end) { st->done = BODY_DONE; return; }

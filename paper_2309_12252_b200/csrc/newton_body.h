@@ -24,6 +24,7 @@ struct BodyArgs {
     int warm;                // buf[0] holds the guess (0: the guess is zero and buf[0] is not read)
     float eta;               // largest boundary mismatch, as a part of max(err, tol), that is accepted
     int burn_cap;            // longest burn-in that is tried (BodyPlan)
+    int expire;              // test aid: every bounded wait runs out (DEER_FLAG_EXPIRE_BODY_WAITS)
     StatusBlock *st;         // [H]
     float *edge;             // [groups][2][n]  states either side of a boundary between two warps
     unsigned *edge_flag;     // [groups]        arrivals at it (left cleared)
@@ -44,6 +45,7 @@ struct AdjArgs {
     int B, T, n, m, H, L;
     int burn, burn_cap;      // burn-in of the first try; longest that another one is worth
     float eta;               // largest boundary mismatch that is accepted, as a part of max|lambda| (and see ADJ_LOCAL)
+    int expire;              // as in BodyArgs
     StatusBlock *st;         // [H]; done = 1 where the launch has done the work (it returns at once where it is set)
     float *edge;             // [boundaries][ADJ_EDGE(n)]  end state of the chain before, start state and scale of the one behind
     unsigned *edge_flag;
@@ -52,7 +54,8 @@ struct AdjArgs {
 
 __host__ __device__ constexpr int ADJ_EDGE(int n) { return 2 * n + 1; }
 
-constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2;       // StatusBlock::done: the loop ended / this form gives up
+// StatusBlock::done: the loop ended / this form gives up / a bounded wait ran out, nothing that was computed counts
+constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3;
 
 // The kernels of one padded state size (newton_kernels.cu).
 struct BodyKernels {

@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
                 __stcg(reinterpret_cast<float4 *>(a.starts + gid * N + c0) + j, make_float4(d[2 * j].x, d[2 * j].y, d[2 * j + 1].x, d[2 * j + 1].y));
         }
         group_sync();
-        if (!tile_wait(&s_bar, phase)) s_abort = 1;
+        // (where it runs out, this step goes on with what it finds, and nothing of it counts)
+        if (a.expire || !tile_wait(&s_bar, phase)) s_abort = 1;
         phase ^= 1u;
         tile_fence_after();
         if (!TWICE) {                                    // (the products are done with the operands)
@@ -436,7 +437,11 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
             __threadfence();
             st->exit_counter = 0u;
             const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits), q = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
-            if (!(e <= 3.402823466e38f) || !(q <= 3.402823466e38f)) {      // beyond f16's range, or not finite at all: the other kernels tell
+            if (*(volatile unsigned *)&st->flags & FLAG_TIMEOUT) {         // rows that were not finished: nothing counts
+                st->err_bits = 0u; st->mis_bits = 0u;
+                st->done = BODY_TIMED_OUT;
+                if (HostResult *h = st->host) h->done = BODY_TIMED_OUT;
+            } else if (!(e <= 3.402823466e38f) || !(q <= 3.402823466e38f)) {      // beyond f16's range, or not finite at all: the other kernels tell
                 st->err_bits = 0u; st->mis_bits = 0u;
                 st->done = BODY_FALL_BACK;
                 if (HostResult *h = st->host) h->done = BODY_FALL_BACK;

@@ -253,3 +253,46 @@ def test_adjoint_tile_beyond_the_range_of_its_operands(bd, t):
         assert MMA_TILE in names and done == 0, names
         for k in got:
             assert np.max(np.abs(got[k] - want[k])) <= 1e-3 * np.max(np.abs(want[k])), k
+
+
+@pytest.mark.parametrize("n,m,B,T,kernel", [(4, 2, 1, 1000, SEG), (24, 10, 5, 1001, SEG), (32, 33, 16, 6001, TILE), (64, 6, 3, 9001, TILE)])
+def test_expired_wait_in_a_body_is_reported(bd, n, m, B, T, kernel):
+    """The whole-loop kernel's wait for the other CTAs and the tile's for its products are bounded: where one runs out the
+    evaluation says so, and the next call on the same workspace is right."""
+    p = synth.gru_params(n, m, seed=11, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=11, tag="c/x")
+    y0 = synth.normal(11, "c/y0", (B, n)) * 0.5
+    pd, xd, yd = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    ws = bd.alloc_workspace(bd.DEER_OP_EVAL, B, T, n, m)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(pd, xd, yd, ws=ws, flags=bd.DEER_FLAG_EXPIRE_BODY_WAITS, check=False))
+    assert kernel in names and r.status == bd.DEER_ERR_DEVICE_TIMEOUT, (names, r.status)
+    r = bd.deer_gru_eval(pd, xd, yd, ws=ws)
+    assert r.status == 0
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-4
+
+
+def test_expired_wait_in_the_adjoint_tile_is_reported(bd):
+    n, m, B, T = 64, 6, 5, 12001
+    p = synth.gru_params(n, m, seed=12, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=12, tag="c/x")
+    y0 = np.zeros((B, n), np.float32)
+    gy = synth.normal(12, "c/gy", (B, T, n))
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    ws = bd.alloc_workspace(bd.DEER_OP_VJP, B, T, n, m)
+    _, names = launched(bd, lambda: bd.deer_gru_vjp(*args, ws=ws, flags=bd.DEER_FLAG_EXPIRE_BODY_WAITS))
+    assert MMA_TILE in names and accepted(ws) == 0
+    assert bd.deer_workspace_status(ws) == bd.DEER_ERR_DEVICE_TIMEOUT
+    got = bd.deer_gru_vjp(*args, ws=ws)
+    assert accepted(ws) == 1 and bd.deer_workspace_status(ws) == bd.DEER_OK
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    assert np.max(np.abs(got["dW_h"].cpu().numpy() - want["dW_h"])) <= 1e-3 * np.max(np.abs(want["dW_h"]))
+
+
+def test_expired_wait_in_the_multihead_loop_is_reported(bd):
+    H, n, m, B, T = 3, 8, 5, 2, 300
+    heads = [bd.GruParamsDev.from_numpy(synth.gru_params(n, m, seed=h, tag="c/gru")) for h in range(H)]
+    x, y0 = dev(synth.x_gaussian(B, T, m, seed=13, tag="c/x")), torch.zeros((B, H, n), device="cuda")
+    with pytest.raises(bd.DeerError):
+        bd.deer_gru_multihead_eval(heads, [1, 2, 4], x, y0, flags=bd.DEER_FLAG_EXPIRE_BODY_WAITS)
+    assert bd.deer_gru_multihead_eval(heads, [1, 2, 4], x, y0)[2] == 0
