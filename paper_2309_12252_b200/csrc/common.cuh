@@ -75,9 +75,11 @@ static inline cudaError_t launch_pdl(bool overlap, void (*kern)(KArgs...), unsig
         }                                                          \
     } while (0)
 
-// What an evaluation reports, written by the kernel that takes the loop decision straight into page-locked host memory.
-struct HostResult {
-    int iters, done, burn;
+// What an evaluation reports, written by the kernel that takes the loop decision straight into page-locked host memory: `done`
+// last, and behind a fence where the host acts on it before it has synchronised.
+struct __align__(16) HostResult {
+    int done, burn;      // (one 64-bit store where nothing else is reported)
+    int iters;
     unsigned err_bits;
     float trace[28];     // err after the first bodies
 };
@@ -175,6 +177,12 @@ __device__ __forceinline__ bool loop_ended(const StatusBlock *st)
 // End of one Newton body (App. B.1 loop): record err, count the body, decide whether the loop goes on
 // (err > tol and fewer than max_iter bodies).  A NaN err fails "err > tol" and ends the loop, as in
 // the listing; an infinite err ends it too.  Single thread.
+__device__ __forceinline__ void post_done(HostResult *h, int done, bool fence)
+{
+    if (fence) __threadfence_system();
+    *(volatile int *)&h->done = done;
+}
+
 __device__ __forceinline__ bool newton_loop_ends(float e, float tol, int k, int max_iter)
 {
     return !(e > tol) || !(e <= 3.402823466e38f) || k + 1 >= max_iter;
@@ -193,7 +201,8 @@ __device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int ma
     if (end) st->done = 1;
     if (HostResult *h = st->host) {
         if (k < HOST_TRACE) h->trace[k] = e;
-        h->iters = k + 1; h->err_bits = bits; h->burn = st->burn; h->done = end;
+        h->iters = k + 1; h->err_bits = bits; h->burn = st->burn;
+        post_done(h, end, false);
     }
 }
 

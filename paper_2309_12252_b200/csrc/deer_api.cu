@@ -1060,6 +1060,19 @@ public:
     HostSlot &operator=(const HostSlot &) = delete;
 };
 
+// Reads the record until the loop or the form has ended there, which is before the launches enqueued behind it have drained,
+// and returns how; 0 after `polls` reads (some 15 ns each), or where the stream has come to its end.
+static int record_posted(const HostResult *hr, cudaStream_t st, unsigned polls)
+{
+    const volatile int *done = &hr->done;
+    for (unsigned k = 1; k <= polls; ++k) {
+        if (const int how = *done) return how;
+        __builtin_ia32_pause();
+        if (k % 1024 == 0 && cudaStreamQuery(st) != cudaErrorNotReady) return *done;         // (an error is sticky: the caller's synchronisation reports it)
+    }
+    return 0;
+}
+
 // ---- evaluations whose bodies are one launch each (newton_body.cuh)
 // The flags that ask for a particular form of the scan are served by the kernels that have that form.
 static bool body_takes(int n, int m, int flags)
@@ -1067,6 +1080,11 @@ static bool body_takes(int n, int m, int flags)
     return !(flags & (DEER_FLAG_GENERIC | DEER_FLAG_MATERIALIZE | DEER_FLAG_TCGEN05 | DEER_FLAG_EXPIRE_WAITS)) &&
            (body_supported(n, m, false) || body_supported(n, m, true));
 }
+
+// Reads of the record before the host waits for the stream.  The bias check answers some 10 us after its launch, without a
+// body; a longer look costs more at the end of an evaluation (a synchronisation that is entered late, 0.7 us) than a form that
+// gives up later gains.
+constexpr unsigned POLLS_BIAS = 1500;
 
 // Runs the Newton loop until it ends or the form gives up (hs->done == BODY_FALL_BACK, the iterate after hs->iters bodies in
 // buf[hs->iters & 1]).
@@ -1133,11 +1151,15 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
         }
         for (int group = 4;; group = 2) {
             const int left = max_iter - hs->iters;
-            for (int j = 0; j < (plan.whole_loop ? 1 : left < group ? left : group); ++j)
+            for (int j = 0; j < (plan.whole_loop ? 1 : left < group ? left : group); ++j) {
+                if (hr && *(volatile int *)&hr->done) break;             // (the bias alone has told, or the loop is over already)
                 if ((rc = launch_newton_body(a, plan, st)) != DEER_OK) return rc;
+            }
             if ((rc = copy_out()) != DEER_OK) return rc;
             if (hr) {
-                DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+                // The next form goes ahead as soon as the record tells that this one has given up.
+                const int end = record_posted(hr, st, POLLS_BIAS);
+                if (end != BODY_FALL_BACK) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
                 hs->iters = hr->iters; hs->done = hr->done; hs->burn = hr->burn; hs->err_last_bits = hr->err_bits;
                 if (hs->done == BODY_TIMED_OUT || (plan.whole_loop && !hs->done)) return DEER_ERR_DEVICE_TIMEOUT;
             } else {

@@ -339,7 +339,7 @@ __global__ void eval_begin_kernel(StatusBlock *st, StatusBlock init, EvalBeginAr
             if (e.b_i && z > e.slow) {
                 init.done = BODY_FALL_BACK;
                 init.burn = (int)fminf(1e6f, -2.3f / __logf(z)) + 1;             // until a tenth is left
-                if (init.host) { init.host->burn = init.burn; init.host->done = init.done; }
+                if (init.host) *reinterpret_cast<volatile unsigned long long *>(init.host) = ((unsigned long long)(unsigned)init.burn << 32) | (unsigned)init.done;
             }
             *st = init;
         }

@@ -73,7 +73,7 @@ __device__ __forceinline__ void body_decide(StatusBlock *st, float eta, int burn
     if (v.counts && (st->done || !v.done)) return;
     st->err_bits = 0u;
     st->done = v.done;
-    if (HostResult *h = st->host) { h->burn = v.burn; h->done = v.done; }
+    if (HostResult *h = st->host) { h->burn = v.burn; post_done(h, v.done, v.done != 0); }
 }
 
 template <int N> struct Body {

@@ -541,7 +541,10 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
                 st->iters = iters + (v.counts ? 1 : 0);
                 st->burn = v.burn;
                 st->done = v.done;
-                if (HostResult *h = st->host) { h->iters = st->iters; h->err_bits = st->err_last_bits; h->burn = v.burn; h->done = v.done; }
+                if (HostResult *h = st->host) {
+                    h->iters = st->iters; h->err_bits = st->err_last_bits; h->burn = v.burn;
+                    post_done(h, v.done, v.done != BODY_DONE);
+                }
             }
         }
         if (v.done) return;
