@@ -42,13 +42,13 @@ __device__ __forceinline__ void st_word(unsigned long long *p, int i, int n, flo
 {
     if (i < n) st_relaxed_u64w(p + i, ((unsigned long long)tag << 32) | __float_as_uint(v));
 }
-__device__ __forceinline__ unsigned wait_word(const unsigned long long *p, unsigned tag, bool &gave_up, unsigned limit)
+__device__ __forceinline__ unsigned wait_word(const unsigned long long *p, unsigned tag, bool &gave_up)
 {
     unsigned long long v = 0;
     for (unsigned spins = 0;; ++spins) {
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
         if ((unsigned)(v >> 32) == tag) break;
-        if (spins > limit) { gave_up = true; break; }
+        if (spins > BODY_SPIN_LIMIT) { gave_up = true; break; }
     }
     return (unsigned)v;
 }
@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
     const float tol = st->tol;
     const int max_iter = st->max_iter;
     __shared__ unsigned red[4][C::WARPS];
-    const unsigned limit = a.expire ? 1u << 10 : BODY_SPIN_LIMIT;        // (expire: besides, the first CTA posts no maxima)
     unsigned long long *const edge_w = reinterpret_cast<unsigned long long *>(a.edge) + (size_t)hd.first_edge * n;
 
     for (unsigned round = 1;; ++round) {
@@ -478,8 +477,8 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         // the boundary behind this CTA: its successor's assumed start was posted when that one's burn-in ended
         if (whole_loop && has_next && grp == G - 1 && g == 7) {
             const unsigned long long *q = edge_w + (size_t)(blockIdx.x + 1) * n + col;
-            if (col < n) mis = max(mis, absdiff_bits(d[2], __uint_as_float(wait_word(q, round, gave_up, limit))));
-            if (col + 1 < n) mis = max(mis, absdiff_bits(d[3], __uint_as_float(wait_word(q + 1, round, gave_up, limit))));
+            if (col < n) mis = max(mis, absdiff_bits(d[2], __uint_as_float(wait_word(q, round, gave_up))));
+            if (col + 1 < n) mis = max(mis, absdiff_bits(d[3], __uint_as_float(wait_word(q + 1, round, gave_up))));
         }
     }
     __syncthreads();
@@ -510,7 +509,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         if (warp == 0) {
             const unsigned e = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[0][lane] : 0u);
             const unsigned q = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[1][lane] : 0u);
-            if (lane == 0 && !(a.expire && blockIdx.x == 0)) {
+            if (lane == 0 && !(a.expire && blockIdx.x == 0)) {             // (expire: nobody's wait for the first CTA ends)
                 __threadfence();                         // this CTA's part of the new iterate is visible before its word
                 st_relaxed_u64w(box + 2 * blockIdx.x, ((unsigned long long)round << 32) | e);
                 st_relaxed_u64w(box + 2 * blockIdx.x + 1, ((unsigned long long)round << 32) | q);
@@ -518,8 +517,8 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         }
         unsigned e = 0u, q = 0u;
         for (int i = tid; i < (int)nctas; i += C::THREADS) {
-            e = max(e, wait_word(box + 2 * i, round, gave_up, limit));
-            q = max(q, wait_word(box + 2 * i + 1, round, gave_up, limit));
+            e = max(e, wait_word(box + 2 * i, round, gave_up));
+            if (!gave_up) q = max(q, wait_word(box + 2 * i + 1, round, gave_up));
         }
         e = __reduce_max_sync(0xffffffffu, e);
         q = __reduce_max_sync(0xffffffffu, q);
