@@ -228,8 +228,8 @@ int deer_gru_eval_diag(const deer_gru_params *params, const float *x, const floa
  * leaves while chunk c is evaluated; each chunk's result is exactly what
  * deer_gru_eval returns for those sequences alone, `iters` and `err` are the
  * largest over the chunks, the status is the worst.  A batch of one chunk runs
- * copy, bodies and copy on `stream`, the result copy enqueued behind the first
- * group of bodies.
+ * copy, bodies and copy on `stream`.  A result is copied once its loop has
+ * ended (results of up to 2 MB behind every group of bodies, without asking).
  *   x_host [B,T,m] host in     y_host [B,T,n] host out
  *   x_dev  [B,T,m], y_dev [B,T,n] : device staging buffers owned by the caller
  *            (y_dev holds the guess on entry if DEER_FLAG_WARM_START, and the

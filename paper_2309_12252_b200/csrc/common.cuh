@@ -76,7 +76,7 @@ static inline cudaError_t launch_pdl(bool overlap, void (*kern)(KArgs...), unsig
     } while (0)
 
 // What an evaluation reports, written by the kernel that takes the loop decision straight into page-locked host memory: `done`
-// last, and behind a fence where the host acts on it before it has synchronised.
+// last, and behind a fence where the host may act on it before it has synchronised (`polled`).
 struct __align__(16) HostResult {
     int done, burn;      // (one 64-bit store where nothing else is reported)
     int iters;
@@ -177,10 +177,16 @@ __device__ __forceinline__ bool loop_ended(const StatusBlock *st)
 // End of one Newton body (App. B.1 loop): record err, count the body, decide whether the loop goes on
 // (err > tol and fewer than max_iter bodies).  A NaN err fails "err > tol" and ends the loop, as in
 // the listing; an infinite err ends it too.  Single thread.
-__device__ __forceinline__ void post_done(HostResult *h, int done, bool fence)
+// fence: the host may act on `done` before it has synchronised.  Else the four words leave as one store.
+__device__ __forceinline__ void post_done(HostResult *h, int done)
 {
-    if (fence) __threadfence_system();
+    __threadfence_system();
     *(volatile int *)&h->done = done;
+}
+__device__ __forceinline__ void post_result(HostResult *h, int done, int burn, int iters, unsigned err_bits, bool fence)
+{
+    *reinterpret_cast<int4 *>(h) = make_int4(fence ? 0 : done, burn, iters, (int)err_bits);
+    if (fence) post_done(h, done);
 }
 
 __device__ __forceinline__ bool newton_loop_ends(float e, float tol, int k, int max_iter)
@@ -188,7 +194,7 @@ __device__ __forceinline__ bool newton_loop_ends(float e, float tol, int k, int 
     return !(e > tol) || !(e <= 3.402823466e38f) || k + 1 >= max_iter;
 }
 
-__device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int max_iter, float *trace)
+__device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int max_iter, float *trace, bool polled = false)
 {
     const unsigned bits = *(volatile unsigned *)&st->err_bits;
     const float e = __uint_as_float(bits);
@@ -201,8 +207,7 @@ __device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int ma
     if (end) st->done = 1;
     if (HostResult *h = st->host) {
         if (k < HOST_TRACE) h->trace[k] = e;
-        h->iters = k + 1; h->err_bits = bits; h->burn = st->burn;
-        post_done(h, end, false);
+        post_result(h, end, st->burn, k + 1, bits, polled && end);
     }
 }
 

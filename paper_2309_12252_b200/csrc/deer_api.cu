@@ -6,6 +6,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <chrono>
 #include <map>
 #include <mutex>
 #include <string>
@@ -1061,16 +1062,16 @@ public:
 };
 
 // Reads the record until the loop or the form has ended there, which is before the launches enqueued behind it have drained,
-// and returns how; 0 after `polls` reads (some 15 ns each), or where the stream has come to its end.
-static int record_posted(const HostResult *hr, cudaStream_t st, unsigned polls)
+// and returns how; 0 after `us` microseconds, or where the stream has come to its end.
+static int record_posted(const HostResult *hr, cudaStream_t st, int us)
 {
     const volatile int *done = &hr->done;
-    for (unsigned k = 1; k <= polls; ++k) {
+    const auto from = std::chrono::steady_clock::now();
+    for (unsigned k = 1;; ++k) {
         if (const int how = *done) return how;
-        __builtin_ia32_pause();
-        if (k % 1024 == 0 && cudaStreamQuery(st) != cudaErrorNotReady) return *done;         // (an error is sticky: the caller's synchronisation reports it)
+        if (k % 16 == 0 && std::chrono::steady_clock::now() - from > std::chrono::microseconds(us)) return 0;
+        if (k % 4096 == 0 && cudaStreamQuery(st) != cudaErrorNotReady) return *done;         // (an error is sticky: the caller's synchronisation reports it)
     }
-    return 0;
 }
 
 // ---- evaluations whose bodies are one launch each (newton_body.cuh)
@@ -1081,17 +1082,17 @@ static bool body_takes(int n, int m, int flags)
            (body_supported(n, m, false) || body_supported(n, m, true));
 }
 
-// Reads of the record before the host waits for the stream.  The bias check answers some 10 us after its launch, without a
-// body; a longer look costs more at the end of an evaluation (a synchronisation that is entered late, 0.7 us) than a form that
-// gives up later gains.
-constexpr unsigned POLLS_BIAS = 1500;
+// How long the record is read before the host waits for the stream, in microseconds.  The bias check answers some 10 us after
+// its launch, without a body; a longer look costs more at the end of an evaluation (a synchronisation that is entered late,
+// 0.7 us) than a form that gives up later gains.
+constexpr int BIAS_US = 20, RESULT_US = 20000;
 
 // Runs the Newton loop until it ends or the form gives up (hs->done == BODY_FALL_BACK, the iterate after hs->iters bodies in
 // buf[hs->iters & 1]).
 template <typename CopyOut>
 static int eval_one_launch(const deer_gru_params *p, const float *x, const float *y0, int B, int T, float tol, int max_iter,
                            const EvalWs &w, float *const (&buf)[2], int flags, cudaStream_t st, StatusBlock *hs, HostResult *hr,
-                           bool &u_done, CopyOut copy_out)
+                           bool &u_done, bool to_host, bool &polled, CopyOut copy_out)
 {
     const int n = p->n, m = p->m;
     const bool need_u = !body_supported(n, m, false);
@@ -1103,6 +1104,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     a.B = B; a.T = T; a.n = n; a.m = m; a.H = 1;
     a.eta = body_eta(n, tol);
     a.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0;
+    a.polled = to_host;
     a.st = w.st; a.edge = w.edge; a.edge_flag = w.edge_flag; a.words = w.words;
     a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
     const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
@@ -1155,11 +1157,12 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
                 if (hr && *(volatile int *)&hr->done) break;             // (the bias alone has told, or the loop is over already)
                 if ((rc = launch_newton_body(a, plan, st)) != DEER_OK) return rc;
             }
-            if ((rc = copy_out()) != DEER_OK) return rc;
+            if ((rc = copy_out(false)) != DEER_OK) return rc;
             if (hr) {
-                // The next form goes ahead as soon as the record tells that this one has given up.
-                const int end = record_posted(hr, st, POLLS_BIAS);
-                if (end != BODY_FALL_BACK) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+                // A result for the host starts on its way, and the next form goes ahead, as soon as the record tells.
+                const int end = record_posted(hr, st, to_host ? RESULT_US : BIAS_US);
+                polled = to_host && end == BODY_DONE;
+                if (end != BODY_FALL_BACK && !polled) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
                 hs->iters = hr->iters; hs->done = hr->done; hs->burn = hr->burn; hs->err_last_bits = hr->err_bits;
                 if (hs->done == BODY_TIMED_OUT || (plan.whole_loop && !hs->done)) return DEER_ERR_DEVICE_TIMEOUT;
             } else {
@@ -1169,11 +1172,17 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
             }
             if (hs->done) break;
         }
-        if (hs->done == BODY_DONE) return DEER_OK;
+        if (hs->done == BODY_DONE) return copy_out(true);
         burn = hs->burn;
     }
     return DEER_OK;                                      // (hs->done == BODY_FALL_BACK)
 }
+
+// Results up to this size are copied to host memory before it is known that they are final: the copy is then enqueued while the
+// bodies run, and one that proves to be in vain takes 40 us of the link at most.  (n = 8, m = 4, B = 4, us per call, early /
+// not: T = 2,000 96 / 97, T = 16,000 (2 MB) 162 / 166, T = 32,000 241 / 240.  What early copies of large results cost: n = m =
+// 32, B = 16, T = 1e5, a cell that remembers for up to 1,000 steps 24.3 / 18.2 ms, random walks 16.4 / 10.9 ms.)
+constexpr size_t HOST_COPY_EARLY = 2 << 20;
 
 static int eval_status(float e, float tol)
 {
@@ -1182,9 +1191,9 @@ static int eval_status(float e, float tol)
 }
 
 // copy_st / copy_ev (optional): the stream the copy to y_host is enqueued on, and an event to order it behind `st`.
-// y_host (optional, host memory): the result is also copied there.  The copy is enqueued behind every
-// group of bodies, after a device-side selection of the buffer that holds the current iterate, so that
-// an evaluation that converges within its first group costs one host synchronisation in all.
+// y_host (optional, host memory): the result is also copied there, after a device-side selection of the buffer that holds the
+// current iterate, once the loop has ended.  A small result is copied behind every group of bodies, whether or not it is the
+// last: an evaluation that converges within its first group then costs one host synchronisation in all.
 static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *y0, int B, int T,
                          float tol, int max_iter, float *y, int *iters, float *err,
                          float *err_trace, void *ws, size_t ws_bytes, int flags, cudaStream_t st,
@@ -1199,9 +1208,17 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     float *buf[2] = {y, w.yalt};
     StatusBlock hs;
     memset(&hs, 0, sizeof(hs));
-    // enqueued behind every group of bodies when the result goes to host memory
-    auto copy_out = [&]() -> int {
-        if (!y_host) return DEER_OK;
+    // ended: the loop has
+    const bool copy_early = N * n * sizeof(float) <= HOST_COPY_EARLY;
+    bool polled = false;                       // the end of the loop was read from the record
+    auto copy_out = [&](bool ended) -> int {
+        if (!y_host || ended == copy_early) return DEER_OK;
+        if (ended && copy_st && polled && hs.done == BODY_DONE && (hs.iters & 1) == 0) {
+            // the record has told that the result is complete, and it is where it belongs: nothing to wait for (three calls less
+            // between the last body and the copy: n = m = 32, B = 16, T = 1e5 6773 -> 6742 us)
+            DEER_CHECK_CUDA(cudaMemcpyAsync(y_host, y, N * n * sizeof(float), cudaMemcpyDeviceToHost, copy_st), "copy result to host");
+            return DEER_OK;
+        }
         size_t words = N * n / 4;
         unsigned blocks = (unsigned)((words + 1023) / 1024);
         const unsigned cap = 4u * (unsigned)num_sms();
@@ -1225,7 +1242,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     bool u_done = false;                       // w.u holds the projected inputs
     bool ended_there = false;                  // the one-launch form ran to the end
     if (one_launch) {
-        if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, u_done, copy_out)) != DEER_OK) return rc;
+        if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, u_done, y_host && !copy_early, polled, copy_out)) != DEER_OK) return rc;
         ended_there = hs.done == BODY_DONE;
         if (burn_in) *burn_in = ended_there ? hs.burn : -hs.burn;      // of the last body; negative: it gave up, what it would have needed
     }
@@ -1300,13 +1317,14 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
                 DEER_KERNEL("newton_control_kernel", st, newton_control_kernel<<<1, 1, 0, st>>>(w.st, tol, max_iter, w.trace));
             }
         }
-        if ((rc = copy_out()) != DEER_OK) return rc;
+        if ((rc = copy_out(false)) != DEER_OK) return rc;
         DEER_CHECK_CUDA(cudaMemcpyAsync(&hs, w.st, 32, cudaMemcpyDeviceToHost, st), "read status");
         DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
         if (hs.flags & FLAG_TIMEOUT) return DEER_ERR_DEVICE_TIMEOUT;
         if (hs.done || enq >= max_iter) break;
         group = 2;
     }
+    if ((rc = copy_out(true)) != DEER_OK) return rc;
     }
     const int k = hs.iters;
     float e;
@@ -1337,7 +1355,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     if (err_trace && k > 0 && !trace_here)
         DEER_CHECK_CUDA(cudaMemcpyAsync(err_trace, w.trace, sizeof(float) * (size_t)(k < ERR_TRACE_CAP ? k : ERR_TRACE_CAP),
                                         cudaMemcpyDeviceToHost, st), "read trace");
-    if (((k & 1) && !y_host) || (err_trace && !trace_here)) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+    if (((k & 1) && !y_host) || (y_host && !copy_early && !copy_st) || (err_trace && !trace_here)) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
     if (iters) *iters = k;
     if (err) *err = e;
     return eval_status(e, tol);
@@ -1722,7 +1740,7 @@ int deer_gru_eval_host(const deer_gru_params *p, const float *x_host, const floa
     }
     DEER_CHECK_CUDA(cudaEventRecord(hp->ev_out, hp->d2h), "record exit event");
     DEER_CHECK_CUDA(cudaStreamWaitEvent(st, hp->ev_out, 0), "wait exit event");
-    DEER_CHECK_CUDA(cudaStreamSynchronize(hp->d2h), "sync");
+    DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
     if (iters) *iters = k_max;
     if (err) *err = e_max;
     return status;

@@ -62,18 +62,18 @@ __device__ __forceinline__ BodyVerdict body_verdict(float e, float mis, float et
 }
 
 // End of a body that is a launch of its own: the last CTA's decision.  Single thread.
-__device__ __forceinline__ void body_decide(StatusBlock *st, float eta, int burn_cap, int T)
+__device__ __forceinline__ void body_decide(StatusBlock *st, float eta, int burn_cap, int T, bool polled)
 {
     const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits);
     const float mis = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
     const BodyVerdict v = body_verdict(e, mis, eta, st->burn, burn_cap, T, st->tol, st->iters, st->max_iter);
     st->mis_bits = 0u;
     st->burn = v.burn;
-    if (v.counts) newton_decide(st, st->tol, st->max_iter, st->trace);
+    if (v.counts) newton_decide(st, st->tol, st->max_iter, st->trace, polled);
     if (v.counts && (st->done || !v.done)) return;
     st->err_bits = 0u;
     st->done = v.done;
-    if (HostResult *h = st->host) { h->burn = v.burn; post_done(h, v.done, v.done != 0); }
+    if (HostResult *h = st->host) { h->burn = v.burn; if (v.done) post_done(h, v.done); }
 }
 
 template <int N> struct Body {
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap, a.T);
+            body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
         }
     }
 }

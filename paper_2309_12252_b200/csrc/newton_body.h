@@ -25,6 +25,7 @@ struct BodyArgs {
     float eta;               // largest boundary mismatch, as a part of max(err, tol), that is accepted
     int burn_cap;            // longest burn-in that is tried (BodyPlan)
     int expire;              // test aid: every bounded wait runs out (DEER_FLAG_EXPIRE_BODY_WAITS)
+    int polled;              // the host reads the result record while the stream runs
     StatusBlock *st;         // [H]
     float *edge;             // [groups][2][n]  states either side of a boundary between two warps
     unsigned *edge_flag;     // [groups]        arrivals at it (left cleared)

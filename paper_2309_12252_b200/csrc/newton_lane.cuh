@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(128) newton_lane_kernel(BodyArgs a)
         if (prevc + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap, a.T);
+            body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
         }
     }
 }

@@ -540,10 +540,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
                 st->iters = iters + (v.counts ? 1 : 0);
                 st->burn = v.burn;
                 st->done = v.done;
-                if (HostResult *h = st->host) {
-                    h->iters = st->iters; h->err_bits = st->err_last_bits; h->burn = v.burn;
-                    post_done(h, v.done, v.done != BODY_DONE);
-                }
+                if (HostResult *h = st->host) post_result(h, v.done, v.burn, st->iters, st->err_last_bits, a.polled || v.done != BODY_DONE);
             }
         }
         if (v.done) return;
@@ -582,7 +579,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap, a.T);
+            body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
         }
     }
     return;

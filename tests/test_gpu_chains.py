@@ -296,3 +296,26 @@ def test_expired_wait_in_the_multihead_loop_is_reported(bd):
     with pytest.raises(bd.DeerError):
         bd.deer_gru_multihead_eval(heads, [1, 2, 4], x, y0, flags=bd.DEER_FLAG_EXPIRE_BODY_WAITS)
     assert bd.deer_gru_multihead_eval(heads, [1, 2, 4], x, y0)[2] == 0
+
+
+@pytest.mark.parametrize("n,m,B,T,bias", [(16, 8, 4, 30000, 6.0), (8, 4, 16, 60000, 6.0), (8, 4, 16, 60000, 0.0), (32, 8, 16, 40000, 0.0)])
+def test_host_call_copies_finished_results_only(bd, n, m, B, T, bias):
+    """The selection of the current iterate goes before a copy of a result to host memory: one per chunk of the call at most,
+    whatever forms give up and however many groups of bodies the loop takes."""
+    p = synth.gru_params(n, m, seed=14, tag="c/gru")
+    p.b_i[n:2 * n] += np.float32(bias)
+    x = walk(synth.x_gaussian(B, T, m, seed=14, tag="c/x"))
+    pd, y0, xd, yd = bd.GruParamsDev.from_numpy(p), torch.zeros((B, n), device="cuda"), torch.empty((B, T, m), device="cuda"), torch.empty((B, T, n), device="cuda")
+    xh, yh = torch.from_numpy(x).pin_memory(), torch.empty((B, T, n), pin_memory=True)
+    ws = bd.alloc_workspace(bd.DEER_OP_EVAL, B, T, n, m)
+    from bench import read_profile
+    bd.lib().deer_profile_enable(1)
+    try:
+        bd.deer_gru_eval_host(pd, xh, y0, yh, xd, yd, ws)
+    finally:
+        bd.lib().deer_profile_enable(0)
+    first = bd.deer_gru_eval_host_chunks(B, T)
+    assert read_profile(bd).get("result_select_kernel", {"launches": 0})["launches"] <= len(first) - 1
+    for lo, hi in zip(first[:-1], first[1:]):          # (bit for bit, also where the iteration of a cell that remembers diverges)
+        alone = bd.deer_gru_eval(pd, dev(x[lo:hi]), y0[lo:hi].contiguous())
+        assert np.array_equal(yh.numpy()[lo:hi], alone.y.cpu().numpy(), equal_nan=True)
