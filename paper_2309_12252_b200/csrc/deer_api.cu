@@ -2110,13 +2110,14 @@ static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int
     }
 }
 
+// did[h]: the gradients of head h, and its part of dx and dy0, are there (empty: of none).
 static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int H, const float *x, const float *y0, const float *y,
                           const float *gy, int B, int T, const deer_gru_grads *dheads, float *dx, float *dy0, const MhWs &w,
-                          cudaStream_t st, bool *did)
+                          cudaStream_t st, std::vector<char> &did)
 {
     const int n = heads[0].n, m = heads[0].m, n3 = 3 * n;
     const size_t N = (size_t)B * T;
-    *did = false;
+    did.clear();
     int rc;
     BodyPlan plan{};
     if (!adjoint_plan(&plan, B, T, n, m, true, strides, H)) return DEER_OK;
@@ -2142,6 +2143,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     a.burn_cap = 512;                                    // (what comes behind goes head by head)
     for (int k = 0; k < ADJ_TRIES; ++k)
         if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
+    DEER_KERNEL("mh_drop_kernel", st, mh_drop_kernel<<<num_sms(), 256, 0, st>>>(w.st, w.dGi, w.dGh, N, H, n3));
     // dW_i, db_i of all heads: one contraction of dG_i [N, H*3n] with x [N, m]
     WgradArgs wa{};
     wa.dG = w.dGi; wa.V = x; wa.T = T; wa.n3 = H * n3; wa.K = m; wa.N = N;
@@ -2174,8 +2176,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     std::vector<StatusBlock> hs((size_t)H);
     DEER_CHECK_CUDA(cudaMemcpyAsync(hs.data(), w.st, sizeof(StatusBlock) * (size_t)H, cudaMemcpyDeviceToHost, st), "read status");
     DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
-    *did = true;
-    for (const StatusBlock &h : hs) *did = *did && h.done == BODY_DONE;    // (a head whose Jacobians hardly decay: head by head)
+    for (const StatusBlock &h : hs) did.push_back(h.done == BODY_DONE);    // (a head whose Jacobians hardly decay goes by itself)
     return DEER_OK;
 }
 
@@ -2250,17 +2251,17 @@ int deer_gru_multihead_vjp(const deer_gru_params *heads, const int *strides, int
     cudaStream_t st = (cudaStream_t)stream;
     MhWs w = carve_mh(ws, H, strides, B, T, n, m);
     if ((rc = check_ws(ws, ws_bytes, w.bytes)) != DEER_OK) return rc;
-    if (mh_batched(n, H, flags)) {
-        bool did = false;
-        if ((rc = mh_vjp_batched(heads, strides, H, x, y0, y, gy, B, T, dheads, dx, dy0, w, st, &did)) != DEER_OK) return rc;
-        if (did) return DEER_OK;
-    }
+    std::vector<char> did;
+    if (mh_batched(n, H, flags) &&
+        (rc = mh_vjp_batched(heads, strides, H, x, y0, y, gy, B, T, dheads, dx, dy0, w, st, did)) != DEER_OK) return rc;
+    const bool batched = !did.empty();
     unsigned timeout_flags = 0;
     int packed_stride = 1;                     // (stride 1: x itself)
     const std::vector<int> order = mh_order(strides, H);
     for (int oi = 0; oi < H; ++oi) {
         const int h = order[(size_t)oi];
         const int s = strides[h], Tp = (T + s - 1) / s, Bs = B * s;
+        if (batched && did[(size_t)h]) continue;
         if (s != packed_stride) {
             { if ((rc = mh_pack(x, w.xs, B, T, s, Tp, m, m, 0, st)) != DEER_OK) return rc; }
             packed_stride = s;
@@ -2272,8 +2273,8 @@ int deer_gru_multihead_vjp(const deer_gru_params *heads, const int *strides, int
         rc = gru_vjp_impl(&heads[h], xs, w.y0s, w.ys, w.gys, Bs, Tp, &dheads[h], dx ? w.dxs : nullptr, dy0 ? w.dy0s : nullptr,
                           w.inner, w.inner_bytes, flags, st);
         if (rc != DEER_OK) return rc;
-        if (dx)     // the heads' input gradients add up, head by head in a fixed order (that of the strides)
-            { if ((rc = mh_unpack(w.dxs, dx, B, T, s, Tp, m, m, 0, oi > 0, st)) != DEER_OK) return rc; }
+        if (dx)     // the heads' input gradients add up, head by head in a fixed order (that of the strides; behind those of a batch)
+            { if ((rc = mh_unpack(w.dxs, dx, B, T, s, Tp, m, m, 0, batched || oi > 0, st)) != DEER_OK) return rc; }
         if (dy0)
             DEER_KERNEL("mh_dy0_reduce_kernel", st, mh_dy0_reduce_kernel<<<mh_blocks((size_t)B * n), 256, 0, st>>>(w.dy0s, dy0, B, s, n, H, h));
         // the inner gradient calls share one status block: keep every head's flags

@@ -39,6 +39,22 @@ __global__ void mh_select_kernel(const StatusBlock *__restrict__ st, float *__re
     }
 }
 
+// Pre-activation gradients of the heads whose adjoint launch gave up: zero, so that the contractions over all heads (dx among
+// them) are those of the others.  Where none did, one look at the status words (2 us).
+__global__ void mh_drop_kernel(const StatusBlock *__restrict__ st, float *__restrict__ dGi, float *__restrict__ dGh, size_t N, int H, int n3)
+{
+    bool any = false;
+    for (int h = threadIdx.x; h < H; h += blockDim.x) any = any || st[h].done != BODY_DONE;
+    if (!__syncthreads_or(any)) return;
+    for (int h = 0; h < H; ++h) {
+        if (st[h].done == BODY_DONE) continue;
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N * n3; i += (size_t)gridDim.x * blockDim.x) {
+            const size_t o = (i / n3 * H + h) * n3 + i % n3;
+            dGi[o] = 0.0f; dGh[o] = 0.0f;
+        }
+    }
+}
+
 // dy0[b, h, i] = sum over the phases p, in order, of dy0s[first_seq[h] + b s + p, i]
 __global__ void mh_dy0_sum_kernel(const BodyHead *__restrict__ heads, const float *__restrict__ dy0s, float *__restrict__ dy0, int B, int T, int n, int H)
 {

@@ -97,3 +97,29 @@ def test_multihead_warm_start_and_argument_checks(bd):
     small = torch.empty(1024, dtype=torch.uint8, device="cuda")
     with pytest.raises(bd.DeerError):
         bd.deer_gru_multihead_eval(hd, st, dev(x), dev(y0), ws=small)
+
+
+@pytest.mark.parametrize("H,n,m,B,T,strides,stubborn", [(4, 8, 16, 3, 3001, [1, 2, 1, 4], [0]), (5, 8, 7, 2, 4000, [2, 1, 4, 1, 2], [1, 3]), (2, 16, 16, 2, 3000, [1, 2], [0, 1])])
+def test_multihead_vjp_redoes_only_the_heads_that_remember(bd, H, n, m, B, T, strides, stubborn):
+    """A head whose Jacobians hardly decay is given up by the launch over all heads; the others' gradients are kept, and dx is the
+    sum of both kinds."""
+    from bench import read_profile
+    heads, st, x, y0 = case(H, n, m, B, T, strides, seed=H + T)
+    for h in stubborn:
+        heads[h].b_i[n:2 * n] += 6.0
+    y32 = oracle.multihead_seq(heads, st, x, y0, np.float32)
+    gy = synth.normal(H + T, "g/mhgy", y32.shape)
+    want = oracle.multihead_bptt(heads, st, x, y0, y32.astype(np.float64), gy, np.float64)
+    args = [bd.GruParamsDev.from_numpy(h) for h in heads], st, dev(x), dev(y0), dev(y32), dev(gy)
+    bd.lib().deer_profile_enable(1)
+    try:
+        g = bd.deer_gru_multihead_vjp(*args)
+    finally:
+        bd.lib().deer_profile_enable(0)
+    assert read_profile(bd)["mh_y0_pack_kernel"]["launches"] == len(stubborn)      # (one per head that goes by itself)
+    for k in ("dW_i", "dW_h", "db_i", "db_h"):
+        for h in range(H):
+            assert rel_inf(g[k][h].cpu().numpy().astype(np.float64), want[k][h]) <= TOL_GRAD, (k, h)
+    assert rel_inf(g["dx"].cpu().numpy().astype(np.float64), want["dx"]) <= TOL_GRAD
+    for h in range(H):
+        assert rel_inf(g["dy0"][:, h].cpu().numpy().astype(np.float64), want["dy0"][:, h]) <= TOL_GRAD, h
