@@ -1112,7 +1112,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE}) {
         BodyPlan plan{};
         if (form == BodyForm::TILE && !aligned32) continue;
-        if (form == BodyForm::ONE_PHASE && (tiles || n <= 8)) break; // (what the tiles give up is for the kernels that multiply the Jacobians out)
+        if (form == BodyForm::ONE_PHASE && tiles) break;             // (what the tiles give up is for the kernels that multiply the Jacobians out)
         const bool have_u = form == BodyForm::LANE ? m > 8 : need_u && form != BodyForm::TILE;
         if (!body_plan(&plan, form, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;
         a.u = have_u ? w.u : nullptr;

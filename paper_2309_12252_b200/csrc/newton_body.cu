@@ -216,6 +216,7 @@ bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have
         p->smem = fixed + k.slot_bytes * (size_t)(p->burn_cap + p->NC * p->L);
         return true;
     }
+    if (n <= 8) return false;
     one_wave_of_chains(p, (const void *)k.one, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.one_smem(kx), body_first_burn(n, 1.0f), B, T, strides, H);
     p->burn_cap = worth_trying(*p, n, m, B);
     return true;

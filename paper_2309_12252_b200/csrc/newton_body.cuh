@@ -86,8 +86,8 @@ template <int N> struct Body {
     }
 };
 
-// EXACT: the products with d are 3 x TF32 as well (n <= 8 and sizes whose solve has always been fp32-accurate); V2: rows
-// are read and written as 8-byte pairs.
+// EXACT: the products with d are 3 x TF32 as well (sizes whose solve has always been fp32-accurate); V2: rows are read and
+// written as 8-byte pairs.  n <= 8 takes a thread per chain instead (newton_lane.cuh).
 template <int N, bool V2, bool EXACT>
 __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_body_kernel(BodyArgs a)
 {

@@ -60,7 +60,7 @@ constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3;
 
 // The kernels of one padded state size (newton_kernels.cu).
 struct BodyKernels {
-    void (*one)(BodyArgs);                     // one-phase (newton_body.cuh)
+    void (*one)(BodyArgs);                     // one-phase (newton_body.cuh); n > 8 only
     void (*seg)(BodyArgs, int, int);           // two-phase (newton_segment.cuh)
     void (*adj)(AdjArgs);                      // adjoint, one-phase (newton_adjoint.cuh)
     void (*(*tile)(int m))(BodyArgs);          // 128 chains per tcgen05 tile (newton_tile.cuh); n = 32, 64 only

@@ -18,7 +18,7 @@ namespace deer {
 template <int N> static BodyKernels kernels_of(bool v2, bool exact)
 {
     BodyKernels k{};
-    k.one = v2 ? newton_body_kernel<N, true, true> : newton_body_kernel<N, false, true>;
+    if constexpr (N > 8) k.one = v2 ? newton_body_kernel<N, true, true> : newton_body_kernel<N, false, true>;
     k.seg = v2 ? newton_segment_kernel<N, true, true> : newton_segment_kernel<N, false, true>;
     if constexpr (N == 16 || N == 32 || N == 64) {
         // single-TF32 products with the update: the sizes whose solve has always run in reduced precision
