@@ -319,3 +319,89 @@ def test_host_call_copies_finished_results_only(bd, n, m, B, T, bias):
     for lo, hi in zip(first[:-1], first[1:]):          # (bit for bit, also where the iteration of a cell that remembers diverges)
         alone = bd.deer_gru_eval(pd, dev(x[lo:hi]), y0[lo:hi].contiguous())
         assert np.array_equal(yh.numpy()[lo:hi], alone.y.cpu().numpy(), equal_nan=True)
+
+
+# ---- the launches are not only made but taken: the kernels behind them do nothing, and the accuracy is the launches' own
+@pytest.mark.parametrize("n,m,B,T,kernel", [
+    (1, 1, 1, 400, SEG), (3, 70, 2, 129, SEG), (12, 5, 3, 401, SEG), (32, 64, 2, 97, SEG), (40, 7, 2, 51, SEG), (24, 10, 16, 6001, SEG),
+    (16, 5, 16, 15001, ONE), (50, 1, 4, 663, ONE), (43, 64, 5, 2003, ONE),
+    (32, 33, 16, 6001, TILE), (32, 3, 3, 40001, TILE), (32, 64, 17, 16001, TILE), (64, 1, 1, 16001, TILE), (64, 64, 7, 2801, TILE),
+    (1, 1, 16, 300001, LANE), (3, 2, 5, 50001, LANE), (4, 3, 16, 50003, LANE), (5, 9, 16, 20001, LANE), (8, 8, 16, 30001, LANE)])
+def test_bodies_are_taken(bd, n, m, B, T, kernel):
+    p = synth.gru_params(n, m, seed=15, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=15, tag="c/x")
+    y0 = synth.normal(15, "c/y0", (B, n)) * 0.5
+    pd, xd, yd = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(pd, xd, yd))
+    assert {k for k in names if k.startswith("newton_")} == {kernel}, names
+    assert not any(k.startswith(("cell_", "scan_", "gen_")) for k in names), names
+    assert r.status == 0 and r.err <= 1e-4
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-5     # (quadratic: far below the last update)
+
+
+@pytest.mark.parametrize("n,m,B,T,x_kind,kernel", [
+    (3, 7, 2, 5001, "noise", WARP), (12, 5, 8, 3001, "noise", WARP), (9, 60, 4, 15001, "noise", WARP), (16, 8, 16, 20001, "noise", WARP),
+    (32, 32, 16, 10001, "noise", WARP), (40, 7, 2, 9001, "noise", WARP), (56, 1, 3, 9001, "noise", WARP),
+    (64, 6, 3, 20001, "noise", MMA_TILE), (64, 64, 16, 4003, "noise", MMA_TILE),
+    (1, 8, 5, 20003, "noise", ROWS), (8, 1, 1, 45, "noise", ROWS), (2, 4, 64, 67, "noise", ROWS), (8, 8, 16, 30001, "noise", ROWS)])
+def test_adjoints_are_taken(bd, n, m, B, T, x_kind, kernel):
+    """Boundaries within 4e-6 of max|lambda| and products of fp32 level: 2e-5 of the largest entry of dx and dy0, and of sums over
+    all positions."""
+    p = synth.gru_params(n, m, 16, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 16, tag="c/x")
+    y0 = synth.normal(16, "c/y0", (B, n)) * 0.3
+    gy = synth.normal(16, "c/gy", (B, T, n))
+    got, want, names, done = gradient(bd, p, x, y0, gy)
+    assert kernel in names and done == 1, names
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        assert np.max(np.abs(got[k] - want[k])) <= 2e-5 * np.max(np.abs(want[k])), k
+
+
+@pytest.mark.parametrize("n,B,T", [(4, 2, 65537), (8, 3, 60001), (16, 1, 9001), (32, 2, 1111), (32, 16, 1300), (64, 1, 515), (64, 5, 193)])
+@pytest.mark.parametrize("reverse", [False, True])
+@pytest.mark.parametrize("decays", [True, False])
+def test_scans_are_taken_where_products_decay(bd, n, B, T, reverse, decays):
+    J = synth.contractive_J(B, T, n, seed=n + T, tag="c/J", scale=1.0)
+    if not decays:
+        J = 0.05 * J + 0.95 * np.eye(n, dtype=np.float32) * np.float32(1.04)
+    ws = bd.alloc_workspace(bd.DEER_OP_SCAN, B, T, n)
+    bd.deer_linrec_scan(dev(J), dev(synth.normal(n + T, "c/b", (B, T, n))), dev(synth.normal(n + T, "c/y0", (B, n))), reverse=reverse, ws=ws)
+    assert accepted(ws) == int(decays)
+
+
+@pytest.mark.parametrize("n,m,B,T", [(32, 32, 16, 6001), (64, 6, 3, 9001)])
+@pytest.mark.parametrize("t", [0, 3000, 5999])
+def test_evaluation_tile_beyond_the_range_of_its_operands(bd, n, m, B, T, t):
+    """An input that f16 halves cannot hold: the tiles give up and the kernels behind do the work."""
+    p = synth.gru_params(n, m, 17, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 17, tag="c/x")
+    x[1, t] *= np.float32(2e4)
+    y0 = synth.normal(17, "c/y0", (B, n)) * 0.5
+    r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)))
+    assert TILE in names and any(k.startswith("cell_") for k in names), names
+    assert r.status == 0
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-4
+
+
+@pytest.mark.parametrize("n,m,B,T", [(32, 32, 16, 6001), (64, 6, 3, 9001)])
+@pytest.mark.parametrize("scale", [1.0, 1e-2, 1e-4])
+def test_evaluation_tile_on_small_inputs(bd, n, m, B, T, scale):
+    """Operands are good to 2^-23 of themselves and, below 2^-6, to 2^-29 absolute.  Without biases the states are as small as the
+    inputs: m + n such errors, weighted by up to 1 / sqrt(n), the 2e-7 absolute of the gates' tanh (half of it with z about 1/2),
+    both summed over some four steps of memory, beside fp32 rounding.  The tanh leads, as it does in the kernels that multiply
+    the Jacobians out: the tile is no further off than they are, but for its operands."""
+    p = synth.gru_params(n, m, 18, tag="c/gru")
+    p.b_i[:] = 0.0
+    p.b_h[:] = 0.0
+    x = synth.x_gaussian(B, T, m, 18, tag="c/x") * np.float32(scale)
+    y0 = np.zeros((B, n), np.float32)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(*args, tol=-1.0, max_iter=6))
+    assert TILE in names, names
+    want = oracle.gru_seq(p, x, y0, np.float64)
+    operands, rounding = 4.0 * (m + n) * 2.0 ** -29 / np.sqrt(n), 4e-6 * np.max(np.abs(want))
+    off = np.max(np.abs(r.y.cpu().numpy() - want))
+    assert off <= operands + 4.0 * 1e-7 + rounding
+    other, names = launched(bd, lambda: bd.deer_gru_eval(*args, tol=-1.0, max_iter=6, flags=bd.DEER_FLAG_MATERIALIZE))
+    assert TILE not in names, names
+    assert off <= operands + 1.5 * np.max(np.abs(other.y.cpu().numpy() - want)) + rounding / 4.0
