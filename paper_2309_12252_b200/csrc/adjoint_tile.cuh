@@ -11,7 +11,8 @@
 // row and step, from the row's largest |lambda|.
 // The pre-activation gradients leave as [position][4n] = (r, z, n hidden, n input): the two that dW_h and dW_i share once.
 //
-// What bounds it: issue slots and the special-function unit in epilogue 1, then the 256-bit stores (a row per lane).
+// What bounds it: latency, as in newton_tile.cuh.  m = 64, 80,000 positions: issue slots 36 % used, special functions 17 %, tensor
+// 22 %, DRAM 4 %; per instruction issued 2.8 warps wait for a load (tensor memory, global), 2.6 at one of a step's three barriers.
 #pragma once
 #include "newton_adjoint.cuh"
 #include "newton_tile.cuh"

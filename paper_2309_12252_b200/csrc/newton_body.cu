@@ -312,7 +312,21 @@ int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 //   n = 64, B = 16, T = 1e3:    - / 2369 / 1247    n = 64, B = 16, T = 1e4:   - / 2828 / 3345
 // Two-phase: one wave (then the whole loop is one launch), two waves from n = 9 on.  One-phase: from half a wave of chains on --
 // below, its steps, a whole cell each, are a serial chain that nothing fills (n <= 8 never comes here: a thread per chain).
-// Sizes without tuned kernels of the other kind always come here.
+// Sizes without tuned kernels of the other kind always come here, to the two-phase kernel up to eight waves: there random walks,
+// whose bodies the long chains of the other run again, break even; white noise does so earlier (B = 16, m = 8, us per evaluation
+// by waves, two-phase / one-phase, white noise then random walks):
+//   n = 12   1.4 312 / 447, 510 / 1200   2.7 446 / 527, 767 / 1507   5.5 836 / 609, 1445 / 1689    10.9 1572 / 792, 2382 / 2194
+//   n = 24   2.2 399 / 657, 617 / 1275   4.5 656 / 799, 1254 / 2095  8.9 1187 / 943, 1828 / 1724   17.8 2426 / 1249, 2946 / 1798
+//   n = 28   4.9 656 / 1068              6.8 883 / 1216              8.6 1126 / 1249, 1603 / 2394
+//   n = 40   3.1 707 / 1171              4.8 888 / 1204              6.6 1223 / 1243               8.5 1562 / 1305
+// A thread per chain, powers of two: by positions per chain of a full GPU (`share`; m = n or 4, B = 16, white noise then random
+// walks, where a try is often lost: thread per chain / multiplied out):
+//   n = 1   13 175 / 208, 128 / 156   30 205 / 235, 141 / 174   42 217 / 302, 162 / 221   84 301 / 541, 226 / 411
+//   n = 2   20 229 / 210, 363 / 306   26 268 / 258, 524 / 477   40 295 / 371, 609 / 537   79 379 / 634, 1025 / 941
+//   n = 4    8 159 / 172, 284 / 231   16 190 / 233, 378 / 318   26 226 / 337, 517 / 450   53 280 / 569, 823 / 737
+//   n = 8    8 339 / 362, 462 / 469   12 365 / 483, 597 / 635   26 439 / 918, 971 / 1172
+// The lines lie where white noise gains more than walks lose (n = 2, 4), and where it begins to gain by a fifth (n = 8); n = 1
+// could start lower.
 bool body_suits(const BodyPlan &p, int n)
 {
     if (p.form == BodyForm::TILE) return true;

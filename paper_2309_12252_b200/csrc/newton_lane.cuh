@@ -5,7 +5,8 @@
 // plain FMAs with the weights as broadcast 16-byte loads.  A warp's 32 chains walk in lockstep through windows of W positions
 // that cp.async has brought into warp-private shared memory (full lines of every chain, one window ahead); the new iterate
 // replaces the old one there and leaves the same way.  Row strides are odd in 16-byte pieces: conflict-free.
-// What bounds it: issue slots and the special-function unit (six of its instructions per state component); n = 1 also HBM.
+// What bounds it: issue slots and latency, with some 14 warps per SM.  n = m = 1, B = 16, T = 3e5: issue slots 54 % used, special
+// functions (six instructions per state component) 32 %, FMA 31 %, DRAM 12 %.
 #pragma once
 #include "newton_body.cuh"
 #include "scan_onepass.cuh"

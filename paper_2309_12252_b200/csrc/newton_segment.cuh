@@ -10,6 +10,8 @@
 //            d <- r + z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d):  9 MMAs of a warp per block of eight columns,
 //            the new d crossing to the other warps of the group through shared memory.
 // A step of phase 2 is some 250 cycles (N = 8: one warp, no exchange).
+// What bounds it: those steps, in series (n = 8, m = 4, B = 16, T = 1e4: issue slots 34 % used; the warps that phase 2 has no
+// chains for wait at the barrier behind it, 5.8 of 16 at a time).
 #pragma once
 #include "newton_body.cuh"
 

@@ -2,18 +2,21 @@
 // see there) with 128 chains in lockstep as the rows of a tcgen05 tile.
 //
 // Per step of a CTA, [128, .] x [., 3n] products by tcgen05.mma.kind::f16 from one thread, accumulators in tensor memory:
-//     x_t W_i^T and y_{t-1} W_h^T   operands as hi + lo f16 halves, three products (good to 2^-23 of the operands: fp32 level)
+//     x_t W_i^T and y_{t-1} W_h^T   operands as hi + lo f16 halves, three products (good to 2^-23 of the operands and, of x and y
+//                                   below 2^-6, to 2^-29 absolute: below the 2e-7 that the gates' tanh is good to)
 //     d_{t-1} W_h^T                 one product (the solve's accuracy is that of its boundaries, see body_verdict)
-// Operands carry powers of two (tile_weight_scale; OP_SCALE, D_SCALE) that keep the halves among the normal f16 numbers and
-// leave in the exponent arithmetic of the epilogue.  A value beyond f16's range turns the body's error into a NaN: the body
+// Operands carry powers of two (tile_weight_scale; OP_SCALE, D_SCALE) that keep the hi halves, and the lo halves of all but small
+// operands, among the normal f16 numbers and leave in the exponent arithmetic of the epilogue.  A value beyond f16's range turns the body's error into a NaN: the body
 // does not count and the evaluation goes on with the other kernels (BODY_FALL_BACK).
 // A row is owned by n/16 threads of one lane, 16 columns each (the warps of a warpgroup see their own 32 tensor-memory lanes):
 // gates, coefficients, the update and the new iterate are elementwise in registers.  Loading is another mapping -- a row's
 // lanes side by side, full lines per request, a step ahead in registers -- and hands the rows over as f16 operands and, in
 // fp32, through `sY`.
 //
-// What bounds it (n = m = 32, B = 16, T = 1e5): the special-function unit, 10 of whose 8-cycle instructions go into a pair of
-// columns, and about as many issue slots; mma.sync spent 2,700 of a warp's 5,400 cycles per 16 rows in the tensor pipe alone.
+// What bounds it: the latency of a step's serial phases with 16 warps per SM (128 registers a thread).  n = m = 32, B = 16,
+// T = 5.6e4: issue slots 49 % used, special functions 29 %, FMA 34 %, ALU 32 %, tensor 15 %, DRAM 27 %; per instruction issued 1.4
+// warps wait for a fixed latency, 1.4 for a load (tensor memory, global), 1.3 at a barrier.  n = 64 (one tile per CTA): issue
+// 38 %, 2.8 at a barrier.  mma.sync spent 2,700 of a warp's 5,400 cycles per 16 rows in the tensor pipe alone.
 #pragma once
 #include "newton_body.cuh"
 #include "tile_umma.cuh"

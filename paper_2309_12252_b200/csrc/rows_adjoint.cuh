@@ -7,7 +7,8 @@
 // p times y_{t-1} and x are its rows of dW_h and dW_i: accumulated in registers over the chain, then over the CTA in a fixed
 // order (slice b of the two-stage reduction; wgrad_final2_kernel adds the slices).  The inputs of the next U positions are
 // requested ahead; no Jacobian, lambda or pre-activation gradient is ever stored.
-// What bounds it: issue slots (about 170 per step and warp, 95 in the burn-in).  Before: a cell that wrote Jacobians, a scan
+// What bounds it: issue slots (about 170 per step and warp, 95 in the burn-in; 55 % used at n = 8, m = 4, B = 16, T = 1e4) and
+// the latency that 11 warps per SM leave.  Before: a cell that wrote Jacobians, a scan
 // that read them, a VJP pass: n = 8, m = 4, B = 16, T = 1e4 92 us, n = m = 8, T = 1e6 6.1 ms.
 #pragma once
 #include <type_traits>

@@ -108,7 +108,8 @@ __device__ __forceinline__ bool tile_wait(uint64_t *bar, unsigned phase)
     return false;
 }
 
-// hi and lo halves of a pair as packed f16: x = hi + lo to 2^-23 of x (values up to 65504)
+// hi and lo halves of a pair as packed f16: x = hi + lo to 2^-23 of x, or 2^-25 where lo is subnormal (|x| below 2^-2; values up
+// to 65504)
 __device__ __forceinline__ void split_f16(float2 x, unsigned &hi, unsigned &lo)
 {
     const __half2 h = __float22half2_rn(x);
