@@ -609,7 +609,7 @@ def step_scan_roofline(m, pk):
         bodies = m["iters"] * m["prof_steps"]            # (a launch may be several bodies, and launches behind the last return at once)
         nbytes = body_bytes_per_position(m["n"], m["dim_in"]) * m["B"] * m["T"]
         return roofline_of_launch(top, nbytes, prof[top]["total_ms"] / bodies, pk,
-                                  dict(note="per Newton body; bound by issue slots and the special-function unit (gates), not by HBM"))
+                                  dict(note="per Newton body; bound by the latency of a step's phases (half of the issue slots used), not by HBM"))
     names = [k for k in prof if is_scan_kernel(k)]
     scan_ms = sum(prof[k]["total_ms"] for k in names)
     launches = sum(prof[k]["launches"] for k in names if k.startswith("scan_")) or (m["prof_steps"] * m["iters"])

@@ -57,9 +57,12 @@ __device__ __forceinline__ int adjoint_burn(const AdjArgs &a, const StatusBlock 
 // End of the launch: were the boundaries good enough?  Single thread.
 __device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool dy0, int burn)
 {
-    auto take = [](unsigned &w) { const float v = __uint_as_float(*(volatile unsigned *)&w); w = 0u; return v; };
-    const float top = take(st->err_bits), mis = take(st->mis_bits), rel = take(st->rel_bits), top_end = take(st->top_end_bits), mis_end = take(st->mis_end_bits);
-    if (*(volatile unsigned *)&st->flags & FLAG_TIMEOUT) { st->burn = 1 << 20; return; }         // (unfinished rows: the kernels behind do the work)
+    // (all words are requested before the first is looked at)
+    const unsigned flags = *(volatile unsigned *)&st->flags;
+    auto word = [](unsigned &w) { return __uint_as_float(*(volatile unsigned *)&w); };
+    const float top = word(st->err_bits), mis = word(st->mis_bits), rel = word(st->rel_bits), top_end = word(st->top_end_bits), mis_end = word(st->mis_end_bits);
+    st->err_bits = 0u; st->mis_bits = 0u; st->rel_bits = 0u; st->top_end_bits = 0u; st->mis_end_bits = 0u;
+    if (flags & FLAG_TIMEOUT) { st->burn = 1 << 20; return; }            // (unfinished rows: the kernels behind do the work)
     // (at the first time step a NaN reaches no boundary and no lambda any more, only the final state and the gradients there)
     const bool inner = top_end <= 3.402823466e38f && mis <= eta * top && rel <= ADJ_LOCAL * eta, end = !dy0 || mis_end <= eta * top_end;
     if (inner && end) { st->done = BODY_DONE; return; }
