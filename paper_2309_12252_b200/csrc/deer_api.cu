@@ -2143,7 +2143,6 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     a.burn_cap = 512;                                    // (what comes behind goes head by head)
     for (int k = 0; k < ADJ_TRIES; ++k)
         if ((rc = launch_newton_adjoint(a, plan, st)) != DEER_OK) return rc;
-    DEER_KERNEL("mh_drop_kernel", st, mh_drop_kernel<<<num_sms(), 256, 0, st>>>(w.st, w.dGi, w.dGh, N, H, n3));
     // dW_i, db_i of all heads: one contraction of dG_i [N, H*3n] with x [N, m]
     WgradArgs wa{};
     wa.dG = w.dGi; wa.V = x; wa.T = T; wa.n3 = H * n3; wa.K = m; wa.N = N;
@@ -2160,7 +2159,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
         DEER_KERNEL("wgrad_mma_kernel", st, wgrad_mma_kernel<<<grid, 32 * ((rows + 15) / 16), 0, st>>>(wa));
     }
     const size_t outs = (size_t)H * n3 * (m + 1);
-    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs + 7) / 8), 256, 0, st>>>(w.partial, P, n3, m, H, w.grads, 0));
+    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs + 7) / 8), 256, 0, st>>>(w.partial, P, n3, m, H, w.grads, 0, nullptr, nullptr, 0));
     // dW_h, db_h: a contraction per head
     WgradArgs wh{};
     wh.dG = w.dGh; wh.V = y; wh.y0 = y0; wh.shifted = 1; wh.T = T; wh.n3 = n3; wh.K = n; wh.N = N;
@@ -2170,7 +2169,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     wh.heads = w.heads; wh.H = H;
     DEER_KERNEL("wgrad_mma_kernel", st, wgrad_mma_kernel<<<dim3(Ph, (n + 63) / 64, H), 32 * ((n3 + 15) / 16), 0, st>>>(wh));
     const size_t outs_h = (size_t)H * n3 * (n + 1);
-    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs_h + 7) / 8), 256, 0, st>>>(w.partial, Ph, n3, n, H, w.grads, 1));
+    DEER_KERNEL("mh_wgrad_final_kernel", st, mh_wgrad_final_kernel<<<(unsigned)((outs_h + 7) / 8), 256, 0, st>>>(w.partial, Ph, n3, n, H, w.grads, 1, dx ? w.st : nullptr, w.dGi, N));
     if (dx && (rc = launch_affine_tiled<true>(w.dGi, w.Wc, nullptr, dx, N, H * n3, m, st)) != DEER_OK) return rc;
     if (dy0) DEER_KERNEL("mh_dy0_sum_kernel", st, mh_dy0_sum_kernel<<<mh_blocks((size_t)B * H * n), 256, 0, st>>>(w.heads, w.dy0all, dy0, B, T, n, H));
     std::vector<StatusBlock> hs((size_t)H);

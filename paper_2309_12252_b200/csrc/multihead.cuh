@@ -39,22 +39,6 @@ __global__ void mh_select_kernel(const StatusBlock *__restrict__ st, float *__re
     }
 }
 
-// Pre-activation gradients of the heads whose adjoint launch gave up: zero, so that the contractions over all heads (dx among
-// them) are those of the others.  Where none did, one look at the status words (2 us).
-__global__ void mh_drop_kernel(const StatusBlock *__restrict__ st, float *__restrict__ dGi, float *__restrict__ dGh, size_t N, int H, int n3)
-{
-    bool any = false;
-    for (int h = threadIdx.x; h < H; h += blockDim.x) any = any || st[h].done != BODY_DONE;
-    if (!__syncthreads_or(any)) return;
-    for (int h = 0; h < H; ++h) {
-        if (st[h].done == BODY_DONE) continue;
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N * n3; i += (size_t)gridDim.x * blockDim.x) {
-            const size_t o = (i / n3 * H + h) * n3 + i % n3;
-            dGi[o] = 0.0f; dGh[o] = 0.0f;
-        }
-    }
-}
-
 // dy0[b, h, i] = sum over the phases p, in order, of dy0s[first_seq[h] + b s + p, i]
 __global__ void mh_dy0_sum_kernel(const BodyHead *__restrict__ heads, const float *__restrict__ dy0s, float *__restrict__ dy0, int B, int T, int n, int H)
 {
@@ -72,26 +56,39 @@ __global__ void mh_dy0_sum_kernel(const BodyHead *__restrict__ heads, const floa
 
 // Second stage of the parameter-gradient reductions over all heads (wgrad_final_kernel with the heads' own outputs):
 // hidden = 0: rows g = h * n3 + ... of ONE contraction [P][H*n3][K+1]; 1: a contraction per head, [H][P][n3][K+1].
-__global__ void mh_wgrad_final_kernel(const float *__restrict__ partial, int P, int n3, int K, int H, const MhGrad *__restrict__ out, int hidden)
+// st, dGi (or null): besides, the input-side pre-activation gradients of the heads whose adjoint launch gave up become zero, so
+// that dx, which is contracted from them next, is the sum over the other heads.  (A look at the status words by the first blocks
+// where none did; by every block of the input weights' sums it took 5 us at 9 heads, as a launch of its own 2.)
+__global__ void mh_wgrad_final_kernel(const float *__restrict__ partial, int P, int n3, int K, int H, const MhGrad *__restrict__ out, int hidden,
+                                      const StatusBlock *__restrict__ st, float *__restrict__ dGi, size_t N)
 {
     const int K1 = K + 1, per = n3 * K1;
     const size_t outs = (size_t)per * H;
     const size_t o = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (o >= outs) return;
-    const int h = (int)(o / per), r = (int)(o % per);
-    const float *src = hidden ? partial + (size_t)h * P * per + r : partial + o;
-    const size_t pitch = hidden ? (size_t)per : outs;
-    float acc = 0.0f;
+    bool any = false;
+    const unsigned droppers = min(gridDim.x, 128u);
+    if (st && blockIdx.x < droppers) for (int h = threadIdx.x; h < H; h += blockDim.x) any = any || st[h].done != BODY_DONE;
+    if (o < outs) {
+        const int h = (int)(o / per), r = (int)(o % per);
+        const float *src = hidden ? partial + (size_t)h * P * per + r : partial + o;
+        const size_t pitch = hidden ? (size_t)per : outs;
+        float acc = 0.0f;
 #pragma unroll 4
-    for (int p = lane; p < P; p += 32) acc += src[p * pitch];
+        for (int p = lane; p < P; p += 32) acc += src[p * pitch];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
-    if (lane == 0) {
-        const int g = r / K1, k = r % K1;
-        float *dW = hidden ? out[h].dW_h : out[h].dW_i, *db = hidden ? out[h].db_h : out[h].db_i;
-        if (k < K) dW[(size_t)g * K + k] = acc;
-        else db[g] = acc;
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+        if (lane == 0) {
+            const int g = r / K1, k = r % K1;
+            float *dW = hidden ? out[h].dW_h : out[h].dW_i, *db = hidden ? out[h].db_h : out[h].db_i;
+            if (k < K) dW[(size_t)g * K + k] = acc;
+            else db[g] = acc;
+        }
+    }
+    if (!__syncthreads_or(any)) return;
+    for (int h = 0; h < H; ++h) {
+        if (st[h].done == BODY_DONE) continue;
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N * n3; i += (size_t)droppers * blockDim.x) dGi[(i / n3 * H + h) * n3 + i % n3] = 0.0f;
     }
 }
 
