@@ -93,7 +93,7 @@ struct ScanWs {
 };
 
 constexpr int VSCAN_L_MIN = 64, VSCAN_BURN = 64, VSCAN_WARPS = 12;
-static_assert(VSCAN_WINDOW <= VSCAN_BURN && VSCAN_BURN <= VSCAN_L_MIN, "every chain but the first has a whole window before it");
+static_assert(VSCAN_BURN % 16 == 0 && VSCAN_WINDOW <= VSCAN_BURN && VSCAN_BURN <= VSCAN_L_MIN, "every chain but the first has a whole window before it");
 
 static int num_sms();
 
@@ -1213,10 +1213,10 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     bool polled = false;                       // the end of the loop was read from the record
     auto copy_out = [&](bool ended) -> int {
         if (!y_host || ended == copy_early) return DEER_OK;
-        if (ended && copy_st && polled && hs.done == BODY_DONE && (hs.iters & 1) == 0) {
+        if (ended && polled && hs.done == BODY_DONE && (hs.iters & 1) == 0) {
             // the record has told that the result is complete, and it is where it belongs: nothing to wait for (three calls less
             // between the last body and the copy: n = m = 32, B = 16, T = 1e5 6773 -> 6742 us)
-            DEER_CHECK_CUDA(cudaMemcpyAsync(y_host, y, N * n * sizeof(float), cudaMemcpyDeviceToHost, copy_st), "copy result to host");
+            DEER_CHECK_CUDA(cudaMemcpyAsync(y_host, y, N * n * sizeof(float), cudaMemcpyDeviceToHost, copy_st ? copy_st : st), "copy result to host");
             return DEER_OK;
         }
         size_t words = N * n / 4;

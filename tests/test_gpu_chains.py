@@ -405,3 +405,17 @@ def test_evaluation_tile_on_small_inputs(bd, n, m, B, T, scale):
     other, names = launched(bd, lambda: bd.deer_gru_eval(*args, tol=-1.0, max_iter=6, flags=bd.DEER_FLAG_MATERIALIZE))
     assert TILE not in names, names
     assert off <= operands + 1.5 * np.max(np.abs(other.y.cpu().numpy() - want)) + rounding / 4.0
+
+
+def test_scan_of_unequal_but_coupled_components_is_taken(bd):
+    """The gradient of a mean over slowly varying sequences: lambda's components differ by orders of magnitude but feed each other,
+    and no fp32 sum has the small ones to more than the large ones' rounding."""
+    n, m, B, T = 64, 4, 8, 2179
+    p = synth.gru_params(n, m, 19, tag="c/gru")
+    x = walk(synth.x_gaussian(B, T, m, 19, tag="c/x"))
+    gy = np.repeat(synth.normal(19, "c/gy", (B, 1, n)) * np.float32(1.0 / T), T, axis=1)
+    gy[:, :, ::2] *= np.float32(1e-4)
+    got, want, names, done = gradient(bd, p, x, np.zeros((B, n), np.float32), gy)
+    assert "scan_verified_kernel" in names and not names & {WARP, MMA_TILE} and done == 1, names
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        assert np.max(np.abs(got[k] - want[k])) <= 2e-5 * np.max(np.abs(want[k])), k
