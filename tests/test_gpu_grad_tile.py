@@ -47,3 +47,20 @@ def test_gradient_in_one_pass_without_dx():
     without = bd.deer_gru_vjp(p, x, y0, y, gy, want_dx=False)
     for k in ("dW_i", "dW_h", "db_i", "db_h"):
         assert torch.equal(with_dx[k], without[k]), k
+
+
+@pytest.mark.parametrize("n,m", [(16, 20), (24, 33), (32, 5), (32, 32), (64, 20), (64, 63)])
+def test_infinite_gradients_stay_infinite(n, m):
+    """One infinite dL/dy among sequences of one step: dx is infinite there, or a NaN where infinities of both signs meet, and
+    the other positions' is what it is without."""
+    p = synth.gru_params(n, m, seed=23, tag="g/gru")
+    x, y0 = synth.x_gaussian(70, 1, m, seed=23, tag="g/x"), synth.normal(23, "g/y0", (70, n)) * np.float32(0.5)
+    gy = synth.normal(23, "g/gy", (70, 1, n))
+    gy[65, 0, 2], gy[3, 0, 1] = np.inf, -np.inf
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    got = bd.deer_gru_vjp(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy))["dx"].cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy.astype(np.float64), np.float64)["dx"]
+    assert np.isinf(want).any() and np.array_equal(got[~np.isfinite(want)], want[~np.isfinite(want)].astype(np.float32), equal_nan=True)
+    at = np.isfinite(want)
+    assert at.sum() == 68 * m and np.linalg.norm(got[at] - want[at]) <= 8e-6 * np.linalg.norm(want[at])
