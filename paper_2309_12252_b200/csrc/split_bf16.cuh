@@ -1,8 +1,10 @@
 // fp32 operands of tcgen05 products as three bf16 parts.
 //
-// Three parts of 8 bits, cut and not rounded, are x exactly (24 bits); six products (hh, hm, mh, mm, hl, lh) leave out 2^-22 of
-// a product, where 3 x TF32 with its cut lo part leaves out some 2^-20.  bf16 has the range of fp32, so no scale is needed.
-// The tensor core cuts when it adds to an accumulator: the large products (hh) get accumulators of their own, or come last.
+// Three parts of 8 bits, each rounded to nearest, are x exactly (the rest behind two has 7 bits at most); six products (hh, hm, mh,
+// mm, hl, lh) leave out 2^-24 of a product at most (2 * 2^-8 * 2^-17), of either sign, where 3 x TF32 with its cut lo part leaves out
+// some 2^-20.  (Parts that are cut leave out up to 2^-21, always towards zero: 3e-8 of a sum on average.)  bf16 has the range of fp32,
+// so no scale is needed.  The tensor core cuts when it adds to an accumulator: the large products (hh) get accumulators of their
+// own, or come last.
 #pragma once
 #include "tile_umma.cuh"
 
@@ -15,13 +17,12 @@ __host__ __device__ constexpr int SPLIT_B(int p) { return p == 0 ? 2 : p == 2 ||
 // x = a + b + c; pairs packed
 __device__ __forceinline__ void split_bf16(float2 x, unsigned &a, unsigned &b, unsigned &c)
 {
-    auto top = [](float v) { return __uint_as_float(__float_as_uint(v) & 0xffff0000u); };
-    auto pack = [](float2 v) { return __byte_perm(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632); };
-    const float2 mone = make_float2(-1.0f, -1.0f);
+    auto pack = [](float2 v) { unsigned d; asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(v.y), "f"(v.x)); return d; };
+    auto left = [](float2 v, unsigned d) { return ffma2(make_float2(__uint_as_float(d << 16), __uint_as_float(d & 0xffff0000u)), make_float2(-1.0f, -1.0f), v); };
     a = pack(x);
-    const float2 r = ffma2(make_float2(top(x.x), top(x.y)), mone, x);
+    const float2 r = left(x, a);
     b = pack(r);
-    c = pack(ffma2(make_float2(top(r.x), top(r.y)), mone, r));
+    c = pack(left(r, b));
 }
 
 // four values' parts into three operands `part` bytes apart

@@ -32,7 +32,7 @@ def test_gradient_in_one_pass(n, m, B, T, scale):
     for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
         a, b = got[k].cpu().numpy().astype(np.float64), want[k]
         # the adjoint's boundaries (4e-6 of max|lambda| each, far less in all but the last place of a few) and gates good to
-        # 3e-7; the contraction adds 2^-22 per product and 64 cuts of 2^-24 between two flushes: below 4e-6 of the norm
+        # 3e-7; the contraction adds 2^-24 per product and 64 cuts of 2^-24 between two flushes: below 4e-6 of the norm
         assert np.linalg.norm(a - b) <= 8e-6 * np.linalg.norm(b), k
 
 
@@ -64,3 +64,29 @@ def test_infinite_gradients_stay_infinite(n, m):
     assert np.isinf(want).any() and np.array_equal(got[~np.isfinite(want)], want[~np.isfinite(want)].astype(np.float32), equal_nan=True)
     at = np.isfinite(want)
     assert at.sum() == 68 * m and np.linalg.norm(got[at] - want[at]) <= 8e-6 * np.linalg.norm(want[at])
+
+
+@pytest.mark.parametrize("n,m", [(16, 8), (24, 33), (32, 31), (32, 64), (64, 1), (64, 6), (64, 31)])
+def test_dx_is_no_further_off_than_fp32_sums(n, m):
+    """Sums whose terms have one sign, so that every cut of an accumulator is on the same side: dx against the error that its
+    sums have in fp32 arithmetic, in order."""
+    p = synth.gru_params(n, m, seed=24, tag="g/gru")
+    p.W_i[:], p.W_h[:] = np.abs(p.W_i), 0.3 * np.abs(p.W_h)
+    p.W_i[2 * n:] *= np.float32(0.2)
+    p.b_i[2 * n:], p.b_h[2 * n:] = -3.0, 1.0                     # dG > 0: h_prev above the candidate, W_hn h + b_hn > 0
+    N = 1500
+    x, h = np.float32(min(0.3, 3 / m)) * np.abs(synth.x_gaussian(N, 1, m, seed=24, tag="g/x")), np.abs(synth.normal(24, "g/y0", (N, n)))
+    gy = np.abs(synth.normal(24, "g/gy", (N, 1, n))) + np.float32(0.1)
+    y = oracle.gru_seq(p, x, h, np.float32)
+    got = bd.deer_gru_vjp(bd.GruParamsDev.from_numpy(p), dev(x), dev(h), dev(y), dev(gy))["dx"].cpu().numpy()[:, 0]
+    u, q = x[:, 0].astype(np.float64) @ p.W_i.T.astype(np.float64) + p.b_i, h.astype(np.float64) @ p.W_h.T.astype(np.float64) + p.b_h
+    r, z = (1 / (1 + np.exp(-u[:, g * n:g * n + n] - q[:, g * n:g * n + n])) for g in (0, 1))
+    c = np.tanh(u[:, 2 * n:] + r * q[:, 2 * n:])
+    dn = gy[:, 0] * (1 - z) * (1 - c * c)
+    dG = np.concatenate([dn * q[:, 2 * n:] * r * (1 - r), gy[:, 0] * (h - c) * z * (1 - z), dn], axis=1)
+    assert (dG > 0).all()
+    want, chain = dG @ p.W_i.astype(np.float64), np.zeros((N, m), np.float32)
+    for k in range(3 * n):
+        chain += dG[:, k, None].astype(np.float32) * p.W_i[k].astype(np.float32)
+    off = lambda a: np.linalg.norm(a - want) / np.linalg.norm(want)
+    assert off(got) <= off(chain), (off(got), off(chain))
