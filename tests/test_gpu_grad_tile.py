@@ -90,3 +90,15 @@ def test_dx_is_no_further_off_than_fp32_sums(n, m):
         chain += dG[:, k, None].astype(np.float32) * p.W_i[k].astype(np.float32)
     off = lambda a: np.linalg.norm(a - want) / np.linalg.norm(want)
     assert off(got) <= off(chain), (off(got), off(chain))
+
+
+@pytest.mark.parametrize("n,m,scale", [(16, 8, 1e-34), (32, 5, 1e-36), (32, 40, 1e-35), (64, 6, 1e-36), (64, 64, 1e-35)])
+def test_small_dx_keeps_its_digits(n, m, scale):
+    """Gradients whose last bf16 part is below what bf16 holds: dx has fp32's accuracy there too."""
+    p = synth.gru_params(n, m, seed=25, tag="g/gru")
+    x, y0 = synth.x_gaussian(100, 1, m, seed=25, tag="g/x"), synth.normal(25, "g/y0", (100, n)) * np.float32(0.5)
+    gy = synth.normal(25, "g/gy", (100, 1, n)) * np.float32(scale)
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    got = bd.deer_gru_vjp(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy))["dx"].cpu().numpy().astype(np.float64)
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy.astype(np.float64), np.float64)["dx"]
+    assert np.linalg.norm((got - want) / scale) <= 2e-6 * np.linalg.norm(want / scale)     # gates and sums 1e-6 (x: rounded to fp32's 2^-24)
