@@ -44,3 +44,39 @@ def test_multihead_gradients_against_the_oracle(H, n, m, B, T, strides):
         for h in range(H):
             assert near(got[k][h], want[h][k]), (k, h)
     assert near(got["dx"], dx) and near(got["dy0"], dy0)
+
+
+@pytest.mark.parametrize("H,n,m,N,one_sign", [
+    (32, 64, 33, 32768, False), (32, 64, 33, 32768, True), (64, 64, 256, 8192, False), (64, 40, 7, 9600, True), (3, 5, 6, 150016, False),
+    (1, 64, 300, 65600, True)])
+def test_sums_over_many_positions(H, n, m, N, one_sign):
+    """The weights' sums in as few slices as the unit's size leaves, over many stages: every head's stride is the length of the
+    sequences, so that each position is a sequence of its own, and the gradients are sums over N positions in 64 bits."""
+    T = 8
+    g = torch.Generator(device="cuda").manual_seed(41)
+    rand = lambda *s: torch.rand(s, generator=g, device="cuda")
+    heads = []
+    for h in range(H):
+        W = [(rand(3 * n, k) * 2 - 1) / n ** 0.5 for k in (m, n)]
+        heads.append(bd.GruParamsDev(n, m, *W, (rand(3 * n) - 0.5) * 0.5, (rand(3 * n) - 0.5) * 0.5))
+    x = rand(N // T, T, m) - (0.0 if one_sign else 0.5)
+    y0 = rand(N // T, H, n) - (0.0 if one_sign else 0.5)
+    gy = rand(N // T, T, H, n) - (0.0 if one_sign else 0.5)
+    got = bd.deer_gru_multihead_vjp(heads, [T] * H, x, y0, torch.zeros_like(gy), gy)
+    X = x.view(N, m).double()
+    for h in range(0, H, 7):
+        p = heads[h]
+        W_i, W_h, b_i, b_h = (t.double() for t in (p.W_i, p.W_h, p.b_i, p.b_h))
+        hp, lam = y0[:, h].double().repeat_interleave(T, 0), gy[:, :, h].reshape(N, n).double()
+        u, q = X @ W_i.T + b_i, hp @ W_h.T + b_h
+        r, z = torch.sigmoid(u[:, :n] + q[:, :n]), torch.sigmoid(u[:, n:2 * n] + q[:, n:2 * n])
+        c = torch.tanh(u[:, 2 * n:] + r * q[:, 2 * n:])
+        dn = lam * (1 - z) * (1 - c * c)
+        dr, dz = dn * q[:, 2 * n:] * r * (1 - r), lam * (hp - c) * z * (1 - z)
+        gi, gh = torch.cat([dr, dz, dn], 1), torch.cat([dr, dz, dn * r], 1)
+        want = dict(dW_i=gi.T @ X, dW_h=gh.T @ hp, db_i=gi.sum(0), db_h=gh.sum(0))
+        for k in want:
+            # 128 additions between two flushes, each cutting half of 2^-23 of what is there, on average half of the whole: 3.8e-6;
+            # the gates 1e-6 (of the terms, which cancel where they have both signs: the biases' sums are held to the terms there)
+            size = want[k].norm() if one_sign or k[1] == "W" else max(want[k].norm(), gi.norm())
+            assert (got[k][h].double() - want[k]).norm() <= 5e-6 * size, (k, h)
