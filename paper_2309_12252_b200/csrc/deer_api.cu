@@ -432,12 +432,19 @@ static int scan_onepass(ScanArgs a, OnePassWs w, bool prep, int flags, cudaStrea
     }
 }
 
+// The limit belongs to the function on the device and not to a launch: it only ever grows, or a call in one thread would lower it
+// between another's opt-in and launch.
 static int opt_in_smem(const void *fn, size_t bytes)
 {
-    if (bytes > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) { set_error(e, "cudaFuncSetAttribute"); return DEER_ERR_CUDA; }
-    }
+    if (bytes <= 48 * 1024) return DEER_OK;
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, size_t> most;
+    int dev = 0;
+    DEER_CHECK_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
+    std::lock_guard<std::mutex> lk(mu);
+    size_t &m = most[{fn, dev}];
+    DEER_CHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(m, bytes)), "cudaFuncSetAttribute");
+    m = std::max(m, bytes);
     return DEER_OK;
 }
 

@@ -12,8 +12,8 @@ from paper_2309_12252_b200 import synth
 pytestmark = pytest.mark.gpu
 
 
-# one kernel launched with shared memory of two sizes: with and without dx
-@pytest.mark.parametrize("jobs", [((64, 6, True), (64, 6, False)), ((32, 32, True), (32, 32, False))])
+# one kernel launched with shared memory of two sizes: with and without dx; two sizes of cell
+@pytest.mark.parametrize("jobs", [((64, 6, True), (64, 6, False)), ((32, 32, True), (32, 32, False)), ((60, 72, True), (62, 100, False))])
 def test_gradients_in_threads(jobs):
     from bench import read_profile
     B, T, count, failed = 1, 65, 300, []
