@@ -14,12 +14,13 @@ namespace deer {
 __host__ __device__ constexpr int SPLIT_A(int p) { return p == 1 ? 2 : p == 2 || p == 4 ? 1 : 0; }
 __host__ __device__ constexpr int SPLIT_B(int p) { return p == 0 ? 2 : p == 2 || p == 3 ? 1 : 0; }
 
-// x = a + b + c; pairs packed
+// x = a + b + c; pairs packed.  The first part of a finite x above bf16's largest (3.39e38; a mask may hold the type's lowest value) is
+// that largest, not infinity; an infinite x has an infinite second part.
 __device__ __forceinline__ void split_bf16(float2 x, unsigned &a, unsigned &b, unsigned &c)
 {
     auto pack = [](float2 v) { unsigned d; asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(v.y), "f"(v.x)); return d; };
     auto left = [](float2 v, unsigned d) { return ffma2(make_float2(__uint_as_float(d << 16), __uint_as_float(d & 0xffff0000u)), make_float2(-1.0f, -1.0f), v); };
-    a = pack(x);
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(a) : "f"(x.y), "f"(x.x));
     const float2 r = left(x, a);
     b = pack(r);
     c = pack(left(r, b));

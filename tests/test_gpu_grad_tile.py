@@ -102,3 +102,21 @@ def test_small_dx_keeps_its_digits(n, m, scale):
     got = bd.deer_gru_vjp(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy))["dx"].cpu().numpy().astype(np.float64)
     want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy.astype(np.float64), np.float64)["dx"]
     assert np.linalg.norm((got - want) / scale) <= 2e-6 * np.linalg.norm(want / scale)     # gates and sums 1e-6 (x: rounded to fp32's 2^-24)
+
+
+@pytest.mark.parametrize("n,m", [(16, 8), (24, 33), (32, 32), (64, 6), (64, 64)])
+def test_inputs_masked_with_the_lowest_value(n, m):
+    """Steps whose first channel holds the type's lowest or largest value: their gates are closed or open for good, their
+    pre-activation gradients zero, and the sums what the other steps give."""
+    p = synth.gru_params(n, m, seed=26, tag="g/gru")
+    x, y0 = synth.x_gaussian(70, 5, m, seed=26, tag="g/x"), synth.normal(26, "g/y0", (70, n)) * np.float32(0.5)
+    top = np.finfo(np.float32).max
+    x[3, 2, 0], x[40, 0, 0], x[69, 4, 0] = -top, top, -top
+    gy = synth.normal(26, "g/gy", (70, 5, n))
+    with np.errstate(over="ignore"):
+        y = oracle.gru_seq(p, x, y0, np.float32)
+        want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy.astype(np.float64), np.float64)
+    got = bd.deer_gru_vjp(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy))
+    for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
+        a, b = got[k].cpu().numpy().astype(np.float64), want[k]
+        assert np.isfinite(b).all() and np.linalg.norm(a - b) <= 8e-6 * np.linalg.norm(b), k

@@ -80,3 +80,29 @@ def test_sums_over_many_positions(H, n, m, N, one_sign):
             # the gates 1e-6 (of the terms, which cancel where they have both signs: the biases' sums are held to the terms there)
             size = want[k].norm() if one_sign or k[1] == "W" else max(want[k].norm(), gi.norm())
             assert (got[k][h].double() - want[k]).norm() <= 5e-6 * size, (k, h)
+
+
+def test_inputs_masked_with_the_lowest_value():
+    """Masked steps hold the type's lowest value in one channel: the projections are finite there, the gates closed or open, and the
+    gradients what the other steps give."""
+    H, n, m, B, T = 3, 8, 20, 4, 60
+    hp = [synth.gru_params(n, m, seed=51 + h, tag="t/gru") for h in range(H)]
+    heads = [bd.GruParamsDev.from_numpy(p) for p in hp]
+    x = synth.x_gaussian(B, T, m, seed=51, tag="t/x")
+    x[1, 7, 3], x[2, 30:33, 0] = np.finfo(np.float32).min, np.finfo(np.float32).min
+    gy = synth.normal(51, "t/gy", (B, T, H, n))
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    xd, y0 = dev(x), torch.zeros((B, H, n), device="cuda")
+    y, _, status = bd.deer_gru_multihead_eval(heads, [1] * H, xd, y0, tol=1e-6)
+    assert status == 0
+    got = bd.deer_gru_multihead_vjp(heads, [1] * H, xd, y0, y, dev(gy))
+    dx = np.zeros((B, T, m))
+    for h in range(H):
+        zero, yn, g = np.zeros((B, n), np.float32), np.ascontiguousarray(y[:, :, h].cpu().numpy()), np.ascontiguousarray(gy[:, :, h])
+        with np.errstate(over="ignore"):
+            assert np.max(np.abs(oracle.gru_seq(hp[h], x, zero, np.float32) - yn)) <= 1e-5
+            want = oracle.gru_bptt(hp[h], x, zero, yn.astype(np.float64), g, np.float64)
+        for k in ("dW_i", "dW_h", "db_i", "db_h"):
+            assert np.linalg.norm(got[k][h].cpu().numpy() - want[k]) <= 8e-6 * np.linalg.norm(want[k]), (k, h)
+        dx += want["dx"]
+    assert np.linalg.norm(got["dx"].cpu().numpy() - dx) <= 8e-6 * np.linalg.norm(dx)
