@@ -95,10 +95,16 @@ enum {
                                    Nothing traps or hangs; the workspace can be used again */
     DEER_FLAG_COEF_ROWS  = 32,  /* deer_gru_cell_jac, n = 16, 32 and 64: write the four coefficient
                                    vectors per position instead of the matrices (see there) */
-    DEER_FLAG_EXPIRE_BODY_WAITS = 64 /* the same test aid for the kernels that run a Newton body, the
+    DEER_FLAG_EXPIRE_BODY_WAITS = 64, /* the same test aid for the kernels that run a Newton body, the
                                    whole loop or the adjoint solve as one launch (evaluations and
                                    gradients): a CTA's wait for the others of a whole-loop launch
                                    and for its tensor-core products give up */
+    DEER_FLAG_EXPIRE_PRODUCT_WAITS = 128 /* the same test aid for the dense products on tensor
+                                   cores before and behind those kernels: the waits of the call's
+                                   first such launch give up; 128 << k: of its launch k.  A gradient
+                                   with 16 <= n <= 64, n % 4 = 0, m <= 64: its contractions; the
+                                   multi-head unit forward: the projection; backward: projection,
+                                   sums of W_i, of W_h, dx */
 };
 
 /* Bytes of workspace needed by `op` at the given sizes (0 if the sizes are

@@ -1395,6 +1395,9 @@ static int launch_vjp_small(const VjpSmallArgs &v, int n, int m, int *P, cudaStr
     }
 }
 
+// do the waits of the call's dense product k run out (test aid)?
+static int expire_product(int flags, int k) { return (flags & DEER_FLAG_EXPIRE_PRODUCT_WAITS << k) != 0; }
+
 // gy_seq (or nullptr): dL/dy is gy_seq [B,n] at every step, and gy a buffer for what has to read it position by position
 static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y0, const float *y,
                         const float *gy, int B, int T, const deer_gru_grads *g, float *dx,
@@ -1496,7 +1499,7 @@ static int gru_vjp_impl(const deer_gru_params *p, const float *x, const float *y
     ga.x = x; ga.y = y; ga.y0 = y0; ga.W_i = p->W_i; ga.dx = dx;
     ga.slices = w.partial;
     ga.N = (int)N; ga.T = T; ga.n = n; ga.m = m;
-    ga.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0;
+    ga.expire = expire_product(flags, 0);
     ga.st = w.st;
     const bool one_pass = !(flags & DEER_FLAG_GENERIC) && N < 0x7fff0000u &&
                           grad_tile_suits(ga, (size_t)(w.partial2 - w.partial) + (size_t)WGRAD_P * n3 * (std::max(m, n) + 1));
@@ -2067,7 +2070,7 @@ static int mh_project(const MhWs &w, const float *x, size_t N, int H, int n, int
     TileGemmArgs a{};
     a.A = x; a.lda = (size_t)m; a.B = w.Wc; a.ldb = (size_t)m; a.bias = w.bc; a.C = w.u;
     a.M = (int)N; a.N = H * 3 * n; a.K = m;
-    a.expire = (flags & DEER_FLAG_EXPIRE_BODY_WAITS) != 0; a.st = w.st;
+    a.expire = expire_product(flags, 0); a.st = w.st;
     return launch_tile_gemm(TileGemm::MAP, a, 1, st);
 }
 
@@ -2126,7 +2129,7 @@ static int mh_eval_batched(const deer_gru_params *heads, const int *strides, int
 // did[h]: the gradients of head h, and its part of dx and dy0, are there (empty: of none).
 static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int H, const float *x, const float *y0, const float *y,
                           const float *gy, int B, int T, const deer_gru_grads *dheads, float *dx, float *dy0, const MhWs &w,
-                          cudaStream_t st, std::vector<char> &did)
+                          int flags, cudaStream_t st, std::vector<char> &did)
 {
     const int n = heads[0].n, m = heads[0].m, n3 = 3 * n;
     const size_t N = (size_t)B * T;
@@ -2143,7 +2146,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     memset(&init, 0, sizeof(init));
     DEER_KERNEL("mh_begin_kernel", st, mh_begin_kernel<<<mh_blocks((size_t)plan.edges + H), 256, 0, st>>>(
                                            w.st, init, H, w.edge_flag, (size_t)plan.edges, nullptr, 0, nullptr, 0));
-    if ((rc = mh_project(w, x, N, H, n, m, 0, st)) != DEER_OK) return rc;
+    if ((rc = mh_project(w, x, N, H, n, m, flags, st)) != DEER_OK) return rc;
     AdjArgs a{};
     a.heads = w.heads;
     a.u = w.u; a.y0 = y0; a.y = y; a.gy = gy;
@@ -2159,7 +2162,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     // dW_i, db_i of all heads: one contraction of dG_i [N, H*3n] with x [N, m]
     TileGemmArgs ga{};
     ga.A = w.dGi; ga.lda = (size_t)H * n3; ga.B = x; ga.ldb = (size_t)m; ga.C = w.partial;
-    ga.M = H * n3; ga.N = m; ga.K = (int)N; ga.st = w.st;
+    ga.M = H * n3; ga.N = m; ga.K = (int)N; ga.expire = expire_product(flags, 1); ga.st = w.st;
     const int P = tile_gemm_slices(ga.M, ga.N, ga.K, MH_P_IN);
     if ((rc = launch_tile_gemm(TileGemm::SUMS, ga, P, st)) != DEER_OK) return rc;
     const size_t outs = (size_t)H * n3 * (m + 1);
@@ -2167,7 +2170,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     // dW_h, db_h: every head's columns of dG_h with its own of y
     TileGemmArgs gh{};
     gh.A = w.dGh; gh.lda = (size_t)H * n3; gh.B = y; gh.ldb = (size_t)H * n; gh.C = w.partial;
-    gh.M = H * n3; gh.N = n; gh.K = (int)N; gh.st = w.st;
+    gh.M = H * n3; gh.N = n; gh.K = (int)N; gh.expire = expire_product(flags, 2); gh.st = w.st;
     gh.heads = w.heads; gh.y0 = y0; gh.T = T; gh.n = n; gh.n3 = n3;
     const int Ph = tile_gemm_slices(gh.M, 1, gh.K, mh_p_hidden(H));
     if ((rc = launch_tile_gemm(TileGemm::SUMS_HEADS, gh, Ph, st)) != DEER_OK) return rc;
@@ -2176,7 +2179,7 @@ static int mh_vjp_batched(const deer_gru_params *heads, const int *strides, int 
     if (dx) {
         TileGemmArgs xa{};
         xa.A = w.dGi; xa.lda = (size_t)H * n3; xa.B = w.Wc; xa.ldb = (size_t)m; xa.C = dx;
-        xa.M = (int)N; xa.N = m; xa.K = H * n3; xa.st = w.st;
+        xa.M = (int)N; xa.N = m; xa.K = H * n3; xa.expire = expire_product(flags, 3); xa.st = w.st;
         if ((rc = launch_tile_gemm(TileGemm::MAP_T, xa, 1, st)) != DEER_OK) return rc;
     }
     if (dy0) DEER_KERNEL("mh_dy0_sum_kernel", st, mh_dy0_sum_kernel<<<mh_blocks((size_t)B * H * n), 256, 0, st>>>(w.heads, w.dy0all, dy0, B, T, n, H));
@@ -2261,7 +2264,7 @@ int deer_gru_multihead_vjp(const deer_gru_params *heads, const int *strides, int
     if ((rc = check_ws(ws, ws_bytes, w.bytes)) != DEER_OK) return rc;
     std::vector<char> did;
     if (mh_batched(n, H, (size_t)B * T, flags) &&
-        (rc = mh_vjp_batched(heads, strides, H, x, y0, y, gy, B, T, dheads, dx, dy0, w, st, did)) != DEER_OK) return rc;
+        (rc = mh_vjp_batched(heads, strides, H, x, y0, y, gy, B, T, dheads, dx, dy0, w, flags, st, did)) != DEER_OK) return rc;
     const bool batched = !did.empty();
     unsigned timeout_flags = 0;
     int packed_stride = 1;                     // (stride 1: x itself)

@@ -12,7 +12,7 @@ struct GradTileArgs {
     float *dx;                   // [N,m] or nullptr
     float *slices;               // [CTAs][grad_tile_slice(n, m)]
     int N, T, n, m;
-    int expire;                  // test aid: the bounded waits run out (DEER_FLAG_EXPIRE_BODY_WAITS)
+    int expire;                  // test aid: the bounded waits of a CTA's last thread run out (DEER_FLAG_EXPIRE_PRODUCT_WAITS)
     StatusBlock *st;
 };
 

@@ -120,3 +120,19 @@ def test_inputs_masked_with_the_lowest_value(n, m):
     for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
         a, b = got[k].cpu().numpy().astype(np.float64), want[k]
         assert np.isfinite(b).all() and np.linalg.norm(a - b) <= 8e-6 * np.linalg.norm(b), k
+
+
+# one run per CTA (the wait behind the last run only), several
+@pytest.mark.parametrize("n,m,B,T", [(16, 8, 3, 64), (32, 33, 2, 97), (60, 7, 1, 65), (32, 32, 8, 5001), (24, 40, 10, 4001), (48, 20, 2, 15001)])
+def test_expired_wait_is_reported(n, m, B, T):
+    """The waits for a run's products run out and the adjoint's do not: the call says so, and the next one on the same workspace
+    gives what one on another does."""
+    p = bd.GruParamsDev.from_numpy(synth.gru_params(n, m, seed=27, tag="g/gru"))
+    x, y0 = dev(synth.x_gaussian(B, T, m, seed=27, tag="g/x")), torch.zeros((B, n), device="cuda")
+    y, gy = bd.deer_gru_eval(p, x, y0).y, dev(synth.normal(27, "g/gy", (B, T, n)))
+    want, ws = bd.deer_gru_vjp(p, x, y0, y, gy), bd.alloc_workspace(bd.DEER_OP_VJP, B, T, n, m)
+    for flags in (bd.DEER_FLAG_EXPIRE_PRODUCT_WAITS, 0):
+        got = bd.deer_gru_vjp(p, x, y0, y, gy, ws=ws, flags=flags)
+        assert bd.deer_workspace_status(ws) == (bd.DEER_ERR_DEVICE_TIMEOUT if flags else bd.DEER_OK)
+    for k, v in want.items():
+        assert torch.equal(got[k], v), k

@@ -106,3 +106,24 @@ def test_inputs_masked_with_the_lowest_value():
             assert np.linalg.norm(got[k][h].cpu().numpy() - want[k]) <= 8e-6 * np.linalg.norm(want[k]), (k, h)
         dx += want["dx"]
     assert np.linalg.norm(got["dx"].cpu().numpy() - dx) <= 8e-6 * np.linalg.norm(dx)
+
+
+# products of one or two stages (no wait but those behind the last one), of several
+@pytest.mark.parametrize("H,n,m,B,T", [(2, 8, 5, 1, 32), (6, 16, 100, 16, 300)])
+def test_expired_waits_are_reported(H, n, m, B, T):
+    """The waits of one dense product run out at a time, and nothing else's: the call says so, and the next one is right."""
+    heads, strides = [bd.GruParamsDev.from_numpy(synth.gru_params(n, m, seed=61 + h, tag="t/gru")) for h in range(H)], [1, 2, 4, 1, 2, 4][:H]
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    x, y0, gy = dev(synth.x_gaussian(B, T, m, seed=61, tag="t/x")), torch.zeros((B, H, n), device="cuda"), dev(synth.normal(61, "t/gy", (B, T, H, n)))
+    ws = bd.alloc_multihead_workspace(heads, strides, B, T, x.device)
+    y = bd.deer_gru_multihead_eval(heads, strides, x, y0)[0]
+    want = bd.deer_gru_multihead_vjp(heads, strides, x, y0, y, gy)
+    expired = lambda call: pytest.raises(bd.DeerError, call).value.status == bd.DEER_ERR_DEVICE_TIMEOUT
+    assert expired(lambda: bd.deer_gru_multihead_eval(heads, strides, x, y0, ws=ws, flags=bd.DEER_FLAG_EXPIRE_PRODUCT_WAITS))
+    again, _, status = bd.deer_gru_multihead_eval(heads, strides, x, y0, ws=ws)
+    assert status == bd.DEER_OK and torch.equal(again, y)
+    for k in range(4):
+        assert expired(lambda: bd.deer_gru_multihead_vjp(heads, strides, x, y0, y, gy, ws=ws, flags=bd.DEER_FLAG_EXPIRE_PRODUCT_WAITS << k)), k
+        got = bd.deer_gru_multihead_vjp(heads, strides, x, y0, y, gy, ws=ws)
+        for name, v in want.items():
+            assert all(torch.equal(a, b) for a, b in zip(got[name], v)), name
