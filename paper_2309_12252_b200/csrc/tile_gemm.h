@@ -16,7 +16,7 @@ struct TileGemmArgs {
     const BodyHead *heads;
     const float *y0;
     int T, n, n3;
-    int expire;              // test aid: the bounded waits run out (DEER_FLAG_EXPIRE_PRODUCT_WAITS)
+    int expire;              // test aid: the bounded waits of a CTA's last thread run out (DEER_FLAG_EXPIRE_PRODUCT_WAITS)
     StatusBlock *st;
     int chunks;              // (set by the launch)
 };
