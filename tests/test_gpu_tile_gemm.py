@@ -11,10 +11,12 @@ pytestmark = pytest.mark.gpu
 
 
 # one column and one stage; sizes that are no multiple of 4 (n, m); a tile's edge in positions (128, 129), inputs (255, 257) and stacked
-# gates (16 heads of 24: 384 = 3 tiles; 11 of 12: a head across two tiles); strides longer than the sequence; one position
+# gates (16 heads of 24: 384 = 3 tiles; 11 of 12: a head across two tiles); strides longer than the sequence; one position; more than a
+# wave of tiles of 128 columns, rows of C on and off 32 bytes
 @pytest.mark.parametrize("H,n,m,B,T,strides", [
     (1, 1, 1, 1, 1, [1]), (2, 4, 8, 1, 128, [1, 2]), (3, 7, 5, 3, 43, [1, 4, 64]), (11, 4, 255, 1, 129, [1, 2, 4, 8, 1, 2, 4, 8, 1, 2, 4]),
     (16, 8, 257, 2, 97, [1, 2, 4, 8] * 4), (2, 64, 32, 2, 33, [1, 3]), (5, 30, 36, 4, 160, [1, 2, 3, 4, 5]), (6, 16, 256, 16, 300, [1, 2, 4, 8, 16, 32]),
+    (3, 6, 257, 16, 1201, [1, 2, 64]), (2, 16, 264, 16, 1201, [1, 4]),
 ])
 def test_multihead_gradients_against_the_oracle(H, n, m, B, T, strides):
     hp = [synth.gru_params(n, m, seed=31 + h, tag="t/gru") for h in range(H)]
