@@ -1,4 +1,4 @@
-// Parameter gradients and dx from the pre-activation gradients in one pass (grad_tile.cuh): host-side interface.
+// Parameter gradients and dx from the pre-activation gradients in one pass (grad_tile.cu): host-side interface.
 #pragma once
 #include "common.cuh"
 

@@ -5,8 +5,8 @@
 // plain FMAs with the weights as broadcast 16-byte loads.  A warp's 32 chains walk in lockstep through windows of W positions
 // that cp.async has brought into warp-private shared memory (full lines of every chain, one window ahead); the new iterate
 // replaces the old one there and leaves the same way.  Row strides are odd in 16-byte pieces: conflict-free.
-// What bounds it: issue slots and latency, with some 14 warps per SM.  n = m = 1, B = 16, T = 3e5: issue slots 54 % used, special
-// functions (six instructions per state component) 32 %, FMA 31 %, DRAM 12 %.
+// What bounds it: issue slots and latency.  n = m = 1, B = 16, T = 3e5, at 94 registers (20 warps fit an SM, 14 were active on average;
+// now 108, 16 fit): issue slots 54 % used, special functions (six instructions per state component) 32 %, FMA 31 %, DRAM 12 %.
 #pragma once
 #include "newton_body.cuh"
 #include "scan_onepass.cuh"
@@ -29,9 +29,10 @@ template <int N, int M> struct Lane {                    // M: input channels, p
 };
 
 // (A CTA per SM named: the compiler, which left to itself aims at more of them, then keeps the cells of the positions that are
-// evaluated side by side in registers.  us per evaluation, without and with: n = m = 1 413 -> 362 and 305 -> 299 (1.6e7 positions, two
-// draws), n = 1, m = 5 616 -> 574, n = 2, m = 4 272 -> 252; n = 2, m = 8 229 -> 231 and n = 1 with projected inputs 448 -> 451, which
-// stay without, as do n = 4 and 8: no difference.  Three CTAs named cost n = 4 and 8 spills, 606 -> 837 us.)
+// evaluated side by side in registers.  us per evaluation, without and with: n = m = 1 (1.6e7 positions, four draws) 413 -> 362,
+// 305 -> 299, 292 -> 286 and 306 -> 301, the last no more than two runs of one side differ; n = 1, m = 5 616 -> 574, n = 2, m = 4
+// 272 -> 252; n = 2, m = 8 229 -> 231 and n = 1 with projected inputs 448 -> 451, which stay without, as do n = 4 and 8: no difference.
+// Three CTAs named cost n = 4 and 8 spills, 606 -> 837 us.)
 template <int N, int M>
 __global__ void __launch_bounds__(128, N <= 2 && M > 0 && N * M <= 8 ? 1 : 0) newton_lane_kernel(BodyArgs a)
 {

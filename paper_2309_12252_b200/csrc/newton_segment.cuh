@@ -9,9 +9,11 @@
 //   phase 2  the chains, 16 in lockstep per group of N / 8 warps (one block of eight state columns each), a step being
 //            d <- r + z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d):  9 MMAs of a warp per block of eight columns,
 //            the new d crossing to the other warps of the group through shared memory.
-// A step of phase 2 is some 250 cycles (N = 8: one warp, no exchange).
-// What bounds it: those steps, in series (n = 8, m = 4, B = 16, T = 1e4: issue slots 34 % used; the warps that phase 2 has no
-// chains for wait at the barrier behind it, 5.8 of 16 at a time).
+// What bounds it: phases in series.  Cycles of a body, read with clock64 by one warp (n = 8, m = 4, B = 16, T = 1e4: 64 chains of 17
+// positions per CTA): phase 1 10,250 (five tiles a warp), 45 steps of burn-in 7,700 (170 a step), the 17 positions owned 10,800 (640 a
+// step, with its old iterate, residual and store), prologue of phase 2 950, exchange with the other CTAs 4,000 ... 10,000.  n = 4, m = 2,
+// T = 1000 (16 chains of 5): 3,500, 30 steps 5,100, 3,550, 1,200, 3,000.  Issue slots 34 % used; the warps that phase 2 has no chains
+// for wait at the barrier behind it, 5.8 of 16 at a time.
 #pragma once
 #include "newton_body.cuh"
 
