@@ -99,13 +99,14 @@ struct StatusBlock {
     int ctl_mode;        // 1: the last CTA of a single-pass scan takes the Newton loop decision
     int max_iter;
     float tol;
-    int burn;            // one-launch bodies: burn-in of their chains, raised when it proves too short
+    int burn;            // one-launch bodies: burn-in of the next body's chains; of a loop that has ended: `need`
     float *trace;        // err after each body (first ERR_TRACE_CAP bodies), or nullptr
     unsigned mis_bits;   // one-launch bodies: largest mismatch between a chain's end and the start its successor assumed
     HostResult *host;    // page-locked host memory, or nullptr
     unsigned top_end_bits, mis_end_bits;     // adjoint launch: max|dy0|, largest mismatch near the first time step
     unsigned rel_bits;   // ... largest mismatch as a part of |lambda| there
-    unsigned pad[43];
+    int need;            // one-launch bodies: longest burn-in that any of them would have needed for the accuracy eta
+    unsigned pad[42];
 };
 static_assert(sizeof(StatusBlock) == 256, "status block is one 256-byte line");
 constexpr int ERR_TRACE_CAP = 1024;

@@ -1082,6 +1082,11 @@ static bool body_takes(int n, int m, int flags)
 // 0.7 us) than a form that gives up later gains.
 constexpr int BIAS_US = 20, RESULT_US = 20000;
 
+// Chains up to this length get the burn-in that each body calls for (body_verdict); with longer ones a try that fails is dearer
+// than what a few steps of them give (n = 1, 224 positions: 370 us either way).  Multi-head units do without: one head whose
+// try fails holds up the others (17 heads of 8: 815 -> 1226 us).
+constexpr int BODY_L_ADAPT = 64;
+
 // Runs the Newton loop until it ends or the form gives up (hs->done == BODY_FALL_BACK, the iterate after hs->iters bodies in
 // buf[hs->iters & 1]).
 template <typename CopyOut>
@@ -1091,7 +1096,8 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
 {
     const int n = p->n, m = p->m;
     const bool need_u = !body_supported(n, m, false);
-    int rc, burn = body_first_burn(n, tol);
+    const int first = body_first_burn(n, tol);
+    int rc, burn = first;
     BodyArgs a{};
     a.h0 = BodyHead{p->W_i, p->W_h, p->b_i, p->b_h, 1, 0};
     a.x = x; a.y0 = y0;
@@ -1117,13 +1123,14 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
         if (burn > plan.burn_cap) { hs->done = BODY_FALL_BACK; continue; }
         a.L = plan.L;
         a.burn_cap = plan.burn_cap;
+        a.adapt = plan.L <= BODY_L_ADAPT;
         a.warm = ((flags & DEER_FLAG_WARM_START) || hs->iters > 0) ? 1 : 0;
         StatusBlock init;
         memset(&init, 0, sizeof(init));
         init.max_iter = max_iter;
         init.tol = tol;
         init.trace = w.trace;
-        init.burn = burn;
+        init.burn = burn == first && !a.warm ? body_start_burn(n, tol, a.adapt != 0) : burn;
         init.iters = hs->iters;
         init.host = hr;
         if (hr) { hr->iters = hs->iters; hr->done = 0; }
@@ -1239,7 +1246,7 @@ static int gru_eval_impl(const deer_gru_params *p, const float *x, const float *
     if (one_launch) {
         if ((rc = eval_one_launch(p, x, y0, B, T, tol, max_iter, w, buf, flags, st, &hs, slot.p, u_done, y_host && !copy_early, polled, copy_out)) != DEER_OK) return rc;
         ended_there = hs.done == BODY_DONE;
-        if (burn_in) *burn_in = ended_there ? hs.burn : -hs.burn;      // of the last body; negative: it gave up, what it would have needed
+        if (burn_in) *burn_in = ended_there ? hs.burn : -hs.burn;      // what its boundaries needed; negative: it gave up, what it would have needed
     }
     if (!one_launch || hs.done != BODY_DONE) {
     const int k0 = hs.iters;                   // bodies that the one-launch form has done
@@ -1774,12 +1781,15 @@ int deer_gru_vjp(const deer_gru_params *p, const float *x, const float *y0, cons
     return gru_vjp_impl(p, x, y0, y, gy, B, T, g, dx, dy0, ws, ws_bytes, flags, (cudaStream_t)stream);
 }
 
-// The burn-in that a gradient's boundaries need, from the one that the evaluation of the same trajectory came to (0: the
-// evaluation tells nothing beyond its first one; negative: it gave up): it goes with the logarithm of the accuracy asked for.
+// The burn-in that a gradient's boundaries need, from the one that the bodies of the same trajectory would have needed for eta
+// (0: they do not tell; negative: the evaluation gave up): it goes with the logarithm of the accuracy asked for.  (Needed / told
+// so, without the tenth and the two, of twelve first layers of 64: 47 / 42, 45 / 45, 39 / 40, 43 / 48, 55 / 52, 46 / 51, 46 / 43,
+// 48 / 53, 40 / 41, 39 / 38, 42 / 43; a try that is too short costs all of its 75 steps.)
 static int adjoint_burn_hint(int burn, int n, float tol)
 {
-    if (abs(burn) <= body_first_burn(n, tol)) return 0;
-    return (int)fmaxf(-1e6f, fminf(1e6f, (float)burn * logf(0.5f * ADJ_ETA) / logf(0.5f * body_eta(n, tol))));
+    if (burn <= 0 && -burn <= body_first_burn(n, tol)) return 0;
+    const float to = logf(0.5f * ADJ_ETA) / logf(0.5f * body_eta(n, tol));
+    return (int)fmaxf(-1e6f, fminf(1e6f, burn > 0 ? 1.1f * to * (float)burn + 2.0f : to * (float)burn));
 }
 
 int deer_gru_classifier_step(const deer_gru_params *l1, const deer_gru_params *l2, const float *W_o,

@@ -49,6 +49,11 @@ bool body_supported(int n, int m, bool have_u)
 float body_eta(int n, float tol) { return reduced(n) ? 1e-3f : tol > 0.0f ? 1e-4f : 4e-6f; }
 int body_first_burn(int n, float tol) { return reduced(n) ? 24 : tol > 0.0f ? 30 : 40; }
 
+// Behind a zero guess the first update is of order one and its boundaries are asked for a twentieth of it: 16 or 24 steps, where
+// a body's time goes with them.  (Rates seen at first bodies, per step: white noise 0.32 ... 0.44, random walks and sinusoids
+// 0.12 ... 0.3; the twentieth takes 0.19 or 0.125.)
+int body_start_burn(int n, float tol, bool adapt) { return tol > 0.0f && adapt ? (reduced(n) ? 16 : 24) : body_first_burn(n, tol); }
+
 // Shared-memory opt-in and CTAs per SM of a kernel, looked up once per kernel, device and shared-memory size.
 static int occupancy_of(const void *kern, int threads, size_t smem)
 {

@@ -26,6 +26,7 @@ struct BodyArgs {
     int burn_cap;            // longest burn-in that is tried (BodyPlan)
     int expire;              // test aid: every bounded wait runs out (DEER_FLAG_EXPIRE_BODY_WAITS)
     int polled;              // the host reads the result record while the stream runs
+    int adapt;               // chains so short that a body's burn-in is its time: no longer than its own accuracy calls for
     StatusBlock *st;         // [H]
     float *edge;             // [groups][2][n]  states either side of a boundary between two warps
     unsigned *edge_flag;     // [groups]        arrivals at it (left cleared)
@@ -75,6 +76,8 @@ struct BodyKernels {
 };
 
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
+constexpr int BODY_BURN_MIN = 8; // ... and have at least this burn-in
+constexpr float BODY_ROUNDING = 2.4e-7f;         // two roundings of a state below one in size
 constexpr int CHAIN_L_MIN = 4;   // ... those of every form but the two-phase one: what boundaries and start states are sized by
 
 // The forms of a body.
@@ -113,8 +116,10 @@ bool body_supported(int n, int m, bool have_u);
 bool body_plan(BodyPlan *p, BodyForm form, int B, int T, int n, int m, bool have_u, const int *strides, int H);
 // Does the form the plan stands for suit the problem, or are the kernels that multiply the Jacobians out faster?
 bool body_suits(const BodyPlan &p, int n);
-// Burn-in a call starts with, and the accuracy asked of the boundaries.
+// Burn-in that a cell as initialised needs for the accuracy asked of the boundaries, that accuracy, and the burn-in of the first
+// body behind a zero guess.
 int body_first_burn(int n, float tol);
+int body_start_burn(int n, float tol, bool adapt);
 float body_eta(int n, float tol);
 int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st);
 

@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(128, N <= 2 && M > 0 && N * M <= 8 ? 1 : 0) ne
         if (prevc + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
+            body_decide(st, a, W, BODY_ROUNDING);
         }
     }
 }

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
     const bool has_next = nk == NC && tab[NC - 1].next, has_prev = tab[0].t0 > 0 && tab[0].t_end > 0;
     const int G = NC >> 4;                               // groups (a power of two)
 
-    int iters = *(volatile int *)&st->iters, burn = *(volatile int *)&st->burn;
+    int iters = *(volatile int *)&st->iters, burn = *(volatile int *)&st->burn, need = 0;
     const float tol = st->tol;
     const int max_iter = st->max_iter;
     __shared__ unsigned red[4][C::WARPS];
@@ -533,7 +533,8 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         }
         const unsigned eb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[2][lane] : 0u);
         const unsigned qb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[3][lane] : 0u);
-        const BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter);
+        const BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter, a.adapt != 0, 0.0f);
+        need = max(need, v.need);
         if (blockIdx.x == 0 && tid == 0) {
             if (v.counts) {
                 if (st->trace && iters < ERR_TRACE_CAP) st->trace[iters] = __uint_as_float(eb);
@@ -542,9 +543,10 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
             }
             if (v.done) {
                 st->iters = iters + (v.counts ? 1 : 0);
-                st->burn = v.burn;
+                const int told = v.done == BODY_DONE ? need : v.burn;
+                st->burn = told;
                 st->done = v.done;
-                if (HostResult *h = st->host) post_result(h, v.done, v.burn, st->iters, st->err_last_bits, a.polled || v.done != BODY_DONE);
+                if (HostResult *h = st->host) post_result(h, v.done, told, st->iters, st->err_last_bits, a.polled || v.done != BODY_DONE);
             }
         }
         if (v.done) return;
@@ -583,7 +585,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
+            body_decide(st, a);
         }
     }
     return;

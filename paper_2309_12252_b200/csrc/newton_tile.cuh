@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
                 st->done = BODY_FALL_BACK;
                 if (HostResult *h = st->host) post_done(h, BODY_FALL_BACK);
             } else {
-                body_decide(st, a.eta, a.burn_cap, a.T, a.polled != 0);
+                body_decide(st, a, 1, BODY_ROUNDING);
             }
         }
     }

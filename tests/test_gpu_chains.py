@@ -64,6 +64,31 @@ def test_bodies(bd, n, m, B, T, x_kind, kernel):
     assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-4
 
 
+@pytest.mark.parametrize("n,m,B,T,bias,warm,kernel", [
+    (8, 4, 16, 9001, 0.0, False, SEG), (8, 4, 16, 9001, 1.0, False, SEG), (24, 5, 2, 3001, 1.0, False, SEG), (24, 5, 2, 3001, 0.0, True, SEG),
+    (16, 5, 16, 15001, 1.0, False, ONE), (32, 33, 16, 6001, 1.0, False, TILE), (64, 3, 3, 12001, 0.0, False, TILE),
+    (64, 3, 3, 12001, 1.0, False, TILE), (64, 3, 3, 12001, 0.0, True, TILE)])
+def test_burn_in_of_each_body_follows_the_cell(bd, n, m, B, T, bias, warm, kernel):
+    """Short chains take the burn-in that their last body's mismatch calls for: cells that forget fast and slowly (update gates
+    biased to keep), and a guess that is near the solution, whose first update asks for more than a twentieth.  Every boundary of
+    the last body is good to 2.4e-7 or a thousandth of the tolerance, the gates to 2e-7, and a cell that forgets a tenth a step
+    carries ten times that."""
+    p = synth.gru_params(n, m, seed=6, tag="c/gru")
+    p.b_i[n:2 * n] += bias
+    x = synth.x_gaussian(B, T, m, seed=6, tag="c/x")
+    y0 = synth.normal(6, "c/y0", (B, n)) * 0.5
+    want = oracle.gru_seq(p, x, y0, np.float32)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    y = dev(want + 1e-2 * synth.normal(6, "c/guess", want.shape)) if warm else None
+    r, names = launched(bd, lambda: bd.deer_gru_eval(*args, y=y, flags=bd.DEER_FLAG_WARM_START if warm else 0))
+    assert kernel in names, names
+    assert r.status == 0 and r.err <= 1e-4
+    assert np.max(np.abs(r.y.cpu().numpy() - want)) <= 1e-5
+    if not warm:
+        exact = bd.deer_gru_eval(*args, flags=bd.DEER_FLAG_MATERIALIZE)
+        assert abs(r.iters - exact.iters) <= 1, (r.iters, exact.iters)
+
+
 @pytest.mark.parametrize("n,m,B,T", [(1, 1, 16, 300001), (8, 4, 4, 1000), (16, 8, 8, 20000), (24, 3, 2, 700), (32, 8, 16, 8000), (64, 6, 2, 9000)])
 def test_cell_that_remembers_for_long(bd, n, m, B, T):
     """The update gate's bias alone keeps the state: no burn-in is tried, the Jacobians are multiplied out."""
