@@ -5,8 +5,12 @@
 // Chains in lockstep, burn-in and verified boundaries as in newton_body.cuh, in descending time.  The state that a chain
 // carries is mu_t = J_{t+1}^T lambda_{t+1}.  With the gates at t and lambda = gy + mu, the hidden-side gradients of the three
 // pre-activations are p = (k_r.lambda, a_z.lambda, k_n.lambda) -- what dW_h, dW_i, dx are contractions of -- and
-//     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands.
-// All products are 3 x TF32 (a one-shot solve).  lambda has no scale that holds everywhere: a sequence's loss may weigh a
+//     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands
+//                                            (a pair of blocks of eight columns is one K step of 16).
+// All products are at fp32 level (a one-shot solve): three TF32 MMAs on split operands up to n = 16, from there on hi + lo f16
+// halves in three m16n8k16 ones, half as many and good to 2^-23 of the operands where those are to 2^-20.  Powers of two
+// (tile_weight_scale, ADJ_OP_SCALE, and per row and step one from the row's largest |lambda|) keep the halves among the normal
+// numbers; a value beyond f16's range makes a NaN, which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a
 // millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
 // the first one.  So a boundary is held to eta of the largest |lambda| of all and, besides, to ADJ_LOCAL eta of the largest
 // |lambda| just before it, over the last ADJ_WINDOW positions of its successor's burn-in (one position alone may be near zero
@@ -14,18 +18,21 @@
 // largest is some third of the largest of all, so that the first rule decides there.
 // One boundary that differs by more leaves StatusBlock::done at 0: the launches enqueued behind this one (a longer burn-in,
 // then the kernels that multiply the Jacobians out) do the work.
-// What bounds it: the latency of chained mma.sync with eight warps per SM (255 registers a thread).  n = m = 32, B = 16, T = 2e4:
-// tensor pipe 48 % active, issue slots 32 % used, DRAM 15 %; per instruction issued 2.6 warps wait for a fixed latency.
+// What bounds it: the latency of chained mma.sync with eight warps per SM (255 registers a thread).  n = m = 32, B = 16, T = 2e4, in
+// TF32: tensor pipe 48 % active, issue slots 32 % used, DRAM 15 %; per instruction issued 2.6 warps wait for a fixed latency.  With
+// f16 halves T = 1e5 takes 850 us where it took 1100.
 // The boundaries that dy0 can still feel -- those less than DY0_REACH burn-ins from the sequence's first step -- are held to
 // eta * max|dy0| as well.
 #pragma once
 #include "newton_body.cuh"
+#include "split_f16.cuh"
 
 namespace deer {
 
 constexpr int DY0_REACH = 8;     // a burn-in takes an error down by about 1e-6 or more; behind eight of them it is below any fp32
 constexpr int ADJ_WINDOW = 8;    // positions before a boundary whose largest |lambda| is its scale
 constexpr float ADJ_LOCAL = 4.0f;
+constexpr float ADJ_OP_SCALE = 4.0f;         // of x and h: values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute
 static_assert(ADJ_WINDOW <= ADJ_BURN && (ADJ_BURN - ADJ_WINDOW) % 4 == 0, "the window is whole steps of every kernel's burn-in");
 
 // A boundary's mismatch as a part of its scale, as the bits of a non-negative float (a NaN stays above all numbers).
@@ -36,6 +43,13 @@ __device__ __forceinline__ unsigned boundary_ratio(unsigned diff, float scale)
 
 template <int N> struct Adj {
     static constexpr int NT = N / 8;
+    // f16 halves from n = 17 on.  Up to 16 the products are few: their halves' conversions and p's scale, which is in the chain, cost
+    // what half the MMAs give.  (us per gradient, TF32 / f16: n = 16, m = 4, 1.28e6 positions 698 / 720; 30 heads of 16 1486 / 1520,
+    // 32 of 8 2147 / 2191; n = 24, m = 16, 1.6e5 390 / 386; n = m = 32 520 / 448; n = 48, m = 32, 64,000 957 / 660; n = 56, m = 8,
+    // 48,000 1100 / 760.)
+    static constexpr bool F16 = NT > 2;
+    static constexpr int KB = F16 ? 2 : 1;               // column blocks of a K step
+    static constexpr int NB = (NT + KB - 1) / KB, PB = (3 * NT + KB - 1) / KB;       // K steps of h and of p
     static constexpr int NS = 3 * N + 2, NS2 = N + 2;    // = 2 (mod 8) records
     static constexpr int SW = N + 4;
     static constexpr bool SS_GLOBAL = N > 48;            // start states in the workspace: the weights of both contractions fill
@@ -43,7 +57,7 @@ template <int N> struct Adj {
     static constexpr size_t smem(int warps, int kx)
     {
         if (SS_GLOBAL) warps = 0;
-        return sizeof(float) * ((size_t)4 * (N / 2 + 4 * kx) * NS + (size_t)4 * (3 * N / 2) * NS2 + 4 * N + (size_t)warps * 16 * SW);
+        return sizeof(float) * ((size_t)16 * (NB + (kx + KB - 1) / KB) * NS + (size_t)16 * PB * NS2 + 4 * N + (size_t)warps * 16 * SW);
     }
 };
 
@@ -77,13 +91,15 @@ template <int N, bool V2>
 __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 3) newton_adjoint_kernel(AdjArgs a)
 {
     using C = Adj<N>;
-    constexpr int NT = C::NT, NS = C::NS, NS2 = C::NS2, SW = C::SW;
+    constexpr int NT = C::NT, KB = C::KB, NB = C::NB, PB = C::PB, NS = C::NS, NS2 = C::NS2, SW = C::SW;
+    constexpr bool F16 = C::F16;
     extern __shared__ __align__(16) float smb[];
+    __shared__ unsigned s_top;
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
     const int n = a.n, m = a.m, H = a.H, L = a.L;
     const bool proj = a.u == nullptr;
-    const int kx = proj ? (m + 7) >> 3 : 0;
+    const int kx = proj ? (m + 8 * KB - 1) / (8 * KB) : 0;               // K steps of x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
 
@@ -94,29 +110,42 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     const unsigned nctas = (unsigned)((groups + nwarps - 1) / nwarps);
     if (blockIdx.x >= nctas) return;
 
-    // ---- weights into shared memory as records {hi(W[c][2p]), hi(W[c][2p+1]), lo, lo}: the B operand of one column block
-    // of one K step is one 128-bit load (weights are not produced by the previous launch: this runs before its end)
-    float4 *sH = reinterpret_cast<float4 *>(smb), *sI = sH + (N / 2) * NS;
-    float4 *sT = sI + 4 * kx * NS;                       // W_h by pairs of rows: the B operand of p W_h
-    float *sb = reinterpret_cast<float *>(sT + (3 * N / 2) * NS2);
-    auto lo = [](float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
-    for (int idx = tid; idx < (N / 2) * 3 * N; idx += blockDim.x) {
-        const int kp = idx % (N / 2), c = idx / (N / 2), gate = c / N, i = c % N;
-        const float *wr = hd.W_h + (size_t)(gate * n + i) * n + 2 * kp;
-        const float v0 = i < n && 2 * kp < n ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < n ? wr[1] : 0.0f;
-        sH[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    // ---- weights into shared memory as records of the four words that a lane needs for a column of a K step: hi of rows 2t, 2t + 1
+    // (and 2t + 8, 2t + 9), and lo of the same: one 128-bit load (weights are not produced by the previous launch: this runs
+    // before its end)
+    uint4 *sH = reinterpret_cast<uint4 *>(smb), *sI = sH + 4 * NB * NS;
+    uint4 *sT = sI + 4 * kx * NS;                        // W_h by rows: the B operand of p W_h
+    float *sb = reinterpret_cast<float *>(sT + 4 * PB * NS2);
+    float wscale = 1.0f, kS = 1.0f;
+    if constexpr (F16) {
+        wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
+        kS = 1.0f / (wscale * ADJ_OP_SCALE);
+    }
+    auto record = [&](auto w, int kt) {                  // w(k): row k of the column
+        const int k = 8 * KB * (kt >> 2) + 2 * (kt & 3);
+        uint4 r;
+        if constexpr (F16) {
+            split_f16(make_float2(w(k) * wscale, w(k + 1) * wscale), r.x, r.z);
+            split_f16(make_float2(w(k + 8) * wscale, w(k + 9) * wscale), r.y, r.w);
+        } else {
+            split_tf32(w(k), r.x, r.z);
+            split_tf32(w(k + 1), r.y, r.w);
+        }
+        return r;
+    };
+    for (int idx = tid; idx < 4 * NB * 3 * N; idx += blockDim.x) {
+        const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
+        const float *wr = hd.W_h + (size_t)(gate * n + i) * n;
+        sH[kt * NS + c] = record([&](int j) { return i < n && j < n ? wr[j] : 0.0f; }, kt);
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
-        const int kp = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
-        const float *wr = hd.W_i + (size_t)(gate * n + i) * m + 2 * kp;
-        const float v0 = i < n && 2 * kp < m ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < m ? wr[1] : 0.0f;
-        sI[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+        const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
+        const float *wr = hd.W_i + (size_t)(gate * n + i) * m;
+        sI[kt * NS + c] = record([&](int j) { return i < n && j < m ? wr[j] : 0.0f; }, kt);
     }
-    for (int idx = tid; idx < (3 * N / 2) * N; idx += blockDim.x) {
-        const int c = idx % N, kp = idx / N, gate = 2 * kp / N, i = 2 * kp % N;
-        const float v0 = c < n && i < n ? hd.W_h[(size_t)(gate * n + i) * n + c] : 0.0f;
-        const float v1 = c < n && i + 1 < n ? hd.W_h[(size_t)(gate * n + i + 1) * n + c] : 0.0f;
-        sT[kp * NS2 + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    for (int idx = tid; idx < 4 * PB * N; idx += blockDim.x) {
+        const int c = idx % N, kt = idx / N;
+        sT[kt * NS2 + c] = record([&](int j) { return j < 3 * N && j % N < n && c < n ? hd.W_h[(size_t)(j / N * n + j % N) * n + c] : 0.0f; }, kt);
     }
     for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
         sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
@@ -236,6 +265,24 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
         float ur_n[U_AHEAD ? NT : 1][4], uz_n[U_AHEAD ? NT : 1][4], un_n[U_AHEAD ? NT : 1][4];
         if constexpr (U_AHEAD) { if (!proj) load_u(ur_n, uz_n, un_n, 0); }
 
+        // block b of a K step of an A operand, row h of this lane: two columns (an accumulator's columns of TF32 in the slots t, t + 4)
+        auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v, float scale) {
+            if constexpr (F16) {
+                split_f16(fmul2(v, make_float2(scale, scale)), hi[2 * b + h], lo[2 * b + h]);
+            } else {
+                split_tf32(v.x, hi[h], lo[h]);
+                split_tf32(v.y, hi[2 + h], lo[2 + h]);
+            }
+        };
+        auto mma = [&](float (&acc)[4], const unsigned (&x)[4], unsigned w0, unsigned w1) {
+            if constexpr (F16) {
+                mma_f16(acc, x, w0, w1);
+            } else {
+                const unsigned w[2] = {w0, w1};
+                mma_tf32(acc, x, w, acc);
+            }
+        };
+
 #pragma unroll 1
         for (int step = s_first; step < s_end; ++step) {
             // (mu stands for lambda = gy + mu in the window: work for eight steps instead of for every one, under the branch that the
@@ -267,32 +314,28 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) { xr[j][q] = 0.0f; xz[j][q] = 0.0f; xn[j][q] = 0.0f; }
-                float2 x0 = act[0] ? ldx(xp[0], 2 * t) : make_float2(0.0f, 0.0f);
-                float2 x1 = act[1] ? ldx(xp[1], 2 * t) : make_float2(0.0f, 0.0f);
+                auto ldxs = [&](int k, float2 (&v)[2 * KB]) {    // rows g, g + 8 at columns 2t .. (and 2t + 8 ..)
+#pragma unroll
+                    for (int q = 0; q < 2 * KB; ++q) v[q] = act[q & 1] ? ldx(xp[q & 1], 8 * KB * k + 8 * (q >> 1) + 2 * t) : make_float2(0.0f, 0.0f);
+                };
+                float2 xc[2 * KB];
+                ldxs(0, xc);
 #pragma unroll 1
                 for (int kk = 0; kk < kx; ++kk) {
                     unsigned ah[4], al[4];
-                    split_tf32(x0.x, ah[0], al[0]);
-                    split_tf32(x1.x, ah[1], al[1]);
-                    split_tf32(x0.y, ah[2], al[2]);
-                    split_tf32(x1.y, ah[3], al[3]);
-                    if (kk + 1 < kx) {
-                        x0 = act[0] ? ldx(xp[0], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
-                        x1 = act[1] ? ldx(xp[1], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
-                    }
-                    const float4 *q0 = sI + (4 * kk + t) * NS + g;
+#pragma unroll
+                    for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], ADJ_OP_SCALE);
+                    if (kk + 1 < kx) ldxs(kk + 1, xc);
+                    const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
                     for (int j = 0; j < NT; ++j) {
-                        {
 #pragma unroll
-                            for (int gate = 0; gate < 3; ++gate) {
-                                const float4 w = q0[gate * N + 8 * j];
-                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                                float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
-                                mma_tf32(acc, al, bh, acc);
-                                mma_tf32(acc, ah, bl, acc);
-                                mma_tf32(acc, ah, bh, acc);
-                            }
+                        for (int gate = 0; gate < 3; ++gate) {
+                            const uint4 w = q0[gate * N + 8 * j];
+                            float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
+                            mma(acc, al, w.x, w.y);
+                            mma(acc, ah, w.z, w.w);
+                            mma(acc, ah, w.x, w.y);
                         }
                     }
                 }
@@ -305,49 +348,81 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
             } else {
                 load_u(xr, xz, xn, 0);
             }
+            if (F16 && !proj) {                          // (in the products' scale: a power of two)
+                const float up = wscale * ADJ_OP_SCALE;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+            }
+            // the state as A operands, and the power of two of p: |p| <= |lambda| / 4 or so, its exponent to 2^9 in every row
+            unsigned ah[NB][4], al[NB][4];
+            if constexpr (F16 && NT % 2) {
+#pragma unroll
+                for (int q = 2; q < 4; ++q) { ah[NB - 1][q] = 0u; al[NB - 1][q] = 0u; }
+            }
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]), ADJ_OP_SCALE);
+            float sc[2] = {1.0f, 1.0f}, kM[2] = {1.0f, 1.0f};
+            if constexpr (F16) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    unsigned q = 0u;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+                        q = max(q, max(__float_as_uint(fabsf(gy[j][2 * h] + d[j][2 * h])), __float_as_uint(fabsf(gy[j][2 * h + 1] + d[j][2 * h + 1]))));
+                    q = max(q, __shfl_xor_sync(0xffffffffu, q, 1));
+                    q = max(q, __shfl_xor_sync(0xffffffffu, q, 2));
+                    const int ex = min(max((int)(q >> 23), 20), 240);
+                    sc[h] = __uint_as_float((unsigned)(127 + 9 - (ex - 127)) << 23);
+                    kM[h] = __uint_as_float((unsigned)(127 - 9 + (ex - 127)) << 23) / wscale;
+                }
+            }
             // ---- hidden half, gates, lambda and the pre-activation gradients, one block of eight columns at a time
-            float p[3][NT][4], zl[NT][4];
+            unsigned ph[PB][4], pl[PB][4];               // p as A operands: block gate * NT + j of eight columns
+            if constexpr (F16 && 3 * NT % 2) {
+#pragma unroll
+                for (int q = 2; q < 4; ++q) { ph[PB - 1][q] = 0u; pl[PB - 1][q] = 0u; }
+            }
+            float zl[NT][4];
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 float (&hr)[4] = xr[j], (&hz)[4] = xz[j];
                 float hq[4] = {0.f, 0.f, 0.f, 0.f};
-                const float4 *q0 = sH + t * NS + 8 * j + g;
+                const uint4 *q0 = sH + t * NS + 8 * j + g;
 #pragma unroll
-                for (int kk = 0; kk < NT; ++kk) {
-                    unsigned ah[4], al[4];
-                    split_tf32(hp[kk][0], ah[0], al[0]); split_tf32(hp[kk][2], ah[1], al[1]);
-                    split_tf32(hp[kk][1], ah[2], al[2]); split_tf32(hp[kk][3], ah[3], al[3]);
+                for (int kk = 0; kk < NB; ++kk)
 #pragma unroll
                     for (int gate = 0; gate < 3; ++gate) {
-                        const float4 w = q0[4 * kk * NS + gate * N];
-                        const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
+                        const uint4 w = q0[4 * kk * NS + gate * N];
                         float (&acc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
-                        mma_tf32(acc, al, bh, acc);
-                        mma_tf32(acc, ah, bl, acc);
-                        mma_tf32(acc, ah, bh, acc);
+                        mma(acc, al[kk], w.x, w.y);
+                        mma(acc, ah[kk], w.z, w.w);
+                        mma(acc, ah[kk], w.x, w.y);
                     }
-                }
                 const int col = 8 * j + 2 * t;
                 const float2 bR = *reinterpret_cast<const float2 *>(sb + col), bZ = *reinterpret_cast<const float2 *>(sb + N + col);
                 const float2 bQ = *reinterpret_cast<const float2 *>(sb + 2 * N + col), bN = *reinterpret_cast<const float2 *>(sb + 3 * N + col);
-                const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f);
+                const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f), k2 = make_float2(kS, kS);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float2 h2 = make_float2(hp[j][2 * h], hp[j][2 * h + 1]);
                     const float2 l2 = fadd2(make_float2(gy[j][2 * h], gy[j][2 * h + 1]), make_float2(d[j][2 * h], d[j][2 * h + 1]));
-                    const float2 q = fadd2(make_float2(hq[2 * h], hq[2 * h + 1]), bQ);
-                    const float2 r = sigmoid2_gate(fadd2(make_float2(hr[2 * h], hr[2 * h + 1]), bR));
-                    const float2 z = sigmoid2_gate(fadd2(make_float2(hz[2 * h], hz[2 * h + 1]), bZ));
-                    const float2 c = tanh2_gate(ffma2(r, q, fadd2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), bN)));
+                    const float2 q = ffma2(make_float2(hq[2 * h], hq[2 * h + 1]), k2, bQ);
+                    const float2 r = sigmoid2_gate(ffma2(make_float2(hr[2 * h], hr[2 * h + 1]), k2, bR));
+                    const float2 z = sigmoid2_gate(ffma2(make_float2(hz[2 * h], hz[2 * h + 1]), k2, bZ));
+                    const float2 c = tanh2_gate(ffma2(r, q, ffma2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), k2, bN)));
                     const float2 omz = ffma2(z, mone, one), omr = ffma2(r, mone, one);
                     const float2 pz = fmul2(fmul2(fmul2(ffma2(c, mone, h2), z), omz), l2);
                     const float2 pa = fmul2(fmul2(omz, ffma2(fmul2(c, mone), c, one)), l2);          // w.r.t. W_in x + b_in
                     const float2 pn = fmul2(pa, r);                                                  // w.r.t. W_hn h + b_hn
                     const float2 pr = fmul2(fmul2(pn, q), omr);
                     const float2 zz = fmul2(z, l2);
-                    p[0][j][2 * h] = pr.x; p[0][j][2 * h + 1] = pr.y;
-                    p[1][j][2 * h] = pz.x; p[1][j][2 * h + 1] = pz.y;
-                    p[2][j][2 * h] = pn.x; p[2][j][2 * h + 1] = pn.y;
+                    const float2 pg[3] = {pr, pz, pn};
+#pragma unroll
+                    for (int gate = 0; gate < 3; ++gate) operand(ph[(gate * NT + j) / KB], pl[(gate * NT + j) / KB], (gate * NT + j) % KB, h, pg[gate], sc[h]);
                     zl[j][2 * h] = zz.x; zl[j][2 * h + 1] = zz.y;
                     if (step >= burn && act[h]) {
                         if (col < n) mb = max(mb, __float_as_uint(fabsf(l2.x)));
@@ -373,23 +448,17 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
             if (step + 1 < s_end) { load_h(hp); load_g(gy); }
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
-                float acc[4] = {zl[j][0], zl[j][1], zl[j][2], zl[j][3]}, cr[4] = {0.f, 0.f, 0.f, 0.f};
-                const float4 *q0 = sT + t * NS2 + 8 * j + g;
+                float acc[4] = {0.f, 0.f, 0.f, 0.f}, cr[4] = {0.f, 0.f, 0.f, 0.f};
+                const uint4 *q0 = sT + t * NS2 + 8 * j + g;
 #pragma unroll
-                for (int gate = 0; gate < 3; ++gate)
+                for (int kk = 0; kk < PB; ++kk) {
+                    const uint4 w = q0[4 * kk * NS2];
+                    mma(cr, pl[kk], w.x, w.y);
+                    mma(cr, ph[kk], w.z, w.w);
+                    mma(acc, ph[kk], w.x, w.y);
+                }
 #pragma unroll
-                    for (int kk = 0; kk < NT; ++kk) {
-                        unsigned ph[4], pl[4];
-                        split_tf32(p[gate][kk][0], ph[0], pl[0]); split_tf32(p[gate][kk][2], ph[1], pl[1]);
-                        split_tf32(p[gate][kk][1], ph[2], pl[2]); split_tf32(p[gate][kk][3], ph[3], pl[3]);
-                        const float4 w = q0[(gate * N / 2 + 4 * kk) * NS2];
-                        const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                        mma_tf32(cr, pl, bh, cr);
-                        mma_tf32(cr, ph, bl, cr);
-                        mma_tf32(acc, ph, bh, acc);
-                    }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? acc[q] + cr[q] : d[j][q];
+                for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? fmaf(acc[q] + cr[q], kM[q >> 1], zl[j][q]) : d[j][q];
             }
         }
         // ---- the state that leaves the first time step: the gradient w.r.t. y0 (wanted or not, it shows what is not finite there)

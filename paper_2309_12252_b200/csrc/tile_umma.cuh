@@ -2,7 +2,7 @@
 // (K-major, SWIZZLE_128B panels of 64 columns), fp32 accumulators in tensor memory.
 #pragma once
 #include "scan_onepass.cuh"
-#include <cuda_fp16.h>
+#include "split_f16.cuh"
 
 namespace deer {
 
@@ -106,37 +106,6 @@ __device__ __forceinline__ bool tile_wait(uint64_t *bar, unsigned phase)
         if (ok) return true;
     }
     return false;
-}
-
-// hi and lo halves of a pair as packed f16: x = hi + lo to 2^-23 of x, or 2^-25 where lo is subnormal (|x| below 2^-2; values up
-// to 65504)
-__device__ __forceinline__ void split_f16(float2 x, unsigned &hi, unsigned &lo)
-{
-    const __half2 h = __float22half2_rn(x);
-    const __half2 l = __float22half2_rn(ffma2(__half22float2(h), make_float2(-1.0f, -1.0f), x));
-    hi = *reinterpret_cast<const unsigned *>(&h);
-    lo = *reinterpret_cast<const unsigned *>(&l);
-}
-__device__ __forceinline__ unsigned pack_f16(float2 x)
-{
-    const __half2 h = __float22half2_rn(x);
-    return *reinterpret_cast<const unsigned *>(&h);
-}
-
-// The power of two that brings the largest of `count` weights (and of a second array) to [2^9, 2^10): with it the lo halves
-// of all but the very smallest are normal f16 numbers.  All threads of the CTA; red: one word.
-__device__ __forceinline__ float tile_weight_scale(const float *w0, int n0, const float *w1, int n1, unsigned *red)
-{
-    unsigned top = 0u;
-    for (int i = threadIdx.x; i < n0; i += blockDim.x) top = max(top, __float_as_uint(fabsf(w0[i])));
-    for (int i = threadIdx.x; i < n1; i += blockDim.x) top = max(top, __float_as_uint(fabsf(w1[i])));
-    if (threadIdx.x == 0) *red = 0u;
-    __syncthreads();
-    top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) atomicMax(red, top);
-    __syncthreads();
-    const int e = min(max((int)(*red >> 23), 40), 220);          // (zero, or beyond any use: the scale stays finite)
-    return __uint_as_float((unsigned)(127 + 9 - (e - 127)) << 23);
 }
 
 }  // namespace deer

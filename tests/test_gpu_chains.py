@@ -444,3 +444,26 @@ def test_scan_of_unequal_but_coupled_components_is_taken(bd):
     assert "scan_verified_kernel" in names and not names & {WARP, MMA_TILE} and done == 1, names
     for k in ("dW_i", "dW_h", "db_i", "db_h", "dx", "dy0"):
         assert np.max(np.abs(got[k] - want[k])) <= 2e-5 * np.max(np.abs(want[k])), k
+
+
+@pytest.mark.parametrize("n,m,B,T,gy_scale,x_scale,kernel", [
+    (9, 3, 40, 700, 1.0, 1.0, WARP), (16, 3, 16, 10001, 1.0, 1.0, WARP), (17, 16, 16, 700, 1.0, 1.0, WARP), (24, 33, 16, 700, 1e-25, 1.0, WARP),
+    (32, 1, 16, 8001, 1e25, 1.0, WARP), (33, 64, 16, 1000, 1.0, 1.0, WARP), (48, 2, 16, 500, 1.0, 1.0, WARP), (57, 15, 16, 300, 1.0, 1.0, WARP),
+    (63, 8, 16, 300, 1.0, 1.0, WARP), (24, 4, 16, 700, 1.0, 3000.0, WARP), (24, 4, 16, 700, 1.0, 2e4, None), (8, 16, 16, 30001, 1.0, 1.0, WARP)])
+def test_adjoint_products_are_at_fp32_level(bd, n, m, B, T, gy_scale, x_scale, kernel):
+    """K steps of 16 with and without their second half, gradients of any magnitude, inputs up to and beyond what the products'
+    halves hold.  A product is good to 2^-22 of its operands and a lambda carries the errors of some ten steps: 2-norms agree to
+    1e-6.  (An input beyond the halves' range is for the kernels behind, and saturates the gates: their 1e-3.)"""
+    p = synth.gru_params(n, m, 8, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, 8, tag="c/x")
+    x[:, :, 0] = np.clip(x[:, :, 0], -4, 4) * np.float32(x_scale)
+    y0 = synth.normal(8, "c/y0", (B, n)) * 0.3
+    y = oracle.gru_seq(p, x, y0, np.float32)
+    gy = (synth.normal(8, "c/gy", (B, T, n)).astype(np.float64) * gy_scale).astype(np.float32)
+    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
+    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True))
+    assert kernel is None or kernel in names, names
+    for k in ("db_i", "db_h", "dx", "dy0"):
+        a, b = got[k].cpu().numpy().astype(np.float64), want[k].astype(np.float64)
+        assert np.linalg.norm(a - b) <= (1e-6 if x_scale == 1.0 else 1e-3) * np.linalg.norm(b), k
