@@ -9,7 +9,7 @@
 //                                            (a pair of blocks of eight columns is one K step of 16).
 // All products are at fp32 level (a one-shot solve): three TF32 MMAs on split operands up to n = 16, from there on hi + lo f16
 // halves in three m16n8k16 ones, half as many and good to 2^-23 of the operands where those are to 2^-20.  Powers of two
-// (tile_weight_scale, ADJ_OP_SCALE, and per row and step one from the row's largest |lambda|) keep the halves among the normal
+// (tile_weight_scale, MMA_OP_SCALE, and per row and step one from the row's largest |lambda|) keep the halves among the normal
 // numbers; a value beyond f16's range makes a NaN, which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a
 // millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
 // the first one.  So a boundary is held to eta of the largest |lambda| of all and, besides, to ADJ_LOCAL eta of the largest
@@ -25,14 +25,12 @@
 // eta * max|dy0| as well.
 #pragma once
 #include "newton_body.cuh"
-#include "split_f16.cuh"
 
 namespace deer {
 
 constexpr int DY0_REACH = 8;     // a burn-in takes an error down by about 1e-6 or more; behind eight of them it is below any fp32
 constexpr int ADJ_WINDOW = 8;    // positions before a boundary whose largest |lambda| is its scale
 constexpr float ADJ_LOCAL = 4.0f;
-constexpr float ADJ_OP_SCALE = 4.0f;         // of x and h: values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute
 static_assert(ADJ_WINDOW <= ADJ_BURN && (ADJ_BURN - ADJ_WINDOW) % 4 == 0, "the window is whole steps of every kernel's burn-in");
 
 // A boundary's mismatch as a part of its scale, as the bits of a non-negative float (a NaN stays above all numbers).
@@ -119,7 +117,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     float wscale = 1.0f, kS = 1.0f;
     if constexpr (F16) {
         wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
-        kS = 1.0f / (wscale * ADJ_OP_SCALE);
+        kS = 1.0f / (wscale * MMA_OP_SCALE);
     }
     auto record = [&](auto w, int kt) {                  // w(k): row k of the column
         const int k = 8 * KB * (kt >> 2) + 2 * (kt & 3);
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 for (int kk = 0; kk < kx; ++kk) {
                     unsigned ah[4], al[4];
 #pragma unroll
-                    for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], ADJ_OP_SCALE);
+                    for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], MMA_OP_SCALE);
                     if (kk + 1 < kx) ldxs(kk + 1, xc);
                     const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
@@ -349,7 +347,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 load_u(xr, xz, xn, 0);
             }
             if (F16 && !proj) {                          // (in the products' scale: a power of two)
-                const float up = wscale * ADJ_OP_SCALE;
+                const float up = wscale * MMA_OP_SCALE;
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -364,7 +362,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]), ADJ_OP_SCALE);
+                for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]), MMA_OP_SCALE);
             float sc[2] = {1.0f, 1.0f}, kM[2] = {1.0f, 1.0f};
             if constexpr (F16) {
 #pragma unroll

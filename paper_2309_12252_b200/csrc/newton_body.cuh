@@ -3,11 +3,12 @@
 //
 // The update solves d_t = J_t d_{t-1} + r_t, r_t = f(y_{t-1}, x_t) - y_t.  The sequences are cut into chains of L
 // positions; sixteen chains advance in lockstep as the sixteen rows of a warp's m16n8k8 MMAs, a step being
-//     [16, m] x [m, 3n] + [16, n] x [n, 3n]      gates: 3 x TF32, so f is good to fp32 level
+//     [16, m] x [m, 3n] + [16, n] x [n, 3n]      gates: hi + lo f16 halves in three MMAs, so f is good to fp32 level
 //     [16, n] x [n, 3n]                          J_t d_{t-1} = z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d)
-// with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragment of one step is the A
-// operand of the next by renaming the contraction index (slots t, t + 4 of a K step hold columns 2t, 2t + 1), so
-// neither J_t, nor its coefficients, nor any chain product is ever formed or stored.
+// with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragments of two blocks of eight
+// columns are the A operand of a K step of 16 as they stand, so neither J_t, nor its coefficients, nor any chain product
+// is ever formed or stored.  Powers of two (tile_weight_scale, MMA_OP_SCALE, MMA_D_SCALE) keep the halves among the normal
+// f16 numbers; a value beyond f16's range makes a NaN, and the body is for the other kernels.
 //
 // What a chain does not know is the update entering it.  It starts `burn` positions early from zero: the error of its
 // entering update is the old error carried through `burn` Jacobians, and the Jacobians of a cell that forgets make it
@@ -23,6 +24,7 @@
 #pragma once
 #include "mma_tf32.cuh"
 #include "newton_body.h"
+#include "split_f16.cuh"
 
 namespace deer {
 
@@ -86,11 +88,17 @@ __device__ __forceinline__ BodyVerdict body_verdict(float e, float mis, float et
 }
 
 // End of a body that is a launch of its own: the last CTA's decision.  unit: what the launch rounds its burn-in up to
-// (a rate that is not adapted to may be underestimated).  Single thread.
-__device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, int unit = 1, float rounding = 0.0f)
+// (a rate that is not adapted to may be underestimated); narrow: its products hold what f16 does.  Single thread.
+__device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, int unit = 1, float rounding = 0.0f, bool narrow = false)
 {
     const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits);
     const float mis = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
+    if (narrow && (!(e <= 3.402823466e38f) || !(mis <= 3.402823466e38f))) {        // beyond f16's range, or not finite at all: the other kernels tell
+        st->err_bits = 0u; st->mis_bits = 0u;
+        st->done = BODY_FALL_BACK;
+        if (HostResult *h = st->host) post_done(h, BODY_FALL_BACK);
+        return;
+    }
     const BodyVerdict v = body_verdict(e, mis, a.eta, a.adapt ? (st->burn + unit - 1) / unit * unit : st->burn, a.burn_cap, a.T, st->tol, st->iters, st->max_iter, a.adapt != 0, rounding);
     st->mis_bits = 0u;
     if (v.need) st->need = max(st->need, v.need);
@@ -102,29 +110,34 @@ __device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, 
     if (HostResult *h = st->host) { h->burn = v.burn; if (v.done) post_done(h, v.done); }
 }
 
+// Scales of x and the states (values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute) and of the update (up to 64;
+// 2^-35 absolute) as f16 operands.
+constexpr float MMA_OP_SCALE = 4.0f, MMA_D_SCALE = 1024.0f;
+
 template <int N> struct Body {
-    static constexpr int NT = N / 8;
-    static constexpr int NS = 3 * N + 2;                 // records per pair of contraction rows: = 2 (mod 8), conflict-free
+    static constexpr int NT = N / 8, NB = (NT + 1) / 2;  // column blocks, K steps
+    static constexpr int NS = 3 * N + 2;                 // records per lane of a K step: = 2 (mod 8), conflict-free
     static constexpr int SW = N + 4;                     // stride of a saved start state
     static constexpr size_t smem(int warps, int kx)      // kx: 8-column blocks of x contracted in the kernel
     {
-        return sizeof(float) * ((size_t)4 * (N / 2 + 4 * kx) * NS + 4 * N + (size_t)warps * 16 * SW);
+        return sizeof(float) * ((size_t)16 * (NB + (kx + 1) / 2) * NS + 4 * N + (size_t)warps * 16 * SW);
     }
 };
 
-// EXACT: the products with d are 3 x TF32 as well (sizes whose solve has always been fp32-accurate); V2: rows are read and
+// EXACT: the products with d are three MMAs as well (sizes whose solve has always been fp32-accurate); V2: rows are read and
 // written as 8-byte pairs.  n <= 8 takes a thread per chain instead (newton_lane.cuh).
 template <int N, bool V2, bool EXACT>
 __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_body_kernel(BodyArgs a)
 {
     using C = Body<N>;
-    constexpr int NT = C::NT, NS = C::NS, SW = C::SW;
+    constexpr int NT = C::NT, NB = C::NB, NS = C::NS, SW = C::SW;
     extern __shared__ __align__(16) float smb[];
+    __shared__ unsigned s_top;
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
     const int n = a.n, m = a.m, H = a.H, L = a.L;
     const bool proj = a.u == nullptr;
-    const int kx = proj ? (m + 7) >> 3 : 0;
+    const int kx = proj ? (m + 15) >> 4 : 0;             // K steps of x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
 
@@ -135,22 +148,28 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
     const unsigned nctas = (unsigned)((groups + nwarps - 1) / nwarps);
     if (blockIdx.x >= nctas) return;
 
-    // ---- weights into shared memory as records {hi(W[c][2p]), hi(W[c][2p+1]), lo, lo}: the B operand of one column block
-    // of one K step is one 128-bit load (weights are not produced by the previous launch: this runs before its end)
-    float4 *sH = reinterpret_cast<float4 *>(smb), *sI = sH + (N / 2) * NS;
-    float *sb = smb + 4 * (size_t)(N / 2 + 4 * kx) * NS;
-    auto lo = [](float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
-    for (int idx = tid; idx < (N / 2) * 3 * N; idx += blockDim.x) {
-        const int kp = idx % (N / 2), c = idx / (N / 2), gate = c / N, i = c % N;
-        const float *wr = hd.W_h + (size_t)(gate * n + i) * n + 2 * kp;
-        const float v0 = i < n && 2 * kp < n ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < n ? wr[1] : 0.0f;
-        sH[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    // ---- weights into shared memory as records of the four words that a lane needs for a column of a K step: hi of rows 2t, 2t + 1
+    // and 2t + 8, 2t + 9, and lo of the same: one 128-bit load (weights are not produced by the previous launch: this runs before
+    // its end)
+    uint4 *sH = reinterpret_cast<uint4 *>(smb), *sI = sH + 4 * NB * NS;
+    float *sb = reinterpret_cast<float *>(sI + 4 * kx * NS);
+    const float wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
+    const float kS = 1.0f / (wscale * MMA_OP_SCALE), kD = 1.0f / (wscale * MMA_D_SCALE);
+    auto record = [&](const float *wr, bool row, int kt, int width) {
+        const int k = 16 * (kt >> 2) + 2 * (kt & 3);
+        auto w = [&](int j) { return row && j < width ? wr[j] * wscale : 0.0f; };
+        uint4 r;
+        split_f16(make_float2(w(k), w(k + 1)), r.x, r.z);
+        split_f16(make_float2(w(k + 8), w(k + 9)), r.y, r.w);
+        return r;
+    };
+    for (int idx = tid; idx < 4 * NB * 3 * N; idx += blockDim.x) {
+        const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
+        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n);
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
-        const int kp = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
-        const float *wr = hd.W_i + (size_t)(gate * n + i) * m + 2 * kp;
-        const float v0 = i < n && 2 * kp < m ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < m ? wr[1] : 0.0f;
-        sI[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+        const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
+        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m);
     }
     for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
         sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
@@ -271,34 +290,29 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) { xr[j][q] = 0.0f; xz[j][q] = 0.0f; xn[j][q] = 0.0f; }
-                float2 x0 = act[0] ? ldx(xp[0], 2 * t) : make_float2(0.0f, 0.0f);
-                float2 x1 = act[1] ? ldx(xp[1], 2 * t) : make_float2(0.0f, 0.0f);
+                auto ldxs = [&](int k, float2 (&v)[4]) {         // rows g, g + 8 at columns 2t .. and 2t + 8 ..
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = act[q & 1] ? ldx(xp[q & 1], 16 * k + 8 * (q >> 1) + 2 * t) : make_float2(0.0f, 0.0f);
+                };
+                float2 xc[4];
+                ldxs(0, xc);
 #pragma unroll 1
                 for (int kk = 0; kk < kx; ++kk) {
                     unsigned ah[4], al[4];
-                    split_tf32(x0.x, ah[0], al[0]);
-                    split_tf32(x1.x, ah[1], al[1]);
-                    split_tf32(x0.y, ah[2], al[2]);
-                    split_tf32(x1.y, ah[3], al[3]);
-                    if (kk + 1 < kx) {
-                        x0 = act[0] ? ldx(xp[0], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
-                        x1 = act[1] ? ldx(xp[1], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
-                    }
-                    const float4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
-                    for (int j = 0; j < NT; ++j) {
-                        {
+                    for (int q = 0; q < 4; ++q) split_f16(fmul2(xc[q], make_float2(MMA_OP_SCALE, MMA_OP_SCALE)), ah[q], al[q]);
+                    if (kk + 1 < kx) ldxs(kk + 1, xc);
+                    const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
-                            for (int gate = 0; gate < 3; ++gate) {
-                                const float4 w = q0[gate * N + 8 * j];
-                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                                float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
-                                mma_tf32(acc, al, bh, acc);
-                                mma_tf32(acc, ah, bl, acc);
-                                mma_tf32(acc, ah, bh, acc);
-                            }
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int gate = 0; gate < 3; ++gate) {
+                            const uint4 w = q0[gate * N + 8 * j];
+                            float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
+                            mma_f16(acc, al, w.x, w.y);
+                            mma_f16(acc, ah, w.z, w.w);
+                            mma_f16(acc, ah, w.x, w.y);
                         }
-                    }
                 }
             } else if constexpr (U_AHEAD) {              // (requested a step ago; the next one's now)
 #pragma unroll
@@ -309,54 +323,68 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
             } else {
                 load_u(xr, xz, xn, 0);
             }
+            if (!proj) {                                 // (in the products' scale: a power of two)
+                const float up = wscale * MMA_OP_SCALE;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+            }
             // ---- hidden half and the update, one block of eight columns at a time
             const bool hid = !zero || __any_sync(0xffffffffu, tt[0] == 0 || tt[1] == 0);     // zero guess: W_h 0 = 0
+            unsigned ah[NB][4], al[NB][4], dh[NB][4], dl[NB][4];
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int j = 2 * k + (q >> 1), e = 2 * (q & 1);
+                    if (j < NT) {
+                        const int jj = j < NT ? j : 0;
+                        split_f16(fmul2(make_float2(hp[jj][e], hp[jj][e + 1]), make_float2(MMA_OP_SCALE, MMA_OP_SCALE)), ah[k][q], al[k][q]);
+                        const float2 ds = fmul2(make_float2(d[jj][e], d[jj][e + 1]), make_float2(MMA_D_SCALE, MMA_D_SCALE));
+                        if constexpr (EXACT) split_f16(ds, dh[k][q], dl[k][q]);
+                        else { dh[k][q] = pack_f16(ds); dl[k][q] = 0u; }
+                    } else {
+                        ah[k][q] = 0u; al[k][q] = 0u; dh[k][q] = 0u; dl[k][q] = 0u;
+                    }
+                }
             float dn[NT][4];
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 {
                     float hr[4] = {xr[j][0], xr[j][1], xr[j][2], xr[j][3]}, hz[4] = {xz[j][0], xz[j][1], xz[j][2], xz[j][3]};
                     float hq[4] = {0.f, 0.f, 0.f, 0.f}, ur[4] = {0.f, 0.f, 0.f, 0.f}, uz[4] = {0.f, 0.f, 0.f, 0.f}, un[4] = {0.f, 0.f, 0.f, 0.f};
-                    const float4 *q0 = sH + t * NS + 8 * j + g;
+                    const uint4 *q0 = sH + t * NS + 8 * j + g;
 #pragma unroll
-                    for (int kk = 0; kk < NT; ++kk) {
-                        {
-                            unsigned ah[4], al[4], dh[4], dl[4];
-                            split_tf32(d[kk][0], dh[0], dl[0]); split_tf32(d[kk][2], dh[1], dl[1]);
-                            split_tf32(d[kk][1], dh[2], dl[2]); split_tf32(d[kk][3], dh[3], dl[3]);
-                            split_tf32(hp[kk][0], ah[0], al[0]); split_tf32(hp[kk][2], ah[1], al[1]);
-                            split_tf32(hp[kk][1], ah[2], al[2]); split_tf32(hp[kk][3], ah[3], al[3]);
+                    for (int kk = 0; kk < NB; ++kk)
 #pragma unroll
-                            for (int gate = 0; gate < 3; ++gate) {
-                                const float4 w = q0[4 * kk * NS + gate * N];
-                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                                float (&hacc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
-                                float (&uacc)[4] = gate == 0 ? ur : gate == 1 ? uz : un;
-                                if (hid) {
-                                    mma_tf32(hacc, al, bh, hacc);
-                                    mma_tf32(hacc, ah, bl, hacc);
-                                    mma_tf32(hacc, ah, bh, hacc);
-                                }
-                                if constexpr (EXACT) {
-                                    mma_tf32(uacc, dl, bh, uacc);
-                                    mma_tf32(uacc, dh, bl, uacc);
-                                }
-                                mma_tf32(uacc, dh, bh, uacc);
+                        for (int gate = 0; gate < 3; ++gate) {
+                            const uint4 w = q0[4 * kk * NS + gate * N];
+                            float (&hacc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
+                            float (&uacc)[4] = gate == 0 ? ur : gate == 1 ? uz : un;
+                            if (hid) {
+                                mma_f16(hacc, al[kk], w.x, w.y);
+                                mma_f16(hacc, ah[kk], w.z, w.w);
+                                mma_f16(hacc, ah[kk], w.x, w.y);
                             }
+                            if constexpr (EXACT) {
+                                mma_f16(uacc, dl[kk], w.x, w.y);
+                                mma_f16(uacc, dh[kk], w.z, w.w);
+                            }
+                            mma_f16(uacc, dh[kk], w.x, w.y);
                         }
-                    }
                     const int col = 8 * j + 2 * t;
                     const float2 bR = *reinterpret_cast<const float2 *>(sb + col), bZ = *reinterpret_cast<const float2 *>(sb + N + col);
                     const float2 bQ = *reinterpret_cast<const float2 *>(sb + 2 * N + col), bN = *reinterpret_cast<const float2 *>(sb + 3 * N + col);
-                    const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f);
+                    const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f), k2 = make_float2(kS, kS);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const float2 h2 = make_float2(hp[j][2 * h], hp[j][2 * h + 1]), y2 = make_float2(yc[j][2 * h], yc[j][2 * h + 1]);
                         const float2 d2 = make_float2(d[j][2 * h], d[j][2 * h + 1]);
-                        const float2 q = fadd2(make_float2(hq[2 * h], hq[2 * h + 1]), bQ);
-                        const float2 r = sigmoid2_gate(fadd2(make_float2(hr[2 * h], hr[2 * h + 1]), bR));
-                        const float2 z = sigmoid2_gate(fadd2(make_float2(hz[2 * h], hz[2 * h + 1]), bZ));
-                        const float2 c = tanh2_gate(ffma2(r, q, fadd2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), bN)));
+                        const float2 q = ffma2(make_float2(hq[2 * h], hq[2 * h + 1]), k2, bQ);
+                        const float2 r = sigmoid2_gate(ffma2(make_float2(hr[2 * h], hr[2 * h + 1]), k2, bR));
+                        const float2 z = sigmoid2_gate(ffma2(make_float2(hz[2 * h], hz[2 * h + 1]), k2, bZ));
+                        const float2 c = tanh2_gate(ffma2(r, q, ffma2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), k2, bN)));
                         const float2 omz = ffma2(z, mone, one), omr = ffma2(r, mone, one);
                         const float2 f = ffma2(omz, c, fmul2(z, h2));
                         const float2 az = fmul2(fmul2(ffma2(c, mone, h2), z), omz);
@@ -365,9 +393,10 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
                         const float2 kr = fmul2(fmul2(kn, q), omr);
                         float2 v = ffma2(y2, mone, f);                                          // r_t = f - y
                         v = ffma2(z, d2, v);
-                        v = ffma2(kr, make_float2(ur[2 * h], ur[2 * h + 1]), v);
-                        v = ffma2(az, make_float2(uz[2 * h], uz[2 * h + 1]), v);
-                        v = ffma2(kn, make_float2(un[2 * h], un[2 * h + 1]), v);
+                        float2 s = fmul2(kr, make_float2(ur[2 * h], ur[2 * h + 1]));
+                        s = ffma2(az, make_float2(uz[2 * h], uz[2 * h + 1]), s);
+                        s = ffma2(kn, make_float2(un[2 * h], un[2 * h + 1]), s);
+                        v = ffma2(s, make_float2(kD, kD), v);
                         dn[j][2 * h] = v.x; dn[j][2 * h + 1] = v.y;
                         if (step >= burn && act[h]) {
                             const float2 yn = fadd2(y2, v);
@@ -460,7 +489,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_bod
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a);
+            body_decide(st, a, 1, 0.0f, true);
         }
     }
 }

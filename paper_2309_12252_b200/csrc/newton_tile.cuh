@@ -453,17 +453,12 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
         if (prev + 1u == gridDim.x) {
             __threadfence();
             st->exit_counter = 0u;
-            const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits), q = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
             if (*(volatile unsigned *)&st->flags & FLAG_TIMEOUT) {         // rows that were not finished: nothing counts
                 st->err_bits = 0u; st->mis_bits = 0u;
                 st->done = BODY_TIMED_OUT;
                 if (HostResult *h = st->host) post_done(h, BODY_TIMED_OUT);
-            } else if (!(e <= 3.402823466e38f) || !(q <= 3.402823466e38f)) {      // beyond f16's range, or not finite at all: the other kernels tell
-                st->err_bits = 0u; st->mis_bits = 0u;
-                st->done = BODY_FALL_BACK;
-                if (HostResult *h = st->host) post_done(h, BODY_FALL_BACK);
             } else {
-                body_decide(st, a, 1, BODY_ROUNDING);
+                body_decide(st, a, 1, BODY_ROUNDING, true);
             }
         }
     }

@@ -467,3 +467,22 @@ def test_adjoint_products_are_at_fp32_level(bd, n, m, B, T, gy_scale, x_scale, k
     for k in ("db_i", "db_h", "dx", "dy0"):
         a, b = got[k].cpu().numpy().astype(np.float64), want[k].astype(np.float64)
         assert np.linalg.norm(a - b) <= (1e-6 if x_scale == 1.0 else 1e-3) * np.linalg.norm(b), k
+
+
+@pytest.mark.parametrize("n,m,B,T,x_scale,y0_scale,kernel", [
+    (16, 5, 16, 15001, 1.0, 0.5, ONE), (12, 16, 16, 40001, 1.0, 0.5, ONE), (49, 17, 4, 663, 1.0, 0.5, ONE), (50, 33, 4, 663, 1.0, 0.5, ONE),
+    (57, 15, 3, 401, 1.0, 0.5, ONE), (62, 70, 4, 300, 1.0, 0.5, ONE), (50, 3, 4, 663, 3000.0, 0.5, ONE), (50, 3, 4, 663, 2e4, 0.5, None),
+    (50, 3, 4, 663, 1.0, 3.0, ONE)])
+def test_one_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, y0_scale, kernel):
+    """K steps of 16 with and without their second half, and inputs and states up to and beyond what the products' halves hold.  The
+    gates are good to 2e-7 and a cell as initialised carries less than ten times that."""
+    p = synth.gru_params(n, m, seed=9, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=9, tag="c/x")
+    x[:, :, 0] = np.clip(x[:, :, 0], -4, 4) * np.float32(x_scale)
+    y0 = np.clip(synth.normal(9, "c/y0", (B, n)), -3, 3) * np.float32(y0_scale)
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
+    assert kernel is None or kernel in names, names
+    assert r.status == 0 and r.err <= 1e-4
+    want = oracle.gru_seq(p, x, y0, np.float64)
+    assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if y0_scale < 1.0 and x_scale == 1.0 else 1e-4)
