@@ -36,12 +36,13 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
     k.adj_tile_smem = [](int m) { return TileAdj::smem((m + 15) & ~15); };
 #endif
     k.one_warps = N > 32 ? 8 : 4;
-    k.seg_warps = Seg<N>::WARPS;
-    k.nc_max = Seg<N>::NC_MAX;
-    k.slot_bytes = Seg<N>::SZ * sizeof(float);
+    k.seg_warps = Seg<N, true>::WARPS;
+    k.nc_max = Seg<N, true>::NC_MAX;
+    k.slot_bytes = Seg<N, true>::SZ * sizeof(float);
     k.one_smem = [](int kx) { return Body<N>::smem(N > 32 ? 8 : 4, kx); };
     k.adj_smem = [](int kx) { return Adj<N>::smem(N > 32 ? 8 : 4, kx); };
-    k.seg_fixed = [](int kx) { return Seg<N>::fixed(kx); };
+    k.seg_fixed = [](int kx) { return Seg<N, true>::fixed(kx); };
+    if constexpr (N == 16) { if (v2 && !exact) k.seg_fixed = [](int kx) { return Seg<N, false>::fixed(kx); }; }
     return k;
 }
 

@@ -8,7 +8,8 @@
 //            coefficients {z, k_r, a_z, k_n, r} [5N] of a position stay in shared memory;
 //   phase 2  the chains, 16 in lockstep per group of N / 8 warps (one block of eight state columns each), a step being
 //            d <- r + z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d):  9 MMAs of a warp per block of eight columns,
-//            the new d crossing to the other warps of the group through shared memory.
+//            the new d crossing to the other warps of the group through shared memory, as the f16
+//            halves of the next step's operand where products are on those.
 // What bounds it: phases in series.  Cycles of a body, read with clock64 by one warp (n = 8, m = 4, B = 16, T = 1e4: 64 chains of 17
 // positions per CTA): phase 1 10,250 (five tiles a warp), 45 steps of burn-in 7,700 (170 a step), the 17 positions owned 10,800 (640 a
 // step, with its old iterate, residual and store), prologue of phase 2 950, exchange with the other CTAs 4,000 ... 10,000.  n = 4, m = 2,
@@ -19,8 +20,14 @@
 
 namespace deer {
 
-template <int N> struct Seg {
+template <int N, bool EXACT> struct Seg {
     static constexpr int NT = N / 8;
+    // f16 halves, as in newton_body.cuh; TF32 for n <= 8, where a block of columns is half of a K step of 16, and for n = 16, whose
+    // single products with the update gain less than the halves' conversions cost.  (us per evaluation, TF32 / f16: n = 24,
+    // 20,000 positions 174 / 164, 8,000 100 / 96; n = 12, 96,000 289 / 281; n = 9, 2,700 78 / 76; n = 32, 16,000 106 / 104; n = 16,
+    // 80,000 231 / 235, 16,000 88 / 90.)
+    static constexpr bool F16 = NT > (EXACT ? 1 : 2);
+    static constexpr int KB = F16 ? 2 : 1, NB = (NT + KB - 1) / KB;      // column blocks of a K step, K steps
     static constexpr int WARPS = N == 8 ? 16 : 8, THREADS = 32 * WARPS;
     static constexpr int GROUPS = NT >= 4 ? 1 : 4 / NT;  // groups of 16 chains at most: one warp of phase 2 per sub-partition (a second
                                                          // one there makes a step of exact products 1.9 times as long)
@@ -31,7 +38,7 @@ template <int N> struct Seg {
     static constexpr int DS = N + (N % 16 == 0 ? 8 : 0);        // stride of an exchanged update
     static constexpr size_t fixed(int kx)                // weights, biases, chain table, start states, exchange buffers
     {
-        return sizeof(float) * ((size_t)4 * (N / 2 + 4 * kx) * NS + 4 * N + (size_t)(NC_MAX + 1) * DS + (size_t)2 * NC_MAX * DS) + 32 * (size_t)NC_MAX;
+        return sizeof(float) * ((size_t)16 * (NB + (kx + KB - 1) / KB) * NS + 4 * N + (size_t)(NC_MAX + 1) * DS + (size_t)2 * NC_MAX * DS) + 32 * (size_t)NC_MAX;
     }
 };
 
@@ -61,16 +68,18 @@ struct SegChain { long long e; int t0, t_end, b, next; };      // e: row of posi
 static_assert(sizeof(SegChain) <= 32, "chain table entry");
 
 template <int N, bool V2, bool EXACT>
-__global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(BodyArgs a, int NC, int whole_loop)
+__global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kernel(BodyArgs a, int NC, int whole_loop)
 {
-    using C = Seg<N>;
-    constexpr int NT = C::NT, NS = C::NS, SZ = C::SZ, DS = C::DS;
+    using C = Seg<N, EXACT>;
+    constexpr int NT = C::NT, KB = C::KB, NB = C::NB, NS = C::NS, SZ = C::SZ, DS = C::DS;
+    constexpr bool F16 = C::F16;
+    __shared__ unsigned s_top;
     extern __shared__ __align__(16) float smb[];
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
     const int n = a.n, m = a.m, H = a.H, L = a.L;
     const bool proj = a.u == nullptr;
-    const int kx = proj ? (m + 7) >> 3 : 0;
+    const int kx = proj ? (m + 8 * KB - 1) / (8 * KB) : 0;               // K steps of x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
 
@@ -79,25 +88,57 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
     const unsigned nctas = (unsigned)((total + NC - 1) / NC);
     if (blockIdx.x >= nctas) return;
 
-    float4 *sH = reinterpret_cast<float4 *>(smb), *sI = sH + (N / 2) * NS;
-    float *sb = smb + 4 * (size_t)(N / 2 + 4 * kx) * NS;
+    uint4 *sH = reinterpret_cast<uint4 *>(smb), *sI = sH + 4 * NB * NS;
+    float *sb = reinterpret_cast<float *>(sI + 4 * kx * NS);
     float *ss = sb + 4 * N;                              // start state of every chain, and of the one behind the last
     float *dx = ss + (C::NC_MAX + 1) * DS;               // exchanged updates [2][NC_MAX][DS]
     SegChain *tab = reinterpret_cast<SegChain *>(dx + 2 * C::NC_MAX * DS);
     float *slots = reinterpret_cast<float *>(tab + C::NC_MAX);
-    auto lo = [](float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
-    for (int idx = tid; idx < (N / 2) * 3 * N; idx += C::THREADS) {
-        const int kp = idx % (N / 2), c = idx / (N / 2), gate = c / N, i = c % N;
-        const float *wr = hd.W_h + (size_t)(gate * n + i) * n + 2 * kp;
-        const float v0 = i < n && 2 * kp < n ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < n ? wr[1] : 0.0f;
-        sH[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+    float wscale = 1.0f, kS = 1.0f, kD = 1.0f;
+    if constexpr (F16) {
+        wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
+        kS = 1.0f / (wscale * MMA_OP_SCALE);
+        kD = 1.0f / (wscale * MMA_D_SCALE);
+    }
+    // weights as records of the four words that a lane needs for a column of a K step (newton_body.cuh)
+    auto record = [&](const float *wr, bool row, int kt, int width) {
+        const int k = 8 * KB * (kt >> 2) + 2 * (kt & 3);
+        auto w = [&](int j) { return row && j < width ? wr[j] * wscale : 0.0f; };
+        uint4 r;
+        if constexpr (F16) {
+            split_f16(make_float2(w(k), w(k + 1)), r.x, r.z);
+            split_f16(make_float2(w(k + 8), w(k + 9)), r.y, r.w);
+        } else {
+            split_tf32(w(k), r.x, r.z);
+            split_tf32(w(k + 1), r.y, r.w);
+        }
+        return r;
+    };
+    for (int idx = tid; idx < 4 * NB * 3 * N; idx += C::THREADS) {
+        const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
+        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n);
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += C::THREADS) {
-        const int kp = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
-        const float *wr = hd.W_i + (size_t)(gate * n + i) * m + 2 * kp;
-        const float v0 = i < n && 2 * kp < m ? wr[0] : 0.0f, v1 = i < n && 2 * kp + 1 < m ? wr[1] : 0.0f;
-        sI[kp * NS + c] = make_float4(v0, v1, lo(v0), lo(v1));
+        const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
+        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m);
     }
+    // block b of a K step of an A operand, row h of this lane: two columns (an accumulator's columns of TF32 in the slots t, t + 4)
+    auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v) {
+        if constexpr (F16) {
+            split_f16(fmul2(v, make_float2(MMA_OP_SCALE, MMA_OP_SCALE)), hi[2 * b + h], lo[2 * b + h]);
+        } else {
+            split_tf32(v.x, hi[h], lo[h]);
+            split_tf32(v.y, hi[2 + h], lo[2 + h]);
+        }
+    };
+    auto mma = [&](float (&acc)[4], const unsigned (&x)[4], unsigned w0, unsigned w1) {
+        if constexpr (F16) {
+            mma_f16(acc, x, w0, w1);
+        } else {
+            const unsigned w[2] = {w0, w1};
+            mma_tf32(acc, x, w, acc);
+        }
+    };
     for (int i = tid; i < N; i += C::THREADS) {
         sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
         sb[N + i] = i < n ? hd.b_h[n + i] + (proj ? hd.b_i[n + i] : 0.0f) : 0.0f;
@@ -176,13 +217,16 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         }
     }
     float nhp[NT][4], ny4[NT][4];
-    float2 nx[2];
+    float2 nx[2 * KB];
     auto fetch = [&]() {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const bool in = tp[h] < tlim[h], lh = in && (!zero || tp[h] == 0), ly = in && !zero;
             const float *hq = tp[h] == 0 ? y0p[h] : yp[h] - yst;
-            if (proj) nx[h] = in ? ldx(xp[h], 2 * t) : make_float2(0.0f, 0.0f);
+            if (proj) {
+#pragma unroll
+                for (int b = 0; b < KB; ++b) nx[2 * b + h] = in ? ldx(xp[h], 8 * b + 2 * t) : make_float2(0.0f, 0.0f);
+            }
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 const float2 v = lh ? ld2(hq, 8 * j + 2 * t, n) : make_float2(0.0f, 0.0f);
@@ -207,7 +251,9 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         for (int h = 0; h < 2; ++h) { tp[h] += dt; slot[h] += dt; yp[h] += dt * yst; xp[h] += dt * xst; }
         float xr[NT][4], xz[NT][4], xn[NT][4];
         if (proj) {
-            float2 x0 = nx[0], x1 = nx[1];
+            float2 xc[2 * KB];
+#pragma unroll
+            for (int q = 0; q < 2 * KB; ++q) xc[q] = nx[q];
             if (left > 1) fetch();
 #pragma unroll
             for (int j = 0; j < NT; ++j)
@@ -216,29 +262,23 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
 #pragma unroll 1
             for (int kk = 0; kk < kx; ++kk) {
                 unsigned ah[4], al[4];
-                split_tf32(x0.x, ah[0], al[0]);
-                split_tf32(x1.x, ah[1], al[1]);
-                split_tf32(x0.y, ah[2], al[2]);
-                split_tf32(x1.y, ah[3], al[3]);
+#pragma unroll
+                for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q]);
                 if (kk + 1 < kx) {
-                    x0 = act[0] ? ldx(xpp[0], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
-                    x1 = act[1] ? ldx(xpp[1], 8 * kk + 8 + 2 * t) : make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int q = 0; q < 2 * KB; ++q) xc[q] = act[q & 1] ? ldx(xpp[q & 1], 8 * KB * (kk + 1) + 8 * (q >> 1) + 2 * t) : make_float2(0.0f, 0.0f);
                 }
-                const float4 *q0 = sI + (4 * kk + t) * NS + g;
+                const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
-                for (int j = 0; j < NT; ++j) {
-                    {
+                for (int j = 0; j < NT; ++j)
 #pragma unroll
-                        for (int gate = 0; gate < 3; ++gate) {
-                            const float4 w = q0[gate * N + 8 * j];
-                            const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                            float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
-                            mma_tf32(acc, al, bh, acc);
-                            mma_tf32(acc, ah, bl, acc);
-                            mma_tf32(acc, ah, bh, acc);
-                        }
+                    for (int gate = 0; gate < 3; ++gate) {
+                        const uint4 w = q0[gate * N + 8 * j];
+                        float (&acc)[4] = gate == 0 ? xr[j] : gate == 1 ? xz[j] : xn[j];
+                        mma(acc, al, w.x, w.y);
+                        mma(acc, ah, w.z, w.w);
+                        mma(acc, ah, w.x, w.y);
                     }
-                }
             }
         } else {
 #pragma unroll
@@ -255,48 +295,59 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
                     xn[j][2 * h] = vn.x; xn[j][2 * h + 1] = vn.y;
                 }
             if (left > 1) fetch();
+            if constexpr (F16) {                         // (in the products' scale: a power of two)
+                const float up = wscale * MMA_OP_SCALE;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+            }
         }
+        unsigned ah[NB][4], al[NB][4];
+        if constexpr (F16 && NT % 2) {
+#pragma unroll
+            for (int q = 2; q < 4; ++q) { ah[NB - 1][q] = 0u; al[NB - 1][q] = 0u; }
+        }
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]));
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
             {
                 float (&hr)[4] = xr[j], (&hz)[4] = xz[j];
                 float hq[4] = {0.f, 0.f, 0.f, 0.f};
                 if (hid) {
-                    const float4 *q0 = sH + t * NS + 8 * j + g;
+                    const uint4 *q0 = sH + t * NS + 8 * j + g;
 #pragma unroll
-                    for (int kk = 0; kk < NT; ++kk) {
-                        {
-                            unsigned ah[4], al[4];
-                            split_tf32(hp[kk][0], ah[0], al[0]); split_tf32(hp[kk][2], ah[1], al[1]);
-                            split_tf32(hp[kk][1], ah[2], al[2]); split_tf32(hp[kk][3], ah[3], al[3]);
+                    for (int kk = 0; kk < NB; ++kk)
 #pragma unroll
-                            for (int gate = 0; gate < 3; ++gate) {
-                                const float4 w = q0[4 * kk * NS + gate * N];
-                                const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                                float (&acc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
-                                mma_tf32(acc, al, bh, acc);
-                                mma_tf32(acc, ah, bl, acc);
-                                mma_tf32(acc, ah, bh, acc);
-                            }
+                        for (int gate = 0; gate < 3; ++gate) {
+                            const uint4 w = q0[4 * kk * NS + gate * N];
+                            float (&acc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
+                            mma(acc, al[kk], w.x, w.y);
+                            mma(acc, ah[kk], w.z, w.w);
+                            mma(acc, ah[kk], w.x, w.y);
                         }
-                    }
                 }
                 const int col = 8 * j + 2 * t;
                 const float2 bR = *reinterpret_cast<const float2 *>(sb + col), bZ = *reinterpret_cast<const float2 *>(sb + N + col);
                 const float2 bQ = *reinterpret_cast<const float2 *>(sb + 2 * N + col), bN = *reinterpret_cast<const float2 *>(sb + 3 * N + col);
-                const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f);
+                const float2 one = make_float2(1.0f, 1.0f), mone = make_float2(-1.0f, -1.0f), k2 = make_float2(kS, kS);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float2 y2 = make_float2(y4[j][2 * h], y4[j][2 * h + 1]);
                     const float2 h2 = make_float2(hp[j][2 * h], hp[j][2 * h + 1]);
-                    const float2 q = fadd2(make_float2(hq[2 * h], hq[2 * h + 1]), bQ);
-                    const float2 r = sigmoid2_gate(fadd2(make_float2(hr[2 * h], hr[2 * h + 1]), bR));
-                    const float2 z = sigmoid2_gate(fadd2(make_float2(hz[2 * h], hz[2 * h + 1]), bZ));
-                    const float2 c = tanh2_gate(ffma2(r, q, fadd2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), bN)));
+                    const float2 q = ffma2(make_float2(hq[2 * h], hq[2 * h + 1]), k2, bQ);
+                    const float2 r = sigmoid2_gate(ffma2(make_float2(hr[2 * h], hr[2 * h + 1]), k2, bR));
+                    const float2 z = sigmoid2_gate(ffma2(make_float2(hz[2 * h], hz[2 * h + 1]), k2, bZ));
+                    const float2 c = tanh2_gate(ffma2(r, q, ffma2(make_float2(xn[j][2 * h], xn[j][2 * h + 1]), k2, bN)));
                     const float2 omz = ffma2(z, mone, one), omr = ffma2(r, mone, one);
                     const float2 f = ffma2(omz, c, fmul2(z, h2));
-                    const float2 az = fmul2(fmul2(ffma2(c, mone, h2), z), omz);
-                    const float2 an = fmul2(omz, ffma2(fmul2(c, mone), c, one));
+                    // (the three coefficients of products with the update carry their scale)
+                    const float2 kd = make_float2(kD, kD), okd = F16 ? fmul2(omz, kd) : omz;
+                    const float2 az = fmul2(fmul2(ffma2(c, mone, h2), z), okd);
+                    const float2 an = fmul2(okd, ffma2(fmul2(c, mone), c, one));
                     const float2 kn = fmul2(an, r);
                     const float2 kr = fmul2(fmul2(kn, q), omr);
                     if (act[h]) {
@@ -320,11 +371,11 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
     float d[4] = {0.f, 0.f, 0.f, 0.f};
     bool next[2] = {false, false}, gave_up = false;
     if (live) {
-        float4 wf[N <= 32 ? NT : 1][3];
-        const float4 *wq = sH + t * NS + 8 * j + g;
+        uint4 wf[N <= 32 ? NB : 1][3];
+        const uint4 *wq = sH + t * NS + 8 * j + g;
         if constexpr (N <= 32) {
 #pragma unroll
-            for (int kk = 0; kk < NT; ++kk)
+            for (int kk = 0; kk < NB; ++kk)
 #pragma unroll
                 for (int gate = 0; gate < 3; ++gate) wf[kk][gate] = wq[4 * kk * NS + gate * N];
         }
@@ -381,29 +432,35 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
                 for (int q = 0; q < 4; ++q) { u[gate][q] = 0.f; v[gate][q] = 0.f; w2[gate][q] = 0.f; }
             const float *xin = xrow + buf * (C::NC_MAX * DS);
 #pragma unroll
-            for (int kk = 0; kk < NT; ++kk) {
-                {
-                    float e4[4];
-                    if constexpr (NT > 1) {
-                        const float2 p0 = *reinterpret_cast<const float2 *>(xin + g * DS + 8 * kk + 2 * t);
-                        const float2 p1 = *reinterpret_cast<const float2 *>(xin + (g + 8) * DS + 8 * kk + 2 * t);
-                        e4[0] = p0.x; e4[1] = p0.y; e4[2] = p1.x; e4[3] = p1.y;
-                    } else {
-                        e4[0] = d[0]; e4[1] = d[1]; e4[2] = d[2]; e4[3] = d[3];
-                    }
-                    unsigned dh[4], dl[4];
-                    split_tf32(e4[0], dh[0], dl[0]); split_tf32(e4[2], dh[1], dl[1]);
-                    split_tf32(e4[1], dh[2], dl[2]); split_tf32(e4[3], dh[3], dl[3]);
+            for (int kk = 0; kk < NB; ++kk) {
+                unsigned dh[4], dl[4];
+                if constexpr (F16) {                     // (the pairs of columns are exchanged as the operand's halves)
 #pragma unroll
-                    for (int gate = 0; gate < 3; ++gate) {
-                        float4 w;
-                        if constexpr (N <= 32) w = wf[kk][gate]; else w = wq[4 * kk * NS + gate * N];
-                        const unsigned bh[2] = {__float_as_uint(w.x), __float_as_uint(w.y)}, bl[2] = {__float_as_uint(w.z), __float_as_uint(w.w)};
-                        mma_tf32(u[gate], dh, bh, u[gate]);
-                        if constexpr (EXACT) {
-                            mma_tf32(v[gate], dl, bh, v[gate]);
-                            mma_tf32(w2[gate], dh, bl, w2[gate]);
+                    for (int q = 0; q < 4; ++q) {
+                        if (2 * kk + (q >> 1) < NT) {
+                            const uint2 p = *reinterpret_cast<const uint2 *>(xin + (g + 8 * (q & 1)) * DS + 16 * kk + 8 * (q >> 1) + 2 * t);
+                            dh[q] = p.x; dl[q] = p.y;
+                        } else {
+                            dh[q] = 0u; dl[q] = 0u;
                         }
+                    }
+                } else {
+                    float2 p[2] = {make_float2(d[0], d[1]), make_float2(d[2], d[3])};
+                    if constexpr (NT > 1) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) p[h] = *reinterpret_cast<const float2 *>(xin + (g + 8 * h) * DS + 8 * kk + 2 * t);
+                    }
+                    operand(dh, dl, 0, 0, p[0]);
+                    operand(dh, dl, 0, 1, p[1]);
+                }
+#pragma unroll
+                for (int gate = 0; gate < 3; ++gate) {
+                    uint4 w;
+                    if constexpr (N <= 32) w = wf[kk][gate]; else w = wq[4 * kk * NS + gate * N];
+                    mma(u[gate], dh, w.x, w.y);
+                    if constexpr (EXACT) {
+                        mma(v[gate], dl, w.x, w.y);
+                        mma(w2[gate], dh, w.z, w.w);
                     }
                 }
             }
@@ -424,8 +481,13 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
                 for (int gate = 0; gate < 3; ++gate) o = ffma2(ck[gate], make_float2(u[gate][2 * h], u[gate][2 * h + 1]), o);
                 d[2 * h] = act ? o.x : d[2 * h];
                 d[2 * h + 1] = act ? o.y : d[2 * h + 1];
-                if constexpr (NT > 1)
+                if constexpr (F16) {
+                    uint2 p;
+                    split_f16(fmul2(make_float2(d[2 * h], d[2 * h + 1]), make_float2(MMA_D_SCALE, MMA_D_SCALE)), p.x, p.y);
+                    *reinterpret_cast<uint2 *>(xout + (g + 8 * h) * DS + col) = p;
+                } else if constexpr (NT > 1) {
                     *reinterpret_cast<float2 *>(xout + (g + 8 * h) * DS + col) = make_float2(d[2 * h], d[2 * h + 1]);
+                }
             }
             if (more) load_coefs();
             group_sync();
@@ -533,7 +595,9 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         }
         const unsigned eb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[2][lane] : 0u);
         const unsigned qb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[3][lane] : 0u);
-        const BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter, a.adapt != 0, 0.0f);
+        BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter, a.adapt != 0, 0.0f);
+        if (F16 && (!(__uint_as_float(eb) <= 3.402823466e38f) || !(__uint_as_float(qb) <= 3.402823466e38f)))
+            v = BodyVerdict{false, BODY_FALL_BACK, burn, 0};         // beyond f16's range, or not finite at all: the other kernels tell
         need = max(need, v.need);
         if (blockIdx.x == 0 && tid == 0) {
             if (v.counts) {
@@ -585,7 +649,7 @@ __global__ void __launch_bounds__(Seg<N>::THREADS, 1) newton_segment_kernel(Body
         if (prev + 1u == nctas) {
             __threadfence();
             st->exit_counter = 0u;
-            body_decide(st, a);
+            body_decide(st, a, 1, 0.0f, F16);
         }
     }
     return;

@@ -486,3 +486,20 @@ def test_one_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, y0_scale,
     assert r.status == 0 and r.err <= 1e-4
     want = oracle.gru_seq(p, x, y0, np.float64)
     assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if y0_scale < 1.0 and x_scale == 1.0 else 1e-4)
+
+
+@pytest.mark.parametrize("n,m,B,T,x_scale,kernel", [
+    (9, 3, 10, 300, 1.0, SEG), (12, 17, 3, 401, 1.0, SEG), (16, 8, 4, 501, 1.0, SEG), (24, 16, 16, 6001, 1.0, SEG), (31, 33, 2, 301, 1.0, SEG),
+    (32, 5, 2, 301, 1.0, SEG), (40, 7, 4, 301, 1.0, SEG), (48, 1, 2, 201, 1.0, SEG), (24, 4, 3, 401, 3000.0, SEG), (24, 4, 3, 401, 2e4, None)])
+def test_two_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, kernel):
+    """As above, for the two-phase form; n = 16 keeps TF32 products, good to 2^-20."""
+    p = synth.gru_params(n, m, seed=10, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=10, tag="c/x")
+    x[:, :, 0] = np.clip(x[:, :, 0], -4, 4) * np.float32(x_scale)
+    y0 = synth.normal(10, "c/y0", (B, n)) * 0.5
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
+    assert kernel is None or kernel in names, names
+    assert r.status == 0 and r.err <= 1e-4
+    want = oracle.gru_seq(p, x, y0, np.float64)
+    assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if x_scale == 1.0 else 1e-4)
