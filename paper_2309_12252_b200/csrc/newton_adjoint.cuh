@@ -432,6 +432,9 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                         };
                         if (a.lam) {
                             st2(a.lam + o * n + col, l2);
+                        } else if (a.packed) {
+                            float *gi = a.dGi + o * 4 * n + col;
+                            st2(gi, pr); st2(gi + n, pz); st2(gi + 2 * n, pn); st2(gi + 3 * n, pa);
                         } else {
                             float *gi = a.dGi + o * 3 * n + col, *gh = a.dGh + o * 3 * n + col;
                             st2(gi, pr); st2(gi + n, pz); st2(gi + 2 * n, pa);

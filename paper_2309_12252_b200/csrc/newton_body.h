@@ -43,6 +43,7 @@ struct AdjArgs {
     const float *gy_seq;     // tiles, or nullptr: [B,n] dL/dy where it is the same at every step of a sequence (gy is not read)
     float *lam;              // [B,T,H,n] out: lambda; or nullptr:
     float *dGi, *dGh;        // [B,T,H,3n] out: gradients w.r.t. the input-side and hidden-side pre-activations
+    int packed;              // one head: dGi receives rows [4n] = (r, z, n hidden, n input) and dGh nothing
     float *dy0;              // or nullptr; row b * H + head (dy0_by_head), else first_seq + sequence
     int dy0_by_head;
     int B, T, n, m, H, L;
