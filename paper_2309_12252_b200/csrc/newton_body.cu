@@ -248,7 +248,8 @@ size_t adjoint_starts(int n) { return n > 48 ? 16 * (size_t)((n + 7) / 8 * 8 + 4
 // of its steps (44 + 16 of them, some 3 us each, more with the channels that a step contracts) until the chains fill the GPU.
 // (B200, us per gradient, here / there, B = 8: n = 9, m = 8 202 / 138 at 6,400 positions, 208 / 200 at 20,000; n = 20, m = 8
 // 228 / 244 at 6,400; n = 28, m = 60 530 / 400 at 6,400, 561 / 737 at 20,000; n = 16, m = 3 219 / 180 at 80,000, 295 / 305 at
-// 160,000; n = 32, m = 3 395 / 263 at 40,000, 436 / 411 at 80,000, m = 64 653 / 465 and 849 / 762 at 80,000 and 160,000;
+// 160,000; n = 32, B = 16, m = 3 295 / 251 at 48,000, 322 / 330 at 64,000, m = 32 374 / 309 at 64,000, 405 / 416 at 96,000, m = 64
+// 494 / 443 at 96,000, 516 / 544 at 128,000;
 // n = 64, here a tile, 728 / 525 at 20,000, 793 / 722 at 40,000, 819 / 881 at 56,000 whatever m.)
 // n <= 4 pads to 8 columns where its own kernels are tuned; n = 64 with m > 64 is no tile's (nor worth its spills early).
 static float adjoint_line(int n, int m)
@@ -258,7 +259,7 @@ static float adjoint_line(int n, int m)
     case 1: case 2: case 4: return 1e30f;
     case 8: return 270000.0f;
     case 16: return 120000.0f * (1.0f + c / 20.0f);
-    case 32: return 70000.0f * (1.0f + c / 35.0f);
+    case 32: return 70000.0f * (1.0f + c / 55.0f);
     case 64: return m <= 64 ? 50000.0f : 250000.0f;
     }
     if (n < 8) return 4000.0f * (1.0f + c / 8.0f);
@@ -317,13 +318,15 @@ int launch_adjoint_tile(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
 //   n = 64, B = 16, T = 1e3:    - / 2369 / 1247    n = 64, B = 16, T = 1e4:   - / 2828 / 3345
 // Two-phase: one wave (then the whole loop is one launch), two waves from n = 9 on.  One-phase: from half a wave of chains on --
 // below, its steps, a whole cell each, are a serial chain that nothing fills (n <= 8 never comes here: a thread per chain).
-// Sizes without tuned kernels of the other kind always come here, to the two-phase kernel up to eight waves: there random walks,
-// whose bodies the long chains of the other run again, break even; white noise does so earlier (B = 16, m = 8, us per evaluation
-// by waves, two-phase / one-phase, white noise then random walks):
-//   n = 12   1.4 312 / 447, 510 / 1200   2.7 446 / 527, 767 / 1507   5.5 836 / 609, 1445 / 1689    10.9 1572 / 792, 2382 / 2194
-//   n = 24   2.2 399 / 657, 617 / 1275   4.5 656 / 799, 1254 / 2095  8.9 1187 / 943, 1828 / 1724   17.8 2426 / 1249, 2946 / 1798
-//   n = 28   4.9 656 / 1068              6.8 883 / 1216              8.6 1126 / 1249, 1603 / 2394
-//   n = 40   3.1 707 / 1171              4.8 888 / 1204              6.6 1223 / 1243               8.5 1562 / 1305
+// Sizes without tuned kernels of the other kind always come here, to the two-phase kernel up to four, five or six waves: there random
+// walks, whose bodies the long chains of the other run again, break even; white noise does so earlier (B = 16, m = 8, us per
+// evaluation, two-phase / one-phase, white noise then random walks, the last before the line and the first behind it):
+//   n = 12   T = 12,000 433 / 386, 669 / 893      T = 16,000 552 / 406, 1100 / 988
+//   n = 20   T = 12,000 566 / 492, 875 / 969      T = 16,000 795 / 498, 1224 / 985
+//   n = 24   T = 12,000 553 / 498, 663 / 759      T = 16,000 781 / 508, 1185 / 1001
+//   n = 28   T = 8,000 614 / 545, 928 / 1012      T = 9,500 722 / 570, 1139 / 1136
+//   n = 40   T = 4,000 652 / 714, 814 / 1076      T = 5,000 803 / 731, 1034 / 1171
+//   n = 48   T = 3,200 774 / 896, 924 / 1270      T = 4,000 919 / 900, 1084 / 1235
 // A thread per chain, powers of two: by positions per chain of a full GPU (`share`; m = n or 4, B = 16, white noise then random
 // walks, where a try is often lost: thread per chain / multiplied out):
 //   n = 1   13 175 / 208, 128 / 156   30 205 / 235, 141 / 174   42 217 / 302, 162 / 221   84 301 / 541, 226 / 411
@@ -340,7 +343,7 @@ bool body_suits(const BodyPlan &p, int n)
     // (n = 1, B = 8, T = 3e3 80 / 92, T = 1e4 96 / 99; n = 2, T = 6e3 114 / 140, T = 1.5e4 142 / 152: above, what a failed try costs
     // on slowly varying inputs, 20 to 30 us, outweighs it)
     if (p.NC > 0 && n <= 2 && (long long)p.max_ctas * p.NC * p.L > (n == 1 ? 20000 : 64000)) return false;
-    if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= 8.0f);
+    if (p.NC > 0) return p.whole_loop || (n > 8 && p.waves <= 2.0f) || (!tuned && n > 8 && p.waves <= (n <= 16 ? 4.0f : n <= 32 ? 5.0f : 6.0f));
     if (!tuned) return true;
     return p.waves >= 0.5f;
 }

@@ -126,8 +126,10 @@ template <int N> struct Body {
 
 // EXACT: the products with d are three MMAs as well (sizes whose solve has always been fp32-accurate); V2: rows are read and
 // written as 8-byte pairs.  n <= 8 takes a thread per chain instead (newton_lane.cuh).
+// (Two CTAs per SM from n = 17 to 32, not three: 168 registers spill.  us per evaluation, three / two: n = 20, 480,000 positions 739 /
+// 649; n = 28, 320,000 832 / 635; n = 30, m = 30, 480,000 1181 / 1033.)
 template <int N, bool V2, bool EXACT>
-__global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : 3) newton_body_kernel(BodyArgs a)
+__global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 3) newton_body_kernel(BodyArgs a)
 {
     using C = Body<N>;
     constexpr int NT = C::NT, NB = C::NB, NS = C::NS, SW = C::SW;
