@@ -272,6 +272,13 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 split_tf32(v.y, hi[2 + h], lo[2 + h]);
             }
         };
+        // the lo halves: of TF32 formed where they are used (kept, they spill at n = 16: 1.28e6 positions 562 -> 580 us)
+        auto low = [&](const unsigned (&hi)[4], unsigned (&lo)[4]) {
+            if constexpr (!F16) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { unsigned h; split_tf32(__uint_as_float(hi[q]), h, lo[q]); }
+            }
+        };
         auto mma = [&](float (&acc)[4], const unsigned (&x)[4], unsigned w0, unsigned w1) {
             if constexpr (F16) {
                 mma_f16(acc, x, w0, w1);
@@ -396,6 +403,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                     for (int gate = 0; gate < 3; ++gate) {
                         const uint4 w = q0[4 * kk * NS + gate * N];
                         float (&acc)[4] = gate == 0 ? hr : gate == 1 ? hz : hq;
+                        low(ah[kk], al[kk]);
                         mma(acc, al[kk], w.x, w.y);
                         mma(acc, ah[kk], w.z, w.w);
                         mma(acc, ah[kk], w.x, w.y);
@@ -449,17 +457,20 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
             if (step + 1 < s_end) { load_h(hp); load_g(gy); }
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
-                float acc[4] = {0.f, 0.f, 0.f, 0.f}, cr[4] = {0.f, 0.f, 0.f, 0.f};
+                float acc[4], cr[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = F16 ? 0.0f : zl[j][q];
                 const uint4 *q0 = sT + t * NS2 + 8 * j + g;
 #pragma unroll
                 for (int kk = 0; kk < PB; ++kk) {
                     const uint4 w = q0[4 * kk * NS2];
+                    low(ph[kk], pl[kk]);
                     mma(cr, pl[kk], w.x, w.y);
                     mma(cr, ph[kk], w.z, w.w);
                     mma(acc, ph[kk], w.x, w.y);
                 }
 #pragma unroll
-                for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? fmaf(acc[q] + cr[q], kM[q >> 1], zl[j][q]) : d[j][q];
+                for (int q = 0; q < 4; ++q) d[j][q] = act[q >> 1] ? (F16 ? fmaf(acc[q] + cr[q], kM[q >> 1], zl[j][q]) : acc[q] + cr[q]) : d[j][q];
             }
         }
         // ---- the state that leaves the first time step: the gradient w.r.t. y0 (wanted or not, it shows what is not finite there)
