@@ -85,8 +85,13 @@ __device__ __forceinline__ void adjoint_decide(StatusBlock *st, float eta, bool 
     st->burn = max(want, burn + 8);
 }
 
-template <int N, bool V2>
-__global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 3) newton_adjoint_kernel(AdjArgs a)
+// CTAS: per SM, at n = 9 to 16 two, which need not spill, or three where many channels are contracted, which leave a step with too
+// little to do beside it.  (us per gradient, three / two: n = 16, m = 8, 240,000 positions 300 / 252, 960,000 572 / 560; m = 24,
+// 640,000 534 / 500; m = 64, 640,000 780 / 922; n = 12, m = 8, 320,000 435 / 396, m = 40 650 / 605; 31 heads of 16 1955 / 1915.)
+template <int N> __host__ __device__ constexpr int adjoint_ctas(int m) { return N > 32 ? 1 : N > 16 ? 2 : N > 8 ? (m > 40 ? 3 : 2) : 3; }
+
+template <int N, bool V2, int CTAS>
+__global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kernel(AdjArgs a)
 {
     using C = Adj<N>;
     constexpr int NT = C::NT, KB = C::KB, NB = C::NB, PB = C::PB, NS = C::NS, NS2 = C::NS2, SW = C::SW;

@@ -238,7 +238,7 @@ bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const in
     if (!adjoint_supported(n, m, have_u)) return false;
     const BodyKernels k = pick(n, (n & 1) == 0);
     if (k.adj_smem(have_u ? 0 : (m + 7) / 8) > BODY_SMEM_MAX) return false;
-    one_wave_of_chains(p, (const void *)k.adj, 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN, B, T, strides, H, 0.8f);
+    one_wave_of_chains(p, (const void *)k.adj(have_u ? 0 : m), 32 * k.one_warps, 16 * k.one_warps, 16, 1, k.adj_smem(have_u ? 0 : (m + 7) / 8), ADJ_BURN, B, T, strides, H, 0.8f);
     return true;
 }
 
@@ -278,9 +278,10 @@ int launch_newton_adjoint(const AdjArgs &a, const BodyPlan &p, cudaStream_t st)
     const bool aligned = (((uintptr_t)a.y | (uintptr_t)a.gy | (uintptr_t)a.y0 | (uintptr_t)a.u | (uintptr_t)a.lam | (uintptr_t)a.dGi |
                            (uintptr_t)a.dGh) & 7) == 0;
     const BodyKernels k = pick(a.n, (a.n & 1) == 0 && aligned);
-    occupancy_of((const void *)k.adj, 32 * p.warps, p.smem);
+    auto kern = k.adj(a.u ? 0 : a.m);
+    occupancy_of((const void *)kern, 32 * p.warps, p.smem);
     DEER_KERNEL("newton_adjoint_kernel", st,
-                k.adj<<<dim3((unsigned)p.max_ctas, (unsigned)a.H), 32 * p.warps, p.smem, st>>>(a));
+                kern<<<dim3((unsigned)p.max_ctas, (unsigned)a.H), 32 * p.warps, p.smem, st>>>(a));
     return DEER_OK;
 }
 

@@ -65,7 +65,7 @@ constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3;
 struct BodyKernels {
     void (*one)(BodyArgs);                     // one-phase (newton_body.cuh); n > 8 only
     void (*seg)(BodyArgs, int, int);           // two-phase (newton_segment.cuh)
-    void (*adj)(AdjArgs);                      // adjoint, one-phase (newton_adjoint.cuh)
+    void (*(*adj)(int m))(AdjArgs);            // adjoint, one-phase (newton_adjoint.cuh); m: channels contracted in the kernel
     void (*(*tile)(int m))(BodyArgs);          // 128 chains per tcgen05 tile (newton_tile.cuh); n = 32, 64 only
     size_t (*tile_smem)(int m);
     int tile_threads, tile_chains;

@@ -24,7 +24,9 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
         // single-TF32 products with the update: the sizes whose solve has always run in reduced precision
         if (v2 && !exact) { k.one = newton_body_kernel<N, true, false>; k.seg = newton_segment_kernel<N, true, false>; }
     }
-    k.adj = v2 ? newton_adjoint_kernel<N, true> : newton_adjoint_kernel<N, false>;
+    constexpr int few = adjoint_ctas<N>(0), many = adjoint_ctas<N>(64);
+    k.adj = v2 ? [](int m) -> void (*)(AdjArgs) { return adjoint_ctas<N>(m) == few ? newton_adjoint_kernel<N, true, few> : newton_adjoint_kernel<N, true, many>; }
+               : [](int m) -> void (*)(AdjArgs) { return adjoint_ctas<N>(m) == few ? newton_adjoint_kernel<N, false, few> : newton_adjoint_kernel<N, false, many>; };
     if constexpr (N == 32 || N == 64) {
         k.tile = [](int m) -> void (*)(BodyArgs) { return m <= 32 ? newton_tile_kernel<N, 1, true> : newton_tile_kernel<N, 64 / N, false>; };
         k.tile_threads = TileBody<N>::THREADS;
