@@ -18,9 +18,9 @@
 // largest is some third of the largest of all, so that the first rule decides there.
 // One boundary that differs by more leaves StatusBlock::done at 0: the launches enqueued behind this one (a longer burn-in,
 // then the kernels that multiply the Jacobians out) do the work.
-// What bounds it: the latency of chained mma.sync with eight warps per SM (255 registers a thread).  n = m = 32, B = 16, T = 2e4, in
-// TF32: tensor pipe 48 % active, issue slots 32 % used, DRAM 15 %; per instruction issued 2.6 warps wait for a fixed latency.  With
-// f16 halves T = 1e5 takes 850 us where it took 1100.
+// What bounds it: the latency of chained mma.sync with eight warps per SM (254 registers a thread).  n = m = 32, B = 16, T = 2e4: tensor
+// pipe 34 % active, issue slots 32 % used, DRAM 17 % (in TF32 48, 32 and 15 %, and 506 us under the profiler where it now takes 396);
+// T = 1e5 takes 820 us where it took 1100.
 // The boundaries that dy0 can still feel -- those less than DY0_REACH burn-ins from the sequence's first step -- are held to
 // eta * max|dy0| as well.
 #pragma once

@@ -19,6 +19,9 @@
 // raised to what the observed decay calls for and the body is run again, or, for a cell that hardly forgets, the
 // evaluation goes on with the kernels that multiply the Jacobians out (BODY_FALL_BACK).
 //
+// What bounds it: the latency of a step's MMAs and gates with eight warps per SM.  n = 28, m = 8, B = 16, T = 2e4: tensor pipe 35 %
+// active, issue slots 32 % used, DRAM 3 %.
+//
 // Nothing waits on another CTA.  Boundaries inside a warp are compared from shared memory; at a boundary between two
 // warps each side leaves its state in global memory and the one that arrives second compares.
 #pragma once
