@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <atomic>
 #include "../../include/deer.h"
+#include "body_verdict.h"
 
 namespace deer {
 
@@ -188,11 +189,6 @@ __device__ __forceinline__ void post_result(HostResult *h, int done, int burn, i
 {
     *reinterpret_cast<int4 *>(h) = make_int4(fence ? 0 : done, burn, iters, (int)err_bits);
     if (fence) post_done(h, done);
-}
-
-__device__ __forceinline__ bool newton_loop_ends(float e, float tol, int k, int max_iter)
-{
-    return !(e > tol) || !(e <= 3.402823466e38f) || k + 1 >= max_iter;
 }
 
 __device__ __forceinline__ void newton_decide(StatusBlock *st, float tol, int max_iter, float *trace, bool polled = false)

@@ -31,65 +31,6 @@
 
 namespace deer {
 
-// What becomes of a body whose update is e and whose largest boundary mismatch is mis, and the burn-in of the next one.
-//
-// Where the loop runs to a tolerance, a body whose boundaries are good to a thousandth of its update is a good quasi-Newton
-// step: it counts.  Far from the solution more than that is lost in Newton's own quadratic error (updates of 1.7, 0.8, 0.05
-// are usual): a twentieth of the update times the update is then good enough.  (Slowly varying inputs, n = 32, B = 16,
-// T = 2e4: two of six bodies were run again for it.)
-//
-// The carried error is about e * rho^burn, so a body shows the rate at which its cell forgets.  What proves too short is raised
-// to what that rate calls for.  Where chains are short, so that a body's time goes with its burn-in (`adapt`), the next body gets
-// the steps that its own accuracy calls for and no more: a quarter of eta of its update (or of the tolerance, whichever is
-// more), or of what counts far from the solution, its update being expected between 0.1 and 2 times this one's square (0.06 ...
-// 0.43 were seen).  Behind a zero guess the rate is not yet the solution's -- slowly varying inputs lost up to half of it from the
-// first body to the second -- so the second one gets a third more.  (Steps per body of a fixed burn-in raised on need, and so:
-// n = 24, B = 5, T = 4,001, random walks 30 53 53 53 -> 24 37 37 42; n = m = 32, B = 16, T = 1e5, white noise 24 24 24 24 -> 16 22
-// 19 15, 1370 -> 1292 us.)
-//
-// `rounding`: what the mismatch is off by where the update is the difference of two rounded states below one in size.
-struct BodyVerdict { bool counts; int done, burn, need; };   // need: the burn-in for eta itself (0: this body does not tell)
-__device__ __forceinline__ BodyVerdict body_verdict(float e, float mis, float eta, int burn, int burn_cap, int T, float tol, int iters, int max_iter, bool adapt, float rounding)
-{
-    BodyVerdict v{true, 0, burn, 0};
-    if (e <= 3.402823466e38f) {                          // (a NaN or Inf ends the loop)
-        const bool to_tol = tol > 0.0f;
-        const float scale = fmaxf(e, to_tol ? tol : 0.0f), thr = eta * scale;
-        const float near = fmaxf(eta, 1e-3f) * scale, most = to_tol ? fmaxf(fmaxf(near, rounding), 0.05f * fminf(e, 1.0f) * e) : thr;
-        const int never = 1 << 20, whole = max(T, burn);                 // (a burn-in of the whole sequence is exact)
-        const float ratio = mis / e;
-        // steps that take an error down to `part` of itself (what is below 1e-7 of the update is rounding)
-        auto steps = [&](float part) { return ratio < 0.7f ? (int)((float)burn * __logf(part) / __logf(fmaxf(ratio, 1e-7f))) : never; };
-        if (!(mis <= 2.0f * rounding)) v.need = min(steps(0.5f * eta), whole);
-        if (!(mis <= (to_tol ? fmaxf(thr, rounding) : thr))) {
-            auto raised = [&](int n) { return min(max(n < never ? n + n / 10 + 4 : n, burn + 8), whole); };
-            const int wn = raised(steps(0.5f * thr / e));
-            if (!(mis <= most)) {
-                v.counts = false;
-                v.burn = wn;
-                if (adapt && to_tol) {
-                    v.burn = min(wn, max(burn + 8, steps(0.25f * most / e) * 5 / 4));
-                    if (raised(steps(0.5f * near / e)) > burn_cap) v.done = BODY_FALL_BACK;        // (the bodies behind it have to be that good)
-                } else if (wn > burn_cap) {
-                    v.done = BODY_FALL_BACK;
-                }
-                return v;
-            }
-            v.burn = min(wn, burn_cap);
-            if (wn > burn_cap && !(mis <= fmaxf(near, rounding))) v.done = BODY_FALL_BACK;         // (it would not do for the next one)
-        }
-        if (adapt && to_tol && e > tol && !v.done) {
-            const float lo = 0.1f * e * e, hi = fminf(e, 2.0f * e * e);
-            const float part = 0.25f * fmaxf(eta * fmaxf(1.0f, tol / hi), 0.05f * fminf(lo, 1.0f));
-            int wn = steps(part) + 1;
-            if (iters == 0) wn += wn / 3;
-            v.burn = min(min(max(wn, BODY_BURN_MIN), burn_cap), whole);
-        }
-    }
-    if (newton_loop_ends(e, tol, iters, max_iter)) v.done = BODY_DONE;
-    return v;
-}
-
 // End of a body that is a launch of its own: the last CTA's decision.  unit: what the launch rounds its burn-in up to
 // (a rate that is not adapted to may be underestimated); narrow: its products hold what f16 does.  Single thread.
 __device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, int unit = 1, float rounding = 0.0f, bool narrow = false)

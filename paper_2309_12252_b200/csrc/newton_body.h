@@ -58,9 +58,6 @@ struct AdjArgs {
 
 __host__ __device__ constexpr int ADJ_EDGE(int n) { return 2 * n + 1; }
 
-// StatusBlock::done: the loop ended / this form gives up / a bounded wait ran out, nothing that was computed counts
-constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3;
-
 // The kernels of one padded state size (newton_kernels.cu).
 struct BodyKernels {
     void (*one)(BodyArgs);                     // one-phase (newton_body.cuh); n > 8 only
@@ -77,8 +74,6 @@ struct BodyKernels {
 };
 
 constexpr int BODY_L_MIN = 3;    // chains are at least this long
-constexpr int BODY_BURN_MIN = 8; // ... and have at least this burn-in
-constexpr float BODY_ROUNDING = 2.4e-7f;         // two roundings of a state below one in size
 constexpr int CHAIN_L_MIN = 4;   // ... those of every form but the two-phase one: what boundaries and start states are sized by
 
 // The forms of a body.

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
     const bool has_next = nk == NC && tab[NC - 1].next, has_prev = tab[0].t0 > 0 && tab[0].t_end > 0;
     const int G = NC >> 4;                               // groups (a power of two)
 
-    int iters = *(volatile int *)&st->iters, burn = *(volatile int *)&st->burn, need = 0;
+    int iters = *(volatile int *)&st->iters, burn = min(*(volatile int *)&st->burn, a.burn_cap), need = 0;       // (the slots end there)
     const float tol = st->tol;
     const int max_iter = st->max_iter;
     __shared__ unsigned red[4][C::WARPS];

@@ -1,0 +1,52 @@
+"""The decision at the end of a one-launch Newton body (csrc/body_verdict.h), as host code."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2309_12252_b200", "csrc")
+
+HARNESS = r'''
+#include "body_verdict.h"
+using namespace deer;
+extern "C" void verdict(float e, float mis, float eta, int burn, int cap, int T, float tol, int iters, int adapt, float rounding, int *out)
+{
+    const BodyVerdict v = body_verdict(e, mis, eta, burn, cap, T, tol, iters, 100, adapt != 0, rounding);
+    out[0] = v.counts; out[1] = v.done; out[2] = v.burn; out[3] = v.need;
+}
+// Bodies whose boundaries forget by `rho` a step, over updates, burn-ins, limits and accuracies: those that end nothing and would
+// have the next body run a burn-in beyond the limit (over), or the same body again with no more of it (stuck).
+extern "C" void sweep(long long *looked_at, long long *over, long long *stuck)
+{
+    *looked_at = *over = *stuck = 0;
+    const float etas[] = {1e-3f, 1e-4f, 4e-6f}, tols[] = {1e-4f, 1e-6f, 1e-2f, -1.0f};
+    for (float eta : etas) for (float tol : tols) for (int cap : {30, 96, 97, 128, 224, 320, 512}) for (int T : {50, 128, 100000})
+    for (int adapt = 0; adapt < 2; ++adapt) for (int iters = 0; iters < 3; ++iters) for (float rounding : {0.0f, BODY_ROUNDING})
+    for (int burn = 8; burn <= cap && burn < T; burn += 1 + burn / 8)          // (from T on every chain starts at its sequence's first step)
+    for (float e = 1e-6f; e < 1e3f; e *= 3.0f) for (float rho = 0.4f; rho < 1.02f; rho += 0.015f) {
+        const BodyVerdict v = body_verdict(e, e * powf(rho, (float)burn), eta, burn, cap, T, tol, iters, 100, adapt != 0, rounding);
+        ++*looked_at;
+        if (!v.done && v.burn > cap) ++*over;
+        if (!v.done && !v.counts && v.burn <= burn) ++*stuck;
+    }
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def V(tmp_path_factory):
+    d = tmp_path_factory.mktemp("verdict")
+    src, lib = str(d / "harness.cpp"), str(d / "harness.so")
+    with open(src, "w") as f:
+        f.write(HARNESS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", lib], check=True)
+    return ctypes.CDLL(lib)
+
+
+def test_no_body_is_given_a_burn_in_beyond_the_limit(V):
+    """The two-phase kernel's shared memory holds the limit's positions and no more."""
+    looked_at, over, stuck = (ctypes.c_longlong() for _ in range(3))
+    V.sweep(ctypes.byref(looked_at), ctypes.byref(over), ctypes.byref(stuck))
+    assert looked_at.value > 1_000_000
+    assert over.value == 0 and stuck.value == 0, (over.value, stuck.value)

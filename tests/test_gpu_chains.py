@@ -89,6 +89,23 @@ def test_burn_in_of_each_body_follows_the_cell(bd, n, m, B, T, bias, warm, kerne
         assert abs(r.iters - exact.iters) <= 1, (r.iters, exact.iters)
 
 
+@pytest.mark.parametrize("n,m,B,T,bias", [(8, 4, 16, 9001, 2.5), (8, 4, 16, 9001, 2.2), (5, 3, 4, 4001, 2.6), (24, 5, 2, 3001, 2.4), (40, 7, 2, 1501, 2.2)])
+@pytest.mark.parametrize("off", [1e-2, 5e-2])
+def test_warm_start_of_a_cell_that_forgets_a_tenth_a_step(bd, n, m, B, T, bias, off):
+    """The first update is small and calls for some hundred steps of burn-in, as many as the two-phase form's shared memory holds
+    or a few more.  (Gates good to 2e-7 and boundaries to a thousandth of the tolerance, carried over some twenty steps.)"""
+    p = synth.gru_params(n, m, seed=6, tag="c/gru")
+    p.b_i[n:2 * n] += np.float32(bias)
+    x = synth.x_gaussian(B, T, m, seed=6, tag="c/x")
+    y0 = synth.normal(6, "c/y0", (B, n)) * 0.5
+    want = oracle.gru_seq(p, x, y0, np.float32)
+    y = dev(want + off * synth.normal(6, "c/guess", want.shape))
+    r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), y=y, flags=bd.DEER_FLAG_WARM_START))
+    assert SEG in names, names
+    assert r.status == 0 and r.err <= 1e-4
+    assert np.max(np.abs(r.y.cpu().numpy() - want)) <= 2e-5
+
+
 @pytest.mark.parametrize("n,m,B,T", [(1, 1, 16, 300001), (8, 4, 4, 1000), (16, 8, 8, 20000), (24, 3, 2, 700), (32, 8, 16, 8000), (64, 6, 2, 9000)])
 def test_cell_that_remembers_for_long(bd, n, m, B, T):
     """The update gate's bias alone keeps the state: no burn-in is tried, the Jacobians are multiplied out."""
