@@ -9,7 +9,7 @@
 //                                            (a pair of blocks of eight columns is one K step of 16).
 // All products are at fp32 level (a one-shot solve): three TF32 MMAs on split operands up to n = 16, from there on hi + lo f16
 // halves in three m16n8k16 ones, half as many and good to 2^-23 of the operands where those are to 2^-20.  Powers of two
-// (tile_weight_scale, MMA_OP_SCALE, and per row and step one from the row's largest |lambda|) keep the halves among the normal
+// (operand_scales, and per row and step one from the row's largest |lambda|) keep the halves among the normal
 // numbers; a value beyond f16's range makes a NaN, which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a
 // millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
 // the first one.  So a boundary is held to eta of the largest |lambda| of all and, besides, to ADJ_LOCAL eta of the largest
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
     constexpr bool F16 = C::F16;
     extern __shared__ __align__(16) float smb[];
     __shared__ unsigned s_top;
+    __shared__ __align__(16) float s_xf[64];
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
     const int n = a.n, m = a.m, H = a.H, L = a.L;
@@ -119,17 +120,18 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
     uint4 *sH = reinterpret_cast<uint4 *>(smb), *sI = sH + 4 * NB * NS;
     uint4 *sT = sI + 4 * kx * NS;                        // W_h by rows: the B operand of p W_h
     float *sb = reinterpret_cast<float *>(sT + 4 * PB * NS2);
-    float wscale = 1.0f, kS = 1.0f;
+    float wscale = 1.0f, unit = 1.0f, kS = 1.0f;
     if constexpr (F16) {
-        wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
-        kS = 1.0f / (wscale * MMA_OP_SCALE);
+        wscale = operand_scales(hd.W_h, hd.W_i, 3 * n, n, proj ? m : 0, MMA_OP_SCALE, MMA_TOP, s_xf, &s_top);
+        unit = wscale * MMA_OP_SCALE;
+        kS = 1.0f / unit;
     }
     auto record = [&](auto w, int kt) {                  // w(k): row k of the column
         const int k = 8 * KB * (kt >> 2) + 2 * (kt & 3);
         uint4 r;
         if constexpr (F16) {
-            split_f16(make_float2(w(k) * wscale, w(k + 1) * wscale), r.x, r.z);
-            split_f16(make_float2(w(k + 8) * wscale, w(k + 9) * wscale), r.y, r.w);
+            split_f16(make_float2(w(k), w(k + 1)), r.x, r.z);
+            split_f16(make_float2(w(k + 8), w(k + 9)), r.y, r.w);
         } else {
             split_tf32(w(k), r.x, r.z);
             split_tf32(w(k + 1), r.y, r.w);
@@ -139,16 +141,16 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
     for (int idx = tid; idx < 4 * NB * 3 * N; idx += blockDim.x) {
         const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
         const float *wr = hd.W_h + (size_t)(gate * n + i) * n;
-        sH[kt * NS + c] = record([&](int j) { return i < n && j < n ? wr[j] : 0.0f; }, kt);
+        sH[kt * NS + c] = record([&](int j) { return i < n && j < n ? wr[j] * wscale : 0.0f; }, kt);
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
         const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
         const float *wr = hd.W_i + (size_t)(gate * n + i) * m;
-        sI[kt * NS + c] = record([&](int j) { return i < n && j < m ? wr[j] : 0.0f; }, kt);
+        sI[kt * NS + c] = record([&](int j) { return i < n && j < m ? wr[j] * (F16 ? unit * pow2_inverse(s_xf[j]) : 1.0f) : 0.0f; }, kt);
     }
     for (int idx = tid; idx < 4 * PB * N; idx += blockDim.x) {
         const int c = idx % N, kt = idx / N;
-        sT[kt * NS2 + c] = record([&](int j) { return j < 3 * N && j % N < n && c < n ? hd.W_h[(size_t)(j / N * n + j % N) * n + c] : 0.0f; }, kt);
+        sT[kt * NS2 + c] = record([&](int j) { return j < 3 * N && j % N < n && c < n ? hd.W_h[(size_t)(j / N * n + j % N) * n + c] * wscale : 0.0f; }, kt);
     }
     for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
         sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
@@ -269,9 +271,9 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
         if constexpr (U_AHEAD) { if (!proj) load_u(ur_n, uz_n, un_n, 0); }
 
         // block b of a K step of an A operand, row h of this lane: two columns (an accumulator's columns of TF32 in the slots t, t + 4)
-        auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v, float scale) {
+        auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v, float2 scale) {
             if constexpr (F16) {
-                split_f16(fmul2(v, make_float2(scale, scale)), hi[2 * b + h], lo[2 * b + h]);
+                split_f16(fmul2(v, scale), hi[2 * b + h], lo[2 * b + h]);
             } else {
                 split_tf32(v.x, hi[h], lo[h]);
                 split_tf32(v.y, hi[2 + h], lo[2 + h]);
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
                 for (int kk = 0; kk < kx; ++kk) {
                     unsigned ah[4], al[4];
 #pragma unroll
-                    for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], MMA_OP_SCALE);
+                    for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], *reinterpret_cast<const float2 *>(s_xf + (F16 ? 16 * kk + 8 * (q >> 1) + 2 * t : 0)));
                     if (kk + 1 < kx) ldxs(kk + 1, xc);
                     const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
@@ -359,11 +361,10 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
                 load_u(xr, xz, xn, 0);
             }
             if (F16 && !proj) {                          // (in the products' scale: a power of two)
-                const float up = wscale * MMA_OP_SCALE;
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= unit; xz[j][q] *= unit; xn[j][q] *= unit; }
             }
             // the state as A operands, and the power of two of p: |p| <= |lambda| / 4 or so, its exponent to 2^9 in every row
             unsigned ah[NB][4], al[NB][4];
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]), MMA_OP_SCALE);
+                for (int h = 0; h < 2; ++h) operand(ah[j / KB], al[j / KB], j % KB, h, make_float2(hp[j][2 * h], hp[j][2 * h + 1]), make_float2(MMA_OP_SCALE, MMA_OP_SCALE));
             float sc[2] = {1.0f, 1.0f}, kM[2] = {1.0f, 1.0f};
             if constexpr (F16) {
 #pragma unroll
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
                     const float2 zz = fmul2(z, l2);
                     const float2 pg[3] = {pr, pz, pn};
 #pragma unroll
-                    for (int gate = 0; gate < 3; ++gate) operand(ph[(gate * NT + j) / KB], pl[(gate * NT + j) / KB], (gate * NT + j) % KB, h, pg[gate], sc[h]);
+                    for (int gate = 0; gate < 3; ++gate) operand(ph[(gate * NT + j) / KB], pl[(gate * NT + j) / KB], (gate * NT + j) % KB, h, pg[gate], make_float2(sc[h], sc[h]));
                     zl[j][2 * h] = zz.x; zl[j][2 * h + 1] = zz.y;
                     if (step >= burn && act[h]) {
                         if (col < n) mb = max(mb, __float_as_uint(fabsf(l2.x)));

@@ -7,8 +7,8 @@
 //     [16, n] x [n, 3n]                          J_t d_{t-1} = z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d)
 // with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragments of two blocks of eight
 // columns are the A operand of a K step of 16 as they stand, so neither J_t, nor its coefficients, nor any chain product
-// is ever formed or stored.  Powers of two (tile_weight_scale, MMA_OP_SCALE, MMA_D_SCALE) keep the halves among the normal
-// f16 numbers; a value beyond f16's range makes a NaN, and the body is for the other kernels.
+// is ever formed or stored.  Powers of two (operand_scales, MMA_D_SCALE) keep the halves among the normal f16 numbers; a
+// value beyond f16's range makes a NaN, and the body is for the other kernels.
 //
 // What a chain does not know is the update entering it.  It starts `burn` positions early from zero: the error of its
 // entering update is the old error carried through `burn` Jacobians, and the Jacobians of a cell that forgets make it
@@ -54,9 +54,10 @@ __device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, 
     if (HostResult *h = st->host) { h->burn = v.burn; if (v.done) post_done(h, v.done); }
 }
 
-// Scales of x and the states (values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute) and of the update (up to 64;
-// 2^-35 absolute) as f16 operands.
+// Scales of the states (values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute: they come from gates that are good to
+// 2e-7) and of the update (up to 64; 2^-35 absolute) as f16 operands, and of a channel's largest weight (operand_scales).
 constexpr float MMA_OP_SCALE = 4.0f, MMA_D_SCALE = 1024.0f;
+constexpr int MMA_TOP = 10;
 
 template <int N> struct Body {
     static constexpr int NT = N / 8, NB = (NT + 1) / 2;  // column blocks, K steps
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     constexpr int NT = C::NT, NB = C::NB, NS = C::NS, SW = C::SW;
     extern __shared__ __align__(16) float smb[];
     __shared__ unsigned s_top;
+    __shared__ __align__(16) float s_xf[64];
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
     const int n = a.n, m = a.m, H = a.H, L = a.L;
@@ -99,11 +101,11 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     // its end)
     uint4 *sH = reinterpret_cast<uint4 *>(smb), *sI = sH + 4 * NB * NS;
     float *sb = reinterpret_cast<float *>(sI + 4 * kx * NS);
-    const float wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
-    const float kS = 1.0f / (wscale * MMA_OP_SCALE), kD = 1.0f / (wscale * MMA_D_SCALE);
-    auto record = [&](const float *wr, bool row, int kt, int width) {
+    const float wscale = operand_scales(hd.W_h, hd.W_i, 3 * n, n, proj ? m : 0, MMA_OP_SCALE, MMA_TOP, s_xf, &s_top);
+    const float unit = wscale * MMA_OP_SCALE, kS = 1.0f / unit, kD = 1.0f / (wscale * MMA_D_SCALE);
+    auto record = [&](const float *wr, bool row, int kt, int width, auto scale) {
         const int k = 16 * (kt >> 2) + 2 * (kt & 3);
-        auto w = [&](int j) { return row && j < width ? wr[j] * wscale : 0.0f; };
+        auto w = [&](int j) { return row && j < width ? wr[j] * scale(j) : 0.0f; };
         uint4 r;
         split_f16(make_float2(w(k), w(k + 1)), r.x, r.z);
         split_f16(make_float2(w(k + 8), w(k + 9)), r.y, r.w);
@@ -111,11 +113,11 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
     };
     for (int idx = tid; idx < 4 * NB * 3 * N; idx += blockDim.x) {
         const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
-        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n);
+        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n, [&](int) { return wscale; });
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += blockDim.x) {
         const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
-        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m);
+        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m, [&](int j) { return unit * pow2_inverse(s_xf[j]); });
     }
     for (int i = tid; i < N; i += blockDim.x) {          // (u holds b_i already)
         sb[i] = i < n ? hd.b_h[i] + (proj ? hd.b_i[i] : 0.0f) : 0.0f;
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 for (int kk = 0; kk < kx; ++kk) {
                     unsigned ah[4], al[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) split_f16(fmul2(xc[q], make_float2(MMA_OP_SCALE, MMA_OP_SCALE)), ah[q], al[q]);
+                    for (int q = 0; q < 4; ++q) split_f16(fmul2(xc[q], *reinterpret_cast<const float2 *>(s_xf + 16 * kk + 8 * (q >> 1) + 2 * t)), ah[q], al[q]);
                     if (kk + 1 < kx) ldxs(kk + 1, xc);
                     const uint4 *q0 = sI + (4 * kk + t) * NS + g;
 #pragma unroll
@@ -270,11 +272,10 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, N > 32 ? 1 : N > 16 ? 2 : 
                 load_u(xr, xz, xn, 0);
             }
             if (!proj) {                                 // (in the products' scale: a power of two)
-                const float up = wscale * MMA_OP_SCALE;
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= unit; xz[j][q] *= unit; xn[j][q] *= unit; }
             }
             // ---- hidden half and the update, one block of eight columns at a time
             const bool hid = !zero || __any_sync(0xffffffffu, tt[0] == 0 || tt[1] == 0);     // zero guess: W_h 0 = 0

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
     constexpr int NT = C::NT, KB = C::KB, NB = C::NB, NS = C::NS, SZ = C::SZ, DS = C::DS;
     constexpr bool F16 = C::F16;
     __shared__ unsigned s_top;
+    __shared__ __align__(16) float s_xf[64];
     extern __shared__ __align__(16) float smb[];
     const BodyHead hd = a.heads ? a.heads[blockIdx.y] : a.h0;
     StatusBlock *st = a.st + blockIdx.y;
@@ -94,16 +95,17 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
     float *dx = ss + (C::NC_MAX + 1) * DS;               // exchanged updates [2][NC_MAX][DS]
     SegChain *tab = reinterpret_cast<SegChain *>(dx + 2 * C::NC_MAX * DS);
     float *slots = reinterpret_cast<float *>(tab + C::NC_MAX);
-    float wscale = 1.0f, kS = 1.0f, kD = 1.0f;
+    float wscale = 1.0f, unit = 1.0f, kS = 1.0f, kD = 1.0f;
     if constexpr (F16) {
-        wscale = tile_weight_scale(hd.W_h, 3 * n * n, hd.W_i, proj ? 3 * n * m : 0, &s_top);
-        kS = 1.0f / (wscale * MMA_OP_SCALE);
+        wscale = operand_scales(hd.W_h, hd.W_i, 3 * n, n, proj ? m : 0, MMA_OP_SCALE, MMA_TOP, s_xf, &s_top);
+        unit = wscale * MMA_OP_SCALE;
+        kS = 1.0f / unit;
         kD = 1.0f / (wscale * MMA_D_SCALE);
     }
     // weights as records of the four words that a lane needs for a column of a K step (newton_body.cuh)
-    auto record = [&](const float *wr, bool row, int kt, int width) {
+    auto record = [&](const float *wr, bool row, int kt, int width, auto scale) {
         const int k = 8 * KB * (kt >> 2) + 2 * (kt & 3);
-        auto w = [&](int j) { return row && j < width ? wr[j] * wscale : 0.0f; };
+        auto w = [&](int j) { return row && j < width ? wr[j] * scale(j) : 0.0f; };
         uint4 r;
         if constexpr (F16) {
             split_f16(make_float2(w(k), w(k + 1)), r.x, r.z);
@@ -116,16 +118,16 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
     };
     for (int idx = tid; idx < 4 * NB * 3 * N; idx += C::THREADS) {
         const int kt = idx % (4 * NB), c = idx / (4 * NB), gate = c / N, i = c % N;
-        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n);
+        sH[kt * NS + c] = record(hd.W_h + (size_t)(gate * n + i) * n, i < n, kt, n, [&](int) { return wscale; });
     }
     for (int idx = tid; idx < 4 * kx * 3 * N; idx += C::THREADS) {
         const int kt = idx % (4 * kx), c = idx / (4 * kx), gate = c / N, i = c % N;
-        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m);
+        sI[kt * NS + c] = record(hd.W_i + (size_t)(gate * n + i) * m, i < n, kt, m, [&](int j) { return F16 ? unit * pow2_inverse(s_xf[j]) : 1.0f; });
     }
     // block b of a K step of an A operand, row h of this lane: two columns (an accumulator's columns of TF32 in the slots t, t + 4)
-    auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v) {
+    auto operand = [&](unsigned (&hi)[4], unsigned (&lo)[4], int b, int h, float2 v, float2 scale = make_float2(MMA_OP_SCALE, MMA_OP_SCALE)) {
         if constexpr (F16) {
-            split_f16(fmul2(v, make_float2(MMA_OP_SCALE, MMA_OP_SCALE)), hi[2 * b + h], lo[2 * b + h]);
+            split_f16(fmul2(v, scale), hi[2 * b + h], lo[2 * b + h]);
         } else {
             split_tf32(v.x, hi[h], lo[h]);
             split_tf32(v.y, hi[2 + h], lo[2 + h]);
@@ -263,7 +265,7 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
             for (int kk = 0; kk < kx; ++kk) {
                 unsigned ah[4], al[4];
 #pragma unroll
-                for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q]);
+                for (int q = 0; q < 2 * KB; ++q) operand(ah, al, q >> 1, q & 1, xc[q], *reinterpret_cast<const float2 *>(s_xf + (F16 ? 16 * kk + 8 * (q >> 1) + 2 * t : 0)));
                 if (kk + 1 < kx) {
 #pragma unroll
                     for (int q = 0; q < 2 * KB; ++q) xc[q] = act[q & 1] ? ldx(xpp[q & 1], 8 * KB * (kk + 1) + 8 * (q >> 1) + 2 * t) : make_float2(0.0f, 0.0f);
@@ -296,11 +298,10 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
                 }
             if (left > 1) fetch();
             if constexpr (F16) {                         // (in the products' scale: a power of two)
-                const float up = wscale * MMA_OP_SCALE;
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= unit; xz[j][q] *= unit; xn[j][q] *= unit; }
             }
         }
         unsigned ah[NB][4], al[NB][4];

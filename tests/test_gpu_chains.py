@@ -520,3 +520,46 @@ def test_two_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, kernel):
     assert r.status == 0 and r.err <= 1e-4
     want = oracle.gru_seq(p, x, y0, np.float64)
     assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if x_scale == 1.0 else 1e-4)
+
+
+def units(m, kind):
+    """A unit per channel: all of them small, all large, or each of its own."""
+    return (np.full(m, 1e-6) if kind == "small" else np.full(m, 1e5) if kind == "large" else 10.0 ** np.linspace(-7, 6, m)).astype(np.float32)
+
+
+@pytest.mark.parametrize("n,m,B,T,kernel", [
+    (9, 3, 10, 300, SEG), (24, 8, 3, 401, SEG), (24, 16, 16, 6001, SEG), (32, 5, 2, 301, SEG), (40, 33, 4, 301, SEG),
+    (12, 16, 16, 40001, ONE), (16, 5, 16, 15001, ONE), (43, 64, 5, 2003, ONE), (62, 20, 4, 663, ONE)])
+@pytest.mark.parametrize("kind", ["small", "large", "mixed"])
+def test_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kernel, kind):
+    """A normalisation folded into the first layer: x s and W_i / s for x and W_i.  The same bounds as of data of order one: the gates'
+    2e-7, less than ten times of it carried, and no other kernel does the work."""
+    p = synth.gru_params(n, m, seed=20, tag="c/gru")
+    s = units(m, kind)
+    p.W_i[:] = p.W_i / s
+    x = synth.x_gaussian(B, T, m, seed=20, tag="c/x") * s
+    y0 = synth.normal(20, "c/y0", (B, n)) * 0.5
+    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
+    assert kernel in names and not any(k.startswith("cell_") for k in names), names
+    assert r.status == 0 and r.err <= 1e-4
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float64))) <= 3e-6
+
+
+@pytest.mark.parametrize("n,m,B,T", [(12, 5, 8, 3001), (17, 16, 16, 700), (32, 32, 16, 8001), (48, 2, 16, 500), (63, 40, 16, 700)])
+@pytest.mark.parametrize("kind", ["small", "large", "mixed"])
+def test_adjoint_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kind):
+    """As above, for the adjoint: 2-norms agree to 1e-6, of dx channel by channel.  (The trajectory that the gradient is taken at is
+    given; its gates are evaluated anew.)"""
+    p = synth.gru_params(n, m, 21, tag="c/gru")
+    s = units(m, kind)
+    p.W_i[:] = p.W_i / s
+    x = synth.x_gaussian(B, T, m, 21, tag="c/x") * s
+    y0 = synth.normal(21, "c/y0", (B, n)) * 0.3
+    gy = synth.normal(21, "c/gy", (B, T, n))
+    got, want, names, done = gradient(bd, p, x, y0, gy)
+    assert WARP in names and done == 1, names
+    for k in ("db_i", "db_h", "dy0"):
+        assert np.linalg.norm(got[k] - want[k]) <= 1e-6 * np.linalg.norm(want[k]), k
+    for c in range(m):
+        assert np.linalg.norm(got["dx"][..., c] - want["dx"][..., c]) <= 1e-6 * np.linalg.norm(want["dx"][..., c]), c
