@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     extern __shared__ __align__(16) unsigned char smem_tile[];
     __shared__ __align__(8) uint64_t bar1, bar2;
     __shared__ unsigned s_tmem, s_top;
+    __shared__ __align__(16) float s_xf[64];
     __shared__ int s_abort[2], s_side[2];               // s_abort: a wait for products 1, 2 ran out (each read behind a sync that
                                                          // follows its writes, and before one that precedes the next)
     unsigned char *sm = (unsigned char *)(((uintptr_t)smem_tile + 1023) & ~(uintptr_t)1023);
@@ -61,8 +62,8 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     const long long tile = blockIdx.x;
 
     // ---- weights, biases, geometry, tensor memory
-    const float wscale = tile_weight_scale(a.h0.W_h, 3 * N * N, a.h0.W_i, 3 * N * m, &s_top);
-    const float kS = 1.0f / (wscale * TILE_OP_SCALE);
+    const float wscale = operand_scales(a.h0.W_h, a.h0.W_i, 3 * N, N, m, TILE_OP_SCALE, TILE_TOP, s_xf, &s_top);
+    const float unit = wscale * TILE_OP_SCALE, kS = 1.0f / unit;
     for (int i = tid; i < (int)WR * (N / 2); i += C::THREADS) {          // rows of W_h in the order n, r, z
         const int k = 2 * (i % (N / 2)), r = i / (N / 2), gate = r < N ? 2 : r / N - 1;
         const float2 v = *reinterpret_cast<const float2 *>(a.h0.W_h + (size_t)(gate * N + r % N) * N + k);
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         const int k = 2 * (i % (kx / 2)), r = i / (kx / 2);
         const float *w = a.h0.W_i + (size_t)r * m + k;
         unsigned hi, lo;
-        split_f16(make_float2(k < m ? w[0] * wscale : 0.0f, k + 1 < m ? w[1] * wscale : 0.0f), hi, lo);
+        split_f16(make_float2(k < m ? w[0] * (unit * pow2_inverse(s_xf[k])) : 0.0f, k + 1 < m ? w[1] * (unit * pow2_inverse(s_xf[k + 1])) : 0.0f), hi, lo);
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, k)) = hi;
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, kx + k)) = lo;
     }
@@ -156,11 +157,10 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
         }
         cp_async_commit();
     };
-    auto put = [&](unsigned char *panel, int row, int k, int klo, float4 v) {
-        const float2 sc = make_float2(TILE_OP_SCALE, TILE_OP_SCALE);
+    auto put = [&](unsigned char *panel, int row, int k, int klo, float4 v, float4 f) {
         uint2 hi, lo;
-        split_f16(fmul2(make_float2(v.x, v.y), sc), hi.x, lo.x);
-        split_f16(fmul2(make_float2(v.z, v.w), sc), hi.y, lo.y);
+        split_f16(fmul2(make_float2(v.x, v.y), make_float2(f.x, f.y)), hi.x, lo.x);
+        split_f16(fmul2(make_float2(v.z, v.w), make_float2(f.z, f.w)), hi.y, lo.y);
         *reinterpret_cast<uint2 *>(panel + panel_off(128, row, k)) = hi;
         *reinterpret_cast<uint2 *>(panel + panel_off(128, row, klo + k)) = lo;
     };
@@ -168,14 +168,15 @@ __global__ void __launch_bounds__(TileAdj::THREADS, 1) adjoint_tile_kernel(AdjAr
     const bool whole = (m & 3) == 0;
     auto put_operands = [&]() {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) put(sH, lr + 32 * i, 4 * lc, N, wanted((x_in >> i) & 1u, yv[i]));
+        for (int i = 0; i < 4; ++i) put(sH, lr + 32 * i, 4 * lc, N, wanted((x_in >> i) & 1u, yv[i]), make_float4(TILE_OP_SCALE, TILE_OP_SCALE, TILE_OP_SCALE, TILE_OP_SCALE));
         const int c = 4 * lc;
         if (c >= kx) return;
+        const float4 f = *reinterpret_cast<const float4 *>(s_xf + c);       // (the channels' units, whatever they are: 888 -> 895 us at m = 64, 320,000 positions)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float4 v = wanted((x_in >> i) & 1u && c < m, xr[i]);
             if (!whole) { v.y = c + 1 < m ? v.y : 0.f; v.z = c + 2 < m ? v.z : 0.f; v.w = c + 3 < m ? v.w : 0.f; }
-            put(sX, lr + 32 * i, c, kx, v);
+            put(sX, lr + 32 * i, c, kx, v, f);
         }
     };
 

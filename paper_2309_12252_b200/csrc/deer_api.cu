@@ -1110,9 +1110,16 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
     const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
     bool tiles = false;
-    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE}) {
+    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE}) {
         BodyPlan plan{};
         if (form == BodyForm::TILE && !aligned32) continue;
+        if (form == BodyForm::TILE && tiles) {           // again, with the inputs in units of its own (in the place of u)
+            if (hs->done != BODY_UNITS) continue;
+            if ((rc = launch_tile_units(a, w.u, st)) != DEER_OK) return rc;
+            u_done = false;
+            a.x = w.u;
+            a.units = 1;
+        }
         if (form == BodyForm::ONE_PHASE && tiles) break;             // (what the tiles give up is for the kernels that multiply the Jacobians out)
         const bool have_u = form == BodyForm::LANE ? m > 8 : need_u && form != BodyForm::TILE;
         if (!body_plan(&plan, form, B, T, n, m, have_u, nullptr, 1) || !body_suits(plan, n)) continue;

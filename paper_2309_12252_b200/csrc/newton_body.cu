@@ -349,6 +349,14 @@ bool body_suits(const BodyPlan &p, int n)
     return p.waves >= 0.5f;
 }
 
+int launch_tile_units(const BodyArgs &a, float *xs, cudaStream_t st)
+{
+    const size_t count = (size_t)a.B * a.T * a.m;
+    const unsigned blocks = (unsigned)std::min<size_t>((count + 1023) / 1024, 8 * (size_t)sm_count());
+    DEER_KERNEL("tile_units_kernel", st, pick(a.n, true).tile_units<<<blocks, 256, 0, st>>>(a.x, xs, count, a.m, a.h0.W_h, a.h0.W_i));
+    return DEER_OK;
+}
+
 int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st)
 {
     const bool aligned = ((((uintptr_t)a.buf[0] | (uintptr_t)a.buf[1] | (uintptr_t)a.y0 | (uintptr_t)a.u) & 7) == 0);

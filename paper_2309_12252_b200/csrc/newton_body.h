@@ -26,6 +26,7 @@ struct BodyArgs {
     int burn_cap;            // longest burn-in that is tried (BodyPlan)
     int expire;              // test aid: every bounded wait runs out (DEER_FLAG_EXPIRE_BODY_WAITS)
     int polled;              // the host reads the result record while the stream runs
+    int units;               // tiles: x comes from launch_tile_units
     int adapt;               // chains so short that a body's burn-in is its time: no longer than its own accuracy calls for
     StatusBlock *st;         // [H]
     float *edge;             // [groups][2][n]  states either side of a boundary between two warps
@@ -65,6 +66,7 @@ struct BodyKernels {
     void (*(*adj)(int m))(AdjArgs);            // adjoint, one-phase (newton_adjoint.cuh); m: channels contracted in the kernel
     void (*(*tile)(int m))(BodyArgs);          // 128 chains per tcgen05 tile (newton_tile.cuh); n = 32, 64 only
     size_t (*tile_smem)(int m);
+    void (*tile_units)(const float *x, float *xs, size_t count, int m, const float *W_h, const float *W_i);
     int tile_threads, tile_chains;
     void (*(*adj_tile)(int m))(AdjArgs);
     size_t (*adj_tile_smem)(int m);
@@ -118,6 +120,8 @@ int body_first_burn(int n, float tol);
 int body_start_burn(int n, float tol, bool adapt);
 float body_eta(int n, float tol);
 int launch_newton_body(const BodyArgs &a, const BodyPlan &p, cudaStream_t st);
+// xs [B,T,m]: x in the units of the tiles' operands, for BodyArgs::units.
+int launch_tile_units(const BodyArgs &a, float *xs, cudaStream_t st);
 
 bool adjoint_supported(int n, int m, bool have_u);
 bool adjoint_plan(BodyPlan *p, int B, int T, int n, int m, bool have_u, const int *strides, int H);

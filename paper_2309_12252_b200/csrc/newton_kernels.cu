@@ -31,6 +31,7 @@ template <int N> static BodyKernels kernels_of(bool v2, bool exact)
         k.tile = [](int m) -> void (*)(BodyArgs) { return m <= 32 ? newton_tile_kernel<N, 1, true> : newton_tile_kernel<N, 64 / N, false>; };
         k.tile_threads = TileBody<N>::THREADS;
         k.tile_chains = TileBody<N>::GROUPS * TileBody<N>::ROWS;
+        k.tile_units = tile_units_kernel<N>;
         k.tile_smem = [](int m) { return TileBody<N>::smem((m + 15) & ~15); };
     }
 #if BODY_N == 64

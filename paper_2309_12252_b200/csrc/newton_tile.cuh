@@ -5,7 +5,7 @@
 //     x_t W_i^T and y_{t-1} W_h^T   operands as hi + lo f16 halves, three products (good to 2^-23 of the operands and, of x and y
 //                                   below 2^-6, to 2^-29 absolute: below the 2e-7 that the gates' tanh is good to)
 //     d_{t-1} W_h^T                 one product (the solve's accuracy is that of its boundaries, see body_verdict)
-// Operands carry powers of two (tile_weight_scale; OP_SCALE, D_SCALE) that keep the hi halves, and the lo halves of all but small
+// Operands carry powers of two (operand_scales; OP_SCALE, D_SCALE) that keep the hi halves, and the lo halves of all but small
 // operands, among the normal f16 numbers and leave in the exponent arithmetic of the epilogue.  A value beyond f16's range turns the body's error into a NaN: the body
 // does not count and the evaluation goes on with the other kernels (BODY_FALL_BACK).
 // A row is owned by n/16 threads of one lane, 16 columns each (the warps of a warpgroup see their own 32 tensor-memory lanes):
@@ -49,7 +49,31 @@ template <int N> struct TileBody {
     }
 };
 
+// Scales of the states (up to 4,094) and of the update.
 constexpr float TILE_OP_SCALE = 16.0f, TILE_D_SCALE = 1024.0f;
+
+// Inputs have the states' scale where every channel's largest weight is of a usual size, 2^-6 to 4: what x contributes to a gate
+// is then held to 2^-27 absolute, up to 64 or more.  Channels in other units are brought to theirs by tile_units_kernel, once per
+// evaluation, and the kernel is launched again (`units`): contributions are held to 2^-31, up to 1,023.  A factor per channel in
+// the loop, where the weights need none, costs the two-tile form its schedule at 128 registers (n = m = 32, B = 16, T = 1e5:
+// 1262 -> 1345 us) and n = 64 a hundredth.
+constexpr int TILE_TOP = 8;
+__device__ __forceinline__ bool tile_usual(const float *xf, float w, int m, int k)
+{
+    if (k >= m) return true;
+    const int e = (int)(__float_as_uint(xf[k]) >> 23) - (int)(__float_as_uint(w * TILE_OP_SCALE) >> 23) + TILE_TOP;
+    return (e >= -6 && e <= 1) || e == -40;                              // (-40: no weights)
+}
+
+// x in the units that the tile kernel's operands have (W_i' comes with its own inverse factors)
+template <int N> __global__ void __launch_bounds__(256) tile_units_kernel(const float *x, float *xs, size_t count, int m, const float *W_h, const float *W_i)
+{
+    __shared__ __align__(16) float s_xf[64];
+    __shared__ unsigned s_top;
+    operand_scales(W_h, W_i, 3 * N, N, m, TILE_OP_SCALE, TILE_TOP, s_xf, &s_top);
+    const size_t step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += step) xs[i] = x[i] * (s_xf[i % (size_t)m] * (1.0f / TILE_OP_SCALE));
+}
 
 template <int N, int XJ, bool TWICE>
 __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(BodyArgs a)
@@ -63,6 +87,7 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
     extern __shared__ __align__(16) unsigned char smem_tile[];
     __shared__ __align__(8) uint64_t s_bars[C::GROUPS];
     __shared__ unsigned s_tmem, s_top;
+    __shared__ __align__(16) float s_xf[64];
     __shared__ int s_aborts[C::GROUPS], s_sides[C::GROUPS][2];
     unsigned char *sm = (unsigned char *)(((uintptr_t)smem_tile + 1023) & ~(uintptr_t)1023);
     const int m = a.m, kx = (m + 15) & ~15;
@@ -82,8 +107,19 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
     const long long total = (long long)a.B * nchain;
 
     // ---- weights, biases, geometry, tensor memory
-    const float wscale = tile_weight_scale(a.h0.W_h, 3 * N * N, a.h0.W_i, 3 * N * m, &s_top);
+    const float wscale = operand_scales(a.h0.W_h, a.h0.W_i, 3 * N, N, m, TILE_OP_SCALE, TILE_TOP, s_xf, &s_top);
     const float kS = 1.0f / (wscale * TILE_OP_SCALE), kD = 1.0f / (wscale * TILE_D_SCALE);
+    if (!a.units) {
+        if (!__syncthreads_and(tile_usual(s_xf, wscale, m, all))) {      // the inputs' units are for tile_units_kernel
+            if (all == 0 && blockIdx.x == 0) {
+                st->done = BODY_UNITS;
+                if (HostResult *h = st->host) { h->burn = st->burn; post_done(h, BODY_UNITS); }
+            }
+            return;
+        }
+        if (all < 64) s_xf[all] = TILE_OP_SCALE;
+        __syncthreads();
+    }
     for (int i = all; i < (int)WR * (N / 2); i += C::THREADS) {          // rows of W_h in the order n, r, z
         const int k = 2 * (i % (N / 2)), r = i / (N / 2), gate = r < N ? 2 : r / N - 1;
         const float2 v = *reinterpret_cast<const float2 *>(a.h0.W_h + (size_t)(gate * N + r % N) * N + k);
@@ -96,7 +132,8 @@ __global__ void __launch_bounds__(TileBody<N>::THREADS, 1) newton_tile_kernel(Bo
         const int k = 2 * (i % (kx / 2)), r = i / (kx / 2);
         const float *w = a.h0.W_i + (size_t)r * m + k;
         unsigned hi, lo;
-        split_f16(make_float2(k < m ? w[0] * wscale : 0.0f, k + 1 < m ? w[1] * wscale : 0.0f), hi, lo);
+        const float unit = wscale * TILE_OP_SCALE;
+        split_f16(make_float2(k < m ? w[0] * (unit * pow2_inverse(s_xf[k])) : 0.0f, k + 1 < m ? w[1] * (unit * pow2_inverse(s_xf[k + 1])) : 0.0f), hi, lo);
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, k)) = hi;
         *reinterpret_cast<unsigned *>(sWi + panel_off(WR, r, kx + k)) = lo;
     }

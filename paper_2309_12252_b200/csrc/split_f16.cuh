@@ -30,22 +30,6 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const unsigned (&a)[4], u
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// The power of two that brings the largest of `count` weights (and of a second array) to [2^9, 2^10): with it the lo halves
-// of all but the very smallest are normal f16 numbers.  All threads of the CTA; red: one word.
-__device__ __forceinline__ float tile_weight_scale(const float *w0, int n0, const float *w1, int n1, unsigned *red)
-{
-    unsigned top = 0u;
-    for (int i = threadIdx.x; i < n0; i += blockDim.x) top = max(top, __float_as_uint(fabsf(w0[i])));
-    for (int i = threadIdx.x; i < n1; i += blockDim.x) top = max(top, __float_as_uint(fabsf(w1[i])));
-    if (threadIdx.x == 0) *red = 0u;
-    __syncthreads();
-    top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) atomicMax(red, top);
-    __syncthreads();
-    const int e = min(max((int)(*red >> 23), 40), 220);          // (zero, or beyond any use: the scale stays finite)
-    return __uint_as_float((unsigned)(127 + 9 - (e - 127)) << 23);
-}
-
 // Powers of two of a cell's f16 operands.  W_h has one, `w`: 2^10, or less where an entry is 16 or more.  The states have one,
 // `states` (a constant of the kernel's), and products are accumulated in units of 1 / (w states).  W_i and x have one per
 // channel k: the largest weight of the channel comes to 2^`top` and x[k] is multiplied by xf[k], what the accumulators' unit leaves,

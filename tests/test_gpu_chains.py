@@ -529,7 +529,8 @@ def units(m, kind):
 
 @pytest.mark.parametrize("n,m,B,T,kernel", [
     (9, 3, 10, 300, SEG), (24, 8, 3, 401, SEG), (24, 16, 16, 6001, SEG), (32, 5, 2, 301, SEG), (40, 33, 4, 301, SEG),
-    (12, 16, 16, 40001, ONE), (16, 5, 16, 15001, ONE), (43, 64, 5, 2003, ONE), (62, 20, 4, 663, ONE)])
+    (12, 16, 16, 40001, ONE), (16, 5, 16, 15001, ONE), (43, 64, 5, 2003, ONE), (62, 20, 4, 663, ONE),
+    (32, 33, 16, 16001, TILE), (32, 5, 16, 8001, TILE), (64, 64, 7, 2801, TILE), (64, 6, 3, 9001, TILE)])
 @pytest.mark.parametrize("kind", ["small", "large", "mixed"])
 def test_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kernel, kind):
     """A normalisation folded into the first layer: x s and W_i / s for x and W_i.  The same bounds as of data of order one: the gates'
@@ -546,9 +547,11 @@ def test_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kernel, 
     assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float64))) <= 3e-6
 
 
-@pytest.mark.parametrize("n,m,B,T", [(12, 5, 8, 3001), (17, 16, 16, 700), (32, 32, 16, 8001), (48, 2, 16, 500), (63, 40, 16, 700)])
+@pytest.mark.parametrize("n,m,B,T,kernel", [
+    (12, 5, 8, 3001, WARP), (17, 16, 16, 700, WARP), (32, 32, 16, 8001, WARP), (48, 2, 16, 500, WARP), (63, 40, 16, 700, WARP),
+    (64, 6, 4, 20001, MMA_TILE), (64, 61, 16, 4003, MMA_TILE)])
 @pytest.mark.parametrize("kind", ["small", "large", "mixed"])
-def test_adjoint_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kind):
+def test_adjoint_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kernel, kind):
     """As above, for the adjoint: 2-norms agree to 1e-6, of dx channel by channel.  (The trajectory that the gradient is taken at is
     given; its gates are evaluated anew.)"""
     p = synth.gru_params(n, m, 21, tag="c/gru")
@@ -558,7 +561,7 @@ def test_adjoint_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, 
     y0 = synth.normal(21, "c/y0", (B, n)) * 0.3
     gy = synth.normal(21, "c/gy", (B, T, n))
     got, want, names, done = gradient(bd, p, x, y0, gy)
-    assert WARP in names and done == 1, names
+    assert kernel in names and done == 1, names
     for k in ("db_i", "db_h", "dy0"):
         assert np.linalg.norm(got[k] - want[k]) <= 1e-6 * np.linalg.norm(want[k]), k
     for c in range(m):
