@@ -16,8 +16,9 @@ using std::min;
 #endif
 
 // StatusBlock::done: the loop ended / this form gives up / a bounded wait ran out, nothing that was computed counts / the tiles
-// take the inputs in units of their own (tile_units_kernel)
-constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3, BODY_UNITS = 4;
+// take the inputs in units of their own (tile_units_kernel) / a value is beyond f16's range, or not finite at all: the kernels
+// without f16 operands tell, and no burn-in is told
+constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3, BODY_UNITS = 4, BODY_BEYOND = 5;
 
 constexpr int BODY_BURN_MIN = 8; // shortest burn-in that is tried
 constexpr float BODY_ROUNDING = 2.4e-7f;         // two roundings of a state below one in size

@@ -1087,7 +1087,7 @@ constexpr int BIAS_US = 20, RESULT_US = 20000;
 // try fails holds up the others (17 heads of 8: 815 -> 1226 us).
 constexpr int BODY_L_ADAPT = 64;
 
-// Runs the Newton loop until it ends or the form gives up (hs->done == BODY_FALL_BACK, the iterate after hs->iters bodies in
+// Runs the Newton loop until it ends or the forms give up (hs->done is not BODY_DONE, the iterate after hs->iters bodies in
 // buf[hs->iters & 1]).
 template <typename CopyOut>
 static int eval_one_launch(const deer_gru_params *p, const float *x, const float *y0, int B, int T, float tol, int max_iter,
@@ -1171,7 +1171,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
                 // A result for the host starts on its way, and the next form goes ahead, as soon as the record tells.
                 const int end = record_posted(hr, st, to_host ? RESULT_US : BIAS_US);
                 polled = to_host && end == BODY_DONE;
-                if (end != BODY_FALL_BACK && !polled) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
+                if ((end == 0 || end == BODY_DONE || end == BODY_TIMED_OUT) && !polled) DEER_CHECK_CUDA(cudaStreamSynchronize(st), "sync");
                 hs->iters = hr->iters; hs->done = hr->done; hs->burn = hr->burn; hs->err_last_bits = hr->err_bits;
                 if (hs->done == BODY_TIMED_OUT || (plan.whole_loop && !hs->done)) return DEER_ERR_DEVICE_TIMEOUT;
             } else {
@@ -1182,9 +1182,10 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
             if (hs->done) break;
         }
         if (hs->done == BODY_DONE) return copy_out(true);
+        if (hs->done == BODY_BEYOND) break;              // (the other forms for this n have no wider range)
         burn = hs->burn;
     }
-    return DEER_OK;                                      // (hs->done == BODY_FALL_BACK)
+    return DEER_OK;                                      // (hs->done == BODY_FALL_BACK or BODY_BEYOND)
 }
 
 // Results up to this size are copied to host memory before it is known that they are final: the copy is then enqueued while the

@@ -37,10 +37,11 @@ __device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, 
 {
     const float e = __uint_as_float(*(volatile unsigned *)&st->err_bits);
     const float mis = __uint_as_float(*(volatile unsigned *)&st->mis_bits);
-    if (narrow && (!(e <= 3.402823466e38f) || !(mis <= 3.402823466e38f))) {        // beyond f16's range, or not finite at all: the other kernels tell
+    if (narrow && (!(e <= 3.402823466e38f) || !(mis <= 3.402823466e38f))) {
         st->err_bits = 0u; st->mis_bits = 0u;
-        st->done = BODY_FALL_BACK;
-        if (HostResult *h = st->host) post_done(h, BODY_FALL_BACK);
+        st->burn = 0;
+        st->done = BODY_BEYOND;
+        if (HostResult *h = st->host) { h->burn = 0; post_done(h, BODY_BEYOND); }
         return;
     }
     const BodyVerdict v = body_verdict(e, mis, a.eta, a.adapt ? (st->burn + unit - 1) / unit * unit : st->burn, a.burn_cap, a.T, st->tol, st->iters, st->max_iter, a.adapt != 0, rounding);

@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(Seg<N, EXACT>::THREADS, 1) newton_segment_kern
         const unsigned qb = __reduce_max_sync(0xffffffffu, lane < C::WARPS ? red[3][lane] : 0u);
         BodyVerdict v = body_verdict(__uint_as_float(eb), __uint_as_float(qb), a.eta, burn, a.burn_cap, a.T, tol, iters, max_iter, a.adapt != 0, 0.0f);
         if (F16 && (!(__uint_as_float(eb) <= 3.402823466e38f) || !(__uint_as_float(qb) <= 3.402823466e38f)))
-            v = BodyVerdict{false, BODY_FALL_BACK, burn, 0};         // beyond f16's range, or not finite at all: the other kernels tell
+            v = BodyVerdict{false, BODY_BEYOND, 0, 0};
         need = max(need, v.need);
         if (blockIdx.x == 0 && tid == 0) {
             if (v.counts) {

@@ -566,3 +566,21 @@ def test_adjoint_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, 
         assert np.linalg.norm(got[k] - want[k]) <= 1e-6 * np.linalg.norm(want[k]), k
     for c in range(m):
         assert np.linalg.norm(got["dx"][..., c] - want["dx"][..., c]) <= 1e-6 * np.linalg.norm(want["dx"][..., c]), c
+
+
+@pytest.mark.parametrize("n,m,B,T,kernel", [(24, 4, 3, 401, SEG), (24, 4, 16, 40001, ONE), (32, 32, 16, 6001, TILE)])
+@pytest.mark.parametrize("slow", [False, True])
+def test_values_beyond_f16_go_to_the_other_kernels_at_once(bd, n, m, B, T, kernel, slow):
+    """What an operand cannot hold is for the kernels without f16 operands: no other form of the same range is tried, whatever an
+    earlier call has left behind (a cell that forgets, or one that was given up because it does not)."""
+    p = synth.gru_params(n, m, seed=22, tag="c/gru")
+    q = synth.gru_params(n, m, seed=22, tag="c/gru")
+    q.b_i[n:2 * n] += np.float32(8.0 if slow else 0.0)
+    x = synth.x_gaussian(B, T, m, seed=22, tag="c/x")
+    y0 = dev(np.zeros((B, n), np.float32))
+    bd.deer_gru_eval(bd.GruParamsDev.from_numpy(q), dev(x), y0)
+    x[1, 100] = 1e9 * np.sign(x[1, 100])
+    r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), y0))
+    assert names & {SEG, ONE, TILE} == {kernel} and any(k.startswith("cell_") for k in names), names
+    assert r.status == 0
+    assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, np.zeros((B, n), np.float32), np.float32))) <= 1e-4
