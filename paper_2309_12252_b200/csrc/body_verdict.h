@@ -76,7 +76,10 @@ DEER_HD BodyVerdict body_verdict(float e, float mis, float eta, int burn, int bu
                 if (adapt && to_tol) {
                     // (no kernel is given more than burn_cap: the two-phase form's shared memory holds no more positions)
                     v.burn = min(min(wn, max(burn + 8, steps(0.25f * most / e) * 5 / 4)), burn_cap);
-                    if (v.burn <= burn || raised(steps(0.5f * near / e)) > burn_cap) v.done = BODY_FALL_BACK;        // (the bodies behind it have to be that good)
+                    if (v.burn <= burn || raised(steps(0.5f * near / e)) > burn_cap) {               // (the bodies behind it have to be that good)
+                        v.done = BODY_FALL_BACK;
+                        v.burn = wn;                     // (what eta would need is what is told: a gradient's first burn-in comes from it)
+                    }
                 } else if (wn > burn_cap) {
                     v.done = BODY_FALL_BACK;
                 }

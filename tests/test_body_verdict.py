@@ -1,5 +1,6 @@
 """The decision at the end of a one-launch Newton body (csrc/body_verdict.h), as host code."""
 import ctypes
+import math
 import os
 import subprocess
 
@@ -50,3 +51,23 @@ def test_no_body_is_given_a_burn_in_beyond_the_limit(V):
     V.sweep(ctypes.byref(looked_at), ctypes.byref(over), ctypes.byref(stuck))
     assert looked_at.value > 1_000_000
     assert over.value == 0 and stuck.value == 0, (over.value, stuck.value)
+
+
+def verdict(V, e, mis, eta, burn, cap, T, tol, iters, adapt, rounding=0.0):
+    out = (ctypes.c_int * 4)()
+    f = ctypes.c_float
+    V.verdict(f(e), f(mis), f(eta), burn, cap, T, f(tol), iters, int(adapt), f(rounding), out)
+    return dict(counts=out[0], done=out[1], burn=out[2], need=out[3])
+
+
+FALL_BACK = 2
+
+
+@pytest.mark.parametrize("rho", [0.93, 0.95, 0.97])
+@pytest.mark.parametrize("eta", [1e-3, 1e-4])
+def test_a_form_that_gives_up_tells_what_its_boundaries_would_need(V, rho, eta):
+    """Whatever the next body would have been given: the steps after which half of eta of the update is left."""
+    e, burn = 1e-2, 30
+    told = [verdict(V, e, e * rho ** burn, eta, burn, 64, 100000, 1e-4, 1, adapt) for adapt in (False, True)]
+    assert all(v["done"] == FALL_BACK and not v["counts"] for v in told), told
+    assert told[0]["burn"] == told[1]["burn"] >= math.log(0.5 * eta) / math.log(rho), told
