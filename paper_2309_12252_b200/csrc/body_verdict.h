@@ -53,21 +53,23 @@ DEER_HD float verdict_log(float x)
 // n = 24, B = 5, T = 4,001, random walks 30 53 53 53 -> 24 37 37 42; n = m = 32, B = 16, T = 1e5, white noise 24 24 24 24 -> 16 22
 // 19 15, 1370 -> 1292 us.)
 //
-// `rounding`: what the mismatch is off by where the update is the difference of two rounded states below one in size.
+// `rounding`: what the mismatch is off by where the update is the difference of two rounded states below one in size.  A carried
+// error of that size looks the same, so it passes only where it is small beside the tolerance: up to 2.5e-3 of that, as much as a
+// good quasi-Newton step leaves anyway.  Below a tolerance of 1e-4 the other kernels finish what rounding makes undecidable here.
 struct BodyVerdict { bool counts; int done, burn, need; };   // need: the burn-in for eta itself (0: this body does not tell)
 DEER_HD BodyVerdict body_verdict(float e, float mis, float eta, int burn, int burn_cap, int T, float tol, int iters, int max_iter, bool adapt, float rounding)
 {
     BodyVerdict v{true, 0, burn, 0};
     if (e <= 3.402823466e38f) {                          // (a NaN or Inf ends the loop)
         const bool to_tol = tol > 0.0f;
-        const float scale = fmaxf(e, to_tol ? tol : 0.0f), thr = eta * scale;
-        const float near = fmaxf(eta, 1e-3f) * scale, most = to_tol ? fmaxf(fmaxf(near, rounding), 0.05f * fminf(e, 1.0f) * e) : thr;
+        const float scale = fmaxf(e, to_tol ? tol : 0.0f), thr = eta * scale, slack = to_tol ? fminf(rounding, 2.5e-3f * tol) : 0.0f;
+        const float near = fmaxf(eta, 1e-3f) * scale, most = to_tol ? fmaxf(fmaxf(near, slack), 0.05f * fminf(e, 1.0f) * e) : thr;
         const int never = 1 << 20, whole = max(T, burn);                 // (a burn-in of the whole sequence is exact)
         const float ratio = mis / e;
         // steps that take an error down to `part` of itself (what is below 1e-7 of the update is rounding)
         auto steps = [&](float part) { return ratio < 0.7f ? (int)((float)burn * verdict_log(part) / verdict_log(fmaxf(ratio, 1e-7f))) : never; };
         if (!(mis <= 2.0f * rounding)) v.need = min(steps(0.5f * eta), whole);
-        if (!(mis <= (to_tol ? fmaxf(thr, rounding) : thr))) {
+        if (!(mis <= fmaxf(thr, slack))) {
             auto raised = [&](int n) { return min(max(n < never ? n + n / 10 + 4 : n, burn + 8), whole); };
             const int wn = raised(steps(0.5f * thr / e));
             if (!(mis <= most)) {
@@ -86,7 +88,7 @@ DEER_HD BodyVerdict body_verdict(float e, float mis, float eta, int burn, int bu
                 return v;
             }
             v.burn = min(wn, burn_cap);
-            if (wn > burn_cap && !(mis <= fmaxf(near, rounding))) v.done = BODY_FALL_BACK;         // (it would not do for the next one)
+            if (wn > burn_cap && !(mis <= fmaxf(near, slack))) v.done = BODY_FALL_BACK;         // (it would not do for the next one)
         }
         if (adapt && to_tol && e > tol && !v.done) {
             const float lo = 0.1f * e * e, hi = fminf(e, 2.0f * e * e);

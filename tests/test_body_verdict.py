@@ -71,3 +71,17 @@ def test_a_form_that_gives_up_tells_what_its_boundaries_would_need(V, rho, eta):
     told = [verdict(V, e, e * rho ** burn, eta, burn, 64, 100000, 1e-4, 1, adapt) for adapt in (False, True)]
     assert all(v["done"] == FALL_BACK and not v["counts"] for v in told), told
     assert told[0]["burn"] == told[1]["burn"] >= math.log(0.5 * eta) / math.log(rho), told
+
+
+@pytest.mark.parametrize("eta", [1e-3, 1e-4])
+@pytest.mark.parametrize("tol", [1e-3, 1e-4, 1e-5, 1e-6, 1e-7, 1e-9])
+@pytest.mark.parametrize("rounding", [0.0, 2.4e-7])
+def test_an_evaluation_does_not_end_on_a_boundary_that_is_off_by_more_than_its_tolerance_allows(V, eta, tol, rounding):
+    """The last body's boundaries are good to 2.5e-3 of the tolerance, whatever its states are rounded to; at 1e-4 rounding is no
+    reason to run it again."""
+    for mis in (1e-12, 1e-10, 3e-9, 6e-8, 1.2e-7, 2.4e-7, 1e-6, 1e-5):
+        v = verdict(V, 0.5 * tol, mis, eta, 30, 512, 100000, tol, 3, False, rounding)
+        if v["counts"]:
+            assert mis <= 2.5e-3 * tol * (1 + 1e-6), mis
+        elif rounding and mis <= 2.4e-7:
+            assert tol < 1e-4, mis
