@@ -57,7 +57,7 @@ constexpr float TILE_OP_SCALE = 16.0f, TILE_D_SCALE = 1024.0f;
 // evaluation, and the kernel is launched again (`units`): contributions are held to 2^-31, up to 1,023.  A factor per channel in
 // the loop, where the weights need none, costs the two-tile form its schedule at 128 registers (n = m = 32, B = 16, T = 1e5:
 // 1262 -> 1345 us) and n = 64 a hundredth.
-constexpr int TILE_TOP = 8;
+constexpr int TILE_TOP = 10;
 __device__ __forceinline__ bool tile_usual(const float *xf, float w, int m, int k)
 {
     if (k >= m) return true;

@@ -30,12 +30,12 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const unsigned (&a)[4], u
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Powers of two of a cell's f16 operands.  W_h has one, `w`: 2^10, or less where an entry is 16 or more.  The states have one,
+// Powers of two of a cell's f16 operands.  W_h has one, `w`: 2^12, or less where an entry is 4 or more.  The states have one,
 // `states` (a constant of the kernel's), and products are accumulated in units of 1 / (w states).  W_i and x have one per
 // channel k: the largest weight of the channel comes to 2^`top` and x[k] is multiplied by xf[k], what the accumulators' unit leaves,
 // which is 2^-top w states times that weight.  x[k] then counts by what it contributes to a gate, in whatever unit it comes: with top =
-// 10 and states = 4 a contribution is good to 2^-22 of itself or 2^-27 absolute, below the 2e-7 of the gates' own arithmetic, up
-// to 16,376.  (One power of two for x and one for both matrices held the same cell in other units, x s and W_i / s, to 3e-4 at s =
+// 10 and states = 4 a contribution is good to 2^-22 of itself or 2^-29 absolute, below the 2e-7 of the gates' own arithmetic, up
+// to 4,094.  (One power of two for x and one for both matrices held the same cell in other units, x s and W_i / s, to 3e-4 at s =
 // 1e-5 and 4e-3 at 1e-6.)
 // All threads of the CTA; xf: 64 words of shared memory (m <= 64; m = 0: none of W_i), red: one.  Returns w.
 __device__ __forceinline__ float operand_scales(const float *W_h, const float *W_i, int rows, int n, int m, float states, int top, float *xf, unsigned *red)
@@ -57,7 +57,7 @@ __device__ __forceinline__ float operand_scales(const float *W_h, const float *W
     __syncthreads();
     const auto exponent = [](unsigned bits, int lo, int hi) { return min(max((int)(bits >> 23) - 127, lo), hi); };     // (zero, or beyond any use: the scales stay finite)
     const auto pow2 = [](int e) { return __uint_as_float((unsigned)(127 + e) << 23); };
-    const float w = pow2(10 - max(exponent(*red, 0, 60) - 3, 0));
+    const float w = pow2(12 - max(exponent(*red, 0, 60) - 1, 0));
     for (int k = threadIdx.x; k < 64; k += blockDim.x) xf[k] = w * states * pow2(exponent(xm[k], -40, 60) - top);
     __syncthreads();
     return w;
