@@ -56,8 +56,9 @@ __device__ __forceinline__ void body_decide(StatusBlock *st, const BodyArgs &a, 
 }
 
 // Scales of the states (values up to 16,376; what is below 2^-5 of one keeps 2^-27 absolute: they come from gates that are good to
-// 2e-7) and of the update (up to 64; 2^-35 absolute) as f16 operands, and of a channel's largest weight (operand_scales).
-constexpr float MMA_OP_SCALE = 4.0f, MMA_D_SCALE = 1024.0f;
+// 2e-7) and of the update (up to 1,023, as behind a y0 of some hundred; 2^-31 absolute: the last body's is the tolerance or less) as
+// f16 operands, and of a channel's largest weight (operand_scales).
+constexpr float MMA_OP_SCALE = 4.0f, MMA_D_SCALE = 64.0f;
 constexpr int MMA_TOP = 10;
 
 template <int N> struct Body {

@@ -603,3 +603,15 @@ def test_a_tolerance_below_what_a_boundary_can_show(bd, n, m, B, T, kernel, tol)
     want = oracle.gru_seq(p, x, y0, np.float64)
     off = [np.max(np.abs(q.y.cpu().numpy() - want)) for q in (r, other)]
     assert off[0] <= 1.5 * off[1] + 2.4e-7, off
+
+
+def test_updates_of_some_hundred_stay_with_the_chains(bd):
+    """A start far from anything that a gate gives: updates of up to 140 on the way, and the chains' f16 operands hold them.  (Much
+    larger ones come of iterations that do not converge in any form.)"""
+    n, m, B, T = 9, 3, 10, 300
+    p = synth.gru_params(n, m, seed=24, tag="c/gru")
+    x = synth.x_gaussian(B, T, m, seed=24, tag="c/x")
+    y0 = np.clip(synth.normal(24, "c/y0", (B, n)), -3, 3) * np.float32(30.0)
+    r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)))
+    assert SEG in names and not any(k.startswith("cell_") for k in names), names
+    assert r.status == 0 and r.err <= 1e-4 and max(r.err_trace[:r.iters]) > 64
