@@ -85,3 +85,21 @@ def test_an_evaluation_does_not_end_on_a_boundary_that_is_off_by_more_than_its_t
             assert mis <= 2.5e-3 * tol * (1 + 1e-6), mis
         elif rounding and mis <= 2.4e-7:
             assert tol < 1e-4, mis
+
+
+@pytest.mark.parametrize("eta", [1e-3, 1e-4])
+def test_the_next_burn_in_follows_the_decay(V, eta):
+    """Short chains: the steps that take the next update's error, of about the square of this one, down to a quarter of what it is
+    asked for, at the rate that this body showed, and a third more behind a zero guess.  Others keep theirs."""
+    e, burn = 0.1, 24
+    for iters in (0, 2):
+        got = []
+        for rho in (0.52, 0.57, 0.62, 0.67, 0.72):            # (0.52^24: what is below 1e-7 of an update is rounding)
+            v = verdict(V, e, e * rho ** burn, eta, burn, 512, 100000, 1e-4, iters, True)
+            assert v["counts"] and not v["done"]
+            want = math.log(0.25 * max(eta, 0.05 * 0.1 * e * e)) / math.log(rho) * (4 / 3 if iters == 0 else 1)
+            assert abs(v["burn"] - max(8, want)) <= 2, (rho, v)
+            got.append(v["burn"])
+            assert verdict(V, e, e * rho ** burn, eta, burn, 512, 100000, 1e-4, iters, False)["burn"] == burn or rho ** burn > eta
+        assert got == sorted(got) and got[-1] >= 1.8 * got[0]
+        assert verdict(V, e, e * 0.72 ** burn, eta, burn, burn, 100000, 1e-4, iters, True)["burn"] == burn

@@ -39,6 +39,11 @@ def walk(x):
     return ((x - x.mean(1, keepdims=True)) / x.std(1, keepdims=True)).astype(np.float32)
 
 
+def behind(names):
+    """Did the kernels that multiply the Jacobians out do a body?"""
+    return any(k.startswith("cell_") for k in names)
+
+
 SEG, ONE, TILE, LANE = "newton_segment_kernel", "newton_body_kernel", "newton_tile_kernel", "newton_lane_kernel"
 
 
@@ -81,7 +86,8 @@ def test_burn_in_of_each_body_follows_the_cell(bd, n, m, B, T, bias, warm, kerne
     args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
     y = dev(want + 1e-2 * synth.normal(6, "c/guess", want.shape)) if warm else None
     r, names = launched(bd, lambda: bd.deer_gru_eval(*args, y=y, flags=bd.DEER_FLAG_WARM_START if warm else 0))
-    assert kernel in names, names
+    # (of the cells that keep more, those of n = 16 and 32 ask for more than is worth trying beside the kernels behind)
+    assert kernel in names and behind(names) == (bias > 0 and n in (16, 32)), names
     assert r.status == 0 and r.err <= 1e-4
     assert np.max(np.abs(r.y.cpu().numpy() - want)) <= 1e-5
     if not warm:
@@ -420,7 +426,7 @@ def test_evaluation_tile_beyond_the_range_of_its_operands(bd, n, m, B, T, t):
     x[1, t] *= np.float32(2e4)
     y0 = synth.normal(17, "c/y0", (B, n)) * 0.5
     r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)))
-    assert TILE in names and any(k.startswith("cell_") for k in names), names
+    assert TILE in names and behind(names), names
     assert r.status == 0
     assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float32))) <= 1e-4
 
@@ -475,14 +481,11 @@ def test_adjoint_products_are_at_fp32_level(bd, n, m, B, T, gy_scale, x_scale, k
     x = synth.x_gaussian(B, T, m, 8, tag="c/x")
     x[:, :, 0] = np.clip(x[:, :, 0], -4, 4) * np.float32(x_scale)
     y0 = synth.normal(8, "c/y0", (B, n)) * 0.3
-    y = oracle.gru_seq(p, x, y0, np.float32)
     gy = (synth.normal(8, "c/gy", (B, T, n)).astype(np.float64) * gy_scale).astype(np.float32)
-    want = oracle.gru_bptt(p, x, y0, y.astype(np.float64), gy, np.float64)
-    args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0), dev(y), dev(gy)
-    got, names = launched(bd, lambda: bd.deer_gru_vjp(*args, want_dx=True))
-    assert kernel is None or kernel in names, names
+    got, want, names, done = gradient(bd, p, x, y0, gy)
+    assert WARP in names and done == (0 if kernel is None else 1), names
     for k in ("db_i", "db_h", "dx", "dy0"):
-        a, b = got[k].cpu().numpy().astype(np.float64), want[k].astype(np.float64)
+        a, b = got[k], want[k].astype(np.float64)
         assert np.linalg.norm(a - b) <= (1e-6 if x_scale == 1.0 else 1e-3) * np.linalg.norm(b), k
 
 
@@ -499,7 +502,7 @@ def test_one_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, y0_scale,
     y0 = np.clip(synth.normal(9, "c/y0", (B, n)), -3, 3) * np.float32(y0_scale)
     args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
     r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
-    assert kernel is None or kernel in names, names
+    assert ONE in names and behind(names) == (kernel is None), names
     assert r.status == 0 and r.err <= 1e-4
     want = oracle.gru_seq(p, x, y0, np.float64)
     assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if y0_scale < 1.0 and x_scale == 1.0 else 1e-4)
@@ -516,7 +519,7 @@ def test_two_phase_products_are_at_fp32_level(bd, n, m, B, T, x_scale, kernel):
     y0 = synth.normal(10, "c/y0", (B, n)) * 0.5
     args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
     r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
-    assert kernel is None or kernel in names, names
+    assert SEG in names and behind(names) == (kernel is None), names
     assert r.status == 0 and r.err <= 1e-4
     want = oracle.gru_seq(p, x, y0, np.float64)
     assert np.max(np.abs(r.y.cpu().numpy() - want)) <= (3e-6 if x_scale == 1.0 else 1e-4)
@@ -542,7 +545,7 @@ def test_products_do_not_depend_on_the_unit_of_an_input(bd, n, m, B, T, kernel, 
     y0 = synth.normal(20, "c/y0", (B, n)) * 0.5
     args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
     r, names = launched(bd, lambda: bd.deer_gru_eval(*args))
-    assert kernel in names and not any(k.startswith("cell_") for k in names), names
+    assert kernel in names and not behind(names), names
     assert r.status == 0 and r.err <= 1e-4
     assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, y0, np.float64))) <= 3e-6
 
@@ -581,7 +584,7 @@ def test_values_beyond_f16_go_to_the_other_kernels_at_once(bd, n, m, B, T, kerne
     bd.deer_gru_eval(bd.GruParamsDev.from_numpy(q), dev(x), y0)
     x[1, 100] = 1e9 * np.sign(x[1, 100])
     r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), y0))
-    assert names & {SEG, ONE, TILE} == {kernel} and any(k.startswith("cell_") for k in names), names
+    assert names & {SEG, ONE, TILE} == {kernel} and behind(names), names
     assert r.status == 0
     assert np.max(np.abs(r.y.cpu().numpy() - oracle.gru_seq(p, x, np.zeros((B, n), np.float32), np.float32))) <= 1e-4
 
@@ -598,7 +601,7 @@ def test_a_tolerance_below_what_a_boundary_can_show(bd, n, m, B, T, kernel, tol)
     args = bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)
     r, names = launched(bd, lambda: bd.deer_gru_eval(*args, tol=tol))
     other = bd.deer_gru_eval(*args, tol=tol, flags=bd.DEER_FLAG_MATERIALIZE)
-    assert kernel in names and any(k.startswith("cell_") for k in names), names
+    assert kernel in names and behind(names), names
     assert r.status == 0 and r.err <= tol or r.status == bd.DEER_NOT_CONVERGED      # (updates of 1e-7 are the rounding of a state near one: they may not end)
     want = oracle.gru_seq(p, x, y0, np.float64)
     off = [np.max(np.abs(q.y.cpu().numpy() - want)) for q in (r, other)]
@@ -613,5 +616,5 @@ def test_updates_of_some_hundred_stay_with_the_chains(bd):
     x = synth.x_gaussian(B, T, m, seed=24, tag="c/x")
     y0 = np.clip(synth.normal(24, "c/y0", (B, n)), -3, 3) * np.float32(30.0)
     r, names = launched(bd, lambda: bd.deer_gru_eval(bd.GruParamsDev.from_numpy(p), dev(x), dev(y0)))
-    assert SEG in names and not any(k.startswith("cell_") for k in names), names
+    assert SEG in names and not behind(names), names
     assert r.status == 0 and r.err <= 1e-4 and max(r.err_trace[:r.iters]) > 64
