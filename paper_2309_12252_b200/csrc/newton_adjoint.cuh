@@ -361,10 +361,11 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
                 load_u(xr, xz, xn, 0);
             }
             if (F16 && !proj) {                          // (in the products' scale: a power of two)
+                const float up = pow2_inverse(kS);
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) { xr[j][q] *= unit; xz[j][q] *= unit; xn[j][q] *= unit; }
+                    for (int q = 0; q < 4; ++q) { xr[j][q] *= up; xz[j][q] *= up; xn[j][q] *= up; }
             }
             // the state as A operands, and the power of two of p: |p| <= |lambda| / 4 or so, its exponent to 2^9 in every row
             unsigned ah[NB][4], al[NB][4];

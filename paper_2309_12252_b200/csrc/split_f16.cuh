@@ -44,16 +44,23 @@ __device__ __forceinline__ float operand_scales(const float *W_h, const float *W
     for (int k = threadIdx.x; k < 64; k += blockDim.x) xm[k] = 0u;
     if (threadIdx.x == 0) *red = 0u;
     __syncthreads();
-    unsigned q = 0u;
-    for (int i = threadIdx.x; i < rows * n; i += blockDim.x) q = max(q, __float_as_uint(fabsf(W_h[i])));
+    const auto largest = [](const float *v, int end, int step) {         // (eight loads in flight: the launch waits for this)
+        unsigned t = 0u;
+        for (int i = threadIdx.x; i < end; i += 8 * step) {
+            float w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = i + j * step < end ? v[i + j * step] : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t = max(t, __float_as_uint(fabsf(w[j])));
+        }
+        return t;
+    };
+    const int threads = blockDim.x, taken = m > 0 ? min(threads / m, 16) * m : 0;    // of W_i a thread to a channel, sixteen at most
+    unsigned q = largest(W_h, rows * n, threads);
+    const unsigned c = (int)threadIdx.x < taken ? largest(W_i, rows * m, taken) : 0u;
     q = __reduce_max_sync(0xffffffffu, q);
     if ((threadIdx.x & 31) == 0) atomicMax(red, q);
-    if (m > 0) {
-        const int per = blockDim.x / m, r0 = threadIdx.x / m, k = threadIdx.x % m;       // a thread to a channel, `per` rows at a time
-        unsigned c = 0u;
-        for (int r = r0; r < rows && r0 < per; r += per) c = max(c, __float_as_uint(fabsf(W_i[r * m + k])));
-        if (c) atomicMax(xm + k, c);
-    }
+    if (c) atomicMax(xm + (int)threadIdx.x % m, c);
     __syncthreads();
     const auto exponent = [](unsigned bits, int lo, int hi) { return min(max((int)(bits >> 23) - 127, lo), hi); };     // (zero, or beyond any use: the scales stay finite)
     const auto pow2 = [](int e) { return __uint_as_float((unsigned)(127 + e) << 23); };
