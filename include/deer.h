@@ -200,7 +200,9 @@ int deer_gru_cell_jac(const deer_gru_params *params, const float *x, const float
  * One global err over the whole batch.
  *   x [B,T,m]   y0 [B,n]   y [B,T,n] out (in: guess if warm start)
  *   tol        : paper default 1e-4 for fp32; a negative tol runs exactly
- *                max_iter bodies; NaN is invalid
+ *                max_iter bodies; NaN is invalid.  The linear solve of the last
+ *                body is good to 2.5e-3 tol or better, the gates to 2e-7: a tol
+ *                of the size of that rounding may not be reached
  *   iters      : host out, number of executed bodies (may be NULL)
  *   err        : host out, last max |y_new - y|       (may be NULL)
  *   err_trace  : host out [max_iter], err after each body, rest untouched (may be NULL)

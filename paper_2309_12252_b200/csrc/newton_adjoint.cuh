@@ -8,10 +8,10 @@
 //     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands
 //                                            (a pair of blocks of eight columns is one K step of 16).
 // All products are at fp32 level (a one-shot solve): three TF32 MMAs on split operands up to n = 16, from there on hi + lo f16
-// halves in three m16n8k16 ones, half as many and good to 2^-23 of the operands where those are to 2^-20.  Powers of two
-// (operand_scales, and per row and step one from the row's largest |lambda|) keep the halves among the normal
-// numbers; a value beyond f16's range makes a NaN, which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a
-// millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
+// halves in three m16n8k16 ones, half as many and good to 2^-22 of the operands (small ones to 2^-27 of a state, 2^-29 of what x
+// contributes to a gate, 2^-34 of the row's largest |lambda|) where those are to 2^-20.  Powers of two (operand_scales, and per row
+// and step one from the row's largest |lambda|) keep the halves among the normal numbers; a value beyond f16's range makes a NaN,
+// which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
 // the first one.  So a boundary is held to eta of the largest |lambda| of all and, besides, to ADJ_LOCAL eta of the largest
 // |lambda| just before it, over the last ADJ_WINDOW positions of its successor's burn-in (one position alone may be near zero
 // where n is small; more would measure a decayed lambda by what it decayed from).  Where all losses weigh alike the window's

@@ -2,7 +2,7 @@
 // linear solve, new iterate and convergence maximum, with nothing but x, the old iterate and the new one in memory.
 //
 // The update solves d_t = J_t d_{t-1} + r_t, r_t = f(y_{t-1}, x_t) - y_t.  The sequences are cut into chains of L
-// positions; sixteen chains advance in lockstep as the sixteen rows of a warp's m16n8k8 MMAs, a step being
+// positions; sixteen chains advance in lockstep as the sixteen rows of a warp's m16n8k16 MMAs, a step being
 //     [16, m] x [m, 3n] + [16, n] x [n, 3n]      gates: hi + lo f16 halves in three MMAs, so f is good to fp32 level
 //     [16, n] x [n, 3n]                          J_t d_{t-1} = z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d)
 // with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragments of two blocks of eight

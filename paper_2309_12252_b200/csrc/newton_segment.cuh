@@ -7,14 +7,14 @@
 //   phase 1  the cell at every position of the CTA once, 16 positions per warp and MMA tile, nothing in series: residual and
 //            coefficients {z, k_r, a_z, k_n, r} [5N] of a position stay in shared memory;
 //   phase 2  the chains, 16 in lockstep per group of N / 8 warps (one block of eight state columns each), a step being
-//            d <- r + z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d):  9 MMAs of a warp per block of eight columns,
-//            the new d crossing to the other warps of the group through shared memory, as the f16
-//            halves of the next step's operand where products are on those.
-// What bounds it: phases in series.  Cycles of a body, read with clock64 by one warp (n = 8, m = 4, B = 16, T = 1e4: 64 chains of 17
-// positions per CTA): phase 1 10,250 (five tiles a warp), 45 steps of burn-in 7,700 (170 a step), the 17 positions owned 10,800 (640 a
-// step, with its old iterate, residual and store), prologue of phase 2 950, exchange with the other CTAs 4,000 ... 10,000.  n = 4, m = 2,
-// T = 1000 (16 chains of 5): 3,500, 30 steps 5,100, 3,550, 1,200, 3,000.  Issue slots 34 % used; the warps that phase 2 has no chains
-// for wait at the barrier behind it, 5.8 of 16 at a time.
+//            d <- r + z.d + k_r.(W_hr d) + a_z.(W_hz d) + k_n.(W_hn d):  9 MMAs of a warp per K step (of 16 columns of d, of
+//            eight in TF32; 3 where products with d are single), the new d crossing to the other warps of the group
+//            through shared memory, as the f16 halves of the next step's operand where products are on those.
+// What bounds it: phases in series.  Cycles of a body, read with clock64 by one warp where burn-ins were 45 steps (n = 8, m = 4, B = 16,
+// T = 1e4: 64 chains of 17 positions per CTA) and 30 (n = 4, m = 2, T = 1000: 16 chains of 5); they now follow the body, 24 ... 40 and 16
+// ... 30.  n = 8: phase 1 10,250 (five tiles a warp), burn-in 170 a step, the 17 positions owned 10,800 (640 a step, with its old
+// iterate, residual and store), prologue of phase 2 950, exchange with the other CTAs 4,000 ... 10,000.  n = 4: 3,500, 170 a step, 3,550,
+// 1,200, 3,000.  Issue slots 34 % used; the warps that phase 2 has no chains for wait at the barrier behind it, 5.8 of 16 at a time.
 #pragma once
 #include "newton_body.cuh"
 

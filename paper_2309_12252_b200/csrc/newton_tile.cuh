@@ -2,8 +2,9 @@
 // see there) with 128 chains in lockstep as the rows of a tcgen05 tile.
 //
 // Per step of a CTA, [128, .] x [., 3n] products by tcgen05.mma.kind::f16 from one thread, accumulators in tensor memory:
-//     x_t W_i^T and y_{t-1} W_h^T   operands as hi + lo f16 halves, three products (good to 2^-23 of the operands and, of x and y
-//                                   below 2^-6, to 2^-29 absolute: below the 2e-7 that the gates' tanh is good to)
+//     x_t W_i^T and y_{t-1} W_h^T   operands as hi + lo f16 halves, three products (good to 2^-22 of the operands and, of small
+//                                   ones, to 2^-29 of a state and 2^-27 or better of what x contributes to a gate (tile_usual):
+//                                   below the 2e-7 that the gates' tanh is good to)
 //     d_{t-1} W_h^T                 one product (the solve's accuracy is that of its boundaries, see body_verdict)
 // Operands carry powers of two (operand_scales; OP_SCALE, D_SCALE) that keep the hi halves, and the lo halves of all but small
 // operands, among the normal f16 numbers and leave in the exponent arithmetic of the epilogue.  A value beyond f16's range turns the body's error into a NaN: the body

@@ -22,7 +22,8 @@ __device__ __forceinline__ unsigned pack_f16(float2 x)
 
 // d += a * b   (m16n8k16, A row-major 16x16, B 16x8, f16 inputs, fp32 accumulate).  It takes the tensor pipe as long as a TF32 MMA of
 // eight columns (8.04 and 8.05 cycles a sub-partition), so a product in three of these on hi + lo f16 halves is half of one in three
-// TF32 MMAs, and good to 2^-23 of its operands where that one is to 2^-20.
+// TF32 MMAs, and good to 2^-22 of its operands where that one is to 2^-20 -- as far as the lo halves are normal f16 numbers, where
+// TF32 has the range of fp32: operands need scales.
 __device__ __forceinline__ void mma_f16(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1)
 {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
