@@ -16,8 +16,8 @@ using std::min;
 #endif
 
 // StatusBlock::done: the loop ended / this form gives up / a bounded wait ran out, nothing that was computed counts / the tiles
-// take the inputs in units of their own (tile_units_kernel) / a value is beyond f16's range, or not finite at all: the kernels
-// without f16 operands tell, and no burn-in is told
+// take the inputs in units of their own (tile_units_kernel) / a value is beyond f16's range, or not finite at all: what runs
+// without such an operand tells, and no burn-in is told
 constexpr int BODY_DONE = 1, BODY_FALL_BACK = 2, BODY_TIMED_OUT = 3, BODY_UNITS = 4, BODY_BEYOND = 5;
 
 constexpr int BODY_BURN_MIN = 8; // shortest burn-in that is tried

@@ -1095,7 +1095,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
                            bool &u_done, bool to_host, bool &polled, CopyOut copy_out)
 {
     const int n = p->n, m = p->m;
-    const bool need_u = !body_supported(n, m, false);
+    bool need_u = !body_supported(n, m, false);
     const int first = body_first_burn(n, tol);
     int rc, burn = first;
     BodyArgs a{};
@@ -1110,8 +1110,14 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
     a.starts = w.J;                                      // (chains x n floats; nothing else is kept there meanwhile)
     const bool aligned32 = (((uintptr_t)buf[0] | (uintptr_t)buf[1]) & 31) == 0 && (((uintptr_t)y0 | (uintptr_t)p->W_h) & 15) == 0;
     bool tiles = false;
-    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE}) {
+    int tried = -1;                                      // the form launched last (the f16 forms have a second try)
+    for (const BodyForm form : {BodyForm::TWO_PHASE, BodyForm::TWO_PHASE, BodyForm::TILE, BodyForm::TILE, BodyForm::LANE, BodyForm::ONE_PHASE, BodyForm::ONE_PHASE}) {
         BodyPlan plan{};
+        if ((int)form == tried && form != BodyForm::TILE) {
+            // What an operand could not hold was most likely an input: projected inputs go to the accumulators, which have fp32's range.
+            if (hs->done != BODY_BEYOND) continue;
+            need_u = true;
+        }
         if (form == BodyForm::TILE && !aligned32) continue;
         if (form == BodyForm::TILE && tiles) {           // again, with the inputs in units of its own (in the place of u)
             if (hs->done != BODY_UNITS) continue;
@@ -1127,6 +1133,7 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
         // n = 32, 64: the two-phase kernel only where it is the whole loop in one launch
         if (form == BodyForm::TWO_PHASE && (n == 32 || n == 64) && aligned32 && m <= 64 && !plan.whole_loop) continue;
         tiles = form == BodyForm::TILE;
+        tried = (int)form;
         if (burn > plan.burn_cap) { hs->done = BODY_FALL_BACK; continue; }
         a.L = plan.L;
         a.burn_cap = plan.burn_cap;
@@ -1182,8 +1189,8 @@ static int eval_one_launch(const deer_gru_params *p, const float *x, const float
             if (hs->done) break;
         }
         if (hs->done == BODY_DONE) return copy_out(true);
-        if (hs->done == BODY_BEYOND) break;              // (the other forms for this n have no wider range)
-        burn = hs->burn;
+        if (hs->done != BODY_BEYOND) burn = hs->burn;
+        else if (tiles || have_u) break;                 // (no other form has a wider range)
     }
     return DEER_OK;                                      // (hs->done == BODY_FALL_BACK or BODY_BEYOND)
 }

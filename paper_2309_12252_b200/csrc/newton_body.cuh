@@ -8,7 +8,7 @@
 // with the gate arithmetic elementwise on the accumulator fragments.  The accumulator fragments of two blocks of eight
 // columns are the A operand of a K step of 16 as they stand, so neither J_t, nor its coefficients, nor any chain product
 // is ever formed or stored.  Powers of two (operand_scales, MMA_D_SCALE) keep the halves among the normal f16 numbers; a
-// value beyond f16's range makes a NaN, and the body is for the other kernels.
+// value beyond f16's range makes a NaN, and the body is run again with projected inputs, or is for the other kernels.
 //
 // What a chain does not know is the update entering it.  It starts `burn` positions early from zero: the error of its
 // entering update is the old error carried through `burn` Jacobians, and the Jacobians of a cell that forgets make it
