@@ -8,7 +8,7 @@
 //     J_t^T lambda = z.lambda + p W_h        [16, 3n] x [3n, n], p's accumulator layout being the A operand as it stands
 //                                            (a pair of blocks of eight columns is one K step of 16).
 // All products are at fp32 level (a one-shot solve): three TF32 MMAs on split operands up to n = 16, from there on hi + lo f16
-// halves in three m16n8k16 ones, half as many and good to 2^-22 of the operands (small ones to 2^-27 of a state, 2^-29 of what x
+// halves in three m16n8k16 ones, half as many and good to 2^-22 of the operands (small ones to 2^-27 of a state and of what x
 // contributes to a gate, 2^-34 of the row's largest |lambda|) where those are to 2^-20.  Powers of two (operand_scales, and per row
 // and step one from the row's largest |lambda|) keep the halves among the normal numbers; a value beyond f16's range makes a NaN,
 // which fails the check below.  lambda has no scale that holds everywhere: a sequence's loss may weigh a millionth of another's, and behind a loss on the last step only lambda decays through every magnitude, down to dx and dy0 at
@@ -31,6 +31,8 @@ namespace deer {
 constexpr int DY0_REACH = 8;     // a burn-in takes an error down by about 1e-6 or more; behind eight of them it is below any fp32
 constexpr int ADJ_WINDOW = 8;    // positions before a boundary whose largest |lambda| is its scale
 constexpr float ADJ_LOCAL = 4.0f;
+constexpr int ADJ_TOP = 12;      // of a channel's largest weight (operand_scales): contributions up to 16,376, held to 2^-27 absolute.  There is no
+                                 // second try with projected inputs here, as an evaluation has it
 static_assert(ADJ_WINDOW <= ADJ_BURN && (ADJ_BURN - ADJ_WINDOW) % 4 == 0, "the window is whole steps of every kernel's burn-in");
 
 // A boundary's mismatch as a part of its scale, as the bits of a non-negative float (a NaN stays above all numbers).
@@ -122,7 +124,7 @@ __global__ void __launch_bounds__(N > 32 ? 256 : 128, CTAS) newton_adjoint_kerne
     float *sb = reinterpret_cast<float *>(sT + 4 * PB * NS2);
     float wscale = 1.0f, unit = 1.0f, kS = 1.0f;
     if constexpr (F16) {
-        wscale = operand_scales(hd.W_h, hd.W_i, 3 * n, n, proj ? m : 0, MMA_OP_SCALE, MMA_TOP, s_xf, &s_top);
+        wscale = operand_scales(hd.W_h, hd.W_i, 3 * n, n, proj ? m : 0, MMA_OP_SCALE, ADJ_TOP, s_xf, &s_top);
         unit = wscale * MMA_OP_SCALE;
         kS = 1.0f / unit;
     }

@@ -476,7 +476,8 @@ def test_scan_of_unequal_but_coupled_components_is_taken(bd):
 @pytest.mark.parametrize("n,m,B,T,gy_scale,x_scale,kernel", [
     (9, 3, 40, 700, 1.0, 1.0, WARP), (16, 3, 16, 10001, 1.0, 1.0, WARP), (17, 16, 16, 700, 1.0, 1.0, WARP), (24, 33, 16, 700, 1e-25, 1.0, WARP),
     (32, 1, 16, 8001, 1e25, 1.0, WARP), (33, 64, 16, 1000, 1.0, 1.0, WARP), (48, 2, 16, 500, 1.0, 1.0, WARP), (57, 15, 16, 300, 1.0, 1.0, WARP),
-    (63, 8, 16, 300, 1.0, 1.0, WARP), (24, 4, 16, 700, 1.0, 3000.0, WARP), (24, 4, 16, 700, 1.0, 2e4, None), (8, 16, 16, 30001, 1.0, 1.0, WARP)])
+    (63, 8, 16, 300, 1.0, 1.0, WARP), (24, 4, 16, 700, 1.0, 3000.0, WARP), (24, 4, 16, 700, 1.0, 2e4, WARP), (24, 4, 16, 700, 1.0, 4e4, None),
+    (8, 16, 16, 30001, 1.0, 1.0, WARP)])
 def test_adjoint_products_are_at_fp32_level(bd, n, m, B, T, gy_scale, x_scale, kernel):
     """K steps of 16 with and without their second half, gradients of any magnitude, inputs up to and beyond what the products'
     halves hold.  A product is good to 2^-22 of its operands and a lambda carries the errors of some ten steps: 2-norms agree to
